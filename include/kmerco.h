@@ -105,12 +105,12 @@ typedef struct {
                               and windows run across read boundaries (a window spanning the
                               end of one read and the start of the next is counted); 0:
                               windows stay inside reads (default). */
-    uint64_t pass_codes;   /* partitioned design: counter increments staged per pass, 1..2^31;
-                              0: 2^31.  A batch with more increments is inserted in several
+    uint64_t pass_codes;   /* counter increments (nhash per window) one pass stages, 1..2^31;
+                              0: as many as suits.  A call with more is inserted in several
                               passes over consecutive parts of its reads; smaller values bound
-                              the scratch memory (about 7 bytes per staged increment with the
-                              counting apply: a 4-byte region code and a 2-byte slice code,
-                              with headroom; about 10 with the compare-and-swap apply). */
+                              the scratch memory (about 10 bytes per staged increment, and
+                              about 25 per window, twice the key's share of that for two-word
+                              keys). */
     uint32_t retry_limit;  /* bound of the device retry loops: compare-and-swap retries of one
                               counter update (Algorithm 3's read-modify-write) and probes of one
                               distinct-set insert.  0: 2^22 and 2^20.  A loop that reaches it

@@ -13,6 +13,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/kmerco.h"
+#include "kmerco_dedup.cuh"
 #include "kmerco_internal.cuh"
 
 using namespace countbf;
@@ -22,6 +23,12 @@ constexpr int kCopyPieces = 8;   // pieces of a host input copied while earlier 
 // (a few milliseconds at most), so the insert does not wait for the device;
 // larger ones are copied and summed by a kernel, which the call waits for.
 constexpr uint64_t kHostBoundReads = 1ull << 16;
+
+// Windows from which an insert call goes by key ranges: below, its dozen
+// launches cost more than the window-by-window kernel takes.  A handle that
+// holds keys already also collects the call's keys into its distinct set.
+constexpr uint64_t kRangesMin = 1ull << 14;
+constexpr uint64_t kRangesMinMore = 1ull << 17;
 
 // Distinct one-word keys above which classification takes the bucket sort
 // (its histogram readback and host-side merge cost more than a full radix
@@ -41,7 +48,8 @@ struct kmerco {
     bool own_stream;
     int update_mode;         // 0 automatic, 1 atomic, 2 partitioned
     uint64_t pass_codes;     // increments staged per partitioned pass
-    int grid_atomic, grid_part, grid_wide;   // insert grids: atomic, partitioned, wide partitioned
+    bool pass_set;           // pass_codes is the caller's: it also bounds a pass's windows
+    int sms, grid_atomic;    // SMs; grid of the window-by-window insert
     uint64_t budget, used;
     uint64_t max_distinct;   // cap of the distinct list; 0: none
     kmerco_alloc_fn alloc_fn;   // caller's device allocator, or NULL for cudaMalloc
@@ -54,8 +62,13 @@ struct kmerco {
     uint64_t *table;         // distinct-key set: cap slots of kw words
     uint64_t cap;
     uint32_t gen;            // generation tag of the set's current keys
+    bool table_ok;           // the set holds exactly the list's keys (built when it is needed)
+    bool table_dirty;        // the set holds keys under the current tag
+    bool list_sorted;        // the list is in ascending order
     uint64_t *dlist;         // distinct keys in arrival order
     uint64_t dlist_cap;
+    uint64_t *dlist2;        // the list's other place: a union is written there
+    uint64_t dlist2_cap;
     uint64_t d_ub;           // upper bound of the distinct keys held
     uint8_t *in_bases;       // staging of host inputs
     uint64_t in_bases_cap;
@@ -86,7 +99,15 @@ struct kmerco {
     cudaEvent_t copy_ev[kCopyPieces + 1], copy_fork;
     bool insert_timed, classify_timed;
     uint64_t launches;       // kernels launched by this handle
-    uint32_t *coarse;        // partitioned design: increment codes per coarse region
+    uint64_t *range_a, *range_b;   // insertion by key ranges: keys, multiplicities, tables
+    uint64_t range_a_cap, range_b_cap;
+    uint32_t *mult;
+    uint64_t mult_cap;
+    unsigned char *range_meta;
+    uint64_t range_meta_cap;
+    uint32_t *union_scratch;
+    uint64_t union_scratch_cap;
+    uint32_t *coarse;        // partitioned update: increment codes per coarse region
     uint64_t coarse_alloc;
     uint32_t *fine;          // ... and per slice
     uint64_t fine_alloc;
@@ -284,16 +305,30 @@ int device_error_status(unsigned err) {
     return KMERCO_OK;
 }
 
-// The distinct-key set must keep its load factor at or below 1/2 for every
-// key the next launch could add: cap >= 2 * (distinct so far + new windows).
-int ensure_set_capacity(kmerco_t *h, uint64_t add) {
-    uint64_t need = h->d_ub + add;
-    if (need <= h->dlist_cap && 2 * need <= h->cap) {
-        h->d_ub = need;
-        return KMERCO_OK;
+// Makes every key of the distinct set read as a free slot: the next
+// generation tag, or a clear once the tags run out.
+int clean_table(kmerco_t *h) {
+    if (!h->table || !h->table_dirty) return KMERCO_OK;
+    if (h->gen + 1 < tag_count(h)) {
+        ++h->gen;
+    } else {
+        KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, h->stream));
+        h->gen = 0;
     }
-    uint64_t D = 0;   // nothing inserted since create or reset: no keys to read back
-    if (h->d_ub) {
+    h->table_dirty = false;
+    return KMERCO_OK;
+}
+
+// Room in the distinct list for `add` more keys, and with want_table the
+// distinct set over all keys held, at a load factor of 1/2 at most for every
+// key the next launch could add: cap >= 2 * (distinct so far + new windows).
+// The set is built when a call first needs it: an insert by key ranges into an
+// empty handle writes the list alone.
+int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
+    uint64_t need = h->d_ub + add;
+    const bool grow_table = want_table && 2 * need > h->cap;
+    uint64_t D = h->d_ub;   // 0: nothing inserted since create or reset
+    if (D && (need > h->dlist_cap || grow_table)) {
         KM_TRY(read_counters(h));
         D = h->ctr_host->distinct;
     }
@@ -314,23 +349,65 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add) {
         h->dlist = (uint64_t *)q;
         h->dlist_cap = want;
     }
-    if (2 * need > h->cap) {
+    if (want_table && 2 * need > h->cap) {
         uint64_t want = 2 * need;
         if (want < h->cap + h->cap / 2) want = h->cap + h->cap / 2;
         if (want < 1024) want = 1024;
         void *q;
         KM_TRY(dev_alloc(h, &q, want * h->kw * 8));
         KM_CUDA(cudaMemsetAsync(q, 0xFF, want * h->kw * 8, h->stream));
-        KM_CUDA(launch_reinsert(h->dlist, D < h->dlist_cap ? D : h->dlist_cap, h->kw,
-                                (uint64_t *)q, want, set_tag(h), nullptr, 0, h->ctr,
+        KM_CUDA(launch_reinsert(h->dlist, D < h->dlist_cap ? D : h->dlist_cap, nullptr, nullptr,
+                                h->kw, (uint64_t *)q, want, set_tag(h), nullptr, 0, h->ctr,
                                 h->G.probe_limit, h->stream));
         h->launches += D ? 1 : 0;
         KM_CUDA(cudaStreamSynchronize(h->stream));
         dev_free(h, h->table, h->cap * h->kw * 8);
         h->table = (uint64_t *)q;
         h->cap = want;
+        h->table_ok = true;
+    } else if (want_table && !h->table_ok) {
+        KM_TRY(clean_table(h));
+        const uint64_t most = D < h->dlist_cap ? D : h->dlist_cap;
+        KM_CUDA(launch_reinsert(h->dlist, most, nullptr, &h->ctr->distinct, h->kw, h->table, h->cap,
+                                set_tag(h), nullptr, 0, h->ctr, h->G.probe_limit, h->stream));
+        h->launches += most ? 1 : 0;
+        h->table_ok = true;
     }
+    if (want_table) h->table_dirty = true;
     h->d_ub = need;
+    return KMERCO_OK;
+}
+
+// Calls that bring at least this share of the keys already held (bounds of
+// both) are merged into the ordered list: a union takes about 10 ps for every
+// key held or new, the distinct set 36 ps for every new one and the list then
+// has to be sorted.
+constexpr uint64_t kMergeShare = 4;
+
+// Room for the union of the list and at most `add` more keys.
+int ensure_union(kmerco_t *h, uint64_t add) {
+    // a bound of what is held will do while the list is small; for a large one the
+    // call waits to learn its length
+    if (h->d_ub && h->d_ub + add > h->dlist2_cap && (h->d_ub + add) * h->kw > (1ull << 28)) {
+        KM_TRY(read_counters(h));
+        h->d_ub = h->ctr_host->distinct;
+    }
+    KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub + add, (uint64_t)h->kw * 8));
+    return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub, add));
+}
+
+// Merges an ascending list of *nb32 or *nb64 keys, at most nb_most, into the
+// handle's ascending list (after ensure_union).
+int merge_keys(kmerco_t *h, const uint64_t *keys, uint64_t nb_most, const unsigned *nb32,
+               const unsigned long long *nb64) {
+    KM_CUDA(launch_union(h->dlist, h->d_ub, keys, nb_most, nb32, nb64, h->kw, h->dlist2,
+                         h->union_scratch, &h->ctr->distinct, h->stream));
+    h->launches += 4;
+    std::swap(h->dlist, h->dlist2);
+    std::swap(h->dlist_cap, h->dlist2_cap);
+    h->d_ub += nb_most;
+    h->table_ok = false;
+    h->list_sorted = true;
     return KMERCO_OK;
 }
 
@@ -363,12 +440,19 @@ int validate(const kmerco_config_t *c) {
     return KMERCO_OK;
 }
 
-// Whether this handle applies counter increments with the partitioned design.
-bool use_partitioned(const kmerco_t *h) {
+// Whether a call of at most `bound` windows applies its increments with the
+// partitioned update.
+bool use_partitioned(const kmerco_t *h, uint64_t bound) {
     if (h->update_mode == 1) return false;
-    const bool able = h->nhash <= kPartMaxHash && h->G.words <= (1ull << (kMaxCoarseShift + 6));
+    const bool able = h->G.words <= (1ull << (kMaxCoarseShift + 6));
     if (h->update_mode == 2) return able;
-    return able && h->G.words >= (1ull << 17);   // smaller countBFs stay L2-resident
+    // smaller countBFs stay L2-resident.  The partitioned update takes about 10 ps
+    // an increment and 3 to 4.3 ps a cell (it reads and writes them all); a random
+    // update 20 ps while the countBF is about the size of L2 (2^25 cells are
+    // 256 MiB), 33 to 60 ps beyond.  A third to nearly all of the windows are
+    // distinct keys.
+    const uint64_t U = bound * (uint64_t)h->nhash, W = h->G.words;
+    return able && W >= (1ull << 17) && U >= (W <= (1ull << 25) ? W : W / 5);
 }
 
 // Trial division; n is at most about 2^24 here.
@@ -410,55 +494,102 @@ bool use_top_sort(uint64_t D, int kw, int bits) {
 
 // ------------------------------------------------------------ insert plan
 
-// How one insert call applies its counter increments (partitioned design),
-// decided on the host from the call's window bound and input size.
+// How one insert call applies its counter increments (partitioned update),
+// decided on the host from the call's window bound.
 struct PartPlan {
     bool part = false, repart = false, count = false;
-    int coarse_shift = 0, slice_shift = 0;
-    uint64_t coarse_cap = 0, fine_cap = 0, nslices = 0, passes = 1;
+    int coarse_shift = 0, slice_shift = 0, slot_bits = 0, w_bits = 0;
+    uint64_t coarse_cap = 0, fine_cap = 0, nslices = 0;
+    uint64_t keys = 0;   // distinct keys whose increments one pass stages
     uint64_t coarse_words() const { return kCoarseBins * coarse_cap; }   // uint32 codes
-    // slice codes: uint16 counting lanes (two per 32-bit word) or uint32 codes
-    bool lane_codes() const { return repart && count; }
-    uint64_t fine_words() const {
-        return !repart ? 0 : lane_codes() ? (nslices * fine_cap + 1) / 2 : nslices * fine_cap;
-    }
+    uint64_t fine_words() const { return repart ? nslices * fine_cap : 0; }
     uint64_t ctr_words() const { return 2 * kCoarseBins + 2 * nslices; }
 };
 
-struct PartBufs {
+// How one insert call runs: window by window, or by key ranges in `passes`
+// passes over consecutive chunks of its reads.
+struct InsertPlan {
+    bool ranges = false;
+    bool fresh = false;      // the handle holds no keys: the first pass writes the list
+    bool merge = false;      // the list stays in order: the call's keys are merged into it
+    uint64_t passes = 1;
+    uint64_t bound = 0;      // windows of the call at most
+    DedupPlan dd;
+    PartPlan pp;
+    // whether the call needs the distinct set
+    bool table() const { return !(ranges && (fresh || merge) && passes == 1); }
+};
+
+struct InsertBufs {
+    DedupBufs dd;
     uint32_t *coarse, *fine;
     unsigned long long *ctr;
 };
 
-// Increment-code buffers sized for one pass of at most pass_codes
-// increments; larger inputs run in several passes over consecutive chunk
-// ranges.  Counting apply for alpha <= 15 (slices of kCountLanes / eta cells,
-// rounded down to a power of two), compare-and-swap apply otherwise or when
-// the slices would be too many for one coarse region.
-PartPlan plan_partition(const kmerco_t *h, uint64_t bound, uint64_t nbytes) {
+// Increment-code buffers sized for one pass of at most pass_codes increments,
+// and for half of a large call's windows: distinct keys are rarely more than
+// half of them, and a second pass takes what is left.  Counting apply (slices of
+// kCountLanes / eta cells, rounded down to a power of two) for alpha <= 15 and
+// enough increments a cell, compare-and-swap apply otherwise or when the slices
+// would be too many for one coarse region.
+PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
     PartPlan pp;
-    if (!use_partitioned(h) || bound == 0) return pp;
+    if (!use_partitioned(h, bound) || bound == 0) return pp;
     pp.part = true;
-    const uint64_t W = h->G.words, U = bound * (uint64_t)h->nhash;
-    const uint64_t part_chunks = (nbytes + kPartChunk - 1) / kPartChunk;
-    pp.passes = (U + h->pass_codes - 1) / h->pass_codes;
-    if (pp.passes > part_chunks) pp.passes = part_chunks;   // a pass takes one chunk at least
-    if (pp.passes < 1) pp.passes = 1;
-    const uint64_t Up = (U + pp.passes - 1) / pp.passes;   // increments per pass, on average
+    const uint64_t W = h->G.words, nh = (uint64_t)h->nhash;
+    pp.keys = std::min(bound, std::max<uint64_t>(h->pass_codes / nh, 1024));
+    if (bound > (1ull << 24)) pp.keys = std::min(pp.keys, (bound + 1) / 2);
+    const uint64_t U = pp.keys * nh;   // increments per pass
     pp.coarse_shift = ceil_log2(W) - 6;
     if (pp.coarse_shift < 0) pp.coarse_shift = 0;
+    pp.slot_bits = ceil_log2((uint64_t)h->eta);
+    pp.w_bits = std::min(32 - pp.coarse_shift - pp.slot_bits, 16);
     int count_shift = 0;
     while ((2ull << count_shift) * (uint64_t)h->eta <= (uint64_t)kCountLanes) ++count_shift;
-    pp.count = h->alpha <= 15 && pp.coarse_shift - count_shift <= kMaxCoarseShift - kSliceShift;
+    // Counting apply: about 1 ps a counter of the countBF; compare-and-swap
+    // apply: 4.3 ps a cell and 2.3 ps an increment more than counting (measured
+    // on 2^24 to 2^29 cells).  A third of the increments staged stand for
+    // distinct keys.
+    const double per_cell = (double)h->eta - 4.3;
+    pp.count = h->alpha <= 15 && pp.coarse_shift - count_shift <= kMaxCoarseShift - kSliceShift &&
+               (double)(bound * nh) / 3 * 2.3 >= per_cell * (double)W;
     pp.slice_shift = pp.count ? count_shift : kSliceShift;
     pp.repart = pp.coarse_shift > pp.slice_shift;
     if (!pp.repart) pp.slice_shift = pp.coarse_shift;
     pp.nslices = (W + (1ull << pp.slice_shift) - 1) >> pp.slice_shift;
-    pp.coarse_cap = Up / kCoarseBins;
+    pp.coarse_cap = U / kCoarseBins;
     pp.coarse_cap = (pp.coarse_cap + pp.coarse_cap / 6 + 4096 + 3) & ~3ull;   // multiple of 4
-    pp.fine_cap = pp.repart ? Up / pp.nslices : 0;
-    pp.fine_cap = (pp.fine_cap + pp.fine_cap / 5 + 1024 + 7) & ~7ull;   // multiple of 8
+    pp.fine_cap = pp.repart ? U / pp.nslices : 0;
+    pp.fine_cap = (pp.fine_cap + pp.fine_cap / 5 + 1024 + 3) & ~3ull;   // multiple of 4
     return pp;
+}
+
+// By key ranges: calls of enough windows, unless the handle limits retries or
+// its list (those limits are the window-by-window kernel's).
+InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool fresh,
+                       bool may_merge = false) {
+    InsertPlan ip;
+    ip.bound = bound;
+    ip.fresh = fresh;
+    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->max_distinct ||
+        h->G.cas_limit != kCasLimit || nbytes < bound)
+        return ip;
+    uint64_t most = kMaxRangeWindows;   // windows one pass takes
+    if (h->pass_set) most = std::min(most, std::max<uint64_t>(h->pass_codes / (uint64_t)h->nhash, 1));
+    ip.passes = (bound + most - 1) / most;
+    const int chunk = dedup_chunk(nbytes);
+    const uint64_t chunks = (nbytes + chunk - 1) / chunk;
+    for (;; ++ip.passes) {
+        if (ip.passes > chunks) ip.passes = chunks;   // a pass takes one chunk at least
+        const uint64_t pc = (chunks + ip.passes - 1) / ip.passes;   // chunks of a pass at most
+        ip.dd = plan_dedup(h->K, std::min(bound, pc * (uint64_t)chunk), pc, chunk);
+        if (ip.dd.on || pc == 1) break;   // else its chunks may hold more windows than a pass takes
+    }
+    ip.ranges = ip.dd.on;
+    if (ip.ranges) ip.pp = plan_partition(h, ip.dd.bound);
+    ip.merge = ip.ranges && !fresh && may_merge && ip.passes == 1 && h->list_sorted &&
+               bound * kMergeShare >= h->d_ub && h->d_ub + bound < 0xFFFFFFFFull;
+    return ip;
 }
 
 // Insert arguments of one call that do not depend on the plan.
@@ -522,96 +653,172 @@ int issue_host_copy(kmerco_t *h, const uint8_t *src, uint8_t *dst, uint64_t nbyt
     return KMERCO_OK;
 }
 
-// Window starts per work unit of an insert call: the partitioned design's
-// chunk, else kChunk, or kSmallChunk when the call's chunks of kChunk would
-// not give every resident block of the GPU one (small inputs).
-uint64_t insert_chunk(const kmerco_t *h, const PartPlan &pp, uint64_t nbytes) {
-    if (pp.part) return kPartChunk;
+// Window starts per work unit of a window-by-window insert: kChunk, or
+// kSmallChunk when the call's chunks of kChunk would not give every resident
+// block of the GPU one (small inputs).
+uint64_t insert_chunk(const kmerco_t *h, uint64_t nbytes) {
     return (nbytes + kChunk - 1) / kChunk < (uint64_t)h->grid_atomic ? kSmallChunk : kChunk;
 }
 
-// All device work of one insert call on stream s, without host
-// synchronisation (so it can be captured): first reads of the chunks, then
-// per pass the insert kernel and, in the partitioned design, repartition and
-// apply.  h->first_read must hold the call's chunks; pb holds pp's buffers.
-// With hc (a host input being copied), each pass is split into up to
-// kCopyPieces launches, each waiting only for the pieces it reads.
-int launch_sample_insert(const kmerco_t *h, InsertArgs a, const PartPlan &pp,
-                         const PartBufs &pb, cudaStream_t s, uint64_t &launches,
-                         const HostCopy *hc = nullptr) {
-    const uint64_t nbytes = a.last - a.first;
-    const uint64_t chunk = insert_chunk(h, pp, nbytes);
-    const uint64_t nchunks = (nbytes + chunk - 1) / chunk;
-    // chunk ranges of the insert launches: per pass, pieces when copying
-    const uint64_t q = hc && pp.passes <= (uint64_t)kCopyPieces
-                           ? std::max<uint64_t>(1, kCopyPieces / pp.passes) : 1;
-    std::vector<uint64_t> cut;   // launch r takes chunks [cut[r], cut[r + 1])
-    for (uint64_t pass = 0; pass < pp.passes; ++pass) {
-        const uint64_t cb = nchunks * pass / pp.passes, ce = nchunks * (pass + 1) / pp.passes;
-        const uint64_t qq = std::min<uint64_t>(q, std::max<uint64_t>(1, ce - cb));
-        for (uint64_t j = 0; j < qq; ++j) cut.push_back(cb + (ce - cb) * j / qq);
+// Chunks of the insert's first_read table at most.
+uint64_t first_read_entries(const kmerco_t *h, const InsertPlan &ip, uint64_t nbytes) {
+    const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
+    return (nbytes + chunk - 1) / chunk;
+}
+
+// Orders stream s after the copies of the pieces holding input bytes [lo, hi).
+int wait_pieces(const HostCopy *hc, uint64_t lo, uint64_t hi, cudaStream_t s) {
+    for (int i = 0; hc && i < hc->npieces; ++i)
+        if (hc->piece_lo(i) < hi && hc->piece_lo(i + 1) > lo)
+            KM_CUDA(cudaStreamWaitEvent(s, hc->ev[i], 0));
+    return KMERCO_OK;
+}
+
+// The increments of one pass's distinct keys, and with e.dlist the distinct list.
+int launch_updates(const kmerco_t *h, const InsertPlan &ip, const InsertBufs &b, EmitArgs e,
+                   cudaStream_t s, uint64_t &launches) {
+    const PartPlan &pp = ip.pp;
+    if (!pp.part) {
+        KM_CUDA(launch_emit_atomic(e, h->kw, h->sms, s));
+        launches += 1;
+        return KMERCO_OK;
     }
-    cut.push_back(nchunks);
-    const uint64_t nr = cut.size() - 1;
-    KM_CUDA(launch_first_read(a.offsets, a.nreads, a.first, nchunks, chunk, h->first_read, s));
-    launches += nchunks ? 1 : 0;
-    a.part = pp.part ? 1 : 0;
-    a.coarse_shift = pp.coarse_shift;
-    a.coarse = pb.coarse;
-    a.coarse_cap = pp.coarse_cap;
-    a.coarse_cursor = pb.ctr;
-    a.coarse_written = pb.ctr ? pb.ctr + kCoarseBins : nullptr;
-    const int grid = !pp.part ? h->grid_atomic : pp.coarse_shift <= 20 ? h->grid_part
-                                                                       : h->grid_wide;
-    uint64_t r = 0;   // next launch range
-    for (uint64_t pass = 0; pass < pp.passes; ++pass) {
-        const uint64_t pass_end = nchunks * (pass + 1) / pp.passes;
-        if (pp.part) KM_CUDA(cudaMemsetAsync(pb.ctr, 0, pp.ctr_words() * 8, s));
-        for (; r < nr && cut[r + 1] <= pass_end && cut[r] < pass_end; ++r) {
-            if (hc) {   // the pieces holding this range's bytes and the K - 1 after it
-                const uint64_t lo = cut[r] * chunk;
-                const uint64_t hi = std::min(cut[r + 1] * chunk + (uint64_t)a.K - 1, nbytes);
-                for (int i = 0; i < hc->npieces; ++i)
-                    if (hc->piece_lo(i) < hi && hc->piece_lo(i + 1) > lo)
-                        KM_CUDA(cudaStreamWaitEvent(s, hc->ev[i], 0));
-            }
-            a.chunk_begin = cut[r];
-            a.nchunks = cut[r + 1];
-            KM_CUDA(launch_insert(a, grid, (int)chunk, s));
-            launches += a.nchunks > a.chunk_begin ? 1 : 0;
-        }
-        if (!pp.part) continue;
-        unsigned long long *fine_cursor = pb.ctr + 2 * kCoarseBins;
-        unsigned long long *fine_written = fine_cursor + pp.nslices;
+    e.coarse_shift = pp.coarse_shift;
+    e.slot_bits = pp.slot_bits;
+    e.w_bits = pp.w_bits;
+    e.coarse = b.coarse;
+    e.coarse_cap = pp.coarse_cap;
+    e.coarse_cursor = b.ctr;
+    e.coarse_written = b.ctr + kCoarseBins;
+    unsigned long long *fine_cursor = b.ctr + 2 * kCoarseBins;
+    unsigned long long *fine_written = fine_cursor + pp.nslices;
+    for (uint64_t k0 = 0; k0 < ip.dd.bound; k0 += pp.keys) {
+        KM_CUDA(cudaMemsetAsync(b.ctr, 0, pp.ctr_words() * 8, s));
+        e.begin = (unsigned)k0;
+        e.end = (unsigned)std::min(k0 + pp.keys, ip.dd.bound);
+        KM_CUDA(launch_emit(e, h->kw, h->sms, s));
         if (pp.repart) {
             PartArgs p;
             p.G = h->G;
             p.coarse_shift = pp.coarse_shift;
+            p.slot_bits = pp.slot_bits;
+            p.w_bits = pp.w_bits;
             p.slice_shift = pp.slice_shift;
-            p.coarse = pb.coarse;
+            p.coarse = b.coarse;
             p.coarse_cap = pp.coarse_cap;
-            p.coarse_written = a.coarse_written;
-            p.fine = pb.fine;
+            p.coarse_written = e.coarse_written;
+            p.fine = b.fine;
             p.fine_cap = pp.fine_cap;
-            p.lane_codes = pp.lane_codes() ? 1 : 0;
+            p.lane_codes = pp.count ? 1 : 0;
             p.fine_cursor = fine_cursor;
             p.fine_written = fine_written;
             p.ctr = h->ctr;
-            KM_CUDA(launch_repartition(p, s));
+            KM_CUDA(launch_repartition(p, h->sms, s));
             launches += 1;
         }
         ApplyArgs ap;
         ap.G = h->G;
+        ap.slot_bits = pp.slot_bits;
+        ap.w_bits = pp.w_bits;
         ap.slice_shift = pp.slice_shift;
-        ap.codes = pp.repart ? pb.fine : pb.coarse;
+        ap.codes = pp.repart ? b.fine : b.coarse;
         ap.cap = pp.repart ? pp.fine_cap : pp.coarse_cap;
-        ap.lane_codes = pp.lane_codes() ? 1 : 0;
-        ap.written = pp.repart ? fine_written : a.coarse_written;
+        ap.lane_codes = pp.repart && pp.count ? 1 : 0;
+        ap.guard = ip.dd.bound * (uint64_t)h->nhash >= (1ull << 32) ? 1 : 0;
+        ap.written = pp.repart ? fine_written : e.coarse_written;
         ap.ctr = h->ctr;
         KM_CUDA(pp.count ? launch_apply_count(ap, pp.nslices, s) : launch_apply(ap, pp.nslices, s));
+        launches += 2;
+    }
+    return KMERCO_OK;
+}
+
+// Where a call to be merged into the list leaves its ascending keys (the place of
+// the windows' keys, which are done with by then).
+uint64_t *merge_input(const InsertPlan &ip, const InsertBufs &b) {
+    return ip.dd.n_fine ? b.dd.b : b.dd.a;
+}
+
+// All device work of one insert call on stream s, without host
+// synchronisation (so it can be captured): first reads of the chunks, then
+// the plan's kernels.  h->first_read must hold the call's chunks; b holds the
+// plan's buffers.  With hc (a host input being copied) the kernels that read
+// the bases are split into up to kCopyPieces launches, each waiting only for
+// the pieces it reads.
+int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
+                         const InsertBufs &b, cudaStream_t s, uint64_t &launches,
+                         const HostCopy *hc = nullptr) {
+    const uint64_t nbytes = a.last - a.first;
+    const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
+    const uint64_t nchunks = (nbytes + chunk - 1) / chunk;
+    KM_CUDA(launch_first_read(a.offsets, a.nreads, a.first, nchunks, chunk, h->first_read, s));
+    launches += nchunks ? 1 : 0;
+    const uint64_t q = hc && hc->npieces > 1 && ip.passes <= (uint64_t)kCopyPieces
+                           ? std::max<uint64_t>(1, kCopyPieces / ip.passes) : 1;
+    for (uint64_t pass = 0; pass < ip.passes; ++pass) {
+        const uint64_t cb = nchunks * pass / ip.passes, ce = nchunks * (pass + 1) / ip.passes;
+        const uint64_t qq = std::min<uint64_t>(q, std::max<uint64_t>(1, ce - cb));
+        for (uint64_t j = 0; j < qq; ++j) {
+            const uint64_t c0 = cb + (ce - cb) * j / qq, c1 = cb + (ce - cb) * (j + 1) / qq;
+            // the pieces holding this range's bytes and the K - 1 after it
+            KM_TRY(wait_pieces(hc, c0 * chunk, std::min(c1 * chunk + (uint64_t)a.K - 1, nbytes), s));
+            if (!ip.ranges) {
+                a.chunk_begin = c0;
+                a.nchunks = c1;
+                KM_CUDA(launch_insert(a, h->grid_atomic, (int)chunk, s));
+                launches += c1 > c0 ? 1 : 0;
+                continue;
+            }
+            KM_CUDA(dedup_pack(ip.dd, b.dd, a, cb, ce - cb, c0, c1, h->sms, s, launches));
+        }
+        if (!ip.ranges) continue;
+        KM_CUDA(dedup_extract(ip.dd, b.dd, a.canonical, ce - cb,
+                              std::min(ce * chunk, nbytes) - cb * chunk, h->sms, s, launches));
+        const bool fresh = ip.fresh && pass == 0;
+        const bool ordered = fresh || ip.merge;
+        KM_CUDA(dedup_finish(ip.dd, b.dd, h->ctr, ce - cb, ordered, fresh, h->sms, s, launches));
+        EmitArgs e = dedup_result(ip.dd, b.dd, h->G, h->ctr, ordered);
+        e.dlist = fresh ? h->dlist : ip.merge ? merge_input(ip, b) : nullptr;
+        KM_TRY(launch_updates(h, ip, b, e, s, launches));
+        if (!ip.table()) continue;
+        // the pass's keys into the distinct set (the first pass of an empty
+        // handle: its list as it stands)
+        KM_CUDA(launch_reinsert(fresh ? h->dlist : e.keys, ip.dd.bound,
+                                fresh ? &e.meta->distinct : &e.meta->out_cursor, nullptr, h->kw,
+                                h->table, h->cap, set_tag(h), fresh ? nullptr : h->dlist,
+                                h->dlist_cap, h->ctr, h->G.probe_limit, s));
         launches += 1;
     }
     return KMERCO_OK;
+}
+
+// The scratch of a plan from the handle's buffers; false when it cannot be
+// had (what was there is then given back).
+bool handle_scratch(kmerco_t *h, const InsertPlan &ip) {
+    const DedupPlan &d = ip.dd;
+    const PartPlan &pp = ip.pp;
+    if (ensure(h, &h->range_a, &h->range_a_cap, d.keys_a()) == KMERCO_OK &&
+        ensure(h, &h->range_b, &h->range_b_cap, d.keys_b()) == KMERCO_OK &&
+        ensure(h, &h->mult, &h->mult_cap, d.mult_words()) == KMERCO_OK &&
+        ensure(h, &h->range_meta, &h->range_meta_cap, d.meta_bytes()) == KMERCO_OK &&
+        (!pp.part ||
+         (ensure(h, &h->coarse, &h->coarse_alloc, pp.coarse_words()) == KMERCO_OK &&
+          (!pp.repart || ensure(h, &h->fine, &h->fine_alloc, pp.fine_words()) == KMERCO_OK) &&
+          ensure(h, &h->part_ctr, &h->part_ctr_alloc, pp.ctr_words()) == KMERCO_OK)))
+        return true;
+    auto give_back = [h](auto **p, uint64_t *cap) {
+        dev_free(h, *p, *cap * sizeof(**p));
+        *p = nullptr;
+        *cap = 0;
+    };
+    give_back(&h->range_a, &h->range_a_cap);
+    give_back(&h->range_b, &h->range_b_cap);
+    give_back(&h->mult, &h->mult_cap);
+    give_back(&h->range_meta, &h->range_meta_cap);
+    give_back(&h->coarse, &h->coarse_alloc);
+    give_back(&h->fine, &h->fine_alloc);
+    give_back(&h->part_ctr, &h->part_ctr_alloc);
+    return false;
 }
 
 }  // namespace
@@ -662,31 +869,41 @@ int kmerco_estimate_bytes(const kmerco_config_t *cfg, uint64_t nreads, uint64_t 
     t.nhash = cfg->nhash;
     t.update_mode = cfg->update_mode;
     t.pass_codes = cfg->pass_codes ? cfg->pass_codes : kMaxBatchCodes;
+    t.pass_set = cfg->pass_codes != 0;
+    t.max_distinct = cfg->max_distinct;
     t.G = make_geometry((cfg->m + (uint64_t)t.eta - 1) / (uint64_t)t.eta, cfg->dim_x, cfg->dim_y,
                         t.alpha, t.nhash);
+    if (cfg->retry_limit) t.G.cas_limit = t.G.probe_limit = cfg->retry_limit;
     const uint64_t kw = (uint64_t)t.kw;
     // ensure(): need + need / 4 + 64 elements
     auto grown = [](uint64_t need, uint64_t elem) { return (need + need / 4 + 64) * elem; };
     uint64_t b = t.G.words * 8 + kCtrBytes;
     if (host_inputs) b += grown(nbytes, 1) + grown(nreads + 1, 8);
     if (windows) {
-        // distinct list and set for every window being a new key
+        // distinct list, and where the call needs it the set, for every window
+        // being a new key
         uint64_t list = windows;
         if (cfg->max_distinct && list > cfg->max_distinct) list = cfg->max_distinct;
-        b += list * kw * 8 + std::max<uint64_t>(2 * windows, 1024) * kw * 8;
-        const PartPlan pp = plan_partition(&t, windows, nbytes);
-        if (pp.part) {
-            b += grown(pp.coarse_words(), 4) + grown(pp.ctr_words(), 8);
-            if (pp.repart) b += grown(pp.fine_words(), 4);
+        b += list * kw * 8;
+        const InsertPlan ip = plan_insert(&t, windows, nbytes, true);
+        if (ip.table()) b += std::max<uint64_t>(2 * windows, 1024) * kw * 8;
+        if (ip.ranges) {
+            b += grown(ip.dd.keys_a(), 8) + grown(ip.dd.keys_b(), 8) +
+                 grown(ip.dd.mult_words(), 4) + grown(ip.dd.meta_bytes(), 1);
+            if (ip.pp.part) {
+                b += grown(ip.pp.coarse_words(), 4) + grown(ip.pp.ctr_words(), 8);
+                if (ip.pp.repart) b += grown(ip.pp.fine_words(), 4);
+            }
         }
-        const uint64_t chunk = pp.part ? kPartChunk : kSmallChunk;   // the most chunks
+        const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : kSmallChunk;   // the most chunks
         b += grown((nbytes + chunk - 1) / chunk, 4);
         // classification of at most `windows` distinct keys
         const uint64_t D = windows;
-        b += 2 * grown(D * kw, 8) + grown(D, 4) + grown(D * kw, 8) +
-             grown(sort_scratch_words(D, kw), 4) + grown(split_scratch_words(D), 8);
-        if (use_top_sort(D, t.kw, 2 * t.K)) b += grown(3 * seg_bounds_entries(D, t.kw) + 1, 8);
-        if (kw == 1 && 2 * t.K >= kHistBits + 8 && D > kBucketSortMin)   // the bucket sort may run
+        b += grown(D, 4) + grown(D * kw, 8) + grown(split_scratch_words(D), 8);
+        const bool sorts = ip.table();   // else the list is written in order
+        if (sorts) b += 2 * grown(D * kw, 8) + grown(sort_scratch_words(D, kw), 4);
+        if (sorts && use_top_sort(D, t.kw, 2 * t.K)) b += grown(3 * seg_bounds_entries(D, t.kw) + 1, 8);
+        if (sorts && kw == 1 && 2 * t.K >= kHistBits + 8 && D > kBucketSortMin)   // the bucket sort may run
             b += grown(kBucketHostWords + kHistBins, 8) +
                  grown(bucket_hist_blocks(D) * kHistBins, 2);
     }
@@ -754,9 +971,10 @@ int kmerco_create_ex(const kmerco_config_t *cfg, kmerco_t **out) {
         if (sms <= 0) sms = 1;
         h->update_mode = cfg->update_mode;
         h->pass_codes = cfg->pass_codes ? cfg->pass_codes : kMaxBatchCodes;
-        h->grid_atomic = sms * insert_blocks_per_sm(h->kw, 0);
-        h->grid_part = sms * insert_blocks_per_sm(h->kw, 1);
-        h->grid_wide = sms * insert_blocks_per_sm(h->kw, 2);
+        h->pass_set = cfg->pass_codes != 0;
+        h->sms = sms;
+        h->grid_atomic = sms * insert_blocks_per_sm(h->kw);
+        h->table_ok = true;   // no keys, no set yet
 
         const uint64_t eta = (uint64_t)h->eta;
         h->G = make_geometry((cfg->m + eta - 1) / eta, cfg->dim_x, cfg->dim_y, h->alpha,
@@ -807,6 +1025,8 @@ void kmerco_destroy(kmerco_t *h) {
         dev_free(h, h->ctr, kCtrBytes);
         dev_free(h, h->table, h->cap * h->kw * 8);
         dev_free(h, h->dlist, h->dlist_cap * h->kw * 8);
+        dev_free(h, h->dlist2, h->dlist2_cap * h->kw * 8);
+        dev_free(h, h->union_scratch, h->union_scratch_cap * 4);
         dev_free(h, h->in_bases, h->in_bases_cap);
         dev_free(h, h->in_offsets, h->in_offsets_cap * 8);
         dev_free(h, h->first_read, h->first_read_cap * 4);
@@ -818,6 +1038,10 @@ void kmerco_destroy(kmerco_t *h) {
         dev_free(h, h->split_scratch, h->split_scratch_cap * 8);
         dev_free(h, h->q_keys, h->q_cap * 16);
         dev_free(h, h->q_est, h->q_cap * 4);
+        dev_free(h, h->range_a, h->range_a_cap * 8);
+        dev_free(h, h->range_b, h->range_b_cap * 8);
+        dev_free(h, h->mult, h->mult_cap * 4);
+        dev_free(h, h->range_meta, h->range_meta_cap);
         dev_free(h, h->coarse, h->coarse_alloc * 4);
         dev_free(h, h->fine, h->fine_alloc * 4);
         dev_free(h, h->part_ctr, h->part_ctr_alloc * 8);
@@ -845,18 +1069,11 @@ int kmerco_reset(kmerco_t *h) {
     if (!h) return KMERCO_EINVAL;
     DeviceGuard guard(h->device);
     KM_CUDA(cudaMemsetAsync(h->G.cells, 0, h->G.words * 8, h->stream));
-    if (h->table && h->d_ub) {
-        // the next generation tag makes every held key read as a free slot;
-        // once the tags run out the table is cleared and they start again
-        if (h->gen + 1 < tag_count(h)) {
-            ++h->gen;
-        } else {
-            KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, h->stream));
-            h->gen = 0;
-        }
-    }
+    KM_TRY(clean_table(h));
     KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), h->stream));
     h->d_ub = 0;
+    h->table_ok = true;
+    h->list_sorted = false;
     h->classified = false;
     h->n_distinct = h->n_trusted = 0;
     h->insert_timed = h->classify_timed = false;
@@ -930,20 +1147,30 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
         }
     }
     if (bound == 0) return KMERCO_OK;   // no window fits in any read
-    KM_TRY(ensure_set_capacity(h, bound));
-
-    PartPlan pp = plan_partition(h, bound, nbytes);
-    if (pp.part &&
-        (ensure(h, &h->coarse, &h->coarse_alloc, pp.coarse_words()) != KMERCO_OK ||
-         (pp.repart && ensure(h, &h->fine, &h->fine_alloc, pp.fine_words()) != KMERCO_OK) ||
-         ensure(h, &h->part_ctr, &h->part_ctr_alloc, pp.ctr_words()) != KMERCO_OK))
-        pp = PartPlan();   // the atomic design when the buffers cannot be had
-    const uint64_t chunk = insert_chunk(h, pp, nbytes);
-    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, (nbytes + chunk - 1) / chunk));
+    InsertPlan ip = plan_insert(h, bound, nbytes, h->d_ub == 0, true);
+    if (ip.ranges && !handle_scratch(h, ip)) {   // window by window when the buffers cannot be had
+        ip = InsertPlan();
+        ip.bound = bound;
+    }
+    if (ip.merge) {
+        const int st = ensure_union(h, bound);
+        if (st == KMERCO_ENOMEM)
+            ip.merge = false;   // the distinct set then
+        else
+            KM_TRY(st);
+    }
+    if (!ip.merge) KM_TRY(ensure_set_capacity(h, bound, ip.table()));
+    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
+    const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
+                             h->part_ctr};
     KM_CUDA(cudaEventRecord(h->ev[0], h->stream));
-    KM_TRY(launch_sample_insert(h, a, pp, PartBufs{h->coarse, h->fine, h->part_ctr}, h->stream,
-                                h->launches, copying ? &hc : nullptr));
+    KM_TRY(launch_sample_insert(h, a, ip, bufs, h->stream, h->launches, copying ? &hc : nullptr));
+    if (ip.merge)
+        KM_TRY(merge_keys(h, merge_input(ip, bufs), bound,
+                          &dedup_result(ip.dd, bufs.dd, h->G, h->ctr, true).meta->distinct, nullptr));
+    if (!ip.table()) h->table_ok = false;   // the list alone was written
+    h->list_sorted = !ip.table();
     KM_CUDA(cudaEventRecord(h->ev[1], h->stream));
     h->insert_timed = true;
     h->classified = false;
@@ -1005,20 +1232,25 @@ int kmerco_classify(kmerco_t *h) {
     const uint64_t D = h->ctr_host->distinct;
     if (D >= 0xFFFFFFFFull) return KMERCO_ENOMEM;   // sort tiles index keys with 32 bits
     const int kw = h->kw;
-    KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D * kw));
-    KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D * kw));
+    const bool in_order = h->list_sorted;
+    if (!in_order) {
+        KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D * kw));
+        KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D * kw));
+        KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap, sort_scratch_words(D, kw)));
+    }
     KM_TRY(ensure(h, &h->est, &h->est_cap, D));
     KM_TRY(wait_result_copies(h, D * kw));
     KM_TRY(ensure(h, &h->split, &h->split_cap, D * kw));
-    KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap, sort_scratch_words(D, kw)));
     KM_TRY(ensure(h, &h->split_scratch, &h->split_scratch_cap, split_scratch_words(D)));
     KM_CUDA(cudaEventRecord(h->ev[2], h->stream));
-    const uint64_t *const distinct_in = h->dlist;   // arrival order; left unchanged
+    const uint64_t *const distinct_in = h->dlist;   // left unchanged
     const uint64_t *sorted = distinct_in;
     const int bits = 2 * h->K;
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
     // (small sets: the radix sort, without the bucket sort's fixed scratch)
-    if (use_top_sort(D, kw, bits)) {
+    if (in_order) {
+        // an insert by key ranges wrote the list in ascending order
+    } else if (use_top_sort(D, kw, bits)) {
         // three stable passes on the top bits (dlist -> alt0 -> alt1 -> alt0),
         // then the segments in shared memory
         const int s0 = bits - kTopSortBits;
@@ -1231,10 +1463,11 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
         KM_CUDA(cudaMemcpyAsync(h->alt0, keys, words * 8, cudaMemcpyHostToDevice, h->stream));
         d_keys = h->alt0;
     }
-    KM_TRY(ensure_set_capacity(h, n));
-    KM_CUDA(launch_reinsert(d_keys, n, h->kw, h->table, h->cap, set_tag(h), h->dlist,
-                            h->dlist_cap, h->ctr, h->G.probe_limit, h->stream));
+    KM_TRY(ensure_set_capacity(h, n, true));
+    KM_CUDA(launch_reinsert(d_keys, n, nullptr, nullptr, h->kw, h->table, h->cap, set_tag(h),
+                            h->dlist, h->dlist_cap, h->ctr, h->G.probe_limit, h->stream));
     h->launches += 1;
+    h->list_sorted = false;
     KM_TRY(read_counters(h));
     KM_TRY(device_error_status(h->ctr_host->error));
     h->classified = false;
@@ -1430,12 +1663,39 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
     KM_TRY(read_counters(src));
     KM_TRY(device_error_status(src->ctr_host->error));
     const DevCounters sc = *src->ctr_host;
-    KM_TRY(ensure_set_capacity(dst, sc.distinct));
+    // ascending lists: copied into an empty handle, merged into an ordered one
+    const bool ordered = src->list_sorted && sc.distinct && !dst->max_distinct &&
+                         dst->G.probe_limit == kProbeLimit;
+    bool listed = false;
+    if (ordered && dst->d_ub == 0) {
+        KM_TRY(ensure_set_capacity(dst, sc.distinct, false));
+        KM_CUDA(cudaMemcpyAsync(dst->dlist, src->dlist, sc.distinct * dst->kw * 8,
+                                cudaMemcpyDeviceToDevice, dst->stream));
+        KM_CUDA(cudaMemcpyAsync(&dst->ctr->distinct, &src->ctr->distinct, sizeof(src->ctr->distinct),
+                                cudaMemcpyDeviceToDevice, dst->stream));
+        dst->table_ok = false;
+        listed = dst->list_sorted = true;
+    } else if (ordered && dst->list_sorted && sc.distinct * kMergeShare >= dst->d_ub &&
+               dst->d_ub + sc.distinct < 0xFFFFFFFFull) {
+        const int st = ensure_union(dst, sc.distinct);
+        if (st != KMERCO_ENOMEM) {
+            KM_TRY(st);
+            KM_TRY(merge_keys(dst, src->dlist, sc.distinct, nullptr, &src->ctr->distinct));
+            listed = true;
+        }
+    }
+    if (!listed) {
+        KM_TRY(ensure_set_capacity(dst, sc.distinct, true));
+        dst->list_sorted = false;
+    }
     KM_CUDA(launch_merge(dst->G.cells, src->G.cells, dst->G, dst->stream));
-    KM_CUDA(launch_reinsert(src->dlist, sc.distinct, dst->kw, dst->table, dst->cap,
-                            set_tag(dst), dst->dlist, dst->dlist_cap, dst->ctr,
-                            dst->G.probe_limit, dst->stream));
-    dst->launches += sc.distinct ? 2 : 1;
+    dst->launches += 1;
+    if (!listed) {
+        KM_CUDA(launch_reinsert(src->dlist, sc.distinct, nullptr, nullptr, dst->kw, dst->table,
+                                dst->cap, set_tag(dst), dst->dlist, dst->dlist_cap, dst->ctr,
+                                dst->G.probe_limit, dst->stream));
+        dst->launches += sc.distinct ? 1 : 0;
+    }
     KM_TRY(read_counters(dst));
     DevCounters dc = *dst->ctr_host;
     dc.windows += sc.windows;
@@ -1487,9 +1747,9 @@ struct kmerco_batch {
     int streams;
     cudaStream_t aux[kBatchStreams];
     cudaEvent_t fork, join[kBatchStreams];
-    PartBufs bufs[kBatchStreams];            // increment-code scratch of each stream
-    uint64_t buf_words[kBatchStreams][3];    // their sizes (coarse, fine, counters)
-    std::vector<PartPlan> plans;             // per sample
+    InsertBufs bufs[kBatchStreams];          // insert scratch of each stream
+    uint64_t buf_bytes[kBatchStreams][7];    // their sizes
+    std::vector<InsertPlan> plans;           // per sample
     std::vector<uint64_t> load;              // per sample: windows, for stream assignment
     // classification graph, replayed while the distinct counts and buffers match
     bool have_cls;
@@ -1581,32 +1841,44 @@ std::vector<int> batch_assign(const kmerco_batch *b, int S) {
 
 // Scratch of every stream, sized for the largest plan of any sample (so any
 // assignment fits).  Returns false when it cannot be had.
+void batch_scratch(InsertBufs &f, void **ptrs[7]) {
+    ptrs[0] = (void **)&f.dd.a;
+    ptrs[1] = (void **)&f.dd.b;
+    ptrs[2] = (void **)&f.dd.mult;
+    ptrs[3] = (void **)&f.dd.meta;
+    ptrs[4] = (void **)&f.coarse;
+    ptrs[5] = (void **)&f.fine;
+    ptrs[6] = (void **)&f.ctr;
+}
+
 bool batch_alloc_scratch(kmerco_batch *b) {
-    uint64_t need[3] = {0, 0, 0};
-    for (const PartPlan &pp : b->plans) {
-        if (!pp.part) continue;
-        need[0] = std::max(need[0], pp.coarse_words());
-        need[1] = std::max(need[1], pp.fine_words());
-        need[2] = std::max(need[2], pp.ctr_words());
+    uint64_t need[7] = {0, 0, 0, 0, 0, 0, 0};
+    for (const InsertPlan &ip : b->plans) {
+        if (!ip.ranges) continue;
+        const uint64_t n[7] = {ip.dd.keys_a() * 8, ip.dd.keys_b() * 8, ip.dd.mult_words() * 4,
+                               ip.dd.meta_bytes(),
+                               ip.pp.part ? ip.pp.coarse_words() * 4 : 0,
+                               ip.pp.part ? ip.pp.fine_words() * 4 : 0,
+                               ip.pp.part ? ip.pp.ctr_words() * 8 : 0};
+        for (int q = 0; q < 7; ++q) need[q] = std::max(need[q], n[q]);
     }
     for (int k = 0; k < kBatchStreams; ++k) {
         if (!b->aux[k] && cudaStreamCreateWithFlags(&b->aux[k], cudaStreamNonBlocking) != cudaSuccess)
             return false;
         if (!b->join[k] && cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming) != cudaSuccess)
             return false;
-        void **ptrs[3] = {(void **)&b->bufs[k].coarse, (void **)&b->bufs[k].fine,
-                          (void **)&b->bufs[k].ctr};
-        const uint64_t elem[3] = {4, 4, 8};
-        for (int q = 0; q < 3; ++q) {
-            if (b->buf_words[k][q] >= need[q]) continue;
+        void **ptrs[7];
+        batch_scratch(b->bufs[k], ptrs);
+        for (int q = 0; q < 7; ++q) {
+            if (b->buf_bytes[k][q] >= need[q]) continue;
             if (*ptrs[q]) {
                 cudaStreamSynchronize(b->aux[k]);
-                raw_free(b->h[0], *ptrs[q], b->buf_words[k][q] * elem[q]);
+                raw_free(b->h[0], *ptrs[q], b->buf_bytes[k][q]);
             }
             *ptrs[q] = nullptr;
-            b->buf_words[k][q] = 0;
-            if (raw_alloc(b->h[0], ptrs[q], need[q] * elem[q]) != KMERCO_OK) return false;
-            b->buf_words[k][q] = need[q];
+            b->buf_bytes[k][q] = 0;
+            if (raw_alloc(b->h[0], ptrs[q], need[q]) != KMERCO_OK) return false;
+            b->buf_bytes[k][q] = need[q];
         }
     }
     return b->fork || cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
@@ -1623,7 +1895,8 @@ int batch_launch_sliced(kmerco_batch *b, int S, bool reset) {
         cudaStream_t st = b->aux[where[i]];
         if (reset) {
             KM_CUDA(cudaMemsetAsync(h->G.cells, 0, h->G.words * 8, st));
-            if (h->table) KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, st));
+            if (h->table && b->plans[i].table())
+                KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, st));
             KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), st));
         }
         const unsigned long long *bo = &b->bound_host[(size_t)i * kBoundOutWords];
@@ -1647,11 +1920,21 @@ int batch_run(kmerco_batch *b, bool reset) {
     return batch_launch(b, b->chunk, b->bpm);
 }
 
+// State of the handles after a batch insert (a replayed graph inserted too).
 void batch_mark_inserted(kmerco_batch *b) {
-    for (kmerco_t *h : b->h) {
+    for (int i = 0; i < b->n; ++i) {
+        kmerco_t *h = b->h[i];
         h->classified = false;
         h->n_distinct = h->n_trusted = 0;
         h->insert_timed = h->classify_timed = false;
+        h->d_ub = std::max(h->d_ub, b->load[i]);
+        if (b->sched == 1 && !b->plans[i].table()) {   // the list alone was written, in order
+            h->table_ok = false;
+            h->list_sorted = true;
+        } else if (b->load[i]) {
+            h->table_ok = h->table_dirty = true;
+            h->list_sorted = false;
+        }
     }
 }
 
@@ -1725,9 +2008,9 @@ void kmerco_batch_destroy(kmerco_batch_t *b) {
             if (b->ev[i]) cudaEventDestroy(b->ev[i]);
         for (int k = 0; k < kBatchStreams; ++k) {
             if (b->aux[k]) cudaStreamSynchronize(b->aux[k]);
-            raw_free(h0, b->bufs[k].coarse, b->buf_words[k][0] * 4);
-            raw_free(h0, b->bufs[k].fine, b->buf_words[k][1] * 4);
-            raw_free(h0, b->bufs[k].ctr, b->buf_words[k][2] * 8);
+            void **ptrs[7];
+            batch_scratch(b->bufs[k], ptrs);
+            for (int q = 0; q < 7; ++q) raw_free(h0, *ptrs[q], b->buf_bytes[k][q]);
             if (b->aux[k]) cudaStreamDestroy(b->aux[k]);
             if (b->join[k]) cudaEventDestroy(b->join[k]);
         }
@@ -1787,7 +2070,7 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
             return KMERCO_EINVAL;
     }
     // capacities (host work; never inside a capture)
-    b->plans.assign(b->n, PartPlan());
+    b->plans.assign(b->n, InsertPlan());
     b->load.assign(b->n, 0);
     for (int i = 0; i < b->n; ++i) {
         kmerco_t *h = b->h[i];
@@ -1796,10 +2079,11 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
         uint64_t bound = bo[0];
         if (h->whole_file)   // the sample's reads are one sequence
             bound = bo[2] - bo[1] >= (uint64_t)h->K ? bo[2] - bo[1] - h->K + 1 : 0;
-        KM_TRY(ensure_set_capacity(h, bound));
+        b->plans[i] = plan_insert(h, bound, bo[2] - bo[1], h->d_ub == 0);
+        // the set too: the persistent schedule inserts into it
+        KM_TRY(ensure_set_capacity(h, bound, bound != 0));
         const uint64_t most = (bo[2] - bo[1] + kSmallChunk - 1) / kSmallChunk;   // chunks at the smallest chunk size
         KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, most ? most : 1));
-        b->plans[i] = plan_partition(h, bound, bo[2] - bo[1]);
         b->load[i] = bound;
     }
     KM_CUDA(cudaStreamSynchronize(b->stream));
@@ -1922,21 +2206,24 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
         const int kw = h->kw;
         // three radix passes and the segments instead of a full radix sort;
         // the bucket sort is not used here (it reads its histogram back)
-        top[i] = 2 * h->K >= kTopSortBits + 12 && D[i] > kBatchTopSortMin;
+        top[i] = !h->list_sorted && 2 * h->K >= kTopSortBits + 12 && D[i] > kBatchTopSortMin;
         if (top[i]) {
             KM_TRY(ensure(h, &h->seg_scratch, &h->seg_scratch_cap,
                           3 * seg_bounds_entries(D[i], kw) + 1));
             KM_TRY(ensure_bucket_host(h));
         }
-        KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D[i] * kw));
-        KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D[i] * kw));
+        if (!h->list_sorted) {
+            KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D[i] * kw));
+            KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D[i] * kw));
+            KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap,
+                          sort_scratch_words(D[i], kw)));
+        }
         KM_TRY(ensure(h, &h->est, &h->est_cap, D[i]));
         if (h->out_pending) {   // the batch writes the lists on its own streams
             KM_CUDA(cudaStreamSynchronize(h->out_stream));
             h->out_pending = false;
         }
         KM_TRY(ensure(h, &h->split, &h->split_cap, D[i] * kw));
-        KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap, sort_scratch_words(D[i], kw)));
         KM_TRY(ensure(h, &h->split_scratch, &h->split_scratch_cap, split_scratch_words(D[i])));
     }
     bool streams_ok = b->fork != nullptr;
@@ -1950,15 +2237,16 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
     // CUDA graph: replayed while every sample's distinct count and buffers
     // are those it was captured with
     std::vector<uint64_t> key;
-    key.reserve((size_t)b->n * 11);
+    key.reserve((size_t)b->n * 12);
     for (int i = 0; i < b->n; ++i) {
         const kmerco_t *h = b->h[i];
-        const uint64_t fields[11] = {h->classified ? ~0ull : D[i], (uint64_t)h->dlist,
+        const uint64_t fields[12] = {h->classified ? ~0ull : D[i], (uint64_t)h->dlist,
                                      (uint64_t)h->alt0, (uint64_t)h->alt1, (uint64_t)h->est,
                                      (uint64_t)h->split, (uint64_t)h->sort_scratch,
                                      (uint64_t)h->split_scratch, (uint64_t)h->ctr,
-                                     (uint64_t)h->G.cells, (uint64_t)h->seg_scratch};
-        key.insert(key.end(), fields, fields + 11);
+                                     (uint64_t)h->G.cells, (uint64_t)h->seg_scratch,
+                                     h->list_sorted ? 1ull : 0ull};
+        key.insert(key.end(), fields, fields + 12);
     }
     if (b->have_cls && key == b->cls_key) {
         KM_CUDA(cudaGraphLaunch(b->cls_exec, b->stream));
@@ -2013,7 +2301,7 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
                     KM_CUDA(big_segment_sort(h->alt0, h->alt1, D[i], h->kw, bits, big, nbig, st));
                     sorted = h->alt0;
                     n_launch += 12;
-                } else {
+                } else if (!h->list_sorted) {
                     KM_CUDA(radix_sort(h->dlist, h->alt0, h->alt1, D[i], h->kw, bits,
                                        h->sort_scratch, &sorted, st));
                     n_launch += D[i] > 1 ? 3 * (uint64_t)passes : 0;

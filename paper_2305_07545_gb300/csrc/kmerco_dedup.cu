@@ -1,0 +1,1946 @@
+// Insertion by key ranges on sm_103a: the windows of a call are brought
+// together by key before anything is counted, so that the countBF sees each
+// distinct K-mer once, with its multiplicity, instead of every window.
+// Saturating increments commute (Algorithm 3 read per counter), so adding a
+// key's multiplicity to its counters at once gives the countBF of adding one
+// per window.
+//
+//   1. pack_kernel: the bases as 2-bit codes and one bit per base that starts
+//      a window to be counted; nothing reads the caller's buffers after it.
+//   2. sample_kernel, splitters_kernel: keys of random windows, sorted; they
+//      cut the key space into ranges that hold about equally many windows.
+//      extract_kernel: per chunk of window starts, every window's canonical
+//      key (rolled from base to base); the chunk's keys are grouped by range
+//      in shared memory and leave as one contiguous piece, with the piece's
+//      range starts in a table.  No key moves by a global atomic.
+//   3. large calls, a second level: the pieces of one range are gathered tile
+//      by tile (row_prefix_kernel, tile_map_kernel say where a tile begins),
+//      cut again by splitters sampled inside the range, and written as tiles
+//      grouped by the finer ranges (refine_kernel).
+//   4. dedup_kernel: one block per final range gathers its windows, finds the
+//      distinct keys and their multiplicities with a shared-memory hash set,
+//      and sorts them.  The ranges are in key order, so the distinct keys
+//      come out in ascending order with nothing left to sort.
+//   5. scan_counts_kernel, then emit_kernel (codes for the partitioned update)
+//      or emit_atomic_kernel: the increments of the distinct keys, and the
+//      distinct list.
+//
+// A range is cut by splitters taken from the data itself, so skewed
+// compositions only move the splitters; one key held by very many windows
+// makes one large range with few distinct keys, which dedup_kernel streams
+// through the same shared memory.  A range with more distinct keys than fit
+// is handled in several rounds over sub-ranges of it.
+//
+// Two-word keys are cut by their top 64 bits (the prefix); equal prefixes stay
+// in one range and are told apart in dedup_kernel.
+#include "kmerco_dedup.cuh"
+#include "kmerco_stage.cuh"
+
+#include <string.h>
+
+#include <algorithm>
+
+namespace countbf {
+namespace {
+
+template <int KW>
+struct Key {
+    uint64_t lo, hi;   // hi is 0 for one-word keys
+    __device__ __forceinline__ bool operator==(const Key &o) const {
+        return lo == o.lo && (KW == 1 || hi == o.hi);
+    }
+    __device__ __forceinline__ bool operator<(const Key &o) const {
+        if (KW == 1) return lo < o.lo;
+        return hi < o.hi || (hi == o.hi && lo < o.lo);
+    }
+};
+
+template <int KW>
+__device__ __forceinline__ Key<KW> load_key(const uint64_t *p, uint64_t i) {
+    Key<KW> k;
+    if (KW == 1) {
+        k.lo = p[i];
+        k.hi = 0;
+    } else {
+        const ulonglong2 v = ((const ulonglong2 *)p)[i];
+        k.lo = v.x;
+        k.hi = v.y;
+    }
+    return k;
+}
+
+template <int KW>
+__device__ __forceinline__ void store_key(uint64_t *p, uint64_t i, const Key<KW> &k) {
+    if (KW == 1) {
+        p[i] = k.lo;
+    } else {
+        ulonglong2 v;
+        v.x = k.lo;
+        v.y = k.hi;
+        ((ulonglong2 *)p)[i] = v;
+    }
+}
+
+// The top min(2K, 64) bits of a key's 2K bits: what ranges are cut by.
+template <int KW>
+__device__ __forceinline__ uint64_t prefix_of(const Key<KW> &k, int K) {
+    if (KW == 1) return k.lo;
+    const int s = 2 * K - 64;   // 2..64
+    return s == 64 ? k.hi : (k.hi << (64 - s)) | (k.lo >> s);
+}
+
+__device__ __forceinline__ int prefix_bits(int K) { return K < 32 ? 2 * K : 64; }
+
+// Bits of x (0 for 0).
+__device__ __forceinline__ int bit_len(uint64_t x) { return 64 - __clzll((long long)x); }
+
+// The canonical one of a window's two strands (InsertArgs::canonical).
+__device__ __forceinline__ Key<1> canonical_key(const Key<1> &f, const Key<1> &r, int mode) {
+    if (mode == 0) return f;
+    if (mode == 1) return r.lo < f.lo ? r : f;
+    uint64_t hf, hr, t;   // the strand with the smaller H_0
+    murmur8(premix8(f.lo), 0u, hf, t);
+    murmur8(premix8(r.lo), 0u, hr, t);
+    return hf < hr ? f : r;
+}
+__device__ __forceinline__ Key<2> canonical_key(const Key<2> &f, const Key<2> &r, int mode) {
+    if (mode == 0) return f;
+    if (mode == 1) return r < f ? r : f;
+    uint64_t hf, hr, t;
+    murmur16(f.lo, f.hi, 0u, hf, t);
+    murmur16(r.lo, r.hi, 0u, hr, t);
+    return hf < hr ? f : r;
+}
+
+// Index of a prefix among the n ranges of n - 1 sorted splitters: how many of
+// those are at or below it.
+// lut[i] = splitters whose (value - lo) >> sh is below i, with kMany set when
+// more than one falls into cell i: one comparison decides nearly every prefix
+// without a branch.  spl is followed by an all-ones value.
+constexpr unsigned kMany = 0x8000u;
+
+__device__ __forceinline__ unsigned find_range(const uint64_t *spl, const uint16_t *lut, unsigned n,
+                                               uint64_t lo, int sh, uint64_t x) {
+    const unsigned e = lut[(unsigned)((x - lo) >> sh)];
+    unsigned a = e & (kMany - 1);
+    a += spl[a] <= x ? 1u : 0u;
+    if (e & kMany)
+        while (spl[a] <= x && spl[a] != ~0ull) ++a;
+    return min(a, n - 1);   // an all-ones prefix passes the end
+}
+
+// Ascending bitonic sort of 1024 * E values, E consecutive ones to a thread in
+// v (1,024 threads); xch: 1024 * E words of shared memory.  Strides inside a
+// thread are register swaps, inside a warp shuffles; only the 15 steps of
+// larger strides go through shared memory (105 of a plain network of 16,384
+// values: 155 -> 20 us for one block).
+template <int E>
+__device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
+    constexpr unsigned P = 1024 * E;
+    const unsigned tid = threadIdx.x, i0 = tid * E;
+    for (unsigned k = 2; k <= P; k <<= 1) {
+        for (unsigned j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32 * E) {   // the partner is in another warp
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; ++e) xch[e * 1024 + tid] = v[e];
+                __syncthreads();
+                const unsigned other = tid ^ (j / E);
+                const bool lower = (i0 & j) == 0, up = (i0 & k) == 0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const uint64_t o = xch[e * 1024 + other];
+                    v[e] = (lower == up) == (o < v[e]) ? o : v[e];
+                }
+            } else if (j >= E) {   // in another lane
+                const bool lower = (i0 & j) == 0, up = (i0 & k) == 0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const uint64_t o = __shfl_xor_sync(0xffffffffu, v[e], j / E);
+                    v[e] = (lower == up) == (o < v[e]) ? o : v[e];
+                }
+            } else {   // in this thread
+#pragma unroll
+                for (int b = E / 2; b > 0; b >>= 1) {
+                    if (b != (int)j) continue;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        if (e & b) continue;
+                        const bool up = ((i0 + e) & k) == 0;
+                        const uint64_t x = v[e], y = v[e | b];
+                        const bool swap = (x > y) == up;
+                        v[e] = swap ? y : x;
+                        v[e | b] = swap ? x : y;
+                    }
+                }
+            }
+        }
+    }
+}
+
+// n - 1 splitters at even ranks of the `valid` smallest of the sorted samples
+// s, and their lookup table, written to global memory; s (32 KiB at least) is
+// overwritten.  lo, last: the least and the largest prefix of the range that
+// they cut.  1,024 threads, n <= kMaxRanges.
+__device__ __forceinline__ void write_splitters(uint64_t *s, unsigned valid, unsigned n,
+                                                uint64_t lo, uint64_t last, uint64_t *spl,
+                                                uint16_t *lut) {
+    static_assert(kMaxRanges <= 1024, "a splitter a thread");
+    constexpr unsigned E = (1u << kLutBits) / 1024;
+    const unsigned j = threadIdx.x;
+    int sh = bit_len(last - lo) - kLutBits;
+    if (sh < 0) sh = 0;
+    uint64_t v = ~0ull;   // the last of the n: what find_range stops at
+    if (valid && j + 1 < n) v = s[(uint64_t)(j + 1) * valid / n];
+    if (j < n) spl[j] = v;
+    __syncthreads();
+    unsigned *cells = (unsigned *)s;   // splitters in every cell of the table
+    for (unsigned i = j; i < (1u << kLutBits); i += 1024) cells[i] = 0;
+    __syncthreads();
+    if (j + 1 < n && valid) {
+        const uint64_t c = (v - lo) >> sh;
+        if (c < (1u << kLutBits)) atomicAdd(cells + c, 1u);
+    }
+    __syncthreads();
+    unsigned c[E], sum = 0;
+#pragma unroll
+    for (unsigned q = 0; q < E; ++q) sum += c[q] = cells[j * E + q];
+    unsigned tot;
+    unsigned pre = block_exclusive_scan<unsigned, 1024>(sum, tot);
+#pragma unroll
+    for (unsigned q = 0; q < E; ++q) {
+        lut[j * E + q] = (uint16_t)(pre | (c[q] > 1 ? kMany : 0u));
+        pre += c[q];
+    }
+}
+
+__device__ __forceinline__ uint64_t mix64(uint64_t x) { return fmix64(x + 0x9E3779B97F4A7C15ull); }
+
+// ---------------------------------------------------------------- 1. pack
+// A pass's bases from its first chunk on as 2-bit codes (InsertArgs' window
+// starts are positions in it), and per window start a bit when the window
+// lies in one read and its K bases are valid.  Bound by the memory it streams:
+// a byte read and 3/8 byte written per base.
+template <int CHUNK>
+__global__ void __launch_bounds__(CHUNK / 16) pack_kernel(InsertArgs a, PackArgs x) {
+    constexpr int NT = CHUNK / 16, kPack32 = ChunkDims<CHUNK>::kPack32;
+    __shared__ StageSmem<CHUNK> S;
+    const int tid = threadIdx.x, K = a.K;
+    unsigned long long my_windows = 0, my_skipped = 0;
+    const unsigned p = (unsigned)tid * 16;
+    const uint64_t *inv64 = (const uint64_t *)S.inv, *brk64 = (const uint64_t *)S.brk;
+    // bit i of an OR over `len` bits from i on, for i < 16, by doubling
+    const auto any_of = [](uint64_t lo, uint64_t hi, int len) {
+        int have = 1;
+        while (have < len) {
+            const int s = min(have, len - have);   // 1..32
+            lo |= (lo >> s) | (hi << (64 - s));
+            hi |= hi >> s;
+            have += s;
+        }
+        return (unsigned)lo & 0xffffu;
+    };
+    for (int i = tid; i < kPack32 / 2; i += NT) S.brk[i] = 0;
+    __syncthreads();
+    for (uint64_t chunk = x.chunk_begin + blockIdx.x; chunk < x.chunk_end; chunk += gridDim.x) {
+        const uint64_t row = chunk - x.chunk0;
+        const unsigned nb = stage_chunk<CHUNK, NT>(a, chunk, S);
+        __syncthreads();
+        unsigned no_window =
+            K > 1 ? any_of(bits_at(brk64, p + 1), bits_at(brk64, p + 65), K - 1) : 0u;
+        if (p + 16 + (unsigned)K > nb + 1) {   // the span ends inside these windows
+            const int left = (int)nb - K - (int)p + 1;   // of the 16, how many fit
+            no_window |= left > 0 ? 0xffffu << left : 0xffffu;
+        }
+        no_window &= 0xffffu;
+        const unsigned bad = any_of(bits_at(inv64, p), bits_at(inv64, p + 64), K) | no_window;
+        x.valid[row * NT + tid] = (uint16_t)~bad;
+        // the codes of the chunk, and of the K - 1 bases and more after the last one
+        const unsigned words = chunk + 1 == x.chunk_last ? kPack32 : NT;
+        for (unsigned t = tid; t < words; t += NT) x.codes[row * NT + t] = S.pk[t];
+        my_windows += 16 - __popc(no_window);
+        my_skipped += __popc(bad & ~no_window);
+        __syncthreads();
+        for (int i = tid; i < kPack32 / 2; i += NT) S.brk[i] = 0;
+        __syncthreads();
+    }
+    // one addition per block: same-address atomics of every warp and chunk
+    // took six times as long as the rest of the kernel
+    unsigned long long w, k;
+    block_exclusive_scan<unsigned long long, NT>(my_windows, w);
+    block_exclusive_scan<unsigned long long, NT>(my_skipped, k);
+    if (tid == 0 && w) {
+        atomicAdd(&a.ctr->windows, w);
+        atomicAdd(&a.ctr->skipped, k);
+        atomicAdd(&a.ctr->inserted, w - k);
+    }
+}
+
+// The forward key of the window at position p of the packed codes (two codes
+// words to a 64-bit word, first base most significant).
+__device__ __forceinline__ void window_at(const uint64_t *codes, uint64_t p, int K, Key<1> &f) {
+    const uint64_t w = p >> 5;
+    const unsigned s = (unsigned)(p & 31) * 2;
+    const uint64_t x0 = codes[w], x1 = codes[w + 1];
+    f.lo = (s ? (x0 << s) | (x1 >> (64 - s)) : x0) >> (64 - 2 * K);
+    f.hi = 0;
+}
+__device__ __forceinline__ void window_at(const uint64_t *codes, uint64_t p, int K, Key<2> &f) {
+    const uint64_t w = p >> 5;
+    const unsigned s = (unsigned)(p & 31) * 2;
+    const uint64_t x0 = codes[w], x1 = codes[w + 1], x2 = codes[w + 2];
+    const uint64_t t0 = s ? (x0 << s) | (x1 >> (64 - s)) : x0;
+    const uint64_t t1 = s ? (x1 << s) | (x2 >> (64 - s)) : x1;
+    const int d = 128 - 2 * K;   // 0..62
+    f.lo = d ? (t1 >> d) | (t0 << (64 - d)) : t1;
+    f.hi = t0 >> d;
+}
+__device__ __forceinline__ Key<1> revcomp(const Key<1> &f, int K) {
+    Key<1> r;
+    r.lo = revcomp64(f.lo, K);
+    r.hi = 0;
+    return r;
+}
+__device__ __forceinline__ Key<2> revcomp(const Key<2> &f, int K) {
+    Key<2> r;
+    revcomp128(f.hi, f.lo, K, r.hi, r.lo);
+    return r;
+}
+
+// ----------------------------------------------------------- 2. splitters
+// One sample per thread: the prefix of the key at a random valid window start
+// (a few tries), else all ones, which sorts last.
+template <int KW>
+__global__ void __launch_bounds__(128) sample_kernel(PackArgs x, int K, int canonical,
+                                                     uint64_t span, unsigned n, uint64_t *out,
+                                                     DedupMeta *meta) {
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool found = false;
+    uint64_t prefix = ~0ull;
+    for (unsigned t = 0; i < n && t < 4 && !found; ++t) {
+        // window starts spread evenly over the pass, jittered
+        const uint64_t slot = (uint64_t)i * span / n, wide = max(span / n, (uint64_t)1);
+        uint64_t p = slot + mix64((uint64_t)i * 4 + t) % wide;
+        if (t >= 2) p = mix64(~((uint64_t)i * 4 + t)) % span;
+        if (!((x.valid[p >> 4] >> (p & 15)) & 1u)) continue;
+        Key<KW> f;
+        window_at((const uint64_t *)x.codes, p, K, f);
+        prefix = prefix_of<KW>(canonical_key(f, revcomp(f, K), canonical), K);
+        found = true;
+    }
+    if (i < n) out[i] = prefix;
+    const unsigned bal = __ballot_sync(0xffffffffu, found);
+    if ((threadIdx.x & 31) == 0 && bal) atomicAdd(&meta->sampled, (unsigned)__popc(bal));
+}
+
+// The block's values sorted into s (1024 * E words of shared memory).
+template <int E>
+__device__ __forceinline__ void sort_into(uint64_t (&v)[E], uint64_t *s) {
+    block_sort<E>(v, s);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) s[threadIdx.x * E + e] = v[e];
+    __syncthreads();
+}
+
+// Sorts the n samples (at most 1024 * E) and takes the splitters of n_ranges
+// ranges.  One block.
+template <int E>
+__global__ void __launch_bounds__(1024) splitters_kernel(const uint64_t *samples, unsigned n,
+                                                         unsigned n_ranges, uint64_t last,
+                                                         uint64_t *spl, uint16_t *lut,
+                                                         const DedupMeta *meta) {
+    extern __shared__ uint64_t s[];
+    uint64_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const unsigned i = e * 1024 + threadIdx.x;
+        v[e] = i < n ? samples[i] : ~0ull;
+    }
+    sort_into<E>(v, s);
+    write_splitters(s, meta->sampled, n_ranges, 0, last, spl, lut);
+}
+
+// ------------------------------------------------- grouping keys by range
+// Shared memory of a block that groups up to TILE keys by up to kMaxRanges
+// ranges.
+template <int KW, int TILE>
+struct __align__(16) GroupSmem {
+    uint64_t keys[TILE * KW];
+    uint64_t spl[kMaxRanges];
+    uint16_t lut[1 << kLutBits];
+    unsigned hist[kMaxRanges + 128];   // zero from the ranges on
+    unsigned start[kMaxRanges + 4];
+    unsigned base;
+};
+
+constexpr unsigned kNoKey = ~0u;
+
+// Exclusive prefix of S.hist[0, n) into S.start (start[n] = the sum), n up to
+// kMaxRanges, by the first warp: a scan by all warps took a tenth of the
+// kernels' instructions.
+template <int KW, int TILE>
+__device__ __forceinline__ void scan_ranges(GroupSmem<KW, TILE> &S, unsigned n) {
+    if (threadIdx.x >= 32) return;
+    const unsigned lane = threadIdx.x, per = (n + 127) / 128 * 4;   // a lane's, four at a time
+    unsigned sum = 0;
+    for (unsigned j = 0; j < per; j += 4) {
+        const uint4 v = *(const uint4 *)(S.hist + lane * per + j);   // zero past n
+        sum += v.x + v.y + v.z + v.w;
+    }
+    unsigned pre = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= (unsigned)o) pre += y;
+    }
+    if (lane == 31) S.start[n] = pre;
+    pre -= sum;
+    for (unsigned j = 0; j < per; j += 4) {
+        const unsigned i = lane * per + j;
+        const uint4 v = *(const uint4 *)(S.hist + i);
+        uint4 o;
+        o.x = pre;
+        o.y = o.x + v.x;
+        o.z = o.y + v.y;
+        o.w = o.z + v.z;
+        pre = o.w + v.w;
+        if (i + 4 <= n) {
+            *(uint4 *)(S.start + i) = o;
+        } else {
+            if (i < n) S.start[i] = o.x;
+            if (i + 1 < n) S.start[i + 1] = o.y;
+            if (i + 2 < n) S.start[i + 2] = o.z;
+        }
+    }
+}
+
+// Copies the first n keys of S.keys to out (16-byte aligned) as a whole.
+template <int KW, int TILE, int NT>
+__device__ __forceinline__ void copy_out(const GroupSmem<KW, TILE> &S, unsigned n, uint64_t *out) {
+    const uint4 *src = (const uint4 *)S.keys;
+    uint4 *dst = (uint4 *)out;
+    const unsigned nv = KW == 1 ? (n + 1) / 2 : n;   // an odd last key takes its padding along
+    for (unsigned i = threadIdx.x; i < nv; i += NT) __stcs(dst + i, src[i]);
+}
+
+// ---------------------------------------------------------------- extract
+// Bound by instruction issue and shared-memory traffic (about 45 instructions
+// a window); it writes one key a window.  Eight consecutive windows a thread:
+// the first key is cut from the packed codes, the others are rolled on by one
+// base.
+template <int KW, int CHUNK, int CANON>
+__global__ void __launch_bounds__(CHUNK / 8, CHUNK >= 4096 ? 2 : 6)
+    extract_kernel(int K, ExtractArgs x) {
+    constexpr int NT = CHUNK / 8;
+    constexpr int PER = 8;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    GroupSmem<KW, CHUNK> &S = *reinterpret_cast<GroupSmem<KW, CHUNK> *>(dyn);
+    const int tid = threadIdx.x;
+    const unsigned nr = x.n_ranges;
+    for (unsigned i = tid; i < nr; i += NT) S.spl[i] = x.spl[i];
+    for (unsigned i = tid; i < kLutStride / 8; i += NT) ((uint4 *)S.lut)[i] = ((const uint4 *)x.lut)[i];
+    const int bits = prefix_bits(K);
+    const int sh = bits > kLutBits ? bits - kLutBits : 0;
+    const uint64_t mask1 = K >= 32 ? ~0ull : (1ull << (2 * K)) - 1;
+    const uint64_t mask_hi = KW == 1 || K >= 64 ? ~0ull : (1ull << (2 * K - 64)) - 1;
+    const uint64_t *codes = (const uint64_t *)x.codes;
+    for (unsigned row = blockIdx.x; row < x.n_chunks; row += gridDim.x) {
+        for (unsigned i = tid; i < nr + 128; i += NT) S.hist[i] = 0;
+        const uint64_t p = (uint64_t)row * CHUNK + (unsigned)tid * PER;
+        const unsigned valid = ((const uint8_t *)x.valid)[p >> 3];
+        Key<KW> f;
+        window_at(codes, p, K, f);
+        Key<KW> r = revcomp(f, K);
+        uint64_t next;   // the bases after the first window, the nearest in the top bits
+        {
+            const uint64_t q = p + (unsigned)K, w = q >> 5;
+            const unsigned s = (unsigned)(q & 31) * 2;
+            next = s ? (codes[w] << s) | (codes[w + 1] >> (64 - s)) : codes[w];
+        }
+        __syncthreads();
+        Key<KW> key[PER];
+        unsigned br[PER];   // range and rank within it
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            key[i] = canonical_key(f, r, CANON);
+            br[i] = kNoKey;
+            if ((valid >> i) & 1u) {
+                const unsigned bin = find_range(S.spl, S.lut, nr, 0, sh, prefix_of<KW>(key[i], K));
+                br[i] = (bin << 16) | atomicAdd(&S.hist[bin], 1u);
+            }
+            const uint64_t c = next >> 62;
+            next <<= 2;
+            if (KW == 1) {
+                f.lo = ((f.lo << 2) | c) & mask1;
+                r.lo = (r.lo >> 2) | ((3 - c) << (2 * K - 2));
+            } else {
+                f.hi = ((f.hi << 2) | (f.lo >> 62)) & mask_hi;
+                f.lo = (f.lo << 2) | c;
+                r.lo = (r.lo >> 2) | (r.hi << 62);
+                r.hi = (r.hi >> 2) | ((3 - c) << (2 * K - 66));
+            }
+        }
+        __syncthreads();
+        scan_ranges(S, nr);
+        __syncthreads();
+        const unsigned n = S.start[nr];
+        if (tid == 0) {
+            // pieces begin at even keys: 16-byte aligned
+            S.base = atomicAdd(&x.meta->cursor, (n + 1) & ~1u);
+            x.piece[row] = S.base;
+        }
+        for (unsigned i = tid; i <= nr; i += NT)
+            x.starts[(uint64_t)i * x.n_chunks + row] = (uint16_t)S.start[i];
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (br[i] != kNoKey)
+                store_key<KW>(S.keys, S.start[br[i] >> 16] + (br[i] & 0xffffu), key[i]);
+        __syncthreads();
+        copy_out<KW, CHUNK, NT>(S, n, x.out + (uint64_t)S.base * KW);
+        // S.keys is written again after the next chunk's barriers
+    }
+}
+
+// ---------------------------------------------------------- runs of keys
+// Brings runs of keys together in shared memory.  Run r (r < n) begins at key
+// src[r] of `from` and its keys come to positions pos[r], pos[r + 1] - 1 less
+// p0 of dst; only positions in [p0, p1) are copied.  Four to sixteen lanes a run,
+// so a warp reads several runs of a sector or two at once; the copies are
+// asynchronous (cp.async), so that each thread has many in flight.  ref: where
+// not null, receives every copied key's place in `from`.
+template <int KW>
+__device__ __forceinline__ void copy_key_async(uint64_t *dst, const uint64_t *src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (KW == 1)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void copies_done() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+template <int KW, int NT>
+__device__ __forceinline__ void gather_runs(const uint64_t *from, const unsigned *src,
+                                            const unsigned *pos, unsigned n, unsigned p0,
+                                            unsigned p1, uint64_t *dst, unsigned *ref = nullptr) {
+    // as many lanes as nearly every run fills
+    const unsigned ls = (p1 - p0) < 8 * n ? 2 : (p1 - p0) < 24 * n ? 3 : 4, step = 1u << ls;
+    const unsigned sub = threadIdx.x & (step - 1);
+    for (unsigned r = threadIdx.x >> ls; r < n; r += NT >> ls) {
+        const unsigned b = pos[r], lo = max(b, p0), hi = min(pos[r + 1], p1);
+        const uint64_t s0 = src[r];
+        for (unsigned q = lo + sub; q < hi; q += step) {
+            copy_key_async<KW>(dst + (uint64_t)(q - p0) * KW, from + (s0 + (q - b)) * KW);
+            if (ref) ref[q - p0] = (unsigned)(s0 + (q - b));
+        }
+    }
+}
+
+// ------------------------------------------------------ 3. second level
+// Row b of the range starts: prefix[b][c] = keys of range b in pieces before
+// piece c; totals[b] = all of them.
+__global__ void __launch_bounds__(1024) row_prefix_kernel(const uint16_t *starts, unsigned n_chunks,
+                                                          uint32_t *prefix, uint32_t *totals) {
+    const uint16_t *r0 = starts + (uint64_t)blockIdx.x * n_chunks, *r1 = r0 + n_chunks;
+    uint32_t *out = prefix + (uint64_t)blockIdx.x * n_chunks;
+    unsigned carry = 0;
+    for (unsigned c0 = 0; c0 < n_chunks; c0 += 4096) {
+        unsigned v[4], sum = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned c = c0 + threadIdx.x * 4 + j;
+            v[j] = c < n_chunks ? (unsigned)r1[c] - r0[c] : 0u;
+            sum += v[j];
+        }
+        unsigned tot;
+        unsigned pre = block_exclusive_scan<unsigned, 1024>(sum, tot) + carry;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned c = c0 + threadIdx.x * 4 + j;
+            if (c < n_chunks) out[c] = pre;
+            pre += v[j];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
+}
+
+// Tile t covers kRefineTile consecutive keys of one range; its range, its
+// place among the range's tiles and the piece that its first key is in.
+__global__ void __launch_bounds__(1024) tile_map_kernel(const uint32_t *totals, unsigned n_ranges,
+                                                        const uint32_t *prefix, unsigned n_chunks,
+                                                        uint32_t *tile_base, TileMap *map,
+                                                        DedupMeta *meta) {
+    __shared__ unsigned base[kMaxRanges + 1];
+    const unsigned tid = threadIdx.x;
+    const unsigned v = tid < n_ranges ? (totals[tid] + kRefineTile - 1) / kRefineTile : 0u;
+    unsigned tot;
+    const unsigned pre = block_exclusive_scan<unsigned, 1024>(v, tot);
+    if (tid < n_ranges) base[tid] = pre;
+    if (tid == 0) base[n_ranges] = tot;
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        for (unsigned i = tid; i <= n_ranges; i += 1024) tile_base[i] = base[i];
+        if (tid == 0) meta->n_tiles = tot;
+    }
+    const unsigned t = blockIdx.x * 1024 + tid;
+    if (t >= tot) return;
+    unsigned lo = 0, hi = n_ranges - 1;   // the last range whose tiles begin at or before t
+    while (lo < hi) {
+        const unsigned m = (lo + hi + 1) / 2;
+        if (base[m] <= t)
+            lo = m;
+        else
+            hi = m - 1;
+    }
+    const uint32_t *row = prefix + (uint64_t)lo * n_chunks;
+    const unsigned p = (t - base[lo]) * kRefineTile;
+    unsigned a = 0, b = n_chunks - 1;   // the last piece with prefix <= p holds key p
+    while (a < b) {
+        const unsigned m = a + (b - a + 1) / 2;
+        if (row[m] <= p)
+            a = m;
+        else
+            b = m - 1;
+    }
+    map[t].range = lo;
+    map[t].piece = a;
+}
+
+// Splitters of the fine ranges inside range b: keys of random places of
+// random pieces' runs.  One block per range.
+template <int KW, int E>
+__global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int K, unsigned n,
+                                                              uint64_t last) {
+    extern __shared__ uint64_t s[];
+    __shared__ unsigned valid;
+    const unsigned b = blockIdx.x;
+    if (threadIdx.x == 0) valid = 0;
+    __syncthreads();
+    const uint64_t lo = b ? x.spl[b - 1] : 0;
+    const uint64_t hi = b + 1 < x.n_ranges ? x.spl[b] : last;
+    uint64_t v[E];
+    unsigned found = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const unsigned i = e * 1024 + threadIdx.x;
+        v[e] = ~0ull;
+        for (unsigned t = 0; i < n && t < 4; ++t) {
+            const uint64_t z = mix64(((uint64_t)b << 32) | (i * 4 + t));
+            const unsigned c = (unsigned)__umul64hi(z, (uint64_t)x.n_chunks);
+            const unsigned s0 = x.starts[(uint64_t)b * x.n_chunks + c];
+            const unsigned m = x.starts[(uint64_t)(b + 1) * x.n_chunks + c] - s0;
+            if (!m) continue;
+            const unsigned o = (unsigned)(((z & 0xffffffffu) * m) >> 32);
+            v[e] = prefix_of<KW>(load_key<KW>(x.in, (uint64_t)x.piece[c] + s0 + o), K);
+            ++found;
+            break;
+        }
+    }
+    if (found) atomicAdd(&valid, found);
+    sort_into<E>(v, s);
+    // as many ranges as this one's windows fill, so that only the fine samples
+    // spread the sizes; the others stay empty (all-ones splitters)
+    const unsigned nf = max(1u, min(x.n_fine, (x.totals[b] + x.target - 1) / x.target));
+    write_splitters(s, valid, nf, lo, hi, x.fine_spl + (uint64_t)b * kMaxRanges,
+                    x.fine_lut + (uint64_t)b * kLutStride);
+    for (unsigned i = nf + threadIdx.x; i < x.n_fine; i += 1024)
+        x.fine_spl[(uint64_t)b * kMaxRanges + i] = ~0ull;
+}
+
+// One tile of a range: gather its keys from the pieces, group them by fine
+// range in shared memory, write them as one contiguous tile with the fine
+// ranges' starts in a table.
+template <int KW>
+struct __align__(16) RefineSmem {
+    GroupSmem<KW, kRefineTile> g;
+    unsigned src[kRefineThreads];
+    unsigned pos[kRefineThreads + 1];
+};
+
+template <int KW>
+__global__ void __launch_bounds__(kRefineThreads, 2) refine_kernel(RefineArgs x, int K,
+                                                                   uint64_t last) {
+    constexpr int NT = kRefineThreads;
+    constexpr int PER = kRefineTile / NT;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    RefineSmem<KW> &S = *reinterpret_cast<RefineSmem<KW> *>(dyn);
+    __shared__ unsigned more;
+    const unsigned tid = threadIdx.x, nf = x.n_fine;
+    const unsigned nt = x.meta->n_tiles;
+    // consecutive tiles per block, so that a range's splitters are loaded once
+    const unsigned t_begin = (unsigned)((uint64_t)nt * blockIdx.x / gridDim.x);
+    const unsigned t_end = (unsigned)((uint64_t)nt * (blockIdx.x + 1) / gridDim.x);
+    unsigned cur = ~0u;
+    uint64_t lo = 0;
+    int sh = 0;
+    for (unsigned t = t_begin; t < t_end; ++t) {
+        const TileMap tm = x.map[t];
+        const unsigned b = tm.range;
+        if (b != cur) {
+            __syncthreads();
+            for (unsigned i = tid; i < nf; i += NT)
+                S.g.spl[i] = x.fine_spl[(uint64_t)b * kMaxRanges + i];
+            for (unsigned i = tid; i < kLutStride / 8; i += NT)
+                ((uint4 *)S.g.lut)[i] = ((const uint4 *)(x.fine_lut + (uint64_t)b * kLutStride))[i];
+            lo = b ? x.spl[b - 1] : 0;
+            sh = bit_len((b + 1 < x.n_ranges ? x.spl[b] : last) - lo) - kLutBits;
+            if (sh < 0) sh = 0;
+            cur = b;
+        }
+        const unsigned local = t - x.tile_base[b];
+        const unsigned p0 = local * kRefineTile;
+        const unsigned n = min((unsigned)kRefineTile, x.totals[b] - p0);
+        const uint32_t *row = x.prefix + (uint64_t)b * x.n_chunks;
+        const uint16_t *st0 = x.starts + (uint64_t)b * x.n_chunks, *st1 = st0 + x.n_chunks;
+        for (unsigned i = tid; i < nf + 128; i += NT) S.g.hist[i] = 0;
+        for (unsigned c0 = tm.piece;; c0 += NT) {
+            const unsigned c = c0 + tid;
+            unsigned p = ~0u, e = ~0u;   // past the last piece: nothing to copy
+            if (c < x.n_chunks) {
+                const unsigned s0 = st0[c];
+                p = row[c];
+                e = p + st1[c] - s0;
+                S.src[tid] = x.piece[c] + s0;
+            }
+            S.pos[tid] = p;
+            if (tid == NT - 1) {
+                S.pos[NT] = e;
+                more = e < p0 + n;   // the tile goes on in the next pieces
+            }
+            __syncthreads();
+            const unsigned nr = min((unsigned)NT, x.n_chunks - c0);
+            if (tid == 0 && nr < NT) S.pos[nr] = x.totals[b];
+            __syncthreads();
+            gather_runs<KW, NT>(x.in, S.src, S.pos, nr, p0, p0 + n, S.g.keys);
+            const bool again = more != 0;
+            __syncthreads();
+            if (!again) break;
+        }
+        copies_done();
+        __syncthreads();
+        Key<KW> key[PER];
+        unsigned br[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const unsigned i = q * NT + tid;
+            br[q] = kNoKey;
+            if (i < n) {
+                key[q] = load_key<KW>(S.g.keys, i);
+                const unsigned bin = find_range(S.g.spl, S.g.lut, nf, lo, sh, prefix_of<KW>(key[q], K));
+                br[q] = (bin << 16) | atomicAdd(&S.g.hist[bin], 1u);
+            }
+        }
+        __syncthreads();
+        scan_ranges(S.g, nf);
+        __syncthreads();
+        const uint64_t tiles_b = x.tile_base[b + 1] - x.tile_base[b];
+        uint16_t *fs = x.fine_starts + (uint64_t)x.tile_base[b] * (nf + 1) + local;
+        for (unsigned i = tid; i <= nf; i += NT) fs[i * tiles_b] = (uint16_t)S.g.start[i];
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (br[q] != kNoKey)
+                store_key<KW>(S.g.keys, S.g.start[br[q] >> 16] + (br[q] & 0xffffu), key[q]);
+        __syncthreads();
+        copy_out<KW, kRefineTile, NT>(S.g, n, x.out + (uint64_t)t * kRefineTile * KW);
+        __syncthreads();
+    }
+}
+
+// -------------------------------------------------------------- 4. dedup
+// A final range as its block reads it: its runs, one in every piece (one level)
+// or in every tile of its coarse range (two levels), the prefixes it spans, and
+// this thread's run of the first NT.
+struct RangeRuns {
+    const uint16_t *row0;
+    unsigned n_runs, first;
+    uint64_t p_lo, p_hi;
+    unsigned src, n;
+
+    __device__ __forceinline__ void load_run(const DedupArgs &x, unsigned r) {
+        src = n = 0;
+        if (r < n_runs) {
+            const unsigned s0 = row0[r];
+            n = (unsigned)row0[(uint64_t)n_runs + r] - s0;
+            src = (x.n_fine ? (first + r) * (unsigned)kRefineTile : x.piece[r]) + s0;
+        }
+    }
+    __device__ __forceinline__ void load(const DedupArgs &x, unsigned g, uint64_t last) {
+        first = 0;
+        if (x.n_fine) {
+            const unsigned b = g / x.n_fine, f = g % x.n_fine;
+            first = x.tile_base[b];
+            n_runs = x.tile_base[b + 1] - first;
+            row0 = x.starts + (uint64_t)first * (x.n_fine + 1) + (uint64_t)f * n_runs;
+            const uint64_t *fs = x.fine_spl + (uint64_t)b * kMaxRanges;
+            p_lo = f ? fs[f - 1] : b ? x.spl[b - 1] : 0;
+            p_hi = f + 1 < x.n_fine ? fs[f] : b + 1 < x.n_ranges ? x.spl[b] : last;
+        } else {
+            n_runs = x.n_chunks;
+            row0 = x.starts + (uint64_t)g * n_runs;
+            p_lo = g ? x.spl[g - 1] : 0;
+            p_hi = g + 1 < x.n_ranges ? x.spl[g] : last;
+        }
+        load_run(x, threadIdx.x);
+    }
+};
+
+template <int KW>
+__device__ __forceinline__ unsigned key_hash(const Key<KW> &k) {
+    uint64_t x = k.lo;
+    if (KW == 2) x ^= rotl64(k.hi, 23) * kMurC2;
+    return (unsigned)((x * 0x9E3779B97F4A7C15ull) >> 32);
+}
+
+constexpr unsigned kRankLimit = 96;     // cuts of up to this many keys are rank sorted
+
+// Exclusive prefix of sub[0, kSubBins2) in place; most: the thread's largest count.
+template <int NT>
+__device__ __forceinline__ void scan_cuts(unsigned *sub, unsigned &most) {
+    constexpr unsigned E = (kSubBins2 + NT - 1) / NT;
+    unsigned v[E], sum = 0;
+    most = 0;
+#pragma unroll
+    for (unsigned j = 0; j < E; ++j) {
+        const unsigned i = threadIdx.x * E + j;
+        v[j] = i < (unsigned)kSubBins2 ? sub[i] : 0u;
+        sum += v[j];
+        most = max(most, v[j]);
+    }
+    unsigned tot;
+    unsigned pre = block_exclusive_scan<unsigned, NT>(sum, tot);
+#pragma unroll
+    for (unsigned j = 0; j < E; ++j) {
+        const unsigned i = threadIdx.x * E + j;
+        if (i < (unsigned)kSubBins2) sub[i] = pre;
+        pre += v[j];
+    }
+}
+
+// Sorts n places (uint16) by the keys key_of gives them: a bitonic network for
+// any length (every compare-exchange puts the smaller key first, partners past
+// the end are skipped).  For ranges whose keys crowd into few cuts.
+template <int NT, typename F>
+__device__ __forceinline__ void bitonic_places(uint16_t *ord, unsigned n, F key_of) {
+    unsigned P = 2;
+    while (P < n) P <<= 1;
+    for (unsigned k = 2; k <= P; k <<= 1) {
+        for (unsigned j = k >> 1; j > 0; j >>= 1) {
+            for (unsigned p = threadIdx.x; p < P / 2; p += NT) {
+                unsigned i, y;
+                if (j == (k >> 1)) {   // the flip: i against its mirror in the k-block
+                    const unsigned blk = p / j, off = p % j;
+                    i = blk * k + off;
+                    y = blk * k + (k - 1 - off);
+                } else {
+                    i = (p / j) * 2 * j + (p % j);
+                    y = i + j;
+                }
+                if (y < n) {
+                    const uint16_t u = ord[i], v = ord[y];
+                    if (key_of(v) < key_of(u)) {
+                        ord[i] = v;
+                        ord[y] = u;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// A block takes one final range at a time.  The range's windows are gathered
+// into shared memory (stage) and equal keys are found without atomics: every
+// window writes its place to its key's slot of a table, and after a barrier
+// looks whose place is there.  Equal key: that window stands for both, and its
+// count goes up.  Another key's: all windows of this key go on to the next free
+// slot together, in a further round.  Nearly all settle in the first round,
+// whose reads and writes have no chain between them (compare-and-swap probing
+// took 1,500 cycles a window and thread, three round trips a probe); the others
+// are listed first, so that the rounds take little.  The
+// windows that stand for their key are ordered by a counting sort on an even
+// cut of the range and ranked inside the cuts; only 16-bit places move.  Four
+// blocks share an SM, and the next range's runs are looked up while this one is
+// sorted.  Ranges of more windows than the stage, or too many
+// unsettled ones, are listed for dedup_big_kernel.
+template <int KW>
+struct __align__(16) SmallSmem {
+    uint64_t stage[kStage<KW> * KW];
+    uint16_t table[kTableSlots];     // then the places in key order
+    unsigned cnt[kStage<KW>];
+    uint16_t list[kStage<KW>];       // places that stand for their keys
+    uint16_t left[kMaxLeft], probe[kMaxLeft];   // unsettled places, and their slots
+    unsigned sub[kSubBins2];
+    unsigned src[kSmallThreads];
+    unsigned pos[kSmallThreads + 1];
+    unsigned lists, crowded, out0;   // lists: entries of left above, of list below
+};
+
+constexpr unsigned kNoPlace = 0xffffu;
+
+template <int KW>
+__global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, int K) {
+    constexpr int NT = kSmallThreads, Q = kStage<KW> / NT;
+    static_assert(kStage<KW> % NT == 0 && kStage<KW> < (int)kTableSlots, "whole rounds, free slots");
+    extern __shared__ __align__(16) unsigned char dyn[];
+    SmallSmem<KW> &S = *reinterpret_cast<SmallSmem<KW> *>(dyn);
+    const unsigned tid = threadIdx.x;
+    const uint64_t last = K >= 32 ? ~0ull : (1ull << (2 * K)) - 1;
+    RangeRuns next;
+    if (blockIdx.x < x.n_total) next.load(x, blockIdx.x, last);
+    for (unsigned g = blockIdx.x; g < x.n_total; g += gridDim.x) {
+        const RangeRuns cur = next;
+        const uint64_t p_lo = cur.p_lo;
+        int sh = bit_len(cur.p_hi - p_lo) - kSubBits2;
+        if (sh < 0) sh = 0;
+        // all windows of the range
+        unsigned n = cur.n;
+        for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
+            n += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
+        unsigned pre = block_exclusive_scan<unsigned, NT>(n, n);
+        if (n == 0 || n > (unsigned)kStage<KW>) {
+            if (tid == 0) {
+                if (n)
+                    x.big[atomicAdd(&x.meta->n_big, 1u)] = g;
+                else
+                    x.counts[g] = 0;
+            }
+            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+            continue;
+        }
+        for (unsigned r0 = 0, m0 = 0; r0 < cur.n_runs; r0 += NT) {
+            RangeRuns seg = cur;
+            if (cur.n_runs > NT) {
+                if (r0) seg.load_run(x, r0 + tid);
+                unsigned m;
+                pre = m0 + block_exclusive_scan<unsigned, NT>(seg.n, m);
+                m0 += m;
+            } else {
+                m0 = n;
+            }
+            S.src[tid] = seg.src;
+            S.pos[tid] = pre;
+            if (tid == 0) S.pos[NT] = m0;
+            __syncthreads();
+            gather_runs<KW, NT>(x.in, S.src, S.pos, min((unsigned)NT, cur.n_runs - r0), 0u, n, S.stage);
+            if (cur.n_runs > NT) __syncthreads();
+        }
+        {
+            const uint4 none = make_uint4(~0u, ~0u, ~0u, ~0u);
+            for (unsigned i = tid; i < kTableSlots / 8; i += NT) ((uint4 *)S.table)[i] = none;
+            for (unsigned i = tid; i < (unsigned)kSubBins2; i += NT) S.sub[i] = 0;
+            if (tid == 0) S.lists = S.crowded = 0;
+        }
+        copies_done();
+        __syncthreads();
+        unsigned slot[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const unsigned i = q * NT + tid;
+            slot[q] = 0;
+            if (i < n) {
+                slot[q] = __umulhi(key_hash(load_key<KW>(S.stage, i)), kTableSlots);
+                S.table[slot[q]] = (uint16_t)i;
+                S.cnt[i] = 0;
+            }
+        }
+        __syncthreads();
+        unsigned rep = 0, left = 0;   // bit q: window q stands for its key / is not settled
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const unsigned i = q * NT + tid;
+            if (i < n) {
+                const unsigned w = S.table[slot[q]];
+                if (w == i || load_key<KW>(S.stage, w) == load_key<KW>(S.stage, i)) {
+                    atomicAdd(&S.cnt[w], 1u);
+                    rep |= (w == i ? 1u : 0u) << q;
+                } else {
+                    left |= 1u << q;
+                }
+            }
+        }
+        // the windows that stand for their keys and the unsettled ones, listed: what
+        // follows touches no others
+        {
+            const unsigned mine = __popc(left) << 16 | __popc(rep);
+            unsigned upto = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, upto, o);
+                if ((tid & 31) >= (unsigned)o) upto += y;
+            }
+            unsigned first = 0;
+            if ((tid & 31) == 31) first = atomicAdd(&S.lists, upto);
+            first = __shfl_sync(0xffffffffu, first, 31) + upto - mine;
+            unsigned a = first & 0xffffu, b = first >> 16;
+            for (; rep; rep &= rep - 1) S.list[a++] = (uint16_t)((__ffs(rep) - 1) * NT + tid);
+            for (; left && b < kMaxLeft; left &= left - 1, ++b) {
+                S.left[b] = (uint16_t)((__ffs(left) - 1) * NT + tid);
+                S.probe[b] = kNoPlace;
+            }
+        }
+        __syncthreads();
+        const unsigned n_left = S.lists >> 16;
+        if (n_left > kMaxLeft) {   // a crowded table: the other kernel's
+            if (tid == 0) x.big[atomicAdd(&x.meta->n_big, 1u)] = g;
+            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+            __syncthreads();
+            continue;
+        }
+        for (bool any = n_left != 0; any;) {
+            // a further round: every window of a key sees the same table and takes
+            // the same free slot
+            for (unsigned p = tid; p < n_left; p += NT) {
+                const unsigned i = S.left[p];
+                if (i == kNoPlace) continue;   // settled
+                unsigned t = S.probe[p];
+                if (t == kNoPlace) t = __umulhi(key_hash(load_key<KW>(S.stage, i)), kTableSlots);
+                do {
+                    t = (t + 1) & (kTableSlots - 1);
+                } while (S.table[t] != kNoPlace);
+                S.probe[p] = (uint16_t)t;
+            }
+            __syncthreads();
+            for (unsigned p = tid; p < n_left; p += NT)
+                if (S.left[p] != kNoPlace) S.table[S.probe[p]] = S.left[p];
+            __syncthreads();
+            bool mine = false;
+            for (unsigned p = tid; p < n_left; p += NT) {
+                const unsigned i = S.left[p];
+                if (i == kNoPlace) continue;
+                const unsigned w = S.table[S.probe[p]];
+                if (w == i || load_key<KW>(S.stage, w) == load_key<KW>(S.stage, i)) {
+                    atomicAdd(&S.cnt[w], 1u);
+                    if (w == i) S.list[atomicAdd(&S.lists, 1u) & 0xffffu] = (uint16_t)i;
+                    S.left[p] = kNoPlace;
+                } else {
+                    mine = true;
+                }
+            }
+            any = __syncthreads_or(mine);
+        }
+        if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+        const unsigned nd = S.lists & 0xffffu;
+        if (!x.ordered) {
+            if (tid == 0) S.out0 = atomicAdd(&x.meta->out_cursor, nd);
+            __syncthreads();
+            for (unsigned p = tid; p < nd; p += NT) {
+                const unsigned i = S.list[p];
+                store_key<KW>(x.out, S.out0 + p, load_key<KW>(S.stage, i));
+                x.mult[S.out0 + p] = S.cnt[i];
+            }
+            __syncthreads();
+            continue;
+        }
+        // their order
+        for (unsigned p = tid; p < nd; p += NT)
+            atomicAdd(&S.sub[(prefix_of<KW>(load_key<KW>(S.stage, S.list[p]), K) - p_lo) >> sh], 1u);
+        if (tid == 0) {
+            S.out0 = atomicAdd(&x.meta->out_cursor, nd);
+            x.places[g] = S.out0;
+            x.counts[g] = nd;
+        }
+        __syncthreads();
+        unsigned most;
+        scan_cuts<NT>(S.sub, most);
+        if (most > kRankLimit) S.crowded = 1;
+        __syncthreads();
+        uint16_t *ord = S.table;   // the table is done with
+        for (unsigned p = tid; p < nd; p += NT) {
+            const unsigned i = S.list[p];
+            const unsigned c = (unsigned)((prefix_of<KW>(load_key<KW>(S.stage, i), K) - p_lo) >> sh);
+            ord[atomicAdd(&S.sub[c], 1u)] = (uint16_t)i;
+        }
+        __syncthreads();
+        const uint64_t at = S.out0;
+        const bool crowded = S.crowded != 0;
+        if (crowded)
+            bitonic_places<NT>(ord, nd, [&](unsigned i) { return load_key<KW>(S.stage, i); });
+        for (unsigned p = tid; p < nd; p += NT) {
+            const unsigned i = ord[p];
+            const Key<KW> k = load_key<KW>(S.stage, i);
+            unsigned rk = p;
+            if (!crowded) {   // a cut's keys end at its cursor and begin at the one before
+                const unsigned c = (unsigned)((prefix_of<KW>(k, K) - p_lo) >> sh);
+                const unsigned a0 = c ? S.sub[c - 1] : 0u, a1 = S.sub[c];
+                if (a1 - a0 > 1) {
+                    rk = a0;
+                    for (unsigned j = a0; j < a1; ++j)
+                        rk += load_key<KW>(S.stage, ord[j]) < k ? 1u : 0u;
+                }
+            }
+            store_key<KW>(x.out, at + rk, k);
+            x.mult[at + rk] = S.cnt[i];
+        }
+        __syncthreads();
+    }
+}
+
+// Ranges of any number of windows, batch by batch: every thread puts keys into
+// an open-addressing table, which counts them; whoever puts a key there first
+// appends its slot to a list, and everything after works on the list.  A range
+// with more distinct keys than the table takes is handled in rounds over
+// sub-ranges [lo, hi) of it: a round that overflows ends below the median of up
+// to 32 of the keys in the table instead (so it leaves some of them out, and the
+// rounds end).
+template <int KW>
+struct __align__(16) DedupSmem {
+    static constexpr int SLOTS = kDedupSlots<KW>;
+    uint64_t stage[kDedupStage<KW> * KW];   // a batch of windows; then uint16 slots in key order
+    uint64_t slot[SLOTS];            // one-word keys: the key; two-word keys: hash and place
+    unsigned ref[KW == 2 ? kDedupStage<KW> : 1];   // two-word keys: places of the batch's windows
+    unsigned cnt[SLOTS];
+    uint16_t list[SLOTS];            // slots in the order they were taken
+    unsigned sub[kSubBins2];         // keys per cut, then the cuts' cursors
+    unsigned src[kDedupThreads];     // runs: first key
+    unsigned pos[kDedupThreads + 1]; // and place among the range's windows
+    unsigned nd, over, crowded, ones, out0, cut;
+    Key<KW> pivot;
+};
+static_assert(kDedupSlots<1> * 2 <= kDedupStage<1> * 8 && kDedupSlots<2> * 2 <= kDedupStage<2> * 16,
+              "the slots in key order take the batch's place");
+
+constexpr uint64_t kFree = ~0ull;
+constexpr int kProbeMax = 192;          // probes after which the table counts as full
+
+// The key in a slot: of two-word keys, where it stands in the input.
+__device__ __forceinline__ Key<1> table_key(const DedupSmem<1> &S, const uint64_t *, unsigned slot) {
+    return Key<1>{S.slot[slot], 0};
+}
+__device__ __forceinline__ Key<2> table_key(const DedupSmem<2> &S, const uint64_t *in, unsigned slot) {
+    return load_key<2>(in, (unsigned)S.slot[slot]);
+}
+
+// Counts one window's key, key `at` of the input.  One-word keys are claimed
+// whole with a 64-bit compare-and-swap.  Two-word keys claim a slot with their
+// hash and their place in the input, and are compared there (the range is in
+// L1), so that no thread waits for another to finish writing a key.
+template <int KW>
+__device__ __forceinline__ void table_add(DedupSmem<KW> &S, const Key<KW> &k, const uint64_t *in,
+                                          unsigned at) {
+    if (KW == 1 && k.lo == kFree) {   // 32-mers of T alone, forward strand
+        atomicAdd(&S.ones, 1u);
+        return;
+    }
+    const unsigned h = key_hash(k);
+    const uint64_t want = KW == 1 ? k.lo : ((uint64_t)h << 32) | at;
+    unsigned slot = __umulhi(h, (unsigned)kDedupSlots<KW>);
+    for (int it = 0; it < kProbeMax; ++it) {
+        unsigned long long *p = (unsigned long long *)S.slot + slot;
+        unsigned long long v = *(volatile unsigned long long *)p;
+        if (v == kFree) {
+            v = atomicCAS(p, (unsigned long long)kFree, (unsigned long long)want);
+            if (v == kFree) {
+                S.list[atomicAdd(&S.nd, 1u)] = (uint16_t)slot;
+                v = want;
+            }
+        }
+        if (KW == 1 ? v == want
+                    : (unsigned)(v >> 32) == h && (v == want || load_key<KW>(in, (unsigned)v) == k)) {
+            atomicAdd(&S.cnt[slot], 1u);
+            return;
+        }
+        if (++slot == (unsigned)kDedupSlots<KW>) slot = 0;
+        if (it >= 16 && *(volatile unsigned *)&S.over) return;   // the round is lost anyway
+    }
+    S.over = 1;
+}
+
+template <int KW>
+__global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x, int K) {
+    constexpr int SLOTS = kDedupSlots<KW>, NT = kDedupThreads;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    DedupSmem<KW> &S = *reinterpret_cast<DedupSmem<KW> *>(dyn);
+    uint16_t *ord = (uint16_t *)S.stage;
+    const unsigned tid = threadIdx.x;
+    for (unsigned i = tid; i < (unsigned)SLOTS; i += NT) {
+        S.slot[i] = kFree;
+        S.cnt[i] = 0;
+    }
+    const uint64_t last = K >= 32 ? ~0ull : (1ull << (2 * K)) - 1;
+    const unsigned n_big = x.meta->n_big;
+    for (unsigned q = blockIdx.x; q < n_big; q += gridDim.x) {
+        const unsigned g = x.big[q];
+        RangeRuns cur;
+        cur.load(x, g, last);
+        const uint64_t p_lo = cur.p_lo;
+        int sh = bit_len(cur.p_hi - p_lo) - kSubBits2;
+        if (sh < 0) sh = 0;
+        unsigned done = 0;   // distinct keys written
+        Key<KW> lo, hi;
+        lo.lo = lo.hi = 0;
+        hi = lo;
+        bool from = false, until = false;   // whether lo and hi bound this round
+        for (bool again = true, begun = false; again;) {
+            __syncthreads();   // the last round's table is cleared
+            if (tid == 0) S.nd = S.over = S.crowded = S.ones = 0;
+            for (unsigned i = tid; i < (unsigned)kSubBins2; i += NT) S.sub[i] = 0;
+            unsigned n_all = 0;
+            for (unsigned r0 = 0; r0 < cur.n_runs; r0 += NT) {
+                RangeRuns seg = cur;
+                if (r0) seg.load_run(x, r0 + tid);
+                unsigned m;
+                const unsigned pre = block_exclusive_scan<unsigned, NT>(seg.n, m);
+                S.src[tid] = seg.src;
+                S.pos[tid] = pre;
+                if (tid == 0) S.pos[NT] = m;
+                n_all += m;
+                __syncthreads();
+                const unsigned nr = min((unsigned)NT, cur.n_runs - r0);
+                for (unsigned p0 = 0; p0 < m; p0 += kDedupStage<KW>) {
+                    const unsigned p1 = min(m, p0 + (unsigned)kDedupStage<KW>);
+                    gather_runs<KW, NT>(x.in, S.src, S.pos, nr, p0, p1, S.stage,
+                                        KW == 2 ? S.ref : nullptr);
+                    copies_done();
+                    __syncthreads();
+                    for (unsigned i = tid; i < p1 - p0; i += NT) {
+                        const Key<KW> k = load_key<KW>(S.stage, i);
+                        if ((from && k < lo) || (until && !(k < hi))) continue;
+                        table_add(S, k, x.in, KW == 2 ? S.ref[i] : 0u);
+                    }
+                    __syncthreads();
+                }
+            }
+            if (!begun) {   // the range's place in the output
+                begun = true;
+                if (tid == 0 && x.ordered) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n_all);
+            }
+            const unsigned nd = S.nd;
+            if (!S.over && !x.ordered) {
+                const bool ones = KW == 1 && S.ones && !until;
+                if (tid == 0) S.out0 = atomicAdd(&x.meta->out_cursor, nd + (ones ? 1u : 0u));
+                __syncthreads();
+                for (unsigned i = tid; i < nd; i += NT) {
+                    const unsigned slot = S.list[i];
+                    store_key<KW>(x.out, S.out0 + i, table_key(S, x.in, slot));
+                    x.mult[S.out0 + i] = S.cnt[slot];
+                }
+                if (ones && tid == 0) {
+                    x.out[S.out0 + nd] = ~0ull;
+                    x.mult[S.out0 + nd] = S.ones;
+                }
+                again = until;
+                lo = hi;
+                from = from || until;
+                until = false;
+            } else if (!S.over) {
+                for (unsigned i = tid; i < nd; i += NT) {
+                    const Key<KW> k = table_key(S, x.in, S.list[i]);
+                    atomicAdd(&S.sub[(prefix_of<KW>(k, K) - p_lo) >> sh], 1u);
+                }
+                __syncthreads();
+                unsigned most;
+                scan_cuts<NT>(S.sub, most);
+                if (most > kRankLimit) S.crowded = 1;
+                __syncthreads();
+                for (unsigned i = tid; i < nd; i += NT) {
+                    const unsigned slot = S.list[i];
+                    const Key<KW> k = table_key(S, x.in, slot);
+                    ord[atomicAdd(&S.sub[(prefix_of<KW>(k, K) - p_lo) >> sh], 1u)] = (uint16_t)slot;
+                }
+                __syncthreads();
+                const uint64_t at = (uint64_t)S.out0 + done;
+                if (!S.crowded) {
+                    // a cut's keys end at its cursor and begin at the one before
+                    for (unsigned i = tid; i < nd; i += NT) {
+                        const unsigned slot = ord[i];
+                        const Key<KW> k = table_key(S, x.in, slot);
+                        const unsigned c = (unsigned)((prefix_of<KW>(k, K) - p_lo) >> sh);
+                        const unsigned a0 = c ? S.sub[c - 1] : 0u, a1 = S.sub[c];
+                        unsigned rk = a0;
+                        if (a1 - a0 > 1)
+                            for (unsigned j = a0; j < a1; ++j)
+                                rk += table_key(S, x.in, ord[j]) < k ? 1u : 0u;
+                        store_key<KW>(x.out, at + rk, k);
+                        x.mult[at + rk] = S.cnt[slot];
+                    }
+                } else {
+                    bitonic_places<NT>(ord, nd, [&](unsigned v) { return table_key(S, x.in, v); });
+                    for (unsigned i = tid; i < nd; i += NT) {
+                        const unsigned slot = ord[i];
+                        store_key<KW>(x.out, at + i, table_key(S, x.in, slot));
+                        x.mult[at + i] = S.cnt[slot];
+                    }
+                }
+                done += nd;
+                if (KW == 1 && S.ones && !until) {   // the largest key there is
+                    if (tid == 0) {
+                        x.out[at + nd] = ~0ull;
+                        x.mult[at + nd] = S.ones;
+                    }
+                    ++done;
+                }
+                again = until;
+                lo = hi;
+                from = from || until;
+                until = false;
+            } else {
+                // too many distinct keys: the round ends below the median of the
+                // first keys found in 32 stretches of the table
+                if (tid == 0) S.cut = 0;
+                __syncthreads();
+                if (tid < 32) {
+                    const unsigned s0 = tid * (SLOTS / 32);
+                    unsigned at = s0;
+                    while (at < s0 + SLOTS / 32 && S.cnt[at] == 0) ++at;
+                    const bool have = at < s0 + SLOTS / 32;
+                    const unsigned held = __ballot_sync(0xffffffffu, have);
+                    Key<KW> k;
+                    k.lo = k.hi = 0;
+                    if (have) k = table_key(S, x.in, at);
+                    unsigned below = 0;
+                    for (int j = 0; j < 32; ++j) {
+                        Key<KW> o;
+                        o.lo = __shfl_sync(0xffffffffu, k.lo, j);
+                        o.hi = KW == 2 ? __shfl_sync(0xffffffffu, k.hi, j) : 0;
+                        below += ((held >> j) & 1u) && o < k ? 1u : 0u;
+                    }
+                    if (have && below && below == (unsigned)__popc(held) / 2) {
+                        S.pivot = k;
+                        S.cut = 1;
+                    }
+                }
+                __syncthreads();
+                hi = S.pivot;
+                until = true;
+                again = S.cut != 0;   // a full stretch of the table holds two keys at least
+                if (!again && tid == 0) atomicOr(&x.ctr->error, kErrProbeLimit);
+            }
+            __syncthreads();
+            for (unsigned i = tid; i < nd; i += NT) {
+                const unsigned slot = S.list[i];
+                S.slot[slot] = kFree;
+                S.cnt[slot] = 0;
+            }
+        }
+        if (tid == 0 && x.ordered) x.counts[g] = done;
+    }
+}
+
+// offsets[g] = distinct keys in ranges before g, offsets[n] = all; one block.
+__global__ void __launch_bounds__(1024) scan_counts_kernel(const uint32_t *counts, unsigned n,
+                                                           uint32_t *offsets, DedupMeta *meta,
+                                                           DevCounters *ctr) {
+    constexpr unsigned E = 16;
+    unsigned carry = 0;
+    for (unsigned i0 = 0; i0 < n; i0 += 1024 * E) {
+        unsigned v[E], sum = 0;
+#pragma unroll
+        for (unsigned j = 0; j < E; ++j) {
+            const unsigned i = i0 + threadIdx.x * E + j;
+            v[j] = i < n ? counts[i] : 0u;
+            sum += v[j];
+        }
+        unsigned tot;
+        unsigned pre = block_exclusive_scan<unsigned, 1024>(sum, tot) + carry;
+#pragma unroll
+        for (unsigned j = 0; j < E; ++j) {
+            const unsigned i = i0 + threadIdx.x * E + j;
+            if (i < n) offsets[i] = pre;
+            pre += v[j];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        offsets[n] = carry;
+        meta->distinct = carry;
+        if (ctr) ctr->distinct = carry;   // the list holds exactly these
+    }
+}
+
+// -------------------------------------------------------- 5. increments
+// Walks distinct keys [begin, end) of the call in ascending order, EMIT_KEYS
+// at a time: ranges hold their keys at places[g], numbered from offsets[g].
+// win: a window of the offsets in shared memory.
+constexpr unsigned kWin = 256;
+
+// The range holding distinct key i (the last g with offsets[g] <= i).
+__device__ __forceinline__ unsigned range_of(const uint32_t *offsets, unsigned n, unsigned i) {
+    unsigned a = 0, b = n - 1;
+    while (a < b) {
+        const unsigned m = a + (b - a + 1) / 2;
+        if (offsets[m] <= i)
+            a = m;
+        else
+            b = m - 1;
+    }
+    return a;
+}
+
+// Loads offsets [g0, g0 + kWin] and places of those ranges into shared memory.
+template <int NT>
+__device__ __forceinline__ void load_window(const EmitArgs &e, unsigned g0, unsigned *off,
+                                            unsigned *plc) {
+    for (unsigned i = threadIdx.x; i <= kWin; i += NT) {
+        const unsigned g = g0 + i;
+        off[i] = g <= e.n_total ? e.offsets[g] : ~0u;
+        if (i < kWin) plc[i] = g < e.n_total ? e.places[g] : 0u;
+    }
+}
+
+// Where key i of the call is in e.keys / e.mult, for i inside the window.
+__device__ __forceinline__ uint64_t place_in(const unsigned *off, const unsigned *plc, unsigned i) {
+    unsigned a = 0, b = kWin - 1;
+    while (a < b) {
+        const unsigned m = (a + b + 1) / 2;
+        if (off[m] <= i)
+            a = m;
+        else
+            b = m - 1;
+    }
+    return (uint64_t)plc[a] + (i - off[a]);
+}
+
+// Partitioned update: one 32-bit code per (distinct key, hash), the cell
+// within its coarse region, the counter within the cell and the increment
+// less one; the codes of a chunk of keys are grouped by region in shared
+// memory and appended to the regions' buffers, one cursor atomic per region.
+// Codes that do not fit, and increments above a code's largest, are added to
+// the countBF directly.
+constexpr int kEmitThreads = 256;
+constexpr int kEmitKeys = 1024;
+
+// Two hashes of four keys a thread are in registers at a time.  MODE: the
+// addressing of the usual countBFs (flat with 2^n counters, flat, two-dimensional;
+// a power of two counters in a cell each), short enough to be unrolled over the
+// keys and hashes; kAnyAddress: the general one, which is not (unrolled, the body
+// would not fit the instruction cache).
+constexpr unsigned kEmitHashes = 2;
+enum AddressMode { kAnyAddress, kFlatPow2, kFlat, kTwoDim };
+
+// Coarse region of hash h, and cell in it and counter in the cell as a code has
+// them (at most 2^30 cells, so a cell's number has 32 bits).
+template <int MODE>
+__device__ __forceinline__ void code_of(const Geometry &G, int coarse_shift, int sb, uint64_t h,
+                                        unsigned &bin, uint32_t &code) {
+    if (MODE == kFlatPow2 || MODE == kFlat) {   // the counter's number is cell and counter
+        const uint64_t g = MODE == kFlatPow2 ? h & G.m_mask : mod_by(h, G.m, G.mag_m);
+        bin = (unsigned)(g >> (coarse_shift + sb));
+        code = (uint32_t)g & ((1u << (coarse_shift + sb)) - 1);
+        return;
+    }
+    uint64_t cell64;
+    unsigned slot;
+    if (MODE == kTwoDim) {
+        cell64 = mod_by(h, G.dim_x, G.mag_x) * G.dim_y + mod_by(h, G.dim_y, G.mag_y);
+        slot = (unsigned)h & (unsigned)(G.eta - 1);
+    } else {
+        address(G, h, cell64, slot);
+    }
+    const unsigned cell = (unsigned)cell64;
+    bin = cell >> coarse_shift;
+    code = ((cell & ((1u << coarse_shift) - 1)) << sb) | slot;
+}
+
+template <int KW, int MODE>
+__global__ void __launch_bounds__(kEmitThreads, 4) emit_kernel(EmitArgs e) {
+    constexpr int NT = kEmitThreads, PER = kEmitKeys / NT;
+    __shared__ uint32_t sorted[kEmitKeys * kEmitHashes];
+    __shared__ uint8_t region[kEmitKeys * kEmitHashes];   // of sorted[i]
+    __shared__ unsigned hist[kCoarseBins], start[kCoarseBins];
+    __shared__ unsigned long long base[kCoarseBins];      // a code's place in e.coarse less its i
+    __shared__ unsigned staged;
+    __shared__ unsigned off[kWin + 1], plc[kWin];
+    const unsigned tid = threadIdx.x, lane = tid & 31;
+    const Geometry &G = e.G;
+    const unsigned D = e.ordered ? e.meta->distinct : e.meta->out_cursor;
+    const unsigned r0 = min(e.begin, D), r1 = min(e.end, D);
+    const unsigned i_begin = r0 + (unsigned)((uint64_t)(r1 - r0) * blockIdx.x / gridDim.x);
+    const unsigned i_end = r0 + (unsigned)((uint64_t)(r1 - r0) * (blockIdx.x + 1) / gridDim.x);
+    if (i_begin >= i_end) return;
+    unsigned g0 = e.ordered ? range_of(e.offsets, e.n_total, i_begin) : 0;
+    const unsigned nh = (unsigned)G.nhash;
+    const int wb = e.w_bits, sb = e.slot_bits;
+    const uint32_t w_most = 1u << wb;   // wb is 16 at most
+    if (e.ordered) load_window<NT>(e, g0, off, plc);
+    else if (tid == 0) off[kWin] = ~0u;   // the keys stand one after the other
+    __syncthreads();
+    for (unsigned i0 = i_begin; i0 < i_end;) {
+        if (off[kWin] <= i0) {   // i0 lies past the window of ranges: the next one
+            __syncthreads();
+            load_window<NT>(e, g0 += kWin, off, plc);
+            __syncthreads();
+            continue;
+        }
+        const unsigned i1 = min(min(i_end, i0 + kEmitKeys), off[kWin]);
+        Key<KW> key[PER];
+        uint32_t w[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const unsigned i = i0 + q * NT + tid;
+            w[q] = 0;
+            if (i < i1) {
+                const uint64_t at = e.ordered ? place_in(off, plc, i) : i;
+                key[q] = load_key<KW>(e.keys, at);
+                w[q] = (uint32_t)min((uint64_t)e.mult[at], G.maxc);
+                if (e.dlist) store_key<KW>(e.dlist, i, key[q]);
+            }
+        }
+        for (unsigned a0 = 0; a0 < nh; a0 += kEmitHashes) {
+            if (tid < kCoarseBins) hist[tid] = 0;
+            __syncthreads();
+            uint32_t code[PER][kEmitHashes];
+            unsigned br[PER][kEmitHashes];
+#pragma unroll(MODE != kAnyAddress ? PER : 1)
+            for (int q = 0; q < PER; ++q) {
+                const uint64_t k1m = KW == 1 ? premix8(key[q].lo) : 0;
+#pragma unroll
+                for (unsigned j = 0; j < kEmitHashes; ++j) {
+                    br[q][j] = kNoKey;
+                    if (w[q] && a0 + j < nh) {
+                        uint64_t h1, h2;
+                        if (KW == 1)
+                            murmur8(k1m, a0 + j, h1, h2);
+                        else
+                            murmur16(key[q].lo, key[q].hi, a0 + j, h1, h2);
+                        unsigned bin;
+                        uint32_t in;
+                        code_of<MODE>(G, e.coarse_shift, sb, h1, bin, in);
+                        const uint32_t wc = min(w[q], w_most);
+                        code[q][j] = (in << wb) | (wc - 1);
+                        br[q][j] = (bin << 16) | atomicAdd(&hist[bin], 1u);
+                        if (wc < w[q]) {
+                            const uint64_t cell = ((uint64_t)bin << e.coarse_shift) | (in >> sb);
+                            sat_add(G.cells, cell, (in & ((1u << sb) - 1)) * (unsigned)G.alpha, G.maxc,
+                                    w[q] - wc, __ldcg(G.cells + cell), G.cas_limit, &e.ctr->error);
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            if (tid < kCoarseBins) {   // warps 0 and 1: prefix over the regions
+                const unsigned n = hist[tid];
+                unsigned incl = n, below = 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= (unsigned)o) incl += t;
+                }
+                if (tid >= 32) {   // warp 1 starts after all of warp 0's regions
+                    below = hist[tid - 32];
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+                }
+                start[tid] = below + incl - n;
+                if (tid == kCoarseBins - 1) staged = below + incl;
+                unsigned long long b0 = ~0ull;
+                if (n) {
+                    b0 = atomicAdd(e.coarse_cursor + tid, (unsigned long long)n);
+                    if (b0 + n > e.coarse_cap) {
+                        b0 = ~0ull;   // region full: these go to the countBF directly
+                    } else {
+                        atomicAdd(e.coarse_written + tid, (unsigned long long)n);
+                        b0 += (uint64_t)tid * e.coarse_cap - (below + incl - n);
+                    }
+                }
+                base[tid] = b0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < PER; ++q)
+#pragma unroll
+                for (unsigned j = 0; j < kEmitHashes; ++j)
+                    if (br[q][j] != kNoKey) {
+                        const unsigned at = start[br[q][j] >> 16] + (br[q][j] & 0xffffu);
+                        sorted[at] = code[q][j];
+                        region[at] = (uint8_t)(br[q][j] >> 16);
+                    }
+            __syncthreads();
+            // runs of a region's codes leave together
+            for (unsigned i = tid, n = staged; i < n; i += NT) {
+                const uint32_t c = sorted[i];
+                const unsigned bin = region[i];
+                const unsigned long long b0 = base[bin];
+                if (b0 != ~0ull) {
+                    __stcs(e.coarse + (b0 + i), c);
+                } else {
+                    const uint64_t cell = ((uint64_t)bin << e.coarse_shift) | (c >> (sb + wb));
+                    const unsigned slot = (c >> wb) & ((1u << sb) - 1);
+                    sat_add(G.cells, cell, slot * (unsigned)G.alpha, G.maxc, (c & (w_most - 1)) + 1ull,
+                            __ldcg(G.cells + cell), G.cas_limit, &e.ctr->error);
+                }
+            }
+            __syncthreads();
+        }
+        i0 = i1;
+    }
+}
+
+// Atomic update: the distinct keys' increments straight into the countBF (an
+// L2-resident one), four first attempts of a key in flight together.
+template <int KW>
+__global__ void __launch_bounds__(kEmitThreads, 4) emit_atomic_kernel(EmitArgs e) {
+    constexpr int NT = kEmitThreads;
+    __shared__ unsigned off[kWin + 1], plc[kWin];
+    const unsigned tid = threadIdx.x;
+    const Geometry &G = e.G;
+    const unsigned D = e.ordered ? e.meta->distinct : e.meta->out_cursor;
+    const unsigned i_begin = (unsigned)((uint64_t)D * blockIdx.x / gridDim.x);
+    const unsigned i_end = (unsigned)((uint64_t)D * (blockIdx.x + 1) / gridDim.x);
+    if (i_begin >= i_end) return;
+    unsigned g0 = e.ordered ? range_of(e.offsets, e.n_total, i_begin) : 0;
+    if (e.ordered) load_window<NT>(e, g0, off, plc);
+    else if (tid == 0) off[kWin] = ~0u;   // the keys stand one after the other
+    __syncthreads();
+    for (unsigned i0 = i_begin; i0 < i_end;) {
+        if (off[kWin] <= i0) {
+            __syncthreads();
+            load_window<NT>(e, g0 += kWin, off, plc);
+            __syncthreads();
+            continue;
+        }
+        const unsigned i1 = min(min(i_end, i0 + NT), off[kWin]);
+        const unsigned i = i0 + tid;
+        i0 = i1;
+        if (i >= i1) continue;
+        const uint64_t at = e.ordered ? place_in(off, plc, i) : i;
+        const Key<KW> key = load_key<KW>(e.keys, at);
+        const uint64_t w = min((uint64_t)e.mult[at], G.maxc);
+        if (e.dlist) store_key<KW>(e.dlist, i, key);
+        const uint64_t k1m = KW == 1 ? premix8(key.lo) : 0;
+        for (int a0 = 0; a0 < G.nhash; a0 += 4) {
+            uint64_t cell[4], cur[4], prev[4];
+            unsigned sh[4];
+            bool need[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                cell[j] = 0;
+                sh[j] = 0;
+                cur[j] = 0;
+                if (a0 + j < G.nhash) {
+                    uint64_t h1, h2;
+                    unsigned slot;
+                    if (KW == 1)
+                        murmur8(k1m, (uint32_t)(a0 + j), h1, h2);
+                    else
+                        murmur16(key.lo, key.hi, (uint32_t)(a0 + j), h1, h2);
+                    address(G, h1, cell[j], slot);
+                    sh[j] = slot * (unsigned)G.alpha;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (a0 + j < G.nhash) cur[j] = __ldcg(G.cells + cell[j]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint64_t room = G.maxc - ((cur[j] >> sh[j]) & G.maxc);
+                need[j] = a0 + j < G.nhash && room != 0;
+                prev[j] = cur[j];
+                if (need[j])
+                    prev[j] = atomicCAS((unsigned long long *)(G.cells + cell[j]),
+                                        (unsigned long long)cur[j],
+                                        (unsigned long long)(cur[j] + (min(w, room) << sh[j])));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (need[j] && prev[j] != cur[j])
+                    sat_add(G.cells, cell[j], sh[j], G.maxc, w, prev[j], G.cas_limit,
+                            &e.ctr->error);
+        }
+    }
+}
+
+// Sub-arrays of DedupBufs::meta.
+struct MetaLayout {
+    uint64_t size = 0;
+    uint64_t take(uint64_t bytes) {
+        const uint64_t at = size;
+        size += (bytes + 255) & ~255ull;
+        return at;
+    }
+    uint64_t meta, codes, valid, samples, spl, lut, piece, starts, places, counts, offsets, big;
+    uint64_t prefix, totals, tile_base, map, fine_spl, fine_lut, fine_starts;
+    explicit MetaLayout(const DedupPlan &p) {
+        meta = take(sizeof(DedupMeta));
+        codes = take(p.chunks * p.chunk / 4 + 64);   // and 128 bases after the last chunk
+        valid = take(p.chunks * p.chunk / 8);
+        samples = take(p.samples * 8ull);
+        spl = take(kMaxRanges * 8ull);
+        lut = take(kLutStride * 2ull);
+        piece = take(p.chunks * 4);
+        starts = take((p.n_ranges + 1ull) * p.chunks * 2);
+        places = take(p.total() * 4);
+        counts = take(p.total() * 4);
+        offsets = take((p.total() + 1) * 4);
+        big = take(p.total() * 4);
+        prefix = totals = tile_base = map = fine_spl = fine_lut = fine_starts = size;
+        if (p.n_fine) {
+            prefix = take((uint64_t)p.n_ranges * p.chunks * 4);
+            totals = take(p.n_ranges * 4ull);
+            tile_base = take((p.n_ranges + 1) * 4ull);
+            map = take(p.tiles() * sizeof(TileMap));
+            fine_spl = take((uint64_t)p.n_ranges * kMaxRanges * 8);
+            fine_lut = take((uint64_t)p.n_ranges * kLutStride * 2);
+            fine_starts = take(p.tiles() * (p.n_fine + 1) * 2);
+        }
+    }
+};
+
+// Values a thread of block_sort holds for n of them (n <= kMaxSamples).
+int sort_items(unsigned n) {
+    int e = 1;
+    while (1024u * e < n) e *= 2;
+    return e;
+}
+
+uint64_t last_prefix(int K) { return K >= 32 ? ~0ull : (1ull << (2 * K)) - 1; }
+
+template <typename F>
+cudaError_t set_smem(F f, size_t bytes) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+#define DD_TRY(call)                              \
+    do {                                          \
+        const cudaError_t e_ = (call);            \
+        if (e_ != cudaSuccess) return e_;         \
+    } while (0)
+
+template <int KW, int CHUNK>
+cudaError_t extract_variant(int K, int canonical, const ExtractArgs &x, unsigned per_sm, int sms,
+                            cudaStream_t s) {
+    constexpr size_t smem = sizeof(GroupSmem<KW, CHUNK>);
+    auto *k = canonical == 0   ? extract_kernel<KW, CHUNK, 0>
+              : canonical == 1 ? extract_kernel<KW, CHUNK, 1> : extract_kernel<KW, CHUNK, 2>;
+    DD_TRY(set_smem(k, smem));
+    const unsigned grid = std::min(x.n_chunks, (unsigned)sms * per_sm);
+    k<<<grid, CHUNK / 8, smem, s>>>(K, x);
+    return cudaGetLastError();
+}
+
+RefineArgs refine_args(const DedupPlan &p, const DedupBufs &d, const MetaLayout &m,
+                       uint64_t n_chunks) {
+    RefineArgs r;
+    r.in = d.a;
+    r.out = d.b;
+    r.n_chunks = (unsigned)n_chunks;
+    r.n_ranges = p.n_ranges;
+    r.n_fine = p.n_fine;
+    r.target = p.target;
+    r.spl = (const uint64_t *)(d.meta + m.spl);
+    r.piece = (const uint32_t *)(d.meta + m.piece);
+    r.prefix = (const uint32_t *)(d.meta + m.prefix);
+    r.totals = (const uint32_t *)(d.meta + m.totals);
+    r.tile_base = (const uint32_t *)(d.meta + m.tile_base);
+    r.starts = (const uint16_t *)(d.meta + m.starts);
+    r.map = (const TileMap *)(d.meta + m.map);
+    r.fine_spl = (uint64_t *)(d.meta + m.fine_spl);
+    r.fine_lut = (uint16_t *)(d.meta + m.fine_lut);
+    r.fine_starts = (uint16_t *)(d.meta + m.fine_starts);
+    r.meta = (DedupMeta *)(d.meta + m.meta);
+    return r;
+}
+
+template <int KW>
+cudaError_t finish_variant(const DedupPlan &p, const DedupBufs &d, DevCounters *ctr,
+                           uint64_t n_chunks, bool ordered, bool fresh, int sms, cudaStream_t s,
+                           uint64_t &launches) {
+    const MetaLayout m(p);
+    DedupMeta *meta = (DedupMeta *)(d.meta + m.meta);
+    const unsigned nc = (unsigned)n_chunks;
+    if (p.n_fine) {
+        const RefineArgs r = refine_args(p, d, m, n_chunks);
+        row_prefix_kernel<<<p.n_ranges, 1024, 0, s>>>(r.starts, nc, (uint32_t *)r.prefix,
+                                                     (uint32_t *)r.totals);
+        const int E = sort_items(p.fine_samples);
+        auto *fk = E == 1 ? fine_splitters_kernel<KW, 1> : E == 2 ? fine_splitters_kernel<KW, 2>
+                 : E == 4 ? fine_splitters_kernel<KW, 4> : E == 8 ? fine_splitters_kernel<KW, 8>
+                 : fine_splitters_kernel<KW, 16>;
+        DD_TRY(set_smem(fk, std::max(E, 4) * 8192));
+        fk<<<p.n_ranges, 1024, std::max(E, 4) * 8192, s>>>(r, p.K, p.fine_samples, last_prefix(p.K));
+        tile_map_kernel<<<(unsigned)((p.tiles() + 1023) / 1024), 1024, 0, s>>>(
+            r.totals, p.n_ranges, r.prefix, nc, (uint32_t *)r.tile_base, (TileMap *)r.map, meta);
+        constexpr size_t smem = sizeof(RefineSmem<KW>);
+        DD_TRY(set_smem(refine_kernel<KW>, smem));
+        const uint64_t grid = std::min<uint64_t>(p.tiles(), (uint64_t)sms * 2);
+        refine_kernel<KW><<<(unsigned)grid, kRefineThreads, smem, s>>>(r, p.K, last_prefix(p.K));
+        launches += 4;
+    }
+    DedupArgs x;
+    x.in = p.n_fine ? d.b : d.a;
+    x.out = p.n_fine ? d.a : d.b;
+    x.mult = d.mult;
+    x.n_chunks = nc;
+    x.n_fine = p.n_fine;
+    x.piece = (const uint32_t *)(d.meta + m.piece);
+    x.tile_base = (const uint32_t *)(d.meta + m.tile_base);
+    x.starts = (const uint16_t *)(d.meta + (p.n_fine ? m.fine_starts : m.starts));
+    x.n_ranges = p.n_ranges;
+    x.n_total = (unsigned)p.total();
+    x.spl = (const uint64_t *)(d.meta + m.spl);
+    x.fine_spl = (const uint64_t *)(d.meta + m.fine_spl);
+    x.places = (uint32_t *)(d.meta + m.places);
+    x.counts = (uint32_t *)(d.meta + m.counts);
+    x.meta = meta;
+    x.ctr = ctr;
+    x.big = (uint32_t *)(d.meta + m.big);
+    x.ordered = ordered ? 1 : 0;
+    constexpr size_t smem = sizeof(SmallSmem<KW>), big_smem = sizeof(DedupSmem<KW>);
+    DD_TRY(set_smem(dedup_kernel<KW>, smem));
+    DD_TRY(set_smem(dedup_big_kernel<KW>, big_smem));
+    const unsigned total = (unsigned)p.total();
+    dedup_kernel<KW><<<std::min(total, (unsigned)sms * 4), kSmallThreads, smem, s>>>(x, p.K);
+    dedup_big_kernel<KW><<<std::min(total, (unsigned)sms * 3), kDedupThreads, big_smem, s>>>(x, p.K);
+    launches += 2;
+    if (!ordered) return cudaGetLastError();
+    scan_counts_kernel<<<1, 1024, 0, s>>>(x.counts, (unsigned)p.total(),
+                                          (uint32_t *)(d.meta + m.offsets), meta, fresh ? ctr : nullptr);
+    launches += 1;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+uint64_t DedupPlan::meta_bytes() const { return MetaLayout(*this).size; }
+
+int dedup_chunk(uint64_t nbytes) {
+    return nbytes / kExtractChunk < 4 * kPlanSms ? kExtractSmall : kExtractChunk;
+}
+
+// Ranges of about `target` windows each, so that few hold more than a dedup
+// block's stage (the splitters' sampling spreads the sizes by a quarter); small calls
+// are cut into at least two ranges per SM while those keep 512 windows.  Up
+// to kMaxRanges ranges in one level; more in two levels of about equally many
+// ranges, so that the runs a block gathers are about equally long at both.
+DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk) {
+    DedupPlan p;
+    p.K = K;
+    p.kw = K <= 32 ? 1 : 2;
+    p.bound = bound;
+    if (bound == 0 || bound > kMaxRangeWindows) return p;
+    // a call of few ranges waits for its largest ones: smaller ones then
+    p.target = bound < (1ull << 25) ? (p.kw == 1 ? 1280 : 896) : (p.kw == 1 ? 1664 : 1152);
+    uint64_t ranges = (bound + p.target - 1) / p.target;
+    ranges = std::max(ranges, std::min<uint64_t>(2 * kPlanSms, bound / 512));
+    if (ranges < 1) ranges = 1;
+    p.chunk = chunk;
+    p.chunks = chunks;
+    if (ranges <= kMaxRanges) {
+        p.n_ranges = (unsigned)ranges;
+    } else {
+        unsigned c = 32;
+        while ((uint64_t)c * c < ranges && c < kMaxRanges) ++c;
+        p.n_ranges = c;
+        const uint64_t mean = (ranges + c - 1) / c;   // and a quarter for the larger ones
+        p.n_fine = (unsigned)std::min<uint64_t>(mean + mean / 4, kMaxRanges);
+        p.fine_samples = std::min(16 * p.n_fine, kMaxSamples);
+    }
+    // sizes spread by about a quarter around their mean; ranges far below a
+    // dedup block's room do with fewer samples
+    p.samples = std::min((bound / ranges < 1024 ? 8 : 32) * p.n_ranges, kMaxSamples);
+    p.on = true;
+    return p;
+}
+
+cudaError_t dedup_pack(const DedupPlan &p, const DedupBufs &d, const InsertArgs &a, uint64_t chunk0,
+                       uint64_t n_chunks, uint64_t begin, uint64_t end, int sms, cudaStream_t s,
+                       uint64_t &launches) {
+    if (begin >= end) return cudaSuccess;
+    const MetaLayout m(p);
+    PackArgs x;
+    x.chunk0 = chunk0;
+    x.chunk_begin = begin;
+    x.chunk_end = end;
+    x.chunk_last = chunk0 + n_chunks;
+    x.codes = (uint32_t *)(d.meta + m.codes);
+    x.valid = (uint16_t *)(d.meta + m.valid);
+    const bool small = p.chunk == kExtractSmall;   // resident blocks of 64 or 256 threads
+    const unsigned grid = (unsigned)std::min<uint64_t>(end - begin, (uint64_t)sms * (small ? 24 : 8));
+    if (small)
+        pack_kernel<kExtractSmall><<<grid, kExtractSmall / 16, 0, s>>>(a, x);
+    else
+        pack_kernel<kExtractChunk><<<grid, kExtractChunk / 16, 0, s>>>(a, x);
+    launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical, uint64_t n_chunks,
+                          uint64_t span, int sms, cudaStream_t s, uint64_t &launches) {
+    const MetaLayout m(p);
+    DedupMeta *meta = (DedupMeta *)(d.meta + m.meta);
+    uint64_t *samples = (uint64_t *)(d.meta + m.samples);
+    PackArgs pa;
+    memset(&pa, 0, sizeof(pa));
+    pa.codes = (uint32_t *)(d.meta + m.codes);
+    pa.valid = (uint16_t *)(d.meta + m.valid);
+    DD_TRY(cudaMemsetAsync(meta, 0, sizeof(DedupMeta), s));
+    const unsigned g = (p.samples + 127) / 128;
+    if (p.kw == 1)
+        sample_kernel<1><<<g, 128, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
+    else
+        sample_kernel<2><<<g, 128, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
+    const int E = sort_items(p.samples);
+    auto *sk = E == 1 ? splitters_kernel<1> : E == 2 ? splitters_kernel<2>
+             : E == 4 ? splitters_kernel<4> : E == 8 ? splitters_kernel<8> : splitters_kernel<16>;
+    DD_TRY(set_smem(sk, std::max(E, 4) * 8192));
+    sk<<<1, 1024, std::max(E, 4) * 8192, s>>>(samples, p.samples, p.n_ranges, last_prefix(p.K),
+                                 (uint64_t *)(d.meta + m.spl), (uint16_t *)(d.meta + m.lut), meta);
+    ExtractArgs x;
+    x.codes = pa.codes;
+    x.valid = pa.valid;
+    x.n_chunks = (unsigned)n_chunks;
+    x.n_ranges = p.n_ranges;
+    x.spl = (const uint64_t *)(d.meta + m.spl);
+    x.lut = (const uint16_t *)(d.meta + m.lut);
+    x.out = d.a;
+    x.piece = (uint32_t *)(d.meta + m.piece);
+    x.starts = (uint16_t *)(d.meta + m.starts);
+    x.meta = meta;
+    launches += 3;
+    if (p.kw == 1)
+        return p.chunk == kExtractSmall
+                   ? extract_variant<1, kExtractSmall>(p.K, canonical, x, 6, sms, s)
+                   : extract_variant<1, kExtractChunk>(p.K, canonical, x, 2, sms, s);
+    return p.chunk == kExtractSmall
+               ? extract_variant<2, kExtractSmall>(p.K, canonical, x, 6, sms, s)
+               : extract_variant<2, kExtractChunk>(p.K, canonical, x, 2, sms, s);
+}
+
+cudaError_t dedup_finish(const DedupPlan &p, const DedupBufs &d, DevCounters *ctr,
+                         uint64_t n_chunks, bool ordered, bool fresh, int sms, cudaStream_t s,
+                         uint64_t &launches) {
+    return p.kw == 1 ? finish_variant<1>(p, d, ctr, n_chunks, ordered, fresh, sms, s, launches)
+                     : finish_variant<2>(p, d, ctr, n_chunks, ordered, fresh, sms, s, launches);
+}
+
+EmitArgs dedup_result(const DedupPlan &p, const DedupBufs &d, const Geometry &G, DevCounters *ctr,
+                      bool ordered) {
+    const MetaLayout m(p);
+    EmitArgs e;
+    memset(&e, 0, sizeof(e));
+    e.G = G;
+    e.keys = p.n_fine ? d.a : d.b;
+    e.mult = d.mult;
+    e.places = (const uint32_t *)(d.meta + m.places);
+    e.offsets = (const uint32_t *)(d.meta + m.offsets);
+    e.n_total = (unsigned)p.total();
+    e.ordered = ordered ? 1 : 0;
+    e.begin = 0;
+    e.end = ~0u;
+    e.ctr = ctr;
+    e.meta = (const DedupMeta *)(d.meta + m.meta);
+    return e;
+}
+
+cudaError_t launch_emit(const EmitArgs &e, int kw, int sms, cudaStream_t s) {
+    const int mode = e.G.eta_log2 < 0 ? kAnyAddress : e.G.dim_x ? kTwoDim : e.G.m_mask ? kFlatPow2 : kFlat;
+    void (*const ks[2][4])(EmitArgs) = {
+        {emit_kernel<1, kAnyAddress>, emit_kernel<1, kFlatPow2>, emit_kernel<1, kFlat>, emit_kernel<1, kTwoDim>},
+        {emit_kernel<2, kAnyAddress>, emit_kernel<2, kFlatPow2>, emit_kernel<2, kFlat>, emit_kernel<2, kTwoDim>}};
+    auto *k = ks[kw - 1][mode];
+    k<<<(unsigned)sms * 4, kEmitThreads, 0, s>>>(e);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_emit_atomic(const EmitArgs &e, int kw, int sms, cudaStream_t s) {
+    if (kw == 1)
+        emit_atomic_kernel<1><<<(unsigned)sms * 4, kEmitThreads, 0, s>>>(e);
+    else
+        emit_atomic_kernel<2><<<(unsigned)sms * 4, kEmitThreads, 0, s>>>(e);
+    return cudaGetLastError();
+}
+
+}  // namespace countbf

@@ -1,78 +1,54 @@
 // Insertion phase of KmerCo (Algorithm 1 with the countBF insert of
 // Algorithm 3) on sm_103a.
 //
-// Work unit: a chunk of consecutive window starts of the flat bases array
-// (kChunk, or kPartChunk in the partitioned design), regardless of read
-// boundaries, so long and short reads balance the same way.  Per chunk a
-// block
-//   1. stages the chunk's bases (plus K-1 halo) in shared memory with
-//      16-byte streaming loads, and marks the read starts inside it in a
-//      break bitmap (no breaks when the reads are one sequence),
-//   2. packs the bases to 2-bit codes (A=0 C=1 G=2 T=3, first base most
-//      significant) with an invalid-base bitmap,
-//   3. keeps the window starts whose K bases are valid and lie in one read,
-//   4. per window: the canonical key (the smaller of forward and reverse
-//      complement by value, or by H_0; Sections 2.2-2.3), k_h MurmurHash3
-//      hashes, one saturating counter increment per hash (Algorithm 3), and
-//      an insert into the distinct-key set (open addressing, linear
-//      probing); keys new to the set are staged in shared memory and
-//      appended to the distinct list with one global atomic per chunk.
+// Two ways lead a call's windows into the countBF and the distinct set:
+//  - by key ranges (kmerco_dedup.cu): the call's distinct keys with their
+//    multiplicities first, then one weighted increment per key and hash; the
+//    kernels that apply those in the partitioned update are here
+//    (repartition_kernel, apply_count_kernel, apply_kernel);
+//  - window by window (insert_kernel, insert_batch_kernel here): for small
+//    calls, handles with a retry limit or a cap on their distinct list, and
+//    when the buffers of the first way cannot be had.
 //
-// Two designs apply the counter increments of step 4:
-//  - atomic: each increment is a compare-and-swap on its 64-bit cell in
-//    global memory;
-//  - partitioned (k_h <= 4, at most 2^30 cells): each increment is emitted
-//    as a 32-bit code (cell within its coarse region, counter within the
-//    cell); the chunk's codes are counting-sorted in shared memory into 64
-//    coarse countBF regions and appended to per-region buffers with one
-//    cursor atomic per region and chunk.  repartition_kernel splits every
-//    region into slices, and one block per slice applies its increments in
-//    shared memory: apply_count_kernel (alpha <= 15) counts them in 32-bit
-//    lanes and adds the counts with saturation (the repartition then writes
-//    each increment as its 16-bit lane index), apply_kernel uses
-//    shared-memory compare-and-swap on the cells.  Either writes the slice
-//    back once.  Increments that do not fit a buffer fall back to the global
-//    compare-and-swap.
-// Saturating increments commute, so both designs give the same countBF.
-#include "kmerco_internal.cuh"
+// insert_kernel: a work unit is a chunk of consecutive window starts of the
+// flat bases array, regardless of read boundaries, so long and short reads
+// balance the same way.  Per chunk a block
+//   1. stages the chunk's bases (plus K-1 halo) in shared memory, 2-bit
+//      packed (A=0 C=1 G=2 T=3, first base most significant), with an
+//      invalid-base bitmap and the read starts inside it in a break bitmap,
+//   2. keeps the window starts whose K bases are valid and lie in one read,
+//   3. per window: the canonical key (the smaller of forward and reverse
+//      complement by value, or by H_0; Sections 2.2-2.3), k_h MurmurHash3
+//      hashes, one saturating counter increment per hash (Algorithm 3), each
+//      a compare-and-swap on its 64-bit cell in global memory, and an insert
+//      into the distinct-key set (open addressing, linear probing); keys new
+//      to the set are staged in shared memory and appended to the distinct
+//      list with one global atomic per chunk.
+//
+// Partitioned update of the first way (at most 2^30 cells): emit_kernel has
+// appended the increments as 32-bit codes to 64 coarse countBF regions;
+// repartition_kernel splits every region into slices, and one block per
+// slice applies its increments in shared memory: apply_count_kernel
+// (alpha <= 15) sums them in 32-bit lanes and adds the sums with saturation
+// (the repartition then writes each increment as its lane index),
+// apply_kernel uses shared-memory compare-and-swap on the cells.  Either
+// writes the slice back once.  Increments that do not fit a buffer are added
+// to the countBF directly.  Saturating increments commute, so every way gives
+// the same countBF.
+#include "kmerco_stage.cuh"
 
 namespace countbf {
 namespace {
 
-// Staging sizes for a chunk of CHUNK window starts.
-template <int CHUNK>
-struct ChunkDims {
-    static constexpr int kPack32 = CHUNK / 16 + 8;   // 16 bases per 32-bit word; chunk + 128 bases
-};
-
-template <int KW, int CHUNK, int PART>
+template <int KW, int CHUNK>
 struct __align__(16) InsertSmem {
-    uint32_t pk[ChunkDims<CHUNK>::kPack32];     // codes; word t at t ^ 1 so pairs read as u64
-    uint16_t inv[ChunkDims<CHUNK>::kPack32];    // bit j of inv[t]: base 16t + j is not ACGTacgt
-    uint32_t brk[ChunkDims<CHUNK>::kPack32 / 2];  // bit q: a read starts at base q of the chunk
+    StageSmem<CHUNK> st;
     uint16_t vpos[CHUNK];                       // valid window starts
     uint64_t fresh[CHUNK * KW];                 // keys new to the distinct set
-    // partitioned design: the chunk's counter-increment codes
-    uint32_t staged[PART ? CHUNK * kPartMaxHash : 1];
-    uint32_t sorted[PART ? CHUNK * kPartMaxHash : 1];
-    uint8_t sbin[PART == 2 ? CHUNK * kPartMaxHash : 1];   // coarse region of staged[i]
-    unsigned hist[PART ? kCoarseBins : 1];
-    unsigned start[PART ? kCoarseBins : 1];
-    unsigned fill[PART ? kCoarseBins : 1];
-    unsigned long long base[PART ? kCoarseBins : 1];
     unsigned nvalid;
     unsigned nfresh;
-    unsigned nupd;
     unsigned long long fresh_base;
 };
-
-// 64 bits of a bitmap starting at bit p.
-__device__ __forceinline__ uint64_t bits_at(const uint64_t *bm, unsigned p) {
-    unsigned w = p >> 6, s = p & 63;
-    uint64_t v = bm[w] >> s;
-    if (s) v |= bm[w + 1] << (64 - s);
-    return v;
-}
 
 __device__ __forceinline__ uint64_t load_cg(const uint64_t *p) { return __ldcg(p); }
 
@@ -138,7 +114,8 @@ __device__ __forceinline__ void sat_increment(uint64_t *cells, uint64_t c, unsig
 // free, so a reset only moves to the next tag instead of clearing the table.
 // Without spare bits (mask 0) a free slot is all ones, cleared at reset.
 // For one-word keys `first` is an already loaded value of the home slot
-// (kEmptyKey - 1 when none was loaded, a value no slot holds).
+// (kEmptyKey - 1 when none was loaded, a value no slot holds); for two-word
+// keys *first2 is, when not null.
 __device__ __forceinline__ bool slot_free(uint64_t top, const SetTag &t) {
     return t.mask ? (top & t.mask) != t.tag : top == kEmptyKey;
 }
@@ -147,7 +124,8 @@ template <int KW>
 __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64_t th,
                                            uint64_t klo, uint64_t khi, const SetTag &t,
                                            uint32_t limit, unsigned *err, uint64_t pol,
-                                           uint64_t first = kEmptyKey - 1) {
+                                           uint64_t first = kEmptyKey - 1,
+                                           const ulonglong2 *first2 = nullptr) {
     uint64_t slot = __umul64hi(th, cap);
     for (uint32_t it = 0;; ++it) {
         if (KW == 1) {
@@ -169,7 +147,7 @@ __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64
             // written), is decided by the 128-bit compare-and-swap, whose
             // result is the slot's real contents.
             const uint64_t whi = khi | t.tag;
-            ulonglong2 v = __ldcg((const ulonglong2 *)(table + 2 * slot));
+            ulonglong2 v = it == 0 && first2 ? *first2 : __ldcg((const ulonglong2 *)(table + 2 * slot));
             for (;;) {
                 if (v.x == klo && v.y == whi) return false;
                 const bool free = t.mask ? slot_free(v.y, t) : (v.x == kEmptyKey || v.y == kEmptyKey);
@@ -191,114 +169,28 @@ __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64
     }
 }
 
-// One chunk of CHUNK window starts (steps 1-5 above) for the sample
+// One chunk of CHUNK window starts (the steps above) for the sample
 // described by `a`; counts its windows into my_windows / my_skipped.
-template <int KW, int CHUNK, int PART>
+template <int KW, int CHUNK>
 __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chunk,
-                                              InsertSmem<KW, CHUNK, PART> &S, uint64_t pol_keep,
+                                              InsertSmem<KW, CHUNK> &S, uint64_t pol_keep,
                                               uint64_t pol_stream,
                                               unsigned long long &my_windows,
                                               unsigned long long &my_skipped) {
     constexpr int kPack32 = ChunkDims<CHUNK>::kPack32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = a.K;
-    const uint64_t total = a.last - a.first;
     const Geometry &G = a.G;
-    const uint64_t c0 = chunk * (uint64_t)CHUNK;
-    const uint64_t e = min(c0 + (uint64_t)(CHUNK + K - 1), total);
-    const unsigned nb = (unsigned)(e - c0);
-    const uintptr_t src = (uintptr_t)(a.bases + c0);
-    const unsigned head = (unsigned)(src & 15);
-    const uintptr_t abase = src - head;
-
-    // 1. read starts inside the chunk's span (none when the reads are one
-    //    sequence); S.brk is zero on entry
-    for (uint64_t r = (uint64_t)a.first_read[chunk] + tid; !a.whole_file && r < a.nreads;
-         r += kInsertThreads) {
-        uint64_t s = a.offsets[r] - a.first;
-        if (s >= c0 + nb) break;
-        if (s < c0) continue;   // only with decreasing offsets, which the host rejects
-        unsigned q = (unsigned)(s - c0);
-        if (q > 0) atomicOr(&S.brk[q >> 5], 1u << (q & 31));
-    }
+    const unsigned nb = stage_chunk<CHUNK, kInsertThreads>(a, chunk, S.st);
     if (tid == 0) {
         S.nvalid = 0;
         S.nfresh = 0;
-        S.nupd = 0;
-    }
-    if (PART && tid < kCoarseBins) {
-        S.hist[tid] = 0;
-        S.fill[tid] = 0;
-    }
-    // 2. bases [16t, 16t + 16) of the span straight from global memory (the
-    //    two 16-byte vectors holding them: whole ones with streaming loads,
-    //    the partial ones at the span's ends bytewise, 'N' outside it), then
-    //    2-bit codes + invalid bits
-    for (int t = tid; t < kPack32; t += kInsertThreads) {
-        uint32_t w[8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned lo = (unsigned)(t + h) << 4;
-            if (lo >= head && lo + 16 <= head + nb) {
-                const uint4 v = __ldcs((const uint4 *)(abase + lo));
-                w[4 * h] = v.x;
-                w[4 * h + 1] = v.y;
-                w[4 * h + 2] = v.z;
-                w[4 * h + 3] = v.w;
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t word = 0;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const unsigned b = lo + 4 * q + k;
-                        const unsigned c = b >= head && b < head + nb
-                                               ? *(const uint8_t *)(abase + b) : (unsigned)'N';
-                        word |= c << (8 * k);
-                    }
-                    w[4 * h + q] = word;
-                }
-            }
-        }
-        // the 16 bytes start `head` bytes into the 32 loaded ones
-        const unsigned hb = (head & 3) * 8;
-        uint32_t x[4];
-        switch (head >> 2) {
-        case 0:
-#pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = __funnelshift_r(w[i], w[i + 1], hb);
-            break;
-        case 1:
-#pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = __funnelshift_r(w[i + 1], w[i + 2], hb);
-            break;
-        case 2:
-#pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = __funnelshift_r(w[i + 2], w[i + 3], hb);
-            break;
-        default:
-#pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = __funnelshift_r(w[i + 3], w[i + 4], hb);
-            break;
-        }
-        uint32_t code = 0, bad = 0;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const unsigned c = (x[j >> 2] >> (8 * (j & 3))) & 0xFFu;
-            const unsigned u = c | 0x20u;
-            const bool ok = (u == 'a') | (u == 'c') | (u == 'g') | (u == 't');
-            const unsigned cd = ((c >> 1) ^ (c >> 2)) & 3u;   // A,a->0 C,c->1 G,g->2 T,t->3
-            code = (code << 2) | (ok ? cd : 0u);
-            bad |= (ok ? 0u : 1u) << j;
-        }
-        S.pk[t ^ 1] = code;
-        S.inv[t] = (uint16_t)bad;
     }
     __syncthreads();
 
-    // 3. window starts: inside one read, K valid bases
-    const uint64_t *inv64 = (const uint64_t *)S.inv;
-    const uint64_t *brk64 = (const uint64_t *)S.brk;
+    // window starts: inside one read, K valid bases
+    const uint64_t *inv64 = (const uint64_t *)S.st.inv;
+    const uint64_t *brk64 = (const uint64_t *)S.st.brk;
     const uint64_t maskK = K == 64 ? ~0ull : ((1ull << K) - 1);
     const uint64_t maskK1 = (1ull << (K - 1)) - 1;
     for (int p0 = 0; p0 < CHUNK; p0 += kInsertThreads) {
@@ -315,10 +207,10 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
     }
     __syncthreads();
 
-    // 4. per valid window: canonical key, hashes, counter updates, set insert
-    for (int i = tid; i < kPack32 / 2; i += kInsertThreads) S.brk[i] = 0;   // for the next chunk
+    // per valid window: canonical key, hashes, counter updates, set insert
+    for (int i = tid; i < kPack32 / 2; i += kInsertThreads) S.st.brk[i] = 0;   // for the next chunk
     const unsigned nvalid = S.nvalid;
-    const uint64_t *pk64 = (const uint64_t *)S.pk;
+    const uint64_t *pk64 = (const uint64_t *)S.st.pk;
     for (unsigned i0 = (unsigned)warp * 32; i0 < nvalid; i0 += kInsertThreads) {
         const unsigned i = i0 + lane;
         const bool active = i < nvalid;
@@ -377,53 +269,10 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
 
         uint64_t table_hash = 0, table_first = kEmptyKey - 1;
         const uint64_t k1m = KW == 1 ? premix8(klo) : 0;
-        if (PART) {
-            // Partitioned design: stage one 32-bit code per increment, the
-            // cell within its coarse region (up to 24 bits) above the counter
-            // within the cell (6 bits), the region itself beside it.  A
-            // window's k_h codes sit together: one reservation per warp.  The
-            // hashes go two per loop trip (a smaller loop body measured
-            // faster than all k_h at once); the distinct-set home slot is
-            // loaded as soon as the first hash gives it.
-            const unsigned nh = (unsigned)G.nhash;   // at most kPartMaxHash
-            const unsigned bal = __ballot_sync(0xffffffffu, active);
-            unsigned base = 0;
-            if (lane == 0 && bal) base = atomicAdd(&S.nupd, nh * (unsigned)__popc(bal));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            base += nh * (unsigned)__popc(bal & ((1u << lane) - 1));
-            if (active) {
-#pragma unroll 2
-                for (unsigned j = 0; j < nh; ++j) {
-                    uint64_t h1, h2, cell;
-                    unsigned slot;
-                    if (KW == 1)
-                        murmur8(k1m, j, h1, h2);
-                    else
-                        murmur16(klo, khi, j, h1, h2);
-                    if (j == 0) {
-                        table_hash = h2;
-                        if (KW == 1)
-                            table_first = load_hint(a.table + __umul64hi(table_hash, a.cap),
-                                                    pol_stream);
-                    }
-                    address(G, h1, cell, slot);
-                    const unsigned bin = (unsigned)(cell >> a.coarse_shift);
-                    const uint32_t code =
-                        ((uint32_t)(cell & ((1ull << a.coarse_shift) - 1)) << 6) | slot;
-                    if (PART == 2) {   // region beside the code
-                        S.staged[base + j] = code;
-                        S.sbin[base + j] = (uint8_t)bin;
-                    } else {           // region in the top 6 bits (coarse_shift <= 20)
-                        S.staged[base + j] = (bin << 26) | code;
-                    }
-                    atomicAdd(&S.hist[bin], 1u);
-                }
-            }
-        }
-        // Atomic design: all loads of a group of four hashes (and, in the
-        // first group, the distinct-set home slot) are issued together, then
-        // all first compare-and-swap attempts; only failed attempts retry.
-        for (int a0 = 0; !PART && a0 < G.nhash; a0 += 4) {
+        // All loads of a group of four hashes (and, in the first group, the
+        // distinct-set home slot) are issued together, then all first
+        // compare-and-swap attempts; only failed attempts retry.
+        for (int a0 = 0; a0 < G.nhash; a0 += 4) {
             uint64_t cell[4], cur[4], prev[4];
             unsigned sh[4], slot[4];
             bool use[4], need[4];
@@ -481,11 +330,9 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
     }
     __syncthreads();
 
-    // 4b. reservations, all in one phase: the distinct-list run of this
-    //     chunk's new keys, and (partitioned design) one cursor atomic per
-    //     coarse region for the chunk's increment codes
+    // the distinct-list run of this chunk's new keys
     const unsigned nfresh = S.nfresh;
-    if (tid == kCoarseBins && nfresh) {
+    if (tid == 0 && nfresh) {
         unsigned long long b = atomicAdd(&a.ctr->distinct, (unsigned long long)nfresh);
         if (b + nfresh > a.dlist_cap) {
             atomicOr(&a.ctr->error, kErrListFull);
@@ -493,67 +340,8 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
         }
         S.fresh_base = b;
     }
-    if (PART) {
-        const unsigned nupd = S.nupd;
-        if (tid < kCoarseBins) {   // warps 0 and 1: prefix over the regions
-            const unsigned n = S.hist[tid];
-            unsigned incl = n, below = 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= (unsigned)o) incl += t;
-            }
-            if (tid >= 32) {   // warp 1 starts after all of warp 0's regions
-                below = S.hist[tid - 32];
-#pragma unroll
-                for (int o = 16; o; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
-            }
-            S.start[tid] = below + incl - n;
-            unsigned long long b0 = ~0ull;
-            if (n) {
-                b0 = atomicAdd(a.coarse_cursor + tid, (unsigned long long)n);
-                if (b0 + n > a.coarse_cap)
-                    b0 = ~0ull;   // region full: these go to the global fallback
-                else
-                    atomicAdd(a.coarse_written + tid, (unsigned long long)n);
-            }
-            S.base[tid] = b0;
-        }
-        __syncthreads();
-        // 4c. counting sort of the codes by coarse region in shared memory
-        for (unsigned i = tid; i < nupd; i += kInsertThreads) {
-            if (PART == 2) {
-                const unsigned bin = S.sbin[i];
-                S.sorted[S.start[bin] + atomicAdd(&S.fill[bin], 1u)] = S.staged[i];
-            } else {
-                const uint32_t c = S.staged[i];
-                const unsigned bin = c >> 26;
-                S.sorted[S.start[bin] + atomicAdd(&S.fill[bin], 1u)] = c & 0x3FFFFFFu;
-            }
-        }
-        __syncthreads();
-        // 4d. one warp per region run: contiguous stores into the region
-        for (unsigned bin = warp; bin < kCoarseBins; bin += kInsertThreads / 32) {
-            const unsigned n = S.hist[bin], s0 = S.start[bin];
-            const unsigned long long b0 = S.base[bin];
-            uint32_t *dst = b0 != ~0ull ? a.coarse + (uint64_t)bin * a.coarse_cap + b0 : nullptr;
-            for (unsigned i = lane; i < n; i += 32) {
-                const uint32_t code = S.sorted[s0 + i];
-                if (dst) {
-                    __stcs(dst + i, code);
-                } else {
-                    const uint64_t cell = ((uint64_t)bin << a.coarse_shift) | (code >> 6);
-                    const unsigned shift = (code & 63u) * (unsigned)G.alpha;
-                    sat_increment(G.cells, cell, shift, G.maxc, load_cg(G.cells + cell),
-                                  G.cas_limit, &a.ctr->error);
-                }
-            }
-        }
-    } else {
-        __syncthreads();
-    }
+    __syncthreads();
 
-    // 5. this chunk's new keys into the distinct list
     if (nfresh) {
         const unsigned long long b = S.fresh_base;
         if (b != ~0ull)
@@ -579,17 +367,15 @@ __device__ __forceinline__ void flush_totals(DevCounters *ctr, unsigned long lon
     k = 0;
 }
 
-template <int KW, int CHUNK, int PART>
+template <int KW, int CHUNK>
 __global__ void __launch_bounds__(kInsertThreads, 4) insert_kernel(InsertArgs a) {
-    // dynamic: the partitioned variants need more than 48 KiB
-    extern __shared__ __align__(16) unsigned char insert_smem[];
-    InsertSmem<KW, CHUNK, PART> &S = *reinterpret_cast<InsertSmem<KW, CHUNK, PART> *>(insert_smem);
-    for (int i = threadIdx.x; i < ChunkDims<CHUNK>::kPack32 / 2; i += kInsertThreads) S.brk[i] = 0;
+    __shared__ InsertSmem<KW, CHUNK> S;
+    for (int i = threadIdx.x; i < ChunkDims<CHUNK>::kPack32 / 2; i += kInsertThreads) S.st.brk[i] = 0;
     __syncthreads();
     const uint64_t pol_keep = policy_keep(), pol_stream = policy_stream();
     unsigned long long my_windows = 0, my_skipped = 0;
     for (uint64_t chunk = a.chunk_begin + blockIdx.x; chunk < a.nchunks; chunk += gridDim.x)
-        process_chunk<KW, CHUNK, PART>(a, chunk, S, pol_keep, pol_stream, my_windows, my_skipped);
+        process_chunk<KW, CHUNK>(a, chunk, S, pol_keep, pol_stream, my_windows, my_skipped);
     flush_totals(a.ctr, my_windows, my_skipped);
 }
 
@@ -602,11 +388,11 @@ template <int KW, int CHUNK>
 __global__ void __launch_bounds__(kInsertThreads, 4) insert_batch_kernel(
     const InsertArgs *args, const unsigned long long *chunk_end, int nsamples,
     unsigned long long total_chunks) {
-    __shared__ InsertSmem<KW, CHUNK, 0> S;
+    __shared__ InsertSmem<KW, CHUNK> S;
     __shared__ InsertArgs A;
     const uint64_t pol_keep = policy_keep(), pol_stream = policy_stream();
     unsigned long long my_windows = 0, my_skipped = 0;
-    for (int i = threadIdx.x; i < ChunkDims<CHUNK>::kPack32 / 2; i += kInsertThreads) S.brk[i] = 0;
+    for (int i = threadIdx.x; i < ChunkDims<CHUNK>::kPack32 / 2; i += kInsertThreads) S.st.brk[i] = 0;
     int s = -1;
     unsigned long long s_begin = 0;
     for (unsigned long long chunk = blockIdx.x; chunk < total_chunks; chunk += gridDim.x) {
@@ -620,8 +406,8 @@ __global__ void __launch_bounds__(kInsertThreads, 4) insert_batch_kernel(
             s_begin = t ? chunk_end[t - 1] : 0;
             __syncthreads();
         }
-        process_chunk<KW, CHUNK, 0>(A, chunk - s_begin, S, pol_keep, pol_stream, my_windows,
-                                        my_skipped);
+        process_chunk<KW, CHUNK>(A, chunk - s_begin, S, pol_keep, pol_stream, my_windows,
+                                 my_skipped);
     }
     if (s >= 0) flush_totals(A.ctr, my_windows, my_skipped);
 }
@@ -726,42 +512,78 @@ __global__ void first_read_batch_kernel(const InsertArgs *args, const unsigned l
     const_cast<uint32_t *>(a.first_read)[local] = (uint32_t)rlo;
 }
 
-// Re-insert keys into a distinct set (growing a set, or merging another
-// handle's keys).  With dlist != nullptr keys new to the set are appended.
+// Insert keys into a distinct set (filling or growing a set, a call's or
+// another handle's distinct keys).  With dlist != nullptr keys new to the set
+// are appended.  n32 / n64: when not null, the number of keys, at most n, is
+// read there.
+// A block takes kReinsertTile keys at a time and reserves the list places of
+// its new keys with one atomic (an atomic per warp, all on one address, took
+// most of the kernel's time).
+constexpr int kReinsertTile = 1024;
+
 template <int KW>
-__global__ void reinsert_kernel(const uint64_t *keys, uint64_t n, uint64_t *table, uint64_t cap,
-                                SetTag tag, uint64_t *dlist, uint64_t dlist_cap, DevCounters *ctr,
-                                uint32_t probe_limit) {
-    const int lane = threadIdx.x & 31;
-    for (uint64_t i0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) & ~31ull; i0 < n;
-         i0 += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t i = i0 + lane;
-        bool isnew = false;
-        uint64_t klo = 0, khi = 0;
-        if (i < n) {
-            klo = keys[i * KW];
-            khi = KW == 2 ? keys[i * KW + 1] : 0;
-            uint64_t h1, h2;
-            if (KW == 1)
-                murmur8(premix8(klo), 0, h1, h2);
-            else
-                murmur16(klo, khi, 0, h1, h2);
-            isnew = set_insert<KW>(table, cap, h2, klo, khi, tag, probe_limit, &ctr->error,
-                                   policy_stream());
+__global__ void __launch_bounds__(256) reinsert_kernel(const uint64_t *keys, uint64_t n,
+                                                       const unsigned *n32,
+                                                       const unsigned long long *n64,
+                                                       uint64_t *table, uint64_t cap, SetTag tag,
+                                                       uint64_t *dlist, uint64_t dlist_cap,
+                                                       DevCounters *ctr, uint32_t probe_limit) {
+    constexpr int PER = kReinsertTile / 256;
+    __shared__ unsigned long long at0;
+    if (n32) n = min(n, (uint64_t)*n32);
+    if (n64) n = min(n, (uint64_t)*n64);
+    for (uint64_t i0 = (uint64_t)blockIdx.x * kReinsertTile; i0 < n;
+         i0 += (uint64_t)gridDim.x * kReinsertTile) {
+        uint64_t klo[PER], khi[PER];
+        unsigned fresh = 0;   // bit q: key q is new
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const uint64_t i = i0 + q * 256 + threadIdx.x;
+            klo[q] = khi[q] = 0;
+            if (i < n) {
+                klo[q] = keys[i * KW];
+                if (KW == 2) khi[q] = keys[i * KW + 1];
+            }
         }
-        if (dlist) {
-            const unsigned bal = __ballot_sync(0xffffffffu, isnew);
-            unsigned long long base = 0;
-            if (lane == 0 && bal) base = atomicAdd(&ctr->distinct, (unsigned long long)__popc(bal));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (isnew) {
-                const uint64_t slot = base + __popc(bal & ((1u << lane) - 1));
-                if (slot < dlist_cap) {
-                    dlist[slot * KW] = klo;
-                    if (KW == 2) dlist[slot * KW + 1] = khi;
-                } else {
-                    atomicOr(&ctr->error, kErrListFull);
-                }
+        uint64_t th[PER], first[PER];
+        ulonglong2 first2[KW == 2 ? PER : 1];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {   // the home slots' loads in flight together
+            uint64_t h1;
+            if (KW == 1)
+                murmur8(premix8(klo[q]), 0, h1, th[q]);
+            else
+                murmur16(klo[q], khi[q], 0, h1, th[q]);
+            first[q] = kEmptyKey - 1;
+            if (i0 + q * 256 + threadIdx.x < n) {
+                const uint64_t home = __umul64hi(th[q], cap);
+                if (KW == 1)
+                    first[q] = load_hint(table + home, policy_stream());
+                else
+                    first2[q] = __ldcg((const ulonglong2 *)(table + 2 * home));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+            if (i0 + q * 256 + threadIdx.x < n &&
+                set_insert<KW>(table, cap, th[q], klo[q], khi[q], tag, probe_limit, &ctr->error,
+                               policy_stream(), first[q], KW == 2 ? &first2[q] : nullptr))
+                fresh |= 1u << q;
+        if (!dlist) continue;
+        unsigned tot;
+        unsigned at = block_exclusive_scan<unsigned, 256>(__popc(fresh), tot);
+        if (threadIdx.x == 0) at0 = tot ? atomicAdd(&ctr->distinct, (unsigned long long)tot) : 0;
+        __syncthreads();
+        const unsigned long long base = at0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (!((fresh >> q) & 1u)) continue;
+            const uint64_t slot = base + at++;
+            if (slot < dlist_cap) {
+                dlist[slot * KW] = klo[q];
+                if (KW == 2) dlist[slot * KW + 1] = khi[q];
+            } else {
+                atomicOr(&ctr->error, kErrListFull);
             }
         }
     }
@@ -788,121 +610,137 @@ __device__ __forceinline__ void repart_scan(const unsigned *v, unsigned *out, un
 }
 
 // Split each coarse region's increment codes into slices of 2^slice_shift
-// cells.  Block (x, y) takes tile x of coarse region y.  MAXF bounds the
-// slices per region (2^(coarse_shift - slice_shift)).  With LANES a slice
-// code is the 16-bit counting lane (counter << slice_shift) | cell of the
-// counting apply, else the 32-bit (cell << 6) | counter.
+// cells.  The blocks walk the tiles of all regions (the regions' code counts
+// are on the device, so an idle pass costs one short launch).  MAXF bounds
+// the slices per region (2^(coarse_shift - slice_shift)).  With LANES a slice
+// code is the counting lane (counter << slice_shift) | cell in its low
+// kLaneBits bits with the increment less one above, else the region's code
+// less the slice's bits.
 template <int MAXF, bool LANES>
 __global__ void __launch_bounds__(kRepartThreads, 3) repartition_kernel(PartArgs p) {
     extern __shared__ uint32_t sorted[];   // the tile's codes grouped by slice
     __shared__ unsigned hist[MAXF], start[MAXF], fill[MAXF];
     __shared__ unsigned long long base[MAXF];
-    const unsigned b = blockIdx.y, tid = threadIdx.x;
-    const uint64_t n = p.coarse_written[b];
-    const uint64_t t0 = (uint64_t)blockIdx.x * kRepartTile;
-    if (t0 >= n) return;
-    const unsigned cnt = (unsigned)min((uint64_t)kRepartTile, n - t0);
-    const int fsh = 6 + p.slice_shift;                            // code >> fsh = slice
+    __shared__ unsigned tiles[kCoarseBins + 1];   // tiles of the regions before each one
+    const unsigned tid = threadIdx.x;
+    if (tid == 0) tiles[0] = 0;
+    if (tid < kCoarseBins)
+        tiles[tid + 1] = (unsigned)((p.coarse_written[tid] + kRepartTile - 1) / kRepartTile);
+    __syncthreads();
+    if (tid == 0)
+        for (int i = 0; i < kCoarseBins; ++i) tiles[i + 1] += tiles[i];
+    __syncthreads();
+    const unsigned total = tiles[kCoarseBins];
+    const int lb = p.slot_bits + p.w_bits;                        // bits under the cell
+    const int fsh = lb + p.slice_shift;                           // code >> fsh = slice
     const unsigned fpc = 1u << (p.coarse_shift - p.slice_shift);  // slices per coarse region
-    for (unsigned f = tid; f < fpc; f += kRepartThreads) {
-        hist[f] = 0;
-        fill[f] = 0;
-    }
-    __syncthreads();
-    // 16 codes per thread, all loads issued before use (the region is 16-byte
-    // aligned: coarse_cap is a multiple of 4 and t0 of kRepartTile)
-    const uint32_t *src = p.coarse + (uint64_t)b * p.coarse_cap + t0;
-    uint32_t c16[16];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const unsigned i = 4 * (tid + j * kRepartThreads);
-        if (i + 4 <= cnt) {
-            const uint4 v = __ldcs((const uint4 *)(src + i));
-            c16[4 * j] = v.x;
-            c16[4 * j + 1] = v.y;
-            c16[4 * j + 2] = v.z;
-            c16[4 * j + 3] = v.w;
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) c16[4 * j + q] = i + q < cnt ? src[i + q] : 0u;
+    const uint32_t smask = (1u << p.slice_shift) - 1, fmask = (1u << fsh) - 1;
+    const uint32_t slot_mask = (1u << p.slot_bits) - 1, w_mask = (1u << p.w_bits) - 1;
+    for (unsigned t = blockIdx.x; t < total; t += gridDim.x) {
+        unsigned b = 0;   // the region of tile t
+        for (unsigned step = kCoarseBins / 2; step; step >>= 1)
+            if (tiles[b + step] <= t) b += step;
+        const uint64_t n = p.coarse_written[b];
+        const uint64_t t0 = (uint64_t)(t - tiles[b]) * kRepartTile;
+        const unsigned cnt = (unsigned)min((uint64_t)kRepartTile, n - t0);
+        for (unsigned f = tid; f < fpc; f += kRepartThreads) {
+            hist[f] = 0;
+            fill[f] = 0;
         }
-    }
+        __syncthreads();
+        // 16 codes per thread, all loads issued before use (the region is 16-byte
+        // aligned: coarse_cap is a multiple of 4 and t0 of kRepartTile)
+        const uint32_t *src = p.coarse + (uint64_t)b * p.coarse_cap + t0;
+        uint32_t c16[16];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const unsigned i = 4 * (tid + j * kRepartThreads);
+        for (int j = 0; j < 4; ++j) {
+            const unsigned i = 4 * (tid + j * kRepartThreads);
+            if (i + 4 <= cnt) {
+                const uint4 v = __ldcs((const uint4 *)(src + i));
+                c16[4 * j] = v.x;
+                c16[4 * j + 1] = v.y;
+                c16[4 * j + 2] = v.z;
+                c16[4 * j + 3] = v.w;
+            } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (i + q < cnt) atomicAdd(&hist[c16[4 * j + q] >> fsh], 1u);
-    }
-    __syncthreads();
-    if (MAXF <= 64) {
-        if (tid < fpc) {
-            unsigned pre = 0;
-            for (unsigned f = 0; f < tid; ++f) pre += hist[f];
-            start[tid] = pre;
-        }
-    } else {
-        repart_scan<(MAXF + kRepartThreads - 1) / kRepartThreads>(hist, start, fpc);
-    }
-    for (unsigned f = tid; f < fpc; f += kRepartThreads) {
-        const unsigned m = hist[f];
-        unsigned long long b0 = ~0ull;
-        if (m) {
-            const uint64_t F = (uint64_t)b * fpc + f;
-            b0 = atomicAdd(p.fine_cursor + F, (unsigned long long)m);
-            if (b0 + m > p.fine_cap)
-                b0 = ~0ull;
-            else
-                atomicAdd(p.fine_written + F, (unsigned long long)m);
-        }
-        base[f] = b0;
-    }
-    __syncthreads();
-    // group the codes by slice, straight from registers
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const unsigned i = 4 * (tid + j * kRepartThreads);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (i + q < cnt) {
-                const unsigned f = c16[4 * j + q] >> fsh;
-                sorted[start[f] + atomicAdd(&fill[f], 1u)] = c16[4 * j + q];
+                for (int q = 0; q < 4; ++q) c16[4 * j + q] = i + q < cnt ? src[i + q] : 0u;
             }
         }
-    }
-    __syncthreads();
-    const uint32_t smask = (1u << p.slice_shift) - 1;
-    for (unsigned i = tid; i < cnt; i += kRepartThreads) {
-        const uint32_t code = sorted[i];
-        const uint32_t word = code >> 6;
-        const unsigned f = word >> p.slice_shift;
-        const unsigned long long b0 = base[f];
-        if (b0 != ~0ull) {
-            const uint64_t F = (uint64_t)b * fpc + f;
-            const uint64_t at = F * p.fine_cap + b0 + (i - start[f]);
-            if (LANES)
-                __stcs((unsigned short *)p.fine + at,
-                       (unsigned short)(((code & 63u) << p.slice_shift) | (word & smask)));
-            else
-                __stcs((uint32_t *)p.fine + at, ((word & smask) << 6) | (code & 63u));
-        } else {
-            const uint64_t cell = ((uint64_t)b << p.coarse_shift) | word;
-            sat_increment(p.G.cells, cell, (code & 63u) * (unsigned)p.G.alpha, p.G.maxc,
-                          load_cg(p.G.cells + cell), p.G.cas_limit, &p.ctr->error);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned i = 4 * (tid + j * kRepartThreads);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q < cnt) atomicAdd(&hist[c16[4 * j + q] >> fsh], 1u);
         }
+        __syncthreads();
+        if (MAXF <= 64) {
+            if (tid < fpc) {
+                unsigned pre = 0;
+                for (unsigned f = 0; f < tid; ++f) pre += hist[f];
+                start[tid] = pre;
+            }
+        } else {
+            repart_scan<(MAXF + kRepartThreads - 1) / kRepartThreads>(hist, start, fpc);
+        }
+        for (unsigned f = tid; f < fpc; f += kRepartThreads) {
+            const unsigned m = hist[f];
+            unsigned long long b0 = ~0ull;
+            if (m) {
+                const uint64_t F = (uint64_t)b * fpc + f;
+                b0 = atomicAdd(p.fine_cursor + F, (unsigned long long)m);
+                if (b0 + m > p.fine_cap)
+                    b0 = ~0ull;
+                else
+                    atomicAdd(p.fine_written + F, (unsigned long long)m);
+            }
+            base[f] = b0;
+        }
+        __syncthreads();
+        // group the codes by slice, straight from registers
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned i = 4 * (tid + j * kRepartThreads);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (i + q < cnt) {
+                    const unsigned f = c16[4 * j + q] >> fsh;
+                    sorted[start[f] + atomicAdd(&fill[f], 1u)] = c16[4 * j + q];
+                }
+            }
+        }
+        __syncthreads();
+        for (unsigned i = tid; i < cnt; i += kRepartThreads) {
+            const uint32_t code = sorted[i];
+            const unsigned f = code >> fsh;
+            const unsigned long long b0 = base[f];
+            const uint32_t slot = (code >> p.w_bits) & slot_mask;
+            if (b0 != ~0ull) {
+                const uint64_t F = (uint64_t)b * fpc + f;
+                const uint64_t at = F * p.fine_cap + b0 + (i - start[f]);
+                const uint32_t out =
+                    LANES ? ((code & w_mask) << kLaneBits) | (slot << p.slice_shift) |
+                                ((code >> lb) & smask)
+                          : code & fmask;
+                __stcs(p.fine + at, out);
+            } else {
+                const uint64_t cell = ((uint64_t)b << p.coarse_shift) | (code >> lb);
+                sat_add(p.G.cells, cell, slot * (unsigned)p.G.alpha, p.G.maxc,
+                        (code & w_mask) + 1ull, load_cg(p.G.cells + cell), p.G.cas_limit,
+                        &p.ctr->error);
+            }
+        }
+        __syncthreads();   // sorted, start and base are free again
     }
 }
 
 // One slice of 2^slice_shift cells per block: load it into shared memory,
 // apply its increment codes with shared-memory compare-and-swap (saturating
-// at 2^alpha - 1), write it back.  LIMITED takes the retry bound from the
-// handle (a retry limit set for testing); the default bound is a constant,
-// which keeps the retry loop measurably faster.  With HALF (alpha divides
-// 32, so no counter straddles the middle of a cell) each update is a 32-bit
-// compare-and-swap on the half-cell that holds the counter.  Slices are
-// 64 KiB, three blocks per SM, so one block's slice load and store overlap
-// the other blocks' updates.
-template <bool LIMITED, bool HALF>
+// at 2^alpha - 1), write it back.  With HALF (alpha divides 32, so no counter
+// straddles the middle of a cell) each update is a 32-bit compare-and-swap on
+// the half-cell that holds the counter.  Slices are 64 KiB, three blocks per
+// SM, so one block's slice load and store overlap the other blocks' updates.
+template <bool HALF>
 __global__ void __launch_bounds__(kCasApplyThreads, 3) apply_kernel(ApplyArgs p) {
     extern __shared__ unsigned long long cells_s[];
     const uint64_t s = blockIdx.x;
@@ -913,8 +751,10 @@ __global__ void __launch_bounds__(kCasApplyThreads, 3) apply_kernel(ApplyArgs p)
     if (n == 0) return;   // no increments for this slice
     for (unsigned i = threadIdx.x; i < nw; i += kCasApplyThreads) cells_s[i] = p.G.cells[w0 + i];
     __syncthreads();
-    const uint32_t *src = (const uint32_t *)p.codes + s * p.cap;   // 16-byte aligned: cap is a multiple of 4
+    const uint32_t *src = p.codes + s * p.cap;   // 16-byte aligned: cap is a multiple of 4
     const uint32_t wmask = (uint32_t)(slice - 1);
+    const uint32_t slot_mask = (1u << p.slot_bits) - 1, inc_mask = (1u << p.w_bits) - 1;
+    const int lb = p.slot_bits + p.w_bits;
     const uint64_t maxc = p.G.maxc;
     const unsigned alpha = (unsigned)p.G.alpha;
     // eight codes per thread in flight (two 16-byte loads), then their updates
@@ -944,18 +784,20 @@ __global__ void __launch_bounds__(kCasApplyThreads, 3) apply_kernel(ApplyArgs p)
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             if (!((valid >> q) & 1u)) continue;   // past the end
-            const unsigned w = (code[q] >> 6) & wmask;
-            const unsigned shift = (code[q] & 63u) * alpha;
+            const unsigned w = (code[q] >> lb) & wmask;
+            const unsigned shift = ((code[q] >> p.w_bits) & slot_mask) * alpha;
+            const unsigned inc = (code[q] & inc_mask) + 1;
             if (HALF) {   // the little-endian half-cell holding the counter
                 unsigned *h32 = (unsigned *)cells_s + 2 * w + (shift >> 5);
                 const unsigned sh = shift & 31u, mc = (unsigned)maxc;
                 unsigned old = *h32;
                 for (uint32_t it = 0;; ++it) {
-                    if (((old >> sh) & mc) == mc) break;
-                    const unsigned prev = atomicCAS(h32, old, old + (1u << sh));
+                    const unsigned room = mc - ((old >> sh) & mc);
+                    if (room == 0) break;
+                    const unsigned prev = atomicCAS(h32, old, old + (min(inc, room) << sh));
                     if (prev == old) break;
                     old = prev;
-                    if (it >= (LIMITED ? p.G.cas_limit : kCasLimit)) {
+                    if (it >= kCasLimit) {
                         atomicOr(&p.ctr->error, kErrCasLimit);
                         break;
                     }
@@ -964,11 +806,13 @@ __global__ void __launch_bounds__(kCasApplyThreads, 3) apply_kernel(ApplyArgs p)
             }
             unsigned long long old = cells_s[w];
             for (uint32_t it = 0;; ++it) {
-                if (((old >> shift) & maxc) == maxc) break;
-                const unsigned long long prev = atomicCAS(cells_s + w, old, old + (1ull << shift));
+                const unsigned long long room = maxc - ((old >> shift) & maxc);
+                if (room == 0) break;
+                const unsigned long long add = inc < room ? inc : room;
+                const unsigned long long prev = atomicCAS(cells_s + w, old, old + (add << shift));
                 if (prev == old) break;
                 old = prev;
-                if (it >= (LIMITED ? p.G.cas_limit : kCasLimit)) {
+                if (it >= kCasLimit) {
                     atomicOr(&p.ctr->error, kErrCasLimit);
                     break;
                 }
@@ -980,15 +824,21 @@ __global__ void __launch_bounds__(kCasApplyThreads, 3) apply_kernel(ApplyArgs p)
 }
 
 // Counting apply (alpha <= 15): one slice of 2^slice_shift cells per block.
-// The slice's increments are counted in 32-bit shared-memory lanes, counter
-// (cell, l) at lane l * 2^slice_shift + cell (a pass stages at most 2^31
-// increments, so a lane cannot wrap).  Then every counter becomes
-// min(old + count, 2^alpha - 1) and the slice is written back once.  With
-// LANES the codes are the 16-bit lanes themselves, else 32-bit
-// (cell << 6) | counter codes.
-template <bool LANES>
+// The slice's increments are summed in 32-bit shared-memory lanes, counter
+// (cell, l) at lane l * 2^slice_shift + cell.  Then every counter becomes
+// min(old + sum, 2^alpha - 1) and the slice is written back once.  With
+// LANES the codes hold the lanes themselves, else cell and counter.
+// A lane's sum is at most k_h times the call's windows; where that could
+// pass 2^32 (p.guard), lanes that already saturate their counter are left
+// alone, which keeps a sum below 2^15 plus the block's increments in flight.
+//
+// The last step costs more than the additions on a countBF with few increments
+// a cell (570 instructions a cell counter by counter), so 4- and 8-bit counters
+// have one that clamps the sums into a packed word and adds the counters of a
+// cell side by side.
+template <int ALPHA, bool LANES>
 __global__ void __launch_bounds__(kApplyThreads, 2) apply_count_kernel(ApplyArgs p) {
-    extern __shared__ uint32_t lanes[];   // one 32-bit count per counter of the slice
+    extern __shared__ __align__(16) uint32_t lanes[];   // one 32-bit sum per counter of the slice
     const uint64_t s = blockIdx.x;
     const uint64_t n = p.written[s];
     if (n == 0) return;   // no increments for this slice
@@ -998,102 +848,103 @@ __global__ void __launch_bounds__(kApplyThreads, 2) apply_count_kernel(ApplyArgs
     const unsigned nw = (unsigned)min(slice, p.G.words - w0);
     const unsigned eta = (unsigned)p.G.eta;
     const unsigned nwords = eta << ssh;
-    for (unsigned i = threadIdx.x; i < nwords; i += kApplyThreads) lanes[i] = 0;
+    if (nwords % 4 == 0) {
+        for (unsigned i = threadIdx.x; i < nwords / 4; i += kApplyThreads)
+            ((uint4 *)lanes)[i] = make_uint4(0, 0, 0, 0);
+    } else {
+        for (unsigned i = threadIdx.x; i < nwords; i += kApplyThreads) lanes[i] = 0;
+    }
     __syncthreads();
-    // 16 bytes per load: 8 lane codes or 4 cell codes; two loads per thread in flight
-    constexpr unsigned kPer = LANES ? 8 : 4;
-    constexpr unsigned kStep = kApplyThreads * 2 * kPer;
+    constexpr unsigned kStep = kApplyThreads * 8;   // two 16-byte loads per thread in flight
     const uint32_t wmask = (uint32_t)(slice - 1);
-    // each slice's codes start 16-byte aligned (cap: a multiple of 8 lanes, 4 cells)
-    const uint16_t *src16 = (const uint16_t *)p.codes + s * p.cap;
-    const uint32_t *src32 = (const uint32_t *)p.codes + s * p.cap;
+    const uint32_t slot_mask = (1u << p.slot_bits) - 1, inc_mask = (1u << p.w_bits) - 1;
+    const int lb = p.slot_bits + p.w_bits;
+    const uint32_t *src = p.codes + s * p.cap;   // 16-byte aligned: cap is a multiple of 4
+    const bool guard = p.guard != 0;
+    const uint32_t sat = (uint32_t)p.G.maxc;
     for (uint64_t i0 = 0; i0 < n; i0 += kStep) {
-        uint32_t code[2 * kPer];
+        uint32_t code[8];
         unsigned valid = 0;
-        const uint64_t i = i0 + threadIdx.x * (uint64_t)kPer;
+        const uint64_t i = i0 + threadIdx.x * 4ull;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const uint64_t j = i + (uint64_t)h * kApplyThreads * kPer;
-            if (j + kPer <= n) {
-                const uint4 v = __ldcs(LANES ? (const uint4 *)(src16 + j) : (const uint4 *)(src32 + j));
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (LANES) {
-                        code[kPer * h + 2 * q] = w[q] & 0xFFFFu;
-                        code[kPer * h + 2 * q + 1] = w[q] >> 16;
-                    } else {
-                        code[kPer * h + q] = w[q];
-                    }
-                }
-                valid |= ((1u << kPer) - 1) << (kPer * h);
+            const uint64_t j = i + (uint64_t)h * kApplyThreads * 4;
+            if (j + 4 <= n) {
+                const uint4 v = __ldcs((const uint4 *)(src + j));
+                code[4 * h] = v.x;
+                code[4 * h + 1] = v.y;
+                code[4 * h + 2] = v.z;
+                code[4 * h + 3] = v.w;
+                valid |= 0xFu << (4 * h);
             } else {
 #pragma unroll
-                for (unsigned q = 0; q < kPer; ++q) {
-                    const bool in = j + q < n;
-                    code[kPer * h + q] = !in ? 0u : LANES ? (uint32_t)src16[j + q] : src32[j + q];
-                    valid |= (in ? 1u : 0u) << (kPer * h + q);
+                for (unsigned q = 0; q < 4; ++q) {
+                    code[4 * h + q] = j + q < n ? src[j + q] : 0u;
+                    valid |= (j + q < n ? 1u : 0u) << (4 * h + q);
                 }
             }
         }
 #pragma unroll
-        for (unsigned q = 0; q < 2 * kPer; ++q) {
+        for (unsigned q = 0; q < 8; ++q) {
             if (!((valid >> q) & 1u)) continue;   // past the end
-            const unsigned c = LANES ? code[q] : ((code[q] & 63u) << ssh) | ((code[q] >> 6) & wmask);
-            atomicAdd(lanes + c, 1u);
+            const uint32_t c = code[q];
+            const unsigned lane = LANES ? c & ((1u << kLaneBits) - 1)
+                                        : (((c >> p.w_bits) & slot_mask) << ssh) | ((c >> lb) & wmask);
+            const unsigned inc = (LANES ? c >> kLaneBits : c & inc_mask) + 1;
+            if (guard && *(volatile uint32_t *)(lanes + lane) >= sat) continue;
+            atomicAdd(lanes + lane, inc);
         }
     }
     __syncthreads();
-    const uint32_t *cnt = lanes;
+    if (ALPHA) {
+        // counters two apart lie in fields of 2 * ALPHA bits, which hold the sum of
+        // a counter and a clamped addend; a carry out of the counter fills it
+        constexpr int A = ALPHA ? ALPHA : 4, F = 2 * A, ETA = 64 / A;
+        constexpr uint64_t kOnes = A == 4 ? 0x0101010101010101ull : 0x0001000100010001ull;
+        constexpr uint64_t kMax = kOnes * ((1ull << A) - 1);
+        for (unsigned i = threadIdx.x; i < nw; i += kApplyThreads) {
+            const uint64_t old = p.G.cells[w0 + i];
+            uint32_t add[2][2] = {{0, 0}, {0, 0}};   // [counter parity][half]
+#pragma unroll
+            for (int l = 0; l < ETA; ++l) {
+                const uint32_t c = min(lanes[((unsigned)l << ssh) | i], (1u << A) - 1);
+                add[l & 1][(l / 2) * F / 32] += c << ((l / 2) * F % 32);
+            }
+            uint64_t out = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint64_t v = ((old >> (h * A)) & kMax) + (((uint64_t)add[h][1] << 32) | add[h][0]);
+                const uint64_t carry = (v >> A) & kOnes;
+                v = (v | ((carry << A) - carry)) & kMax;
+                out |= v << (h * A);
+            }
+            p.G.cells[w0 + i] = out;
+        }
+        return;
+    }
     const unsigned alpha = (unsigned)p.G.alpha;
     const uint64_t maxc = p.G.maxc;
     for (unsigned i = threadIdx.x; i < nw; i += kApplyThreads) {
         const uint64_t old = p.G.cells[w0 + i];
         uint64_t out = 0;
         for (unsigned l = 0; l < eta; ++l) {
-            const uint64_t v = ((old >> (l * alpha)) & maxc) + cnt[((uint64_t)l << ssh) | i];
+            const uint64_t v = ((old >> (l * alpha)) & maxc) + lanes[((uint64_t)l << ssh) | i];
             out |= (v < maxc ? v : maxc) << (l * alpha);
         }
         p.G.cells[w0 + i] = out;
     }
 }
 
-// Launch insert_kernel<KW, CHUNK, PART> (g blocks), or with g == 0 report its
-// resident blocks per SM in *per_sm.
-template <int KW, int CHUNK, int PART>
-cudaError_t insert_variant(const InsertArgs *a, unsigned g, cudaStream_t s, int *per_sm) {
-    const int smem = (int)sizeof(InsertSmem<KW, CHUNK, PART>);
-    cudaError_t e = cudaFuncSetAttribute(insert_kernel<KW, CHUNK, PART>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, insert_kernel<KW, CHUNK, PART>,
-                                                             kInsertThreads, smem);
-    insert_kernel<KW, CHUNK, PART><<<g, kInsertThreads, smem, s>>>(*a);
-    return cudaGetLastError();
-}
-
-// part: 0 atomic design; 1 partitioned, region bits inside the codes
-// (coarse_shift <= 20); 2 partitioned, regions beside the codes.
-cudaError_t dispatch_insert(const InsertArgs *a, int kw, int part, unsigned g, cudaStream_t s,
-                            int *per_sm, int chunk = kChunk) {
-    if (part == 0 && chunk == kSmallChunk)
-        return kw == 1 ? insert_variant<1, kSmallChunk, 0>(a, g, s, per_sm)
-                       : insert_variant<2, kSmallChunk, 0>(a, g, s, per_sm);
-    if (part == 1 && kw == 1) return insert_variant<1, kPartChunk, 1>(a, g, s, per_sm);
-    if (part == 1) return insert_variant<2, kPartChunk, 1>(a, g, s, per_sm);
-    if (part == 2 && kw == 1) return insert_variant<1, kPartChunk, 2>(a, g, s, per_sm);
-    if (part == 2) return insert_variant<2, kPartChunk, 2>(a, g, s, per_sm);
-    if (kw == 1) return insert_variant<1, kChunk, 0>(a, g, s, per_sm);
-    return insert_variant<2, kChunk, 0>(a, g, s, per_sm);
-}
-
 }  // namespace
 
-int insert_blocks_per_sm(int kw, int part) {
+int insert_blocks_per_sm(int kw) {
     int n = 0;
-    if (dispatch_insert(nullptr, kw, part, 0, 0, &n) != cudaSuccess) n = 0;
-    return n > 0 ? n : 1;
+    const cudaError_t e =
+        kw == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<1, kChunk>,
+                                                                kInsertThreads, 0)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<2, kChunk>,
+                                                                kInsertThreads, 0);
+    return e == cudaSuccess && n > 0 ? n : 1;
 }
 
 cudaError_t launch_window_bound(const uint64_t *offsets, uint64_t nreads, int K, DevCounters *ctr,
@@ -1157,16 +1008,14 @@ cudaError_t launch_insert_batch(const InsertArgs *args, const unsigned long long
     return cudaGetLastError();
 }
 
-cudaError_t launch_repartition(const PartArgs &p, cudaStream_t s) {
-    const uint64_t tiles = (p.coarse_cap + kRepartTile - 1) / kRepartTile;
-    if (tiles == 0) return cudaSuccess;
+cudaError_t launch_repartition(const PartArgs &p, int sms, cudaStream_t s) {
     if (p.coarse_shift - p.slice_shift > kMaxCoarseShift - kSliceShift ||
         p.coarse_shift <= p.slice_shift)
         return cudaErrorInvalidValue;
     const int smem = kRepartTile * (int)sizeof(uint32_t);
-    const dim3 grid((unsigned)tiles, kCoarseBins);
-    if (p.lane_codes && ((uint64_t)p.G.eta << p.slice_shift) > (uint64_t)kCountLanes)
-        return cudaErrorInvalidValue;   // a lane must fit 16 bits
+    if (p.lane_codes && (((uint64_t)p.G.eta << p.slice_shift) > (uint64_t)kCountLanes ||
+                         p.w_bits > 32 - kLaneBits))
+        return cudaErrorInvalidValue;   // a lane must fit its bits
     // slices per coarse region: up to 64, 1,024 or kMaxFine (2,048)
     const int fbits = p.coarse_shift - p.slice_shift;
     void (*k)(PartArgs) =
@@ -1177,18 +1026,16 @@ cudaError_t launch_repartition(const PartArgs &p, cudaStream_t s) {
                                       : repartition_kernel<kMaxFine, false>);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, kRepartThreads, smem, s>>>(p);
+    const uint64_t tiles = (p.coarse_cap + kRepartTile - 1) / kRepartTile * kCoarseBins;
+    k<<<(unsigned)(tiles < (uint64_t)sms * 3 ? tiles : (uint64_t)sms * 3), kRepartThreads, smem, s>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_apply(const ApplyArgs &p, uint64_t nslices, cudaStream_t s) {
     if (nslices == 0) return cudaSuccess;
-    if (p.lane_codes || p.cap % 4) return cudaErrorInvalidValue;   // 32-bit codes, 16-byte aligned
+    if (p.lane_codes || p.cap % 4) return cudaErrorInvalidValue;   // 16-byte aligned slices
     const size_t smem = (size_t)8 << p.slice_shift;
-    const bool half = 32 % p.G.alpha == 0;
-    void (*k)(ApplyArgs) = p.G.cas_limit == kCasLimit
-                               ? (half ? apply_kernel<false, true> : apply_kernel<false, false>)
-                               : (half ? apply_kernel<true, true> : apply_kernel<true, false>);
+    void (*k)(ApplyArgs) = 32 % p.G.alpha == 0 ? apply_kernel<true> : apply_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(8 << kSliceShift));
     if (e != cudaSuccess) return e;
@@ -1200,8 +1047,11 @@ cudaError_t launch_apply_count(const ApplyArgs &p, uint64_t nslices, cudaStream_
     if (nslices == 0) return cudaSuccess;
     const size_t smem = ((size_t)p.G.eta << p.slice_shift) * 4;
     if (smem > (size_t)kCountLanes * 4 || p.G.alpha > 15) return cudaErrorInvalidValue;
-    if (p.cap % (p.lane_codes ? 8 : 4)) return cudaErrorInvalidValue;   // 16-byte aligned slices
-    void (*k)(ApplyArgs) = p.lane_codes ? apply_count_kernel<true> : apply_count_kernel<false>;
+    if (p.cap % 4) return cudaErrorInvalidValue;   // 16-byte aligned slices
+    void (*k)(ApplyArgs) =
+        p.G.alpha == 4   ? (p.lane_codes ? apply_count_kernel<4, true> : apply_count_kernel<4, false>)
+        : p.G.alpha == 8 ? (p.lane_codes ? apply_count_kernel<8, true> : apply_count_kernel<8, false>)
+                         : (p.lane_codes ? apply_count_kernel<0, true> : apply_count_kernel<0, false>);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kCountLanes * 4);
     if (e != cudaSuccess) return e;
@@ -1212,24 +1062,29 @@ cudaError_t launch_apply_count(const ApplyArgs &p, uint64_t nslices, cudaStream_
 cudaError_t launch_insert(const InsertArgs &a, int grid, int chunk, cudaStream_t s) {
     if (a.nchunks <= a.chunk_begin) return cudaSuccess;
     const uint64_t n = a.nchunks - a.chunk_begin;
-    const uint64_t g = n < (uint64_t)grid ? n : (uint64_t)grid;
-    const int part = !a.part ? 0 : a.coarse_shift <= 20 ? 1 : 2;
-    if ((part ? kPartChunk : chunk) != chunk) return cudaErrorInvalidValue;
-    return dispatch_insert(&a, a.K <= 32 ? 1 : 2, part, (unsigned)g, s, nullptr, chunk);
+    const unsigned g = (unsigned)(n < (uint64_t)grid ? n : (uint64_t)grid);
+    if (chunk != kChunk && chunk != kSmallChunk) return cudaErrorInvalidValue;
+    void (*k)(InsertArgs) = a.K <= 32 ? (chunk == kChunk ? insert_kernel<1, kChunk>
+                                                         : insert_kernel<1, kSmallChunk>)
+                                      : (chunk == kChunk ? insert_kernel<2, kChunk>
+                                                         : insert_kernel<2, kSmallChunk>);
+    k<<<g, kInsertThreads, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_reinsert(const uint64_t *keys, uint64_t n, int kw, uint64_t *table,
-                            uint64_t cap, SetTag tag, uint64_t *dlist, uint64_t dlist_cap,
-                            DevCounters *ctr, uint32_t probe_limit, cudaStream_t s) {
+cudaError_t launch_reinsert(const uint64_t *keys, uint64_t n, const unsigned *n32,
+                            const unsigned long long *n64, int kw, uint64_t *table, uint64_t cap,
+                            SetTag tag, uint64_t *dlist, uint64_t dlist_cap, DevCounters *ctr,
+                            uint32_t probe_limit, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    uint64_t blocks = (n + 255) / 256;
-    if (blocks > 65536) blocks = 65536;
+    uint64_t blocks = (n + kReinsertTile - 1) / kReinsertTile;
+    if (blocks > 152 * 8) blocks = 152 * 8;   // resident ones: the rest by stride
     if (kw == 1)
-        reinsert_kernel<1><<<(unsigned)blocks, 256, 0, s>>>(keys, n, table, cap, tag, dlist, dlist_cap,
-                                                             ctr, probe_limit);
+        reinsert_kernel<1><<<(unsigned)blocks, 256, 0, s>>>(keys, n, n32, n64, table, cap, tag, dlist,
+                                                             dlist_cap, ctr, probe_limit);
     else
-        reinsert_kernel<2><<<(unsigned)blocks, 256, 0, s>>>(keys, n, table, cap, tag, dlist, dlist_cap,
-                                                             ctr, probe_limit);
+        reinsert_kernel<2><<<(unsigned)blocks, 256, 0, s>>>(keys, n, n32, n64, table, cap, tag, dlist,
+                                                             dlist_cap, ctr, probe_limit);
     return cudaGetLastError();
 }
 

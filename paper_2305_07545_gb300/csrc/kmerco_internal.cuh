@@ -13,11 +13,11 @@ constexpr uint64_t kEmptyKey = ~0ull;      // empty slot of the distinct-key set
                                            // no canonical key is all ones
 constexpr int kChunk = 2048;               // window starts per insert work unit
 constexpr int kSmallChunk = 512;           // the same for inputs too small to fill the GPU
-constexpr int kPartChunk = 1024;           // the same in the partitioned update design
-constexpr int kPartMaxHash = 4;            // hashes the partitioned design stages per window
+constexpr int kPartMaxHash = 4;            // hashes the partitioned update groups at a time
 constexpr int kCoarseBins = 64;            // coarse countBF regions of the partitioned design
 constexpr int kSliceShift = 13;            // 2^13 cells (64 KiB) per shared-memory slice
 constexpr int kMaxCoarseShift = 24;        // cell-in-region bits of an increment code
+constexpr int kLaneBits = 14;              // lane bits of a counting-apply code
 constexpr int kMaxFine = 1 << (kMaxCoarseShift - kSliceShift);   // slices per coarse region
 constexpr uint64_t kMaxBatchCodes = 1ull << 31;   // increments staged per partitioned pass
 constexpr int kRepartTile = 8192;          // codes per repartition block
@@ -213,6 +213,25 @@ __device__ __forceinline__ void address(const Geometry &G, uint64_t h, uint64_t 
     }
 }
 
+// Saturating addition of w to the counter at `shift` of cell c: w saturating
+// increments of Algorithm 3 at once.  `old` is a recent read of the cell.
+__device__ __forceinline__ void sat_add(uint64_t *cells, uint64_t c, unsigned shift, uint64_t maxc,
+                                        uint64_t w, uint64_t old, uint32_t limit, unsigned *err) {
+    for (uint32_t it = 0;; ++it) {
+        const uint64_t v = (old >> shift) & maxc, room = maxc - v;
+        if (room == 0) return;   // saturated: stays at the maximum
+        const uint64_t add = w < room ? w : room;
+        const uint64_t prev = atomicCAS((unsigned long long *)(cells + c), (unsigned long long)old,
+                                        (unsigned long long)(old + (add << shift)));
+        if (prev == old) return;
+        old = prev;
+        if (it >= limit) {
+            atomicOr(err, kErrCasLimit);
+            return;
+        }
+    }
+}
+
 // ------------------------------------------------------------ block scan
 // Exclusive prefix sum of one value per thread across a block of NT threads
 // (a multiple of 32, at most 1024): warp shuffles, then a scan of the warp
@@ -303,24 +322,18 @@ struct InsertArgs {
     uint64_t *dlist;             // distinct keys in arrival order
     uint64_t dlist_cap;
     DevCounters *ctr;
-    // partitioned update design (part != 0)
-    int part;
-    int coarse_shift;                      // coarse region = cell >> coarse_shift
-    uint32_t *coarse;                      // kCoarseBins regions of coarse_cap codes
-    uint64_t coarse_cap;
-    unsigned long long *coarse_cursor;     // codes reserved per region
-    unsigned long long *coarse_written;    // codes written per region (a prefix)
 };
 
+// Increment codes (32 bits): cell within its coarse region, then slot_bits of
+// counter within the cell, then w_bits of the increment less one.
 struct PartArgs {
     Geometry G;
-    int coarse_shift;
+    int coarse_shift, slot_bits, w_bits;
     int slice_shift;                       // fine slice = cell >> slice_shift
-    const uint32_t *coarse;
+    const uint32_t *coarse;                // kCoarseBins regions of coarse_cap codes
     uint64_t coarse_cap;
     const unsigned long long *coarse_written;
-    void *fine;                            // one region of fine_cap codes per slice:
-                                           // uint16 lane codes when lane_codes, else uint32
+    uint32_t *fine;                        // one region of fine_cap codes per slice
     uint64_t fine_cap;
     int lane_codes;                        // slice codes are counting-apply lanes
     unsigned long long *fine_cursor;
@@ -330,11 +343,12 @@ struct PartArgs {
 
 struct ApplyArgs {
     Geometry G;
+    int slot_bits, w_bits;
     int slice_shift;                       // cells per slice = 2^slice_shift
-    const void *codes;                     // one region of cap codes per slice:
-                                           // uint16 lane codes when lane_codes, else uint32
+    const uint32_t *codes;                 // one region of cap codes per slice
     uint64_t cap;
     int lane_codes;
+    int guard;                             // a lane's sum could pass 2^32
     const unsigned long long *written;     // codes per slice
     DevCounters *ctr;
 };
@@ -345,12 +359,10 @@ cudaError_t launch_first_read(const uint64_t *offsets, uint64_t nreads, uint64_t
                               uint64_t nchunks, uint64_t chunk, uint32_t *first_read,
                               cudaStream_t s);
 // chunk: the window starts per work unit the call was planned with (kChunk
-// or kSmallChunk in the atomic design, kPartChunk in the partitioned one).
+// or kSmallChunk).
 cudaError_t launch_insert(const InsertArgs &a, int grid, int chunk, cudaStream_t s);
-// Resident insert blocks per SM; part: 0 atomic design, 1 partitioned with
-// region bits inside the codes (coarse_shift <= 20), 2 partitioned (wide).
-int insert_blocks_per_sm(int kw, int part);
-cudaError_t launch_repartition(const PartArgs &p, cudaStream_t s);
+int insert_blocks_per_sm(int kw);   // resident insert blocks per SM
+cudaError_t launch_repartition(const PartArgs &p, int sms, cudaStream_t s);
 
 // Batched insertion (atomic design): many samples, each with its own
 // InsertArgs (device array), chunks of all samples in one index space with
@@ -369,11 +381,22 @@ cudaError_t launch_apply(const ApplyArgs &p, uint64_t nslices, cudaStream_t s);
 // kCountLanes), then added to the counters with saturation.
 constexpr int kCountLanes = 16384;
 cudaError_t launch_apply_count(const ApplyArgs &p, uint64_t nslices, cudaStream_t s);
-// Insert n keys into a distinct set; when dlist is not null, keys new to the
-// set are appended to it (ctr->distinct counts them).
-cudaError_t launch_reinsert(const uint64_t *keys, uint64_t n, int kw, uint64_t *table,
-                            uint64_t cap, SetTag tag, uint64_t *dlist, uint64_t dlist_cap,
-                            DevCounters *ctr, uint32_t probe_limit, cudaStream_t s);
+// Insert keys into a distinct set: n of them, or as many as *n32 / *n64 says
+// (device memory, when not null), at most n.  When dlist is not null, keys new
+// to the set are appended to it (ctr->distinct counts them).
+cudaError_t launch_reinsert(const uint64_t *keys, uint64_t n, const unsigned *n32,
+                            const unsigned long long *n64, int kw, uint64_t *table, uint64_t cap,
+                            SetTag tag, uint64_t *dlist, uint64_t dlist_cap, DevCounters *ctr,
+                            uint32_t probe_limit, cudaStream_t s);
+
+// out = the union of two ascending lists without repetition (out overlaps neither).
+// a has *distinct keys (at most na_most) and b *nb32 or *nb64 (whichever is not
+// null; at most nb_most); *distinct becomes the union's length.  scratch needs
+// union_scratch_words(na_most, nb_most) words.
+uint64_t union_scratch_words(uint64_t na, uint64_t nb);
+cudaError_t launch_union(const uint64_t *a, uint64_t na_most, const uint64_t *b, uint64_t nb_most,
+                         const unsigned *nb32, const unsigned long long *nb64, int kw, uint64_t *out,
+                         unsigned *scratch, unsigned long long *distinct, cudaStream_t s);
 
 // Radix sort of n keys of kw words (1 or 2) on their low `bits` bits.  The
 // sorted keys end in *result, which is one of in, alt0 or alt1; in is left
