@@ -65,6 +65,9 @@ struct kmerco {
     bool table_ok;           // the set holds exactly the list's keys (built when it is needed)
     bool table_dirty;        // the set holds keys under the current tag
     bool list_sorted;        // the list is in ascending order
+    uint8_t *sure;           // list key i has more than tau windows in the countBF
+    uint64_t sure_cap;
+    bool sure_ok;            // ... of the list and the countBF as they are
     uint64_t *dlist;         // distinct keys in arrival order
     uint64_t dlist_cap;
     uint64_t *dlist2;        // the list's other place: a union is written there
@@ -406,7 +409,7 @@ int merge_keys(kmerco_t *h, const uint64_t *keys, uint64_t nb_most, const unsign
     std::swap(h->dlist, h->dlist2);
     std::swap(h->dlist_cap, h->dlist2_cap);
     h->d_ub += nb_most;
-    h->table_ok = false;
+    h->table_ok = h->sure_ok = false;
     h->list_sorted = true;
     return KMERCO_OK;
 }
@@ -511,6 +514,7 @@ struct PartPlan {
 struct InsertPlan {
     bool ranges = false;
     bool fresh = false;      // the handle holds no keys: the first pass writes the list
+    bool sure = false;       // the list is the call's keys: which are sure is written too
     bool merge = false;      // the list stays in order: the call's keys are merged into it
     uint64_t passes = 1;
     uint64_t bound = 0;      // windows of the call at most
@@ -779,6 +783,8 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
         KM_CUDA(dedup_finish(ip.dd, b.dd, h->ctr, ce - cb, ordered, fresh, h->sms, s, launches));
         EmitArgs e = dedup_result(ip.dd, b.dd, h->G, h->ctr, ordered);
         e.dlist = fresh ? h->dlist : ip.merge ? merge_input(ip, b) : nullptr;
+        e.sure = fresh && ip.sure ? h->sure : nullptr;
+        e.tau = h->tau;
         KM_TRY(launch_updates(h, ip, b, e, s, launches));
         if (!ip.table()) continue;
         // the pass's keys into the distinct set (the first pass of an empty
@@ -884,7 +890,7 @@ int kmerco_estimate_bytes(const kmerco_config_t *cfg, uint64_t nreads, uint64_t 
         // being a new key
         uint64_t list = windows;
         if (cfg->max_distinct && list > cfg->max_distinct) list = cfg->max_distinct;
-        b += list * kw * 8;
+        b += list * kw * 8 + grown(windows, 1);
         const InsertPlan ip = plan_insert(&t, windows, nbytes, true);
         if (ip.table()) b += std::max<uint64_t>(2 * windows, 1024) * kw * 8;
         if (ip.ranges) {
@@ -1027,6 +1033,7 @@ void kmerco_destroy(kmerco_t *h) {
         dev_free(h, h->dlist, h->dlist_cap * h->kw * 8);
         dev_free(h, h->dlist2, h->dlist2_cap * h->kw * 8);
         dev_free(h, h->union_scratch, h->union_scratch_cap * 4);
+        dev_free(h, h->sure, h->sure_cap);
         dev_free(h, h->in_bases, h->in_bases_cap);
         dev_free(h, h->in_offsets, h->in_offsets_cap * 8);
         dev_free(h, h->first_read, h->first_read_cap * 4);
@@ -1073,7 +1080,7 @@ int kmerco_reset(kmerco_t *h) {
     KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), h->stream));
     h->d_ub = 0;
     h->table_ok = true;
-    h->list_sorted = false;
+    h->list_sorted = h->sure_ok = false;
     h->classified = false;
     h->n_distinct = h->n_trusted = 0;
     h->insert_timed = h->classify_timed = false;
@@ -1160,6 +1167,7 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
             KM_TRY(st);
     }
     if (!ip.merge) KM_TRY(ensure_set_capacity(h, bound, ip.table()));
+    ip.sure = !ip.table() && ip.fresh && ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
     KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
     const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
@@ -1171,6 +1179,7 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
                           &dedup_result(ip.dd, bufs.dd, h->G, h->ctr, true).meta->distinct, nullptr));
     if (!ip.table()) h->table_ok = false;   // the list alone was written
     h->list_sorted = !ip.table();
+    h->sure_ok = ip.sure;
     KM_CUDA(cudaEventRecord(h->ev[1], h->stream));
     h->insert_timed = true;
     h->classified = false;
@@ -1360,11 +1369,10 @@ int kmerco_classify(kmerco_t *h) {
         if (D > 1) h->launches += 3 * (uint64_t)passes;
     }
 sorted_done:
-    KM_CUDA(launch_classify_query(sorted, D, kw, h->G, h->tau, h->est, h->stream));
-    h->est_exact = false;
-    KM_CUDA(launch_split(sorted, h->est, D, kw, h->tau, h->split, h->split_scratch, h->ctr,
-                         h->stream));
-    if (D > 0) h->launches += 4;   // query + three split kernels
+    h->est_exact = false;   // est holds the keys' bits
+    KM_CUDA(launch_classify(sorted, D, kw, h->G, h->tau, in_order && h->sure_ok ? h->sure : nullptr,
+                            h->est, h->split, h->split_scratch, h->ctr, h->stream));
+    if (D > 0) h->launches += 3;   // mark, scan, scatter
     KM_CUDA(cudaEventRecord(h->ev[3], h->stream));
     KM_TRY(read_counters(h));
     h->sorted = sorted;
@@ -1448,6 +1456,7 @@ int kmerco_set_counters(kmerco_t *h, const uint64_t *src, uint64_t nwords) {
     DeviceGuard guard(h->device);
     KM_CUDA(cudaMemcpyAsync(h->G.cells, src, nwords * 8, cudaMemcpyDefault, h->stream));
     KM_CUDA(cudaStreamSynchronize(h->stream));
+    h->sure_ok = false;   // other counters
     h->classified = false;
     return KMERCO_OK;
 }
@@ -1467,7 +1476,7 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
     KM_CUDA(launch_reinsert(d_keys, n, nullptr, nullptr, h->kw, h->table, h->cap, set_tag(h),
                             h->dlist, h->dlist_cap, h->ctr, h->G.probe_limit, h->stream));
     h->launches += 1;
-    h->list_sorted = false;
+    h->list_sorted = h->sure_ok = false;
     KM_TRY(read_counters(h));
     KM_TRY(device_error_status(h->ctr_host->error));
     h->classified = false;
@@ -1664,6 +1673,7 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
     KM_TRY(device_error_status(src->ctr_host->error));
     const DevCounters sc = *src->ctr_host;
     // ascending lists: copied into an empty handle, merged into an ordered one
+    dst->sure_ok = false;
     const bool ordered = src->list_sorted && sc.distinct && !dst->max_distinct &&
                          dst->G.probe_limit == kProbeLimit;
     bool listed = false;
@@ -1731,7 +1741,7 @@ struct kmerco_batch {
     std::vector<unsigned long long> chunk_end, bound_host;
     std::vector<const char *> p_bases;       // inputs of the planned launch
     std::vector<const uint64_t *> p_offs;
-    std::vector<uint32_t> graph_gen;         // distinct-set generation of each handle at capture
+    std::vector<uint64_t> graph_key;         // what the captured launches hold of every handle
     std::vector<uint64_t> p_nreads;
     bool planned, tuned, have_graph;
     int chunk, bpm;
@@ -1920,6 +1930,14 @@ int batch_run(kmerco_batch *b, bool reset) {
     return batch_launch(b, b->chunk, b->bpm);
 }
 
+// What a captured insert of a handle holds of it: its generation tag and buffers
+// (a later insert into the handle alone may move them).
+void handle_key(const kmerco_t *h, std::vector<uint64_t> &key) {
+    const uint64_t f[6] = {h->gen, (uint64_t)h->dlist, (uint64_t)h->table, (uint64_t)h->first_read,
+                           (uint64_t)h->sure, h->dlist_cap};
+    key.insert(key.end(), f, f + 6);
+}
+
 // State of the handles after a batch insert (a replayed graph inserted too).
 void batch_mark_inserted(kmerco_batch *b) {
     for (int i = 0; i < b->n; ++i) {
@@ -1928,9 +1946,11 @@ void batch_mark_inserted(kmerco_batch *b) {
         h->n_distinct = h->n_trusted = 0;
         h->insert_timed = h->classify_timed = false;
         h->d_ub = std::max(h->d_ub, b->load[i]);
+        h->sure_ok = false;
         if (b->sched == 1 && !b->plans[i].table()) {   // the list alone was written, in order
             h->table_ok = false;
             h->list_sorted = true;
+            h->sure_ok = b->plans[i].sure;
         } else if (b->load[i]) {
             h->table_ok = h->table_dirty = true;
             h->list_sorted = false;
@@ -2029,7 +2049,12 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
     bool same = b->planned && reset && b->have_graph;
     for (int i = 0; same && i < b->n; ++i)
         same = b->p_bases[i] == bases[i] && b->p_offs[i] == offsets[i] &&
-               b->p_nreads[i] == nreads[i] && b->h[i]->gen == b->graph_gen[i];
+               b->p_nreads[i] == nreads[i];
+    if (same) {
+        std::vector<uint64_t> key;
+        for (const kmerco_t *h : b->h) handle_key(h, key);
+        same = key == b->graph_key;
+    }
     if (same) {
         KM_CUDA(cudaGraphLaunch(b->exec, b->stream));
         b->launches += b->total_chunks ? 2 : 0;
@@ -2082,6 +2107,8 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
         b->plans[i] = plan_insert(h, bound, bo[2] - bo[1], h->d_ub == 0);
         // the set too: the persistent schedule inserts into it
         KM_TRY(ensure_set_capacity(h, bound, bound != 0));
+        b->plans[i].sure = !b->plans[i].table() && b->plans[i].fresh &&
+                           ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
         const uint64_t most = (bo[2] - bo[1] + kSmallChunk - 1) / kSmallChunk;   // chunks at the smallest chunk size
         KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, most ? most : 1));
         b->load[i] = bound;
@@ -2153,8 +2180,8 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
             }
             b->graph = g;
             b->have_graph = true;
-            b->graph_gen.resize(b->n);   // the tags the graph's launches carry
-            for (int i = 0; i < b->n; ++i) b->graph_gen[i] = b->h[i]->gen;
+            b->graph_key.clear();
+            for (const kmerco_t *h : b->h) handle_key(h, b->graph_key);
             KM_CUDA(cudaGraphLaunch(b->exec, b->stream));
         }
     } else {
@@ -2237,16 +2264,17 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
     // CUDA graph: replayed while every sample's distinct count and buffers
     // are those it was captured with
     std::vector<uint64_t> key;
-    key.reserve((size_t)b->n * 12);
+    key.reserve((size_t)b->n * 13);
     for (int i = 0; i < b->n; ++i) {
         const kmerco_t *h = b->h[i];
-        const uint64_t fields[12] = {h->classified ? ~0ull : D[i], (uint64_t)h->dlist,
+        const uint64_t fields[13] = {h->classified ? ~0ull : D[i], (uint64_t)h->dlist,
                                      (uint64_t)h->alt0, (uint64_t)h->alt1, (uint64_t)h->est,
                                      (uint64_t)h->split, (uint64_t)h->sort_scratch,
                                      (uint64_t)h->split_scratch, (uint64_t)h->ctr,
                                      (uint64_t)h->G.cells, (uint64_t)h->seg_scratch,
-                                     h->list_sorted ? 1ull : 0ull};
-        key.insert(key.end(), fields, fields + 12);
+                                     h->list_sorted ? 1ull : 0ull,
+                                     h->sure_ok ? (uint64_t)h->sure : 0ull};
+        key.insert(key.end(), fields, fields + 13);
     }
     if (b->have_cls && key == b->cls_key) {
         KM_CUDA(cudaGraphLaunch(b->cls_exec, b->stream));
@@ -2287,7 +2315,7 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
                 cudaStream_t st = b->aux[k];
                 const int bits = 2 * h->K, passes = (bits + kRadixBits - 1) / kRadixBits;
                 const uint64_t *sorted = h->dlist;
-                uint64_t n_launch = D[i] ? 4 : 0;   // query + three split kernels
+                uint64_t n_launch = D[i] ? 3 : 0;   // mark, scan, scatter
                 if (top[i]) {   // as in kmerco_classify; long runs are checked below
                     const int s0 = bits - kTopSortBits;
                     const uint64_t nbe = seg_bounds_entries(D[i], h->kw);
@@ -2306,9 +2334,9 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
                                        h->sort_scratch, &sorted, st));
                     n_launch += D[i] > 1 ? 3 * (uint64_t)passes : 0;
                 }
-                KM_CUDA(launch_classify_query(sorted, D[i], h->kw, h->G, h->tau, h->est, st));
-                KM_CUDA(launch_split(sorted, h->est, D[i], h->kw, h->tau, h->split,
-                                     h->split_scratch, h->ctr, st));
+                KM_CUDA(launch_classify(sorted, D[i], h->kw, h->G, h->tau,
+                                        h->list_sorted && h->sure_ok ? h->sure : nullptr, h->est,
+                                        h->split, h->split_scratch, h->ctr, st));
                 h->launches += n_launch;
                 b->launches += n_launch;
                 h->sorted = sorted;
@@ -2364,11 +2392,10 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
         bool any;
         KM_TRY(sort_long_runs(h, D[i], 2 * h->K, h->bucket_host[0], &any, b->stream));
         if (!any) continue;
-        KM_CUDA(launch_classify_query(h->alt0, D[i], h->kw, h->G, h->tau, h->est, b->stream));
-        KM_CUDA(launch_split(h->alt0, h->est, D[i], h->kw, h->tau, h->split, h->split_scratch,
-                             h->ctr, b->stream));
-        h->launches += 4;
-        b->launches += 4;
+        KM_CUDA(launch_classify(h->alt0, D[i], h->kw, h->G, h->tau, nullptr, h->est, h->split,
+                                h->split_scratch, h->ctr, b->stream));
+        h->launches += 3;
+        b->launches += 3;
         KM_CUDA(cudaMemcpyAsync(h->ctr_host, h->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost,
                                 b->stream));
         KM_CUDA(cudaStreamSynchronize(b->stream));

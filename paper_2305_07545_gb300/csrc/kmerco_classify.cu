@@ -13,14 +13,13 @@
 //    insertion or bitonic sort).  A single bin too large for shared memory
 //    is left to radix_sort.
 //  - query: per key, k_h hashes and the minimum counter, 0 if any is 0.
-//  - split: stable partition on est > tau (trustworthy first).
+//  - classify: whether a key's estimate exceeds tau, and the stable partition on
+//    it (trustworthy first).
 //  - merge: counter-wise min(a + b, 2^alpha - 1) of two countBFs.
 #include "kmerco_internal.cuh"
 
 namespace countbf {
 namespace {
-
-constexpr int kWarps = kSortThreads / 32;
 
 // The 8-bit digit at bit `shift` of a key (a digit may straddle the two
 // words of a two-word key).
@@ -247,124 +246,168 @@ __global__ void query_kernel(const uint64_t *keys, uint64_t n, int K, Geometry G
     }
 }
 
-// Algorithm 5 as far as Algorithm 2 needs it.  The split asks only whether
-// est > tau, and est is the minimum of the key's k_h counters, so the first
-// counter at or below tau decides "erroneous": the remaining counters of that
-// key are not read.  est[i] is then exact for every trustworthy key (all k_h
-// counters read) and, for an erroneous key, the minimum of the counters read
-// so far, which is at most tau; Algorithm 5's 0 for an empty counter is that
-// minimum too.  Each lane works through its keys one counter per iteration
-// (a finished key makes room for the lane's next key at once), so every
-// iteration keeps one random counter read per lane in flight.
+// Algorithm 5 as far as Algorithm 2 needs it: bit i of `bits` says that key i's
+// estimate exceeds tau, tile_cnt[t] how many of tile t do.  The estimate is the
+// minimum of the key's k_h counters, so the first counter at or below tau
+// decides "erroneous" and the key's other counters are not read.  A key whose
+// `sure` byte is set has more than tau windows in this countBF, which never
+// underestimates: it is trustworthy without a look at its counters (these would
+// be all k_h of them; without the bytes the 86% of erroneous keys cost one read
+// each, the others four: 7.5 instead of 4.4 ms for 2.1e8 keys in a 4 GiB
+// countBF).
+//
+// Bound by random reads.  Each lane works through its 16 keys of a tile one
+// counter per iteration (a decided key makes room for the lane's next key at
+// once), so every iteration keeps one random counter read per lane in flight;
+// the next key is loaded meanwhile.
 template <int KW>
-__global__ void __launch_bounds__(256) classify_query_kernel(const uint64_t *keys, uint64_t n,
-                                                             Geometry G, uint32_t tau,
-                                                             uint32_t *est) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint64_t klo = keys[i * KW], khi = KW == 2 ? keys[i * KW + 1] : 0;
-    uint64_t k1m = KW == 1 ? premix8(klo) : 0;
-    unsigned j = 0;
-    uint64_t best = ~0ull;
-    for (;;) {
-        uint64_t h1, h2, cell;
-        unsigned slot;
-        if (KW == 1)
-            murmur8(k1m, j, h1, h2);
-        else
-            murmur16(klo, khi, j, h1, h2);
-        address(G, h1, cell, slot);
-        const uint64_t v = (__ldg(G.cells + cell) >> (slot * (unsigned)G.alpha)) & G.maxc;
-        best = v < best ? v : best;
-        if (++j < (unsigned)G.nhash && best > tau) continue;
-        est[i] = (uint32_t)best;
-        i += stride;
-        if (i >= n) break;
-        klo = keys[i * KW];
-        khi = KW == 2 ? keys[i * KW + 1] : 0;
-        k1m = KW == 1 ? premix8(klo) : 0;
-        j = 0;
-        best = ~0ull;
-    }
-}
-
-// Trusted keys per split tile.  A tile of kSplitTile keys is read in 16
-// rounds of kSortThreads consecutive keys (coalesced), key tile0 + 256j + tid.
-__global__ void __launch_bounds__(kSortThreads) split_count_kernel(const uint32_t *est, uint64_t n,
-                                                                   uint32_t tau, uint64_t *tile_cnt) {
-    const uint64_t tile0 = (uint64_t)blockIdx.x * kSplitTile;
-    unsigned c = 0;
+__global__ void __launch_bounds__(kSortThreads, 8) classify_mark_kernel(
+    const uint64_t *keys, uint64_t n, Geometry G, uint32_t tau, const uint8_t *sure, uint32_t *bits,
+    uint64_t *tile_cnt) {
+    constexpr int PER = kSplitTile / kSortThreads;
+    __shared__ unsigned total;
+    const unsigned tid = threadIdx.x, lane = tid & 31;
+    for (uint64_t tile = blockIdx.x; tile * kSplitTile < n; tile += gridDim.x) {
+        const uint64_t t0 = tile * kSplitTile + tid;
+        if (tid == 0) total = 0;
+        unsigned trusted = 0, todo = 0;   // bit j: key t0 + 256 j
 #pragma unroll
-    for (int j = 0; j < kSplitTile / kSortThreads; ++j) {
-        const uint64_t i = tile0 + (uint64_t)j * kSortThreads + threadIdx.x;
-        c += (i < n) && est[i] > tau;
+        for (int j = 0; j < PER; ++j) {
+            const uint64_t i = t0 + (uint64_t)j * kSortThreads;
+            if (i < n) {
+                if (sure && sure[i])
+                    trusted |= 1u << j;
+                else
+                    todo |= 1u << j;
+            }
+        }
+        __syncthreads();
+        if (todo) {
+            unsigned cur = __ffs(todo) - 1;
+            todo &= todo - 1;
+            uint64_t i = t0 + (uint64_t)cur * kSortThreads;
+            uint64_t klo = keys[i * KW], khi = KW == 2 ? keys[i * KW + 1] : 0;
+            unsigned nxt = todo ? __ffs(todo) - 1 : cur;
+            i = t0 + (uint64_t)nxt * kSortThreads;
+            uint64_t nlo = keys[i * KW], nhi = KW == 2 ? keys[i * KW + 1] : 0;
+            uint64_t k1m = KW == 1 ? premix8(klo) : 0;
+            unsigned a = 0;
+            for (;;) {
+                uint64_t h1, h2, cell;
+                unsigned slot;
+                if (KW == 1)
+                    murmur8(k1m, a, h1, h2);
+                else
+                    murmur16(klo, khi, a, h1, h2);
+                address(G, h1, cell, slot);
+                const uint64_t v = (__ldg(G.cells + cell) >> (slot * (unsigned)G.alpha)) & G.maxc;
+                if (v > tau) {
+                    if (++a < (unsigned)G.nhash) continue;
+                    trusted |= 1u << cur;
+                }
+                if (!todo) break;
+                cur = nxt;
+                todo &= todo - 1;
+                klo = nlo;
+                khi = nhi;
+                k1m = KW == 1 ? premix8(klo) : 0;
+                a = 0;
+                if (todo) {
+                    nxt = __ffs(todo) - 1;
+                    i = t0 + (uint64_t)nxt * kSortThreads;
+                    nlo = keys[i * KW];
+                    if (KW == 2) nhi = keys[i * KW + 1];
+                }
+            }
+        }
+        __syncwarp();
+        unsigned mine = 0, word = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const unsigned b = __ballot_sync(0xffffffffu, (trusted >> j) & 1u);
+            mine += __popc(b);
+            if (lane == (unsigned)j) word = b;   // the warp's 32 keys of round j
+        }
+        // words in key order: round j's eight warps stand together
+        if (lane < (unsigned)PER && tile * kSplitTile + lane * kSortThreads + (tid & ~31u) < n)
+            bits[(tile * kSplitTile + lane * kSortThreads + (tid & ~31u)) / 32] = word;
+        if (lane == 0) atomicAdd(&total, mine);
+        __syncthreads();
+        if (tid == 0) tile_cnt[tile] = total;
+        __syncthreads();
     }
-    unsigned long long tot;
-    block_exclusive_scan<unsigned long long, kSortThreads>(c, tot);
-    if (threadIdx.x == 0) tile_cnt[blockIdx.x] = tot;
 }
 
 // Exclusive scan of tile counts in place (one block); total -> ctr->trusted.
-__global__ void __launch_bounds__(kSortThreads) split_scan_kernel(uint64_t *tile_cnt,
-                                                                  uint64_t ntiles, DevCounters *ctr) {
+__global__ void __launch_bounds__(1024) split_scan_kernel(uint64_t *tile_cnt, uint64_t ntiles,
+                                                          DevCounters *ctr) {
+    constexpr unsigned E = 8;
     unsigned long long carry = 0;
-    for (uint64_t s0 = 0; s0 < ntiles; s0 += kSortThreads) {
-        const uint64_t idx = s0 + threadIdx.x;
-        unsigned long long v = idx < ntiles ? tile_cnt[idx] : 0ull, tot;
-        unsigned long long pre = block_exclusive_scan<unsigned long long, kSortThreads>(v, tot) + carry;
-        if (idx < ntiles) tile_cnt[idx] = pre;
+    for (uint64_t s0 = 0; s0 < ntiles; s0 += 1024 * E) {
+        unsigned long long v[E], sum = 0, tot;
+#pragma unroll
+        for (unsigned j = 0; j < E; ++j) {
+            const uint64_t idx = s0 + threadIdx.x * E + j;
+            v[j] = idx < ntiles ? tile_cnt[idx] : 0ull;
+            sum += v[j];
+        }
+        unsigned long long pre = block_exclusive_scan<unsigned long long, 1024>(sum, tot) + carry;
+#pragma unroll
+        for (unsigned j = 0; j < E; ++j) {
+            const uint64_t idx = s0 + threadIdx.x * E + j;
+            if (idx < ntiles) tile_cnt[idx] = pre;
+            pre += v[j];
+        }
         carry += tot;
     }
     if (threadIdx.x == 0) ctr->trusted = carry;
 }
 
-// Stable split of one tile: trustworthy keys (est > tau) go after the
-// trustworthy keys of earlier tiles, erroneous keys after all trustworthy
-// keys and the erroneous keys of earlier tiles, both in key order.  The tile
-// is read in 16 coalesced rounds; a key's rank comes from its warp's ballot
-// and the counts of the (round, warp) segments before it.
+// Stable split of one tile: trustworthy keys (their bit is set) go after the
+// trustworthy keys of earlier tiles, erroneous keys after all trustworthy keys
+// and the erroneous keys of earlier tiles, both in key order.  A key's rank
+// comes from its word of 32 bits and the scanned counts of the words before it.
+// Bound by the memory it streams: a key read and written once.
 template <int KW>
 __global__ void __launch_bounds__(kSortThreads) split_scatter_kernel(const uint64_t *keys,
-                                                                     const uint32_t *est, uint64_t n,
-                                                                     uint32_t tau,
+                                                                     const uint32_t *bits, uint64_t n,
                                                                      const uint64_t *tile_pre,
                                                                      const DevCounters *ctr,
                                                                      uint64_t *out) {
-    constexpr int kRounds = kSplitTile / kSortThreads;
-    __shared__ unsigned seg[kRounds * kWarps];   // trusted keys per (round, warp), then their prefix
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kRounds = kSplitTile / kSortThreads, kWords = kSplitTile / 32;
+    static_assert(kWords <= kSortThreads, "a word a thread");
+    __shared__ unsigned word[kWords], before[kWords];
+    const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t tile0 = (uint64_t)blockIdx.x * kSplitTile;
-    unsigned bal[kRounds];
+    unsigned w = 0;
+    if (tid < kWords && tile0 + tid * 32 < n) w = bits[tile0 / 32 + tid];
+    uint64_t key[kRounds][KW];
 #pragma unroll
-    for (int j = 0; j < kRounds; ++j) {
-        const uint64_t i = tile0 + (uint64_t)j * kSortThreads + threadIdx.x;
-        bal[j] = __ballot_sync(0xffffffffu, i < n && est[i] > tau);
-        if (lane == 0) seg[j * kWarps + warp] = __popc(bal[j]);
+    for (int j = 0; j < kRounds; ++j) {   // in flight across the scan
+        const uint64_t i = tile0 + (uint64_t)j * kSortThreads + tid;
+#pragma unroll
+        for (int q = 0; q < KW; ++q) key[j][q] = i < n ? keys[i * KW + q] : 0;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {   // segments in key order: round-major, then warp
-        unsigned acc = 0;
-        for (int q = 0; q < kRounds * kWarps; ++q) {
-            const unsigned v = seg[q];
-            seg[q] = acc;
-            acc += v;
-        }
+    unsigned tot;
+    const unsigned pre = block_exclusive_scan<unsigned, kSortThreads>(__popc(w), tot);
+    if (tid < kWords) {
+        word[tid] = w;
+        before[tid] = pre;
     }
     __syncthreads();
     const uint64_t T = ctr->trusted;
     const uint64_t tpre = tile_pre[blockIdx.x];   // trusted keys before this tile
+    const uint64_t epre = T + (tile0 - tpre);
     const unsigned lt = (1u << lane) - 1;
 #pragma unroll
     for (int j = 0; j < kRounds; ++j) {
-        const uint64_t i = tile0 + (uint64_t)j * kSortThreads + threadIdx.x;
-        if (i >= n) continue;
-        const uint64_t off = i - tile0;   // keys of the tile before this one
-        const uint64_t tr_before = seg[j * kWarps + warp] + __popc(bal[j] & lt);
-        const uint64_t o = (bal[j] >> lane) & 1u ? tpre + tr_before
-                                                : T + (tile0 - tpre) + (off - tr_before);
+        const unsigned off = j * kSortThreads + tid;   // keys of the tile before this one
+        if (tile0 + off >= n) continue;
+        const unsigned b = word[j * (kSortThreads / 32) + warp];
+        const unsigned tr = before[j * (kSortThreads / 32) + warp] + __popc(b & lt);
+        const uint64_t o = (b >> lane) & 1u ? tpre + tr : epre + (off - tr);
 #pragma unroll
-        for (int w = 0; w < KW; ++w) out[o * KW + w] = keys[i * KW + w];
+        for (int q = 0; q < KW; ++q) out[o * KW + q] = key[j][q];
     }
 }
 
@@ -1162,32 +1205,25 @@ cudaError_t launch_query(const uint64_t *keys, uint64_t n, int kw, int K, Geomet
     return cudaGetLastError();
 }
 
-cudaError_t launch_classify_query(const uint64_t *keys, uint64_t n, int kw, Geometry G,
-                                  uint32_t tau, uint32_t *est, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    const unsigned g = grid_for(n, 256, 152 * 8);
-    if (kw == 1)
-        classify_query_kernel<1><<<g, 256, 0, s>>>(keys, n, G, tau, est);
-    else
-        classify_query_kernel<2><<<g, 256, 0, s>>>(keys, n, G, tau, est);
-    return cudaGetLastError();
-}
-
 uint64_t split_scratch_words(uint64_t n) { return (n + kSplitTile - 1) / kSplitTile + 1; }
 
-cudaError_t launch_split(const uint64_t *keys, const uint32_t *est, uint64_t n, int kw,
-                         uint32_t tau, uint64_t *out, uint64_t *scratch, DevCounters *ctr,
-                         cudaStream_t s) {
+cudaError_t launch_classify(const uint64_t *keys, uint64_t n, int kw, Geometry G, uint32_t tau,
+                            const uint8_t *sure, uint32_t *bits, uint64_t *out, uint64_t *scratch,
+                            DevCounters *ctr, cudaStream_t s) {
     if (n == 0) return cudaMemsetAsync(&ctr->trusted, 0, sizeof(ctr->trusted), s);
     const uint64_t ntiles = (n + kSplitTile - 1) / kSplitTile;
-    split_count_kernel<<<(unsigned)ntiles, kSortThreads, 0, s>>>(est, n, tau, scratch);
-    split_scan_kernel<<<1, kSortThreads, 0, s>>>(scratch, ntiles, ctr);
+    const unsigned g = (unsigned)(ntiles < 152 * 8 ? ntiles : 152 * 8);
     if (kw == 1)
-        split_scatter_kernel<1><<<(unsigned)ntiles, kSortThreads, 0, s>>>(keys, est, n, tau, scratch,
-                                                                          ctr, out);
+        classify_mark_kernel<1><<<g, kSortThreads, 0, s>>>(keys, n, G, tau, sure, bits, scratch);
     else
-        split_scatter_kernel<2><<<(unsigned)ntiles, kSortThreads, 0, s>>>(keys, est, n, tau, scratch,
-                                                                          ctr, out);
+        classify_mark_kernel<2><<<g, kSortThreads, 0, s>>>(keys, n, G, tau, sure, bits, scratch);
+    split_scan_kernel<<<1, 1024, 0, s>>>(scratch, ntiles, ctr);
+    if (kw == 1)
+        split_scatter_kernel<1><<<(unsigned)ntiles, kSortThreads, 0, s>>>(keys, bits, n, scratch, ctr,
+                                                                          out);
+    else
+        split_scatter_kernel<2><<<(unsigned)ntiles, kSortThreads, 0, s>>>(keys, bits, n, scratch, ctr,
+                                                                          out);
     return cudaGetLastError();
 }
 

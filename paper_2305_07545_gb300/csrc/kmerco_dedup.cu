@@ -1477,6 +1477,7 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_kernel(EmitArgs e) {
                 key[q] = load_key<KW>(e.keys, at);
                 w[q] = (uint32_t)min((uint64_t)e.mult[at], G.maxc);
                 if (e.dlist) store_key<KW>(e.dlist, i, key[q]);
+                if (e.sure) e.sure[i] = w[q] > e.tau;
             }
         }
         for (unsigned a0 = 0; a0 < nh; a0 += kEmitHashes) {
@@ -1600,6 +1601,7 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_atomic_kernel(EmitArgs e
         const Key<KW> key = load_key<KW>(e.keys, at);
         const uint64_t w = min((uint64_t)e.mult[at], G.maxc);
         if (e.dlist) store_key<KW>(e.dlist, i, key);
+        if (e.sure) e.sure[i] = w > e.tau;
         const uint64_t k1m = KW == 1 ? premix8(key.lo) : 0;
         for (int a0 = 0; a0 < G.nhash; a0 += 4) {
             uint64_t cell[4], cur[4], prev[4];

@@ -102,7 +102,9 @@ struct EmitArgs {
     unsigned n_total;        // ranges
     int ordered;             // keys in the order of the ranges (places, offsets), else as they stand
     unsigned begin, end;     // distinct keys of this pass
-    uint64_t *dlist;         // distinct list to write (handles without keys), or null
+    uint64_t *dlist;         // distinct list to write, or null
+    uint8_t *sure;           // key i has more than tau windows (or null)
+    uint32_t tau;
     int coarse_shift, slot_bits, w_bits;
     uint32_t *coarse;
     uint64_t coarse_cap;

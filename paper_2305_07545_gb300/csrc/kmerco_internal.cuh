@@ -446,16 +446,14 @@ cudaError_t bucket_place_and_sort(const uint64_t *in, uint64_t *out, uint64_t n,
 
 cudaError_t launch_query(const uint64_t *keys, uint64_t n, int kw, int K, Geometry G,
                          uint32_t *est, cudaStream_t s);
-// Algorithm 5 only as far as the split on tau needs it (classify_query_kernel):
-// est exact for keys above tau, at most tau otherwise.
-cudaError_t launch_classify_query(const uint64_t *keys, uint64_t n, int kw, Geometry G,
-                                  uint32_t tau, uint32_t *est, cudaStream_t s);
-// est > tau split, stable: trusted keys to out[0, T), erroneous to out[T, n);
-// T written to ctr->trusted.  scratch needs split_scratch_words(n) uint64.
+// Algorithm 2's split of n keys: trusted keys (estimate > tau) to out[0, T),
+// erroneous to out[T, n), both in order; T written to ctr->trusted.  A key with
+// a nonzero `sure` byte (null: none) is known to be trusted.  bits needs n / 32 + 1
+// words, scratch split_scratch_words(n).
 uint64_t split_scratch_words(uint64_t n);
-cudaError_t launch_split(const uint64_t *keys, const uint32_t *est, uint64_t n, int kw,
-                         uint32_t tau, uint64_t *out, uint64_t *scratch, DevCounters *ctr,
-                         cudaStream_t s);
+cudaError_t launch_classify(const uint64_t *keys, uint64_t n, int kw, Geometry G, uint32_t tau,
+                            const uint8_t *sure, uint32_t *bits, uint64_t *out, uint64_t *scratch,
+                            DevCounters *ctr, cudaStream_t s);
 cudaError_t launch_merge(uint64_t *dst, const uint64_t *src, Geometry G, cudaStream_t s);
 // pos[i] = lower bound of probe i (kw words) in n sorted keys.
 cudaError_t launch_lower_bound(const uint64_t *keys, uint64_t n, int kw, const uint64_t *probes,

@@ -121,3 +121,49 @@ def test_all_ones_key():
     g = gpu_run(b, o, 32, 1 << 16, 4, 3, 2, forward_only=True)
     ref = check(g, b, o, 32, 4, 3, 2, forward_only=True)
     assert ref.distinct_lo[-1] == np.uint64(0xFFFFFFFFFFFFFFFF)
+
+
+def test_batch_replay_after_a_handle_moved_its_list():
+    # a captured batch insert writes a handle's list; inserting into the handle
+    # alone merges that list into another buffer: the batch must not replay into
+    # the old one
+    parts = [readsim.scaled("tiny", 2500, seed_offset=60 + i).generate() for i in range(3)]
+    dev = [(_dev(b), _dev(o)) for b, o in parts]
+    stream = torch.cuda.Stream()
+    fs = [kc.CountBF(21, 1 << 20, 4, 3, 2, stream=stream.cuda_stream) for _ in range(2)]
+    with kc.Batch(fs) as batch:
+        batch.schedule(1, 2)
+        for turn in range(3):
+            batch.insert([dev[0][0], dev[1][0]], [dev[0][1], dev[1][1]])
+            if turn == 1:
+                fs[0].insert(*dev[2])
+            batch.classify()
+            for i, f in enumerate(fs):
+                b, o = parts[i]
+                if turn == 1 and i == 0:
+                    b = np.concatenate([b, parts[2][0]])
+                    o = np.concatenate([o, parts[2][1][1:] + o[-1]])
+                keys, est = f.distinct()
+                g = dict(stats=f.stats(), counters=f.counters(), keys=keys, est=est,
+                         trusted=f.trusted(), erroneous=f.erroneous())
+                check(g, b, o, 21, 4, 3, 2)
+    for f in fs:
+        f.close()
+
+
+def test_replaced_counters_decide_the_split():
+    # keys with more than tau windows are trustworthy without a look at their
+    # counters only while the counters are those of their windows
+    b, o = readsim.scaled("tiny", 2000, seed_offset=77).generate()
+    with kc.CountBF(21, 1 << 20, 4, 3, 2) as bf:
+        bf.insert(_dev(b), _dev(o))
+        cells = bf.counters()
+        kc.kmerco_set_counters(bf.h, np.zeros_like(cells), len(cells))
+        bf.classify()
+        assert bf.stats()["trustworthy"] == 0
+        kc.kmerco_set_counters(bf.h, cells, len(cells))
+        bf.classify()
+        keys, est = bf.distinct()
+        g = dict(stats=bf.stats(), counters=bf.counters(), keys=keys, est=est,
+                 trusted=bf.trusted(), erroneous=bf.erroneous())
+    check(g, b, o, 21, 4, 3, 2)
