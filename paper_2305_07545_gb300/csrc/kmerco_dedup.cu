@@ -7,8 +7,9 @@
 //
 //   1. pack_kernel: the bases as 2-bit codes and one bit per base that starts
 //      a window to be counted; nothing reads the caller's buffers after it.
-//   2. sample_kernel, splitters_kernel: keys of random windows, sorted; they
-//      cut the key space into ranges that hold about equally many windows.
+//   2. sample_kernel, rank_kernel: keys of random windows and their ranks; the
+//      ones at even ranks cut the key space into ranges that hold about
+//      equally many windows.
 //      extract_kernel: per chunk of window starts, every window's canonical
 //      key (rolled from base to base); the chunk's keys are grouped by range
 //      in shared memory and leave as one contiguous piece, with the piece's
@@ -133,7 +134,7 @@ __device__ __forceinline__ unsigned find_range(const uint64_t *spl, const uint16
 // v (1,024 threads); xch: 1024 * E words of shared memory.  Strides inside a
 // thread are register swaps, inside a warp shuffles; only the 15 steps of
 // larger strides go through shared memory (105 of a plain network of 16,384
-// values: 155 -> 20 us for one block).
+// values).
 template <int E>
 __device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
     constexpr unsigned P = 1024 * E;
@@ -178,26 +179,18 @@ __device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
     }
 }
 
-// n - 1 splitters at even ranks of the `valid` smallest of the sorted samples
-// s, and their lookup table, written to global memory; s (32 KiB at least) is
-// overwritten.  lo, last: the least and the largest prefix of the range that
-// they cut.  1,024 threads, n <= kMaxRanges.
-__device__ __forceinline__ void write_splitters(uint64_t *s, unsigned valid, unsigned n,
-                                                uint64_t lo, uint64_t last, uint64_t *spl,
-                                                uint16_t *lut) {
+// The lookup table of n - 1 splitters of the range [lo, last], v the thread's
+// (1,024 threads, n <= kMaxRanges); cells: 32 KiB of shared memory.
+__device__ __forceinline__ void write_lut(unsigned *cells, uint64_t v, bool any, unsigned n,
+                                          uint64_t lo, uint64_t last, uint16_t *lut) {
     static_assert(kMaxRanges <= 1024, "a splitter a thread");
     constexpr unsigned E = (1u << kLutBits) / 1024;
     const unsigned j = threadIdx.x;
     int sh = bit_len(last - lo) - kLutBits;
     if (sh < 0) sh = 0;
-    uint64_t v = ~0ull;   // the last of the n: what find_range stops at
-    if (valid && j + 1 < n) v = s[(uint64_t)(j + 1) * valid / n];
-    if (j < n) spl[j] = v;
-    __syncthreads();
-    unsigned *cells = (unsigned *)s;   // splitters in every cell of the table
     for (unsigned i = j; i < (1u << kLutBits); i += 1024) cells[i] = 0;
     __syncthreads();
-    if (j + 1 < n && valid) {
+    if (j + 1 < n && any) {   // splitters in every cell of the table
         const uint64_t c = (v - lo) >> sh;
         if (c < (1u << kLutBits)) atomicAdd(cells + c, 1u);
     }
@@ -308,57 +301,84 @@ __device__ __forceinline__ Key<2> revcomp(const Key<2> &f, int K) {
 }
 
 // ----------------------------------------------------------- 2. splitters
-// One sample per thread: the prefix of the key at a random valid window start
-// (a few tries), else all ones, which sorts last.
+constexpr unsigned kSampleTile = 1024;   // samples a block sorts
+
+// Prefixes of the keys at n random valid window starts of the pass's `span` bases (a
+// few tries each), as sorted tiles of kSampleTile; the last one is filled up with
+// all ones.  Whole prefixes: copies of a repeat have long beginnings in common,
+// and cutting by their top 31 bits left more than twice as many windows in some
+// ranges (dedup_big_kernel 2.8 instead of 1.8 ms for 3.8e8 two-word windows).
 template <int KW>
-__global__ void __launch_bounds__(128) sample_kernel(PackArgs x, int K, int canonical,
-                                                     uint64_t span, unsigned n, uint64_t *out,
-                                                     DedupMeta *meta) {
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int canonical,
+                                                      uint64_t span, unsigned n,
+                                                      uint64_t *samples, DedupMeta *meta) {
+    __shared__ uint64_t xch[kSampleTile];
+    const unsigned i = blockIdx.x * kSampleTile + threadIdx.x;
+    uint64_t v[1] = {~0ull};
     bool found = false;
-    uint64_t prefix = ~0ull;
-    for (unsigned t = 0; i < n && t < 4 && !found; ++t) {
-        // window starts spread evenly over the pass, jittered
+    for (unsigned t = 0; t < 4 && i < n && !found; ++t) {
+        // window starts spread evenly over the pass, jittered; then anywhere
         const uint64_t slot = (uint64_t)i * span / n, wide = max(span / n, (uint64_t)1);
-        uint64_t p = slot + mix64((uint64_t)i * 4 + t) % wide;
-        if (t >= 2) p = mix64(~((uint64_t)i * 4 + t)) % span;
-        if (!((x.valid[p >> 4] >> (p & 15)) & 1u)) continue;
+        const uint64_t z = mix64((uint64_t)i * 4 + t);
+        const uint64_t at = t < 2 ? slot + __umul64hi(z, wide) : __umul64hi(z, span);
+        if (!((x.valid[at >> 4] >> (at & 15)) & 1u)) continue;
         Key<KW> f;
-        window_at((const uint64_t *)x.codes, p, K, f);
-        prefix = prefix_of<KW>(canonical_key(f, revcomp(f, K), canonical), K);
+        window_at((const uint64_t *)x.codes, at, K, f);
+        v[0] = prefix_of<KW>(canonical_key(f, revcomp(f, K), canonical), K);
         found = true;
     }
-    if (i < n) out[i] = prefix;
-    const unsigned bal = __ballot_sync(0xffffffffu, found);
-    if ((threadIdx.x & 31) == 0 && bal) atomicAdd(&meta->sampled, (unsigned)__popc(bal));
+    const int c = __syncthreads_count(found);
+    if (threadIdx.x == 0 && c) atomicAdd(&meta->sampled, (unsigned)c);
+    block_sort<1>(v, xch);
+    samples[i] = v[0];
 }
 
-// The block's values sorted into s (1024 * E words of shared memory).
-template <int E>
-__device__ __forceinline__ void sort_into(uint64_t (&v)[E], uint64_t *s) {
-    block_sort<E>(v, s);
+// The samples of even ranks among the n of all tiles become the n_ranges - 1
+// splitters.  Block b ranks tile b: a sample's place in it, and by bisection its
+// places in the other tiles (all of them in shared memory; of equal samples the
+// ones of earlier tiles come first).  The last block to finish builds the lookup
+// table.  One block that sorted all samples took 20 us for 4,096 of them and 80 for
+// 16,384, a fifth to a third of a piece of 5e5 windows.
+__global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples, unsigned n,
+                                                    unsigned n_ranges, uint64_t last,
+                                                    DedupMeta *meta, uint64_t *spl,
+                                                    uint16_t *lut) {
+    extern __shared__ ulonglong2 s2[];
+    __shared__ bool is_last;
+    uint64_t *const s = (uint64_t *)s2;
+    const unsigned tid = threadIdx.x, own = blockIdx.x;
+    for (unsigned i = tid; i < n / 2; i += 1024) s2[i] = ((const ulonglong2 *)samples)[i];
     __syncthreads();
+    const uint64_t v = s[own * kSampleTile + tid];
+    unsigned rank = tid;
+    for (unsigned c = 0; c < n / kSampleTile; ++c) {
+        if (c == own) continue;
+        const uint64_t *const t = s + c * kSampleTile;
+        unsigned at = 0;   // samples of the tile in front of v
 #pragma unroll
-    for (int e = 0; e < E; ++e) s[threadIdx.x * E + e] = v[e];
-    __syncthreads();
-}
-
-// Sorts the n samples (at most 1024 * E) and takes the splitters of n_ranges
-// ranges.  One block.
-template <int E>
-__global__ void __launch_bounds__(1024) splitters_kernel(const uint64_t *samples, unsigned n,
-                                                         unsigned n_ranges, uint64_t last,
-                                                         uint64_t *spl, uint16_t *lut,
-                                                         const DedupMeta *meta) {
-    extern __shared__ uint64_t s[];
-    uint64_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const unsigned i = e * 1024 + threadIdx.x;
-        v[e] = i < n ? samples[i] : ~0ull;
+        for (unsigned step = kSampleTile / 2; step; step >>= 1)
+            if (t[at + step - 1] < v || (c < own && t[at + step - 1] == v)) at += step;
+        rank += at + (t[at] < v || (c < own && t[at] == v) ? 1 : 0);
     }
-    sort_into<E>(v, s);
-    write_splitters(s, meta->sampled, n_ranges, 0, last, spl, lut);
+    const unsigned valid = meta->sampled;
+    if (rank < valid) {   // splitter k - 1 is the sample of rank k * valid / n_ranges
+        const uint64_t r = rank;
+        for (uint64_t k = (r * n_ranges + valid - 1) / valid;
+             k < n_ranges && k * valid / n_ranges == r; ++k)
+            if (k) spl[k - 1] = v;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) is_last = atomicAdd(&meta->ranked, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    uint64_t f = ~0ull;   // the last of the n: what find_range stops at
+    if (valid && tid + 1 < n_ranges)
+        f = __ldcg(spl + tid);
+    else if (tid < n_ranges)
+        spl[tid] = f;
+    write_lut((unsigned *)s, f, valid != 0, n_ranges, 0, last, lut);
 }
 
 // ------------------------------------------------- grouping keys by range
@@ -641,14 +661,20 @@ __global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int 
         }
     }
     if (found) atomicAdd(&valid, found);
-    sort_into<E>(v, s);
+    block_sort<E>(v, s);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) s[threadIdx.x * E + e] = v[e];
+    __syncthreads();
     // as many ranges as this one's windows fill, so that only the fine samples
     // spread the sizes; the others stay empty (all-ones splitters)
     const unsigned nf = max(1u, min(x.n_fine, (x.totals[b] + x.target - 1) / x.target));
-    write_splitters(s, valid, nf, lo, hi, x.fine_spl + (uint64_t)b * kMaxRanges,
-                    x.fine_lut + (uint64_t)b * kLutStride);
-    for (unsigned i = nf + threadIdx.x; i < x.n_fine; i += 1024)
-        x.fine_spl[(uint64_t)b * kMaxRanges + i] = ~0ull;
+    const unsigned j = threadIdx.x;
+    uint64_t f = ~0ull;
+    if (valid && j + 1 < nf) f = s[(uint64_t)(j + 1) * valid / nf];
+    if (j < x.n_fine) x.fine_spl[(uint64_t)b * kMaxRanges + j] = f;
+    __syncthreads();
+    write_lut((unsigned *)s, f, valid != 0, nf, lo, hi, x.fine_lut + (uint64_t)b * kLutStride);
 }
 
 // One tile of a range: gather its keys from the pieces, group them by fine
@@ -1645,6 +1671,8 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_atomic_kernel(EmitArgs e
     }
 }
 
+unsigned round_up(unsigned n, unsigned to) { return (n + to - 1) / to * to; }
+
 // Sub-arrays of DedupBufs::meta.
 struct MetaLayout {
     uint64_t size = 0;
@@ -1659,7 +1687,7 @@ struct MetaLayout {
         meta = take(sizeof(DedupMeta));
         codes = take(p.chunks * p.chunk / 4 + 64);   // and 128 bases after the last chunk
         valid = take(p.chunks * p.chunk / 8);
-        samples = take(p.samples * 8ull);
+        samples = take(round_up(p.samples, kSampleTile) * 8ull);
         spl = take(kMaxRanges * 8ull);
         lut = take(kLutStride * 2ull);
         piece = take(p.chunks * 4);
@@ -1830,9 +1858,11 @@ DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk) {
         p.n_fine = (unsigned)std::min<uint64_t>(mean + mean / 4, kMaxRanges);
         p.fine_samples = std::min(16 * p.n_fine, kMaxSamples);
     }
-    // sizes spread by about a quarter around their mean; ranges far below a
-    // dedup block's room do with fewer samples
-    p.samples = std::min((bound / ranges < 1024 ? 8 : 32) * p.n_ranges, kMaxSamples);
+    // sixteen spread the sizes by a quarter around their mean; ranges far below a
+    // dedup block's room do with eight (with eight for 900 two-word windows a range,
+    // many ranges went to dedup_big_kernel: 112 us of a 370 us call, now 21 of 260)
+    const unsigned per_range = p.n_fine ? 32 : bound / ranges * 2 <= p.target ? 8 : 16;
+    p.samples = std::min(per_range * p.n_ranges, kMaxSamples);
     p.on = true;
     return p;
 }
@@ -1863,23 +1893,20 @@ cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical,
                           uint64_t span, int sms, cudaStream_t s, uint64_t &launches) {
     const MetaLayout m(p);
     DedupMeta *meta = (DedupMeta *)(d.meta + m.meta);
-    uint64_t *samples = (uint64_t *)(d.meta + m.samples);
     PackArgs pa;
     memset(&pa, 0, sizeof(pa));
     pa.codes = (uint32_t *)(d.meta + m.codes);
     pa.valid = (uint16_t *)(d.meta + m.valid);
     DD_TRY(cudaMemsetAsync(meta, 0, sizeof(DedupMeta), s));
-    const unsigned g = (p.samples + 127) / 128;
-    if (p.kw == 1)
-        sample_kernel<1><<<g, 128, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
-    else
-        sample_kernel<2><<<g, 128, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
-    const int E = sort_items(p.samples);
-    auto *sk = E == 1 ? splitters_kernel<1> : E == 2 ? splitters_kernel<2>
-             : E == 4 ? splitters_kernel<4> : E == 8 ? splitters_kernel<8> : splitters_kernel<16>;
-    DD_TRY(set_smem(sk, std::max(E, 4) * 8192));
-    sk<<<1, 1024, std::max(E, 4) * 8192, s>>>(samples, p.samples, p.n_ranges, last_prefix(p.K),
-                                 (uint64_t *)(d.meta + m.spl), (uint16_t *)(d.meta + m.lut), meta);
+    uint64_t *samples = (uint64_t *)(d.meta + m.samples);
+    const unsigned n = round_up(p.samples, kSampleTile), tiles = n / kSampleTile;
+    const size_t smem = std::max(n * sizeof(uint64_t), sizeof(unsigned) << kLutBits);
+    auto *sk = p.kw == 1 ? sample_kernel<1> : sample_kernel<2>;
+    sk<<<tiles, 1024, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
+    DD_TRY(set_smem(rank_kernel, smem));
+    rank_kernel<<<tiles, 1024, smem, s>>>(samples, n, p.n_ranges, last_prefix(p.K), meta,
+                                          (uint64_t *)(d.meta + m.spl),
+                                          (uint16_t *)(d.meta + m.lut));
     ExtractArgs x;
     x.codes = pa.codes;
     x.valid = pa.valid;

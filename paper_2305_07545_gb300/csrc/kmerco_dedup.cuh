@@ -27,16 +27,17 @@ constexpr int kSubBits2 = 9;
 constexpr int kSubBins2 = (1 << kSubBits2) + 1;   // the range's last prefix may open one more
 constexpr uint64_t kMaxRangeWindows = 1ull << 31;   // of one pass (32-bit key indexes)
 constexpr uint64_t kPlanSms = 152;       // SMs of a GB300: plans follow from the input alone
-constexpr unsigned kMaxSamples = 16384;  // samples one block sorts in shared memory
+constexpr unsigned kMaxSamples = 16384;  // samples that cut a level's ranges, at most
 
 struct DedupMeta {
     unsigned cursor;       // keys reserved by extract_kernel
     unsigned out_cursor;   // keys reserved by dedup_kernel
     unsigned distinct;     // distinct keys of the call
     unsigned n_tiles;      // refine tiles
-    unsigned sampled;      // valid samples
+    unsigned sampled;      // samples that are keys
+    unsigned ranked;       // blocks of rank_kernel that are done
     unsigned n_big;        // ranges left to dedup_big_kernel
-    unsigned pad[2];
+    unsigned pad;
 };
 
 struct TileMap {

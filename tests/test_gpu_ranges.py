@@ -167,3 +167,23 @@ def test_replaced_counters_decide_the_split():
         g = dict(stats=bf.stats(), counters=bf.counters(), keys=keys, est=est,
                  trusted=bf.trusted(), erroneous=bf.erroneous())
     check(g, b, o, 21, 4, 3, 2)
+
+
+@pytest.mark.parametrize("K", [21, 40])
+def test_uneven_reads_and_few_windows(K):
+    # runs of empty and short reads at the chunks' borders, long ones over several
+    # chunks; then a call of which nearly no window counts, so that there are
+    # fewer samples than ranges
+    st = readsim.Stream(K)
+    lens = np.concatenate([np.zeros(3000, np.int64), [33000], st.integers(9000, 8).astype(np.int64),
+                           [1023, 1, 4096, 0, 0, 12001], st.integers(200, 300).astype(np.int64)])
+    o = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    b = readsim.ASCII[st.integers(int(o[-1]), 4).astype(np.uint8)]
+    g = gpu_run(b, o, K, 1 << 18, 4, 3, 2)
+    check(g, b, o, K, 4, 3, 2)
+    b = np.full(70000, ord("N"), np.uint8)
+    o = np.array([0, 70000], np.uint64)
+    for at in (0, 35000, 70000 - K - 9):
+        b[at:at + K + 9] = readsim.ASCII[st.integers(K + 9, 4).astype(np.uint8)]
+    g = gpu_run(b, o, K, 1 << 18, 4, 3, 2)
+    check(g, b, o, K, 4, 3, 2)
