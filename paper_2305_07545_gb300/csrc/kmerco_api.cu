@@ -99,7 +99,8 @@ struct kmerco {
                              // for the trustworthy ones
     cudaEvent_t ev[4];
     cudaStream_t copy_stream;                      // host input copies (created on first use)
-    cudaEvent_t copy_ev[kCopyPieces + 1], copy_fork;
+    cudaEvent_t copy_ev[kCopyPieces + 1];          // of the reads' pieces, of the offsets
+    cudaEvent_t copy_fork, input_read;             // input_read: the staged inputs have been read
     bool insert_timed, classify_timed;
     uint64_t launches;       // kernels launched by this handle
     uint64_t *range_a, *range_b;   // insertion by key ranges: keys, multiplicities, tables
@@ -630,23 +631,36 @@ struct HostCopy {
     uint64_t piece_lo(int i) const { return nbytes * (uint64_t)i / (uint64_t)npieces; }
 };
 
-// Issue the copy of nbytes host bytes src -> dst in pieces on the handle's
-// copy stream, after the work already queued on the handle's stream (the
-// previous call may still read dst).
-int issue_host_copy(kmerco_t *h, const uint8_t *src, uint8_t *dst, uint64_t nbytes,
-                    HostCopy &hc) {
+// The copy stream, ready to overwrite the input staging.  On the handle's own
+// stream nothing but the handle's calls is queued, so the copies wait only until
+// the last insert has read the staging (its first kernels: sixteen pieces of one
+// sample then move while the pieces before are counted, 12.1 -> 11.4 ms); on a
+// caller's stream, or into buffers that are new, they come after everything queued.
+int fork_copies(kmerco_t *h, bool new_buffers) {
     if (!h->copy_stream) {
         bool ok = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&h->copy_fork, cudaEventDisableTiming) == cudaSuccess;
+                  cudaEventCreateWithFlags(&h->copy_fork, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&h->input_read, cudaEventDisableTiming) == cudaSuccess;
         for (int i = 0; ok && i <= kCopyPieces; ++i)
             ok = cudaEventCreateWithFlags(&h->copy_ev[i], cudaEventDisableTiming) == cudaSuccess;
         if (!ok) return KMERCO_ECUDA;
     }
+    if (h->own_stream && !new_buffers) {
+        KM_CUDA(cudaStreamWaitEvent(h->copy_stream, h->input_read, 0));
+    } else {
+        KM_CUDA(cudaEventRecord(h->copy_fork, h->stream));
+        KM_CUDA(cudaStreamWaitEvent(h->copy_stream, h->copy_fork, 0));
+    }
+    return KMERCO_OK;
+}
+
+// Issue the copy of nbytes host bytes src -> dst in pieces on the copy stream
+// (after fork_copies).
+int issue_host_copy(kmerco_t *h, const uint8_t *src, uint8_t *dst, uint64_t nbytes,
+                    HostCopy &hc) {
     hc.nbytes = nbytes;
     hc.npieces = nbytes >= (8ull << 20) ? kCopyPieces : 1;
     hc.ev = h->copy_ev;
-    KM_CUDA(cudaEventRecord(h->copy_fork, h->stream));
-    KM_CUDA(cudaStreamWaitEvent(h->copy_stream, h->copy_fork, 0));
     for (int i = 0; i < hc.npieces; ++i) {
         const uint64_t lo = hc.piece_lo(i), hi = hc.piece_lo(i + 1);
         if (hi > lo)
@@ -748,10 +762,10 @@ uint64_t *merge_input(const InsertPlan &ip, const InsertBufs &b) {
 // the plan's kernels.  h->first_read must hold the call's chunks; b holds the
 // plan's buffers.  With hc (a host input being copied) the kernels that read
 // the bases are split into up to kCopyPieces launches, each waiting only for
-// the pieces it reads.
+// the pieces it reads; input_read is recorded when the input has been read.
 int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
                          const InsertBufs &b, cudaStream_t s, uint64_t &launches,
-                         const HostCopy *hc = nullptr) {
+                         const HostCopy *hc = nullptr, cudaEvent_t input_read = nullptr) {
     const uint64_t nbytes = a.last - a.first;
     const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
     const uint64_t nchunks = (nbytes + chunk - 1) / chunk;
@@ -775,6 +789,7 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
             }
             KM_CUDA(dedup_pack(ip.dd, b.dd, a, cb, ce - cb, c0, c1, h->sms, s, launches));
         }
+        if (input_read && pass + 1 == ip.passes) KM_CUDA(cudaEventRecord(input_read, s));
         if (!ip.ranges) continue;
         KM_CUDA(dedup_extract(ip.dd, b.dd, a.canonical, ce - cb,
                               std::min(ce * chunk, nbytes) - cb * chunk, h->sms, s, launches));
@@ -1062,6 +1077,7 @@ void kmerco_destroy(kmerco_t *h) {
         for (int i = 0; i <= kCopyPieces; ++i)
             if (h->copy_ev[i]) cudaEventDestroy(h->copy_ev[i]);
         if (h->copy_fork) cudaEventDestroy(h->copy_fork);
+        if (h->input_read) cudaEventDestroy(h->input_read);
         if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
         if (h->out_ready) cudaEventDestroy(h->out_ready);
         if (h->out_done) cudaEventDestroy(h->out_done);
@@ -1103,15 +1119,20 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
     if (host_offsets) {   // checked and summed on the device too
         // the offsets go first: a check that waits for them then does not wait
         // for the reads' bytes queued behind them on the copy engine
+        const uint64_t *old_off = h->in_offsets;
+        const uint8_t *old_bases = h->in_bases;
+        const uint64_t nb = host_bases && offsets[nreads] > offsets[0] ? offsets[nreads] - offsets[0] : 0;
         KM_TRY(ensure(h, &h->in_offsets, &h->in_offsets_cap, nreads + 1));
+        if (nb) KM_TRY(ensure(h, &h->in_bases, &h->in_bases_cap, nb));
+        KM_TRY(fork_copies(h, h->in_offsets != old_off || h->in_bases != old_bases));
         KM_CUDA(cudaMemcpyAsync(h->in_offsets, offsets, (nreads + 1) * 8, cudaMemcpyHostToDevice,
-                                h->stream));
+                                h->copy_stream));
+        KM_CUDA(cudaEventRecord(h->copy_ev[kCopyPieces], h->copy_stream));
+        KM_CUDA(cudaStreamWaitEvent(h->stream, h->copy_ev[kCopyPieces], 0));
         d_off = h->in_offsets;
-        if (host_bases && offsets[nreads] > offsets[0]) {
+        if (nb) {
             // the reads' bytes start moving now, while the offsets are checked;
             // the insert launches wait only for the pieces they read
-            const uint64_t nb = offsets[nreads] - offsets[0];
-            KM_TRY(ensure(h, &h->in_bases, &h->in_bases_cap, nb));
             KM_TRY(issue_host_copy(h, (const uint8_t *)bases + offsets[0], h->in_bases, nb, hc));
             copying = true;
         }
@@ -1146,7 +1167,9 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
             d_bases = (const uint8_t *)bases + first;
         } else {   // copied piece by piece on the copy stream (issued above when it could be)
             if (!copying) {
+                const uint8_t *old = h->in_bases;
                 KM_TRY(ensure(h, &h->in_bases, &h->in_bases_cap, nbytes));
+                KM_TRY(fork_copies(h, h->in_bases != old));
                 KM_TRY(issue_host_copy(h, (const uint8_t *)bases + first, h->in_bases, nbytes, hc));
                 copying = true;
             }
@@ -1173,7 +1196,8 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
     const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
                              h->part_ctr};
     KM_CUDA(cudaEventRecord(h->ev[0], h->stream));
-    KM_TRY(launch_sample_insert(h, a, ip, bufs, h->stream, h->launches, copying ? &hc : nullptr));
+    KM_TRY(launch_sample_insert(h, a, ip, bufs, h->stream, h->launches, copying ? &hc : nullptr,
+                                copying || host_offsets ? h->input_read : nullptr));
     if (ip.merge)
         KM_TRY(merge_keys(h, merge_input(ip, bufs), bound,
                           &dedup_result(ip.dd, bufs.dd, h->G, h->ctr, true).meta->distinct, nullptr));

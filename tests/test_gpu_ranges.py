@@ -187,3 +187,39 @@ def test_uneven_reads_and_few_windows(K):
         b[at:at + K + 9] = readsim.ASCII[st.integers(K + 9, 4).astype(np.uint8)]
     g = gpu_run(b, o, K, 1 << 18, 4, 3, 2)
     check(g, b, o, K, 4, 3, 2)
+
+
+@pytest.mark.parametrize("own_stream", [True, False])
+@pytest.mark.parametrize("pass_codes", [0, 40000])
+def test_pieces_copied_while_earlier_ones_are_counted(own_stream, pass_codes):
+    # pieces of many sizes from one pinned buffer each, without a wait between them;
+    # on a caller's stream a piece is written by a copy queued there right before
+    parts = [readsim.scaled("tiny", n, seed_offset=300 + i).generate()
+             for i, n in enumerate((3000, 40, 2500, 1, 3600, 700))]
+    stream = torch.cuda.Stream()
+    bf = kc.CountBF(21, 1 << 20, 4, 3, 2, pass_codes=pass_codes,
+                    stream=None if own_stream else stream.cuda_stream)
+    pinned = [(torch.from_numpy(b).pin_memory(), torch.from_numpy(o.view(np.int64)).pin_memory())
+              for b, o in parts]
+    if own_stream:
+        for b, o in pinned:
+            bf.insert(b, o)
+    else:
+        for b, o in pinned:
+            src = b.cuda()
+            b.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                torch.cuda._sleep(2_000_000)
+                b.copy_(src, non_blocking=True)
+            bf.insert(b, o)
+            torch.cuda.synchronize()
+    bf.classify()
+    keys, est = bf.distinct()
+    g = dict(stats=bf.stats(), counters=bf.counters(), keys=keys, est=est,
+             trusted=bf.trusted(), erroneous=bf.erroneous())
+    bf.close()
+    offs = [np.zeros(1, np.uint64)]
+    for _, o in parts:
+        offs.append(o[1:] + offs[-1][-1])
+    check(g, np.concatenate([b for b, _ in parts]), np.concatenate(offs), 21, 4, 3, 2)
