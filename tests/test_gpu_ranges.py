@@ -223,3 +223,14 @@ def test_pieces_copied_while_earlier_ones_are_counted(own_stream, pass_codes):
     for _, o in parts:
         offs.append(o[1:] + offs[-1][-1])
     check(g, np.concatenate([b for b, _ in parts]), np.concatenate(offs), 21, 4, 3, 2)
+
+
+@pytest.mark.parametrize("K", [21, 40])
+@pytest.mark.parametrize("nhash", [3, 6, 7])
+@pytest.mark.parametrize("alpha,m,dims", [(8, 0, (401, 409)), (4, 1 << 22, None), (8, 1100003, None)])
+def test_codes_of_three_hashes(K, nhash, alpha, m, dims):
+    # the partitioned increments with two and with three hashes a pass, keys that
+    # are no multiple of a block's
+    b, o = _uniform(1801, 151, seed=nhash + K)
+    g = gpu_run(b, o, K, m, alpha, nhash, 2, dims=dims)
+    check(g, b, o, K, alpha, nhash, 2, cross_check=False)
