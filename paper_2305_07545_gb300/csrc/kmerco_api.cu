@@ -397,7 +397,8 @@ int ensure_union(kmerco_t *h, uint64_t add) {
         h->d_ub = h->ctr_host->distinct;
     }
     KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub + add, (uint64_t)h->kw * 8));
-    return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub, add));
+    // several passes: each one's list into what is held by then
+    return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub + add, add));
 }
 
 // Merges an ascending list of *nb32 or *nb64 keys, at most nb_most, into the
@@ -516,19 +517,26 @@ struct InsertPlan {
     bool ranges = false;
     bool fresh = false;      // the handle holds no keys: the first pass writes the list
     bool sure = false;       // the list is the call's keys: which are sure is written too
-    bool merge = false;      // the list stays in order: the call's keys are merged into it
+    bool merge = false;      // the list stays in order: every pass's keys but the ones that
+                             // begin a list are merged into it
     uint64_t passes = 1;
     uint64_t bound = 0;      // windows of the call at most
     DedupPlan dd;
     PartPlan pp;
     // whether the call needs the distinct set
-    bool table() const { return !(ranges && (fresh || merge) && passes == 1); }
+    bool table() const { return !(ranges && (merge || (fresh && passes == 1))); }
+    uint64_t merges() const { return merge ? passes - (fresh ? 1 : 0) : 0; }
 };
 
 struct InsertBufs {
     DedupBufs dd;
     uint32_t *coarse, *fine;
     unsigned long long *ctr;
+    // of a call that merges: the list, the other buffer it is merged into (they
+    // take turns), and the keys held before, at most
+    uint64_t *list, *list2;
+    unsigned *union_scratch;
+    uint64_t held;
 };
 
 // Increment-code buffers sized for one pass of at most pass_codes increments,
@@ -579,7 +587,9 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->max_distinct ||
         h->G.cas_limit != kCasLimit || nbytes < bound)
         return ip;
-    uint64_t most = kMaxRangeWindows;   // windows one pass takes
+    // windows one pass takes (1.9e9 two-word windows: 239 ms with their classification
+    // in one pass, 244 in two that keep to the ranges' target)
+    uint64_t most = kMaxRangeWindows;
     if (h->pass_set) most = std::min(most, std::max<uint64_t>(h->pass_codes / (uint64_t)h->nhash, 1));
     ip.passes = (bound + most - 1) / most;
     const int chunk = dedup_chunk(nbytes);
@@ -592,8 +602,10 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     }
     ip.ranges = ip.dd.on;
     if (ip.ranges) ip.pp = plan_partition(h, ip.dd.bound);
-    ip.merge = ip.ranges && !fresh && may_merge && ip.passes == 1 && h->list_sorted &&
-               bound * kMergeShare >= h->d_ub && h->d_ub + bound < 0xFFFFFFFFull;
+    // (a call of several passes into an empty handle would else put its keys into a
+    // set and sort them: 2.4e9 windows 170 ms and 50 to classify, merged 143 and 28)
+    ip.merge = ip.ranges && may_merge && h->d_ub + bound < 0xFFFFFFFFull &&
+               (fresh ? ip.passes > 1 : h->list_sorted && bound * kMergeShare >= h->d_ub);
     return ip;
 }
 
@@ -773,6 +785,7 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
     launches += nchunks ? 1 : 0;
     const uint64_t q = hc && hc->npieces > 1 && ip.passes <= (uint64_t)kCopyPieces
                            ? std::max<uint64_t>(1, kCopyPieces / ip.passes) : 1;
+    uint64_t *list = b.list, *list2 = b.list2;
     for (uint64_t pass = 0; pass < ip.passes; ++pass) {
         const uint64_t cb = nchunks * pass / ip.passes, ce = nchunks * (pass + 1) / ip.passes;
         const uint64_t qq = std::min<uint64_t>(q, std::max<uint64_t>(1, ce - cb));
@@ -801,6 +814,13 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
         e.sure = fresh && ip.sure ? h->sure : nullptr;
         e.tau = h->tau;
         KM_TRY(launch_updates(h, ip, b, e, s, launches));
+        if (ip.merge && !fresh) {
+            const uint64_t before = std::min(b.held + pass * ip.dd.bound, b.held + ip.bound);
+            KM_CUDA(launch_union(list, before, e.dlist, ip.dd.bound, &e.meta->distinct, nullptr,
+                                 h->kw, list2, b.union_scratch, &h->ctr->distinct, s));
+            launches += 4;
+            std::swap(list, list2);
+        }
         if (!ip.table()) continue;
         // the pass's keys into the distinct set (the first pass of an empty
         // handle: its list as it stands)
@@ -1182,25 +1202,33 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
         ip = InsertPlan();
         ip.bound = bound;
     }
+    uint64_t held = 0;
     if (ip.merge) {
         const int st = ensure_union(h, bound);
         if (st == KMERCO_ENOMEM)
             ip.merge = false;   // the distinct set then
         else
             KM_TRY(st);
+        held = h->d_ub;
     }
-    if (!ip.merge) KM_TRY(ensure_set_capacity(h, bound, ip.table()));
-    ip.sure = !ip.table() && ip.fresh && ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
+    // a call merged once writes its list into the other buffer alone
+    if (!ip.merge || ip.passes > 1)
+        KM_TRY(ensure_set_capacity(h, bound, ip.table()));
+    else
+        h->d_ub += bound;
+    ip.sure = !ip.table() && ip.fresh && ip.passes == 1 &&
+              ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
     KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
     const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
-                             h->part_ctr};
+                             h->part_ctr, h->dlist, h->dlist2, h->union_scratch, held};
     KM_CUDA(cudaEventRecord(h->ev[0], h->stream));
     KM_TRY(launch_sample_insert(h, a, ip, bufs, h->stream, h->launches, copying ? &hc : nullptr,
                                 copying || host_offsets ? h->input_read : nullptr));
-    if (ip.merge)
-        KM_TRY(merge_keys(h, merge_input(ip, bufs), bound,
-                          &dedup_result(ip.dd, bufs.dd, h->G, h->ctr, true).meta->distinct, nullptr));
+    if (ip.merges() & 1) {
+        std::swap(h->dlist, h->dlist2);
+        std::swap(h->dlist_cap, h->dlist2_cap);
+    }
     if (!ip.table()) h->table_ok = false;   // the list alone was written
     h->list_sorted = !ip.table();
     h->sure_ok = ip.sure;

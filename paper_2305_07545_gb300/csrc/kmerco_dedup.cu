@@ -1854,6 +1854,9 @@ DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk) {
     } else {
         unsigned c = 32;
         while ((uint64_t)c * c < ranges && c < kMaxRanges) ++c;
+        // with the quarter, no more fine ranges than there may be
+        c = std::max(c, (unsigned)std::min<uint64_t>((ranges * 5 / 4 + kMaxRanges - 1) / kMaxRanges,
+                                                     kMaxRanges));
         p.n_ranges = c;
         const uint64_t mean = (ranges + c - 1) / c;   // and a quarter for the larger ones
         p.n_fine = (unsigned)std::min<uint64_t>(mean + mean / 4, kMaxRanges);

@@ -234,3 +234,23 @@ def test_codes_of_three_hashes(K, nhash, alpha, m, dims):
     b, o = _uniform(1801, 151, seed=nhash + K)
     g = gpu_run(b, o, K, m, alpha, nhash, 2, dims=dims)
     check(g, b, o, K, alpha, nhash, 2, cross_check=False)
+
+
+@pytest.mark.parametrize("K", [21, 40])
+@pytest.mark.parametrize("passes", [2, 3, 4])
+def test_passes_merged_into_the_list(K, passes):
+    # a call of several passes into an empty handle, and one into a handle that holds
+    # keys: every pass's keys are merged into the ascending list
+    parts = [readsim.scaled("single", n, seed_offset=400 + i).generate()
+             for i, n in enumerate((2400, 2000))]
+    windows = 2400 * (150 - K + 1)
+    dev = [(_dev(b), _dev(o)) for b, o in parts]   # read by every pass: kept until the end
+    with kc.CountBF(K, 1 << 20, 4, 3, 2, pass_codes=windows * 3 // passes + 3) as bf:
+        for b, o in dev:
+            bf.insert(b, o)
+        bf.classify()
+        keys, est = bf.distinct()
+        g = dict(stats=bf.stats(), counters=bf.counters(), keys=keys, est=est,
+                 trusted=bf.trusted(), erroneous=bf.erroneous())
+    offs = np.concatenate([parts[0][1], parts[1][1][1:] + parts[0][1][-1]])
+    check(g, np.concatenate([b for b, _ in parts]), offs, K, 4, 3, 2)
