@@ -51,7 +51,8 @@ PROFILE_SUMMARIES = {"single": PROFILE_SUMMARY,
                      "repeats55": os.path.join(ROOT, "profiles", "insert_phase_repeats.md")}
 SECONDARY = {"repeats": "repeats55"}   # workload timed after the headline one, same reads
 INSERT_SOURCES = [os.path.join(ROOT, "paper_2305_07545_gb300", "csrc", f)
-                  for f in ("kmerco_insert.cu", "kmerco_internal.cuh")]
+                  for f in ("kmerco_insert.cu", "kmerco_internal.cuh", "kmerco_stage.cuh",
+                            "kmerco_dedup.cu", "kmerco_dedup.cuh", "kmerco_union.cu")]
 
 
 def describe(w: readsim.Workload) -> str:
@@ -129,9 +130,9 @@ def roofline_of_insert(inserted: int, nhash: int, key_words: int, input_bytes: i
     sector_bytes = inserted * 64 * nhash
     return {"bound": "hbm", "achieved": achieved, "peak": peak_gbs, "unit": "GB/s",
             "frac": achieved / peak_gbs, "traffic": traffic,
-            "kernel": "insert phase: every kernel of one kmerco_insert call (insert_kernel: "
-                      "pack, canonical, hash, distinct set, increment staging; in the "
-                      "partitioned design also repartition_kernel and the apply kernel)",
+            "kernel": "insert phase: every kernel of one kmerco_insert call (by key ranges: "
+                      "pack, sample, extract, refine, dedup, emit, repartition, apply, union; "
+                      "small calls window by window)",
             "model": "word-granular: k_h x (8-byte cell read + write) + key written and "
                      "read once per inserted K-mer, plus the input",
             "algorithmic_bytes_per_kmer": per_kmer,

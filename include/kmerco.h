@@ -175,8 +175,8 @@ int kmerco_paper_dims(uint64_t n, double fpp, uint64_t *dim_x, uint64_t *dim_y);
  * Device bytes a handle with options *cfg holds at most after one
  * kmerco_insert of nreads reads (nbytes bases, `windows` windows: the sum of
  * max(0, len - K + 1), or the whole-file count) and one kmerco_classify:
- * the countBF, a distinct set and list sized for every window being a new
- * key, the increment-code buffers of the update design the call would take,
+ * the countBF, a distinct list (and a set, where the call needs one) sized for
+ * every window being a new key, the key-range and increment-code buffers of the update design the call would take,
  * the classification buffers for that many distinct keys, and with
  * host_inputs != 0 the staging copy of the reads.  This is the figure a
  * scheduler can admit a job by, and give the handle as its hbm_budget.
@@ -210,8 +210,9 @@ void kmerco_destroy(kmerco_t *h);
  * summed on the host, so the call does not wait for the device; device
  * offsets, and host offsets of more reads, are summed by a kernel whose
  * result the call waits for (copied ahead of the reads, so the wait is for
- * the offsets and the kernel only).  A call that has to grow the distinct set
- * also waits for the keys already held.
+ * the offsets and the kernel only).  A call that has to grow the distinct set or
+ * list may also wait to learn how many keys are held.  Device inputs are read by
+ * the call's kernels: keep them until the handle's stream has passed them.
  * Errors: EINVAL (NULL pointer with nreads > 0, nreads >= 2^32 - 1,
  * decreasing offsets); ENOMEM; ECUDA.
  */
