@@ -349,6 +349,9 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
         if (D) KM_CUDA(cudaMemcpyAsync(q, h->dlist, (D < h->dlist_cap ? D : h->dlist_cap) * h->kw * 8,
                                        cudaMemcpyDeviceToDevice, h->stream));
         KM_CUDA(cudaStreamSynchronize(h->stream));
+        // the sorted keys may be the list itself, and the getters read them still
+        // when the call fails further on
+        if (h->sorted == h->dlist) h->sorted = (uint64_t *)q;
         dev_free(h, h->dlist, h->dlist_cap * h->kw * 8);
         h->dlist = (uint64_t *)q;
         h->dlist_cap = want;

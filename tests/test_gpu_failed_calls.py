@@ -1,0 +1,58 @@
+"""A call that fails for memory leaves the handle as it was.
+
+The handle's results are read again after the refused call: keys, estimates,
+both lists and the countBF have to be those of the calls that succeeded.  The
+caller's allocator hands freed blocks out again at once, so results that are
+read from a freed buffer would hold the filler that the test puts there.
+"""
+import numpy as np
+import pytest
+
+import readsim
+
+torch = pytest.importorskip("torch")
+import paper_2305_07545_gb300 as kc  # noqa: E402
+from test_gpu_parity import _dev, check  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _results(bf):
+    keys, est = bf.distinct()
+    return dict(stats=bf.stats(), counters=bf.counters(), keys=keys, est=est,
+                trusted=bf.trusted(), erroneous=bf.erroneous())
+
+
+def _held(K, b, o, **kw):
+    """Device bytes of a handle after one insert and a classification."""
+    with kc.CountBF(K, 1 << 18, 4, 3, 2, **kw) as bf:
+        bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        return bf.stats()["device_bytes"]
+
+
+@pytest.mark.parametrize("K", [21, 40])
+@pytest.mark.parametrize("allocator", [None, "torch"])
+def test_results_after_an_insert_whose_set_does_not_fit(K, allocator):
+    # the second call moves the list (1.1e6 bytes a key word) and then finds no room
+    # for the set, which is twice as large
+    b, o = readsim.random_reads(17000 // (150 - K + 1) + 1, 150, 150, seed=5)
+    b2, o2 = readsim.random_reads(120000 // (150 - K + 1) + 1, 150, 150, seed=6)
+    kw = 1 if K <= 32 else 2
+    budget = _held(K, b, o) + 1_200_000 * kw
+    with kc.CountBF(K, 1 << 18, 4, 3, 2, hbm_budget=budget, allocator=allocator) as bf:
+        bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        d2 = _dev(b2), _dev(o2)
+        with pytest.raises(kc.KmercoError) as e:
+            bf.insert(*d2)
+        assert e.value.status == kc.ENOMEM
+        filler = [torch.full((n,), -1, dtype=torch.int64, device="cuda")
+                  for n in (1 << 14, 17000 * kw, 1 << 16, 1 << 18)]
+        torch.cuda.synchronize()
+        check(_results(bf), b, o, K, 4, 3, 2)
+        probes = bf.distinct()[0][::97].copy()
+        ranks = np.zeros(len(probes), np.uint64)
+        kc.kmerco_rank_of(bf.h, probes, len(probes), ranks)
+        assert np.array_equal(ranks, np.arange(0, bf.stats()["distinct"], 97, dtype=np.uint64))
+        del filler
