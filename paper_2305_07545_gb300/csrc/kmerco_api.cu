@@ -1522,10 +1522,14 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
     DeviceGuard guard(h->device);
     const uint64_t words = n * h->kw;
     const uint64_t *d_keys = keys;
-    if (!is_device_ptr(keys)) {   // stage host keys in the classification buffer
-        KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, words));
-        KM_CUDA(cudaMemcpyAsync(h->alt0, keys, words * 8, cudaMemcpyHostToDevice, h->stream));
-        d_keys = h->alt0;
+    if (!is_device_ptr(keys)) {
+        // staged in a sort buffer; not in the one that holds the classified keys,
+        // which the getters read still when the call fails further on
+        const bool second = h->sorted && h->sorted == h->alt0;
+        uint64_t **stage = second ? &h->alt1 : &h->alt0;
+        KM_TRY(ensure(h, stage, second ? &h->alt1_cap : &h->alt0_cap, words));
+        KM_CUDA(cudaMemcpyAsync(*stage, keys, words * 8, cudaMemcpyHostToDevice, h->stream));
+        d_keys = *stage;
     }
     KM_TRY(ensure_set_capacity(h, n, true));
     KM_CUDA(launch_reinsert(d_keys, n, nullptr, nullptr, h->kw, h->table, h->cap, set_tag(h),

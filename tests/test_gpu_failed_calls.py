@@ -56,3 +56,29 @@ def test_results_after_an_insert_whose_set_does_not_fit(K, allocator):
         kc.kmerco_rank_of(bf.h, probes, len(probes), ranks)
         assert np.array_equal(ranks, np.arange(0, bf.stats()["distinct"], 97, dtype=np.uint64))
         del filler
+
+
+@pytest.mark.parametrize("K", [20, 21, 40])   # the sort ends in either of its buffers
+def test_results_after_an_add_whose_set_does_not_fit(K):
+    # calls of a few windows go to the distinct set, so the list is sorted into a
+    # buffer of its own; the added keys are staged on the device before the set is
+    # found not to fit
+    parts = [readsim.random_reads(40, 150, 150, seed=7 + i) for i in range(2)]
+    kw = 1 if K <= 32 else 2
+    more = np.arange(60000 * kw, dtype=np.uint64)
+    with kc.CountBF(K, 1 << 18, 4, 3, 2) as bf:
+        for b, o in parts:
+            bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        held = bf.stats()["device_bytes"]
+    # the staging (a quarter more than the keys) and the list fit, the set does not
+    with kc.CountBF(K, 1 << 18, 4, 3, 2, hbm_budget=held + 1_300_000 * kw) as bf:
+        for b, o in parts:
+            bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        with pytest.raises(kc.KmercoError) as e:
+            kc.kmerco_add_distinct(bf.h, more, 60000)
+        assert e.value.status == kc.ENOMEM
+        (b1, o1), (b2, o2) = parts
+        check(_results(bf), np.concatenate([b1, b2]), np.concatenate([o1, o2[1:] + o1[-1]]),
+              K, 4, 3, 2)
