@@ -111,6 +111,7 @@ struct kmerco {
     uint64_t range_meta_cap;
     uint32_t *union_scratch;
     uint64_t union_scratch_cap;
+    bool scratch_busy;       // an insert is securing its buffers: its scratch stays
     uint32_t *coarse;        // partitioned update: increment codes per coarse region
     uint64_t coarse_alloc;
     uint32_t *fine;          // ... and per slice
@@ -200,20 +201,53 @@ void raw_free(const kmerco_t *h, void *p, uint64_t bytes) {
     cudaFree(p);
 }
 
-int dev_alloc(kmerco_t *h, void **p, uint64_t bytes) {
-    *p = nullptr;
-    if (bytes == 0) bytes = 16;
-    if (h->budget && h->used + bytes > h->budget) return KMERCO_ENOMEM;
-    KM_TRY(raw_alloc(h, p, bytes));
-    h->used += bytes;
-    return KMERCO_OK;
-}
-
 void dev_free(kmerco_t *h, void *p, uint64_t bytes) {
     if (!p) return;
     if (bytes == 0) bytes = 16;
     raw_free(h, p, bytes);
     h->used -= bytes;
+}
+
+// Gives back what the handle holds only to make its next insert quicker: the
+// scratch of an insert by key ranges, the list's other place, and the sure bytes
+// (keys are then classified by their counters).
+void release_scratch(kmerco_t *h) {
+    auto give_back = [h](auto **p, uint64_t *cap, uint64_t elem) {
+        dev_free(h, *p, *cap * elem);
+        *p = nullptr;
+        *cap = 0;
+    };
+    give_back(&h->range_a, &h->range_a_cap, 8);
+    give_back(&h->range_b, &h->range_b_cap, 8);
+    give_back(&h->mult, &h->mult_cap, 4);
+    give_back(&h->range_meta, &h->range_meta_cap, 1);
+    give_back(&h->coarse, &h->coarse_alloc, 4);
+    give_back(&h->fine, &h->fine_alloc, 4);
+    give_back(&h->part_ctr, &h->part_ctr_alloc, 8);
+    give_back(&h->dlist2, &h->dlist2_cap, (uint64_t)h->kw * 8);
+    give_back(&h->union_scratch, &h->union_scratch_cap, 4);
+    give_back(&h->sure, &h->sure_cap, 1);
+    h->sure_ok = false;
+}
+
+// Memory that a call cannot do without; where there is none left, the scratch of
+// earlier inserts makes room.
+int dev_alloc(kmerco_t *h, void **p, uint64_t bytes) {
+    *p = nullptr;
+    if (bytes == 0) bytes = 16;
+    const auto take = [&] {
+        if (h->budget && h->used + bytes > h->budget) return KMERCO_ENOMEM;
+        return raw_alloc(h, p, bytes);
+    };
+    int st = take();
+    if (st == KMERCO_ENOMEM && !h->scratch_busy) {
+        const uint64_t used = h->used;
+        release_scratch(h);
+        if (h->used < used) st = take();
+    }
+    KM_TRY(st);
+    h->used += bytes;
+    return KMERCO_OK;
 }
 
 // Make *p hold at least `need` elements of `elem` bytes (contents dropped).
@@ -836,33 +870,39 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
     return KMERCO_OK;
 }
 
-// The scratch of a plan from the handle's buffers; false when it cannot be
-// had (what was there is then given back).
-bool handle_scratch(kmerco_t *h, const InsertPlan &ip) {
+// The buffers of a plan from the handle's: the ranges' scratch, the list, the set
+// or the union's buffers, first reads.  `held` becomes the keys held before, at most.
+int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) {
     const DedupPlan &d = ip.dd;
     const PartPlan &pp = ip.pp;
-    if (ensure(h, &h->range_a, &h->range_a_cap, d.keys_a()) == KMERCO_OK &&
-        ensure(h, &h->range_b, &h->range_b_cap, d.keys_b()) == KMERCO_OK &&
-        ensure(h, &h->mult, &h->mult_cap, d.mult_words()) == KMERCO_OK &&
-        ensure(h, &h->range_meta, &h->range_meta_cap, d.meta_bytes()) == KMERCO_OK &&
-        (!pp.part ||
-         (ensure(h, &h->coarse, &h->coarse_alloc, pp.coarse_words()) == KMERCO_OK &&
-          (!pp.repart || ensure(h, &h->fine, &h->fine_alloc, pp.fine_words()) == KMERCO_OK) &&
-          ensure(h, &h->part_ctr, &h->part_ctr_alloc, pp.ctr_words()) == KMERCO_OK)))
-        return true;
-    auto give_back = [h](auto **p, uint64_t *cap) {
-        dev_free(h, *p, *cap * sizeof(**p));
-        *p = nullptr;
-        *cap = 0;
-    };
-    give_back(&h->range_a, &h->range_a_cap);
-    give_back(&h->range_b, &h->range_b_cap);
-    give_back(&h->mult, &h->mult_cap);
-    give_back(&h->range_meta, &h->range_meta_cap);
-    give_back(&h->coarse, &h->coarse_alloc);
-    give_back(&h->fine, &h->fine_alloc);
-    give_back(&h->part_ctr, &h->part_ctr_alloc);
-    return false;
+    if (ip.ranges) {
+        KM_TRY(ensure(h, &h->range_a, &h->range_a_cap, d.keys_a()));
+        KM_TRY(ensure(h, &h->range_b, &h->range_b_cap, d.keys_b()));
+        KM_TRY(ensure(h, &h->mult, &h->mult_cap, d.mult_words()));
+        KM_TRY(ensure(h, &h->range_meta, &h->range_meta_cap, d.meta_bytes()));
+        if (pp.part) {
+            KM_TRY(ensure(h, &h->coarse, &h->coarse_alloc, pp.coarse_words()));
+            if (pp.repart) KM_TRY(ensure(h, &h->fine, &h->fine_alloc, pp.fine_words()));
+            KM_TRY(ensure(h, &h->part_ctr, &h->part_ctr_alloc, pp.ctr_words()));
+        }
+    }
+    if (ip.merge) {
+        const int st = ensure_union(h, ip.bound);
+        if (st == KMERCO_ENOMEM)
+            ip.merge = false;   // the distinct set then
+        else
+            KM_TRY(st);
+    }
+    held = h->d_ub;
+    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
+    // a call merged once writes its list into the other buffer alone
+    if (!ip.merge || ip.passes > 1)
+        KM_TRY(ensure_set_capacity(h, ip.bound, ip.table()));
+    else
+        h->d_ub += ip.bound;
+    ip.sure = !ip.table() && ip.fresh && ip.passes == 1 &&
+              ensure(h, &h->sure, &h->sure_cap, ip.bound) == KMERCO_OK;
+    return KMERCO_OK;
 }
 
 }  // namespace
@@ -1201,27 +1241,19 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
     }
     if (bound == 0) return KMERCO_OK;   // no window fits in any read
     InsertPlan ip = plan_insert(h, bound, nbytes, h->d_ub == 0, true);
-    if (ip.ranges && !handle_scratch(h, ip)) {   // window by window when the buffers cannot be had
+    uint64_t held = 0;
+    h->scratch_busy = ip.ranges;
+    int st = secure_insert(h, ip, nbytes, held);
+    h->scratch_busy = false;
+    if (st == KMERCO_ENOMEM && ip.ranges) {
+        // window by window, which needs the list and the set alone (24 bytes a
+        // window and key word instead of 34 and more)
+        release_scratch(h);
         ip = InsertPlan();
         ip.bound = bound;
+        st = secure_insert(h, ip, nbytes, held);
     }
-    uint64_t held = 0;
-    if (ip.merge) {
-        const int st = ensure_union(h, bound);
-        if (st == KMERCO_ENOMEM)
-            ip.merge = false;   // the distinct set then
-        else
-            KM_TRY(st);
-        held = h->d_ub;
-    }
-    // a call merged once writes its list into the other buffer alone
-    if (!ip.merge || ip.passes > 1)
-        KM_TRY(ensure_set_capacity(h, bound, ip.table()));
-    else
-        h->d_ub += bound;
-    ip.sure = !ip.table() && ip.fresh && ip.passes == 1 &&
-              ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
-    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
+    KM_TRY(st);
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
     const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
                              h->part_ctr, h->dlist, h->dlist2, h->union_scratch, held};
@@ -1992,9 +2024,9 @@ int batch_run(kmerco_batch *b, bool reset) {
 // What a captured insert of a handle holds of it: its generation tag and buffers
 // (a later insert into the handle alone may move them).
 void handle_key(const kmerco_t *h, std::vector<uint64_t> &key) {
-    const uint64_t f[6] = {h->gen, (uint64_t)h->dlist, (uint64_t)h->table, (uint64_t)h->first_read,
-                           (uint64_t)h->sure, h->dlist_cap};
-    key.insert(key.end(), f, f + 6);
+    const uint64_t f[7] = {h->gen, (uint64_t)h->dlist, (uint64_t)h->table, (uint64_t)h->first_read,
+                           (uint64_t)h->sure, h->dlist_cap, h->sure_cap};
+    key.insert(key.end(), f, f + 7);
 }
 
 // State of the handles after a batch insert (a replayed graph inserted too).
@@ -2166,10 +2198,10 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
         b->plans[i] = plan_insert(h, bound, bo[2] - bo[1], h->d_ub == 0);
         // the set too: the persistent schedule inserts into it
         KM_TRY(ensure_set_capacity(h, bound, bound != 0));
-        b->plans[i].sure = !b->plans[i].table() && b->plans[i].fresh &&
-                           ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
         const uint64_t most = (bo[2] - bo[1] + kSmallChunk - 1) / kSmallChunk;   // chunks at the smallest chunk size
         KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, most ? most : 1));
+        b->plans[i].sure = !b->plans[i].table() && b->plans[i].fresh &&
+                           ensure(h, &h->sure, &h->sure_cap, bound) == KMERCO_OK;
         b->load[i] = bound;
     }
     KM_CUDA(cudaStreamSynchronize(b->stream));

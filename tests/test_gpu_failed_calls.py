@@ -82,3 +82,43 @@ def test_results_after_an_add_whose_set_does_not_fit(K):
         (b1, o1), (b2, o2) = parts
         check(_results(bf), np.concatenate([b1, b2]), np.concatenate([o1, o2[1:] + o1[-1]]),
               K, 4, 3, 2)
+
+
+@pytest.mark.parametrize("K", [21, 40])
+@pytest.mark.parametrize("share", [24.3, 27, 30, 33, 34.5, 36, 40, 60])
+def test_a_budget_that_holds_the_list_and_the_set_is_enough(K, share):
+    # 24 bytes a window and key word hold the list and the set; the scratch of an
+    # insert by key ranges is taken only where it leaves room for what has to be had,
+    # and goes when the classification needs the memory
+    reads = 60
+    b, o = readsim.random_reads(reads, 150, 150, seed=11)
+    b, o = np.tile(b, 30), np.arange(30 * reads + 1, dtype=np.uint64) * np.uint64(150)
+    kw = 1 if K <= 32 else 2
+    windows = 30 * reads * (150 - K + 1)
+    with kc.CountBF(K, 1 << 18, 4, 3, 2) as bf:
+        base = bf.stats()["device_bytes"]
+    distinct = reads * (150 - K + 1)
+    # classification: two sort buffers, the lists, bits, and the sorts' small scratch
+    budget = base + int(share * kw * windows) + 60 * kw * distinct + (1 << 16)
+    with kc.CountBF(K, 1 << 18, 4, 3, 2, hbm_budget=budget) as bf:
+        bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        check(_results(bf), b, o, K, 4, 3, 2)
+        assert bf.stats()["device_bytes"] <= budget
+
+
+def test_scratch_of_an_insert_makes_room_for_later_calls():
+    # an insert by key ranges that fits holds its scratch on; classification and the
+    # query's staging need more than what is left beside it
+    K = 31
+    b, o = readsim.random_reads(2000, 150, 150, seed=12)
+    with kc.CountBF(K, 1 << 18, 4, 3, 2) as bf:
+        bf.insert(_dev(b), _dev(o))
+        kc.kmerco_sync(bf.h)
+        budget = bf.stats()["device_bytes"] + 4096
+    with kc.CountBF(K, 1 << 18, 4, 3, 2, hbm_budget=budget) as bf:
+        bf.insert(_dev(b), _dev(o))
+        bf.classify()
+        check(_results(bf), b, o, K, 4, 3, 2)
+        q = np.arange(100000, dtype=np.uint64)
+        assert len(bf.query(q)) == len(q)
