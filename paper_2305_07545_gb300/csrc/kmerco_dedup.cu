@@ -803,12 +803,16 @@ struct RangeRuns {
             row0 = x.starts + (uint64_t)first * (x.n_fine + 1) + (uint64_t)f * n_runs;
             const uint64_t *fs = x.fine_spl + (uint64_t)b * kMaxRanges;
             p_lo = f ? fs[f - 1] : b ? x.spl[b - 1] : 0;
-            p_hi = f + 1 < x.n_fine ? fs[f] : b + 1 < x.n_ranges ? x.spl[b] : last;
+            // unused splitters are all ones: the last range in use ends where its
+            // coarse one does (taken for all the key space, its keys fall into one
+            // cut and the block sorts them by the whole bitonic network)
+            const uint64_t end = b + 1 < x.n_ranges ? x.spl[b] : last;
+            p_hi = f + 1 < x.n_fine ? min(fs[f], end) : end;
         } else {
             n_runs = x.n_chunks;
             row0 = x.starts + (uint64_t)g * n_runs;
             p_lo = g ? x.spl[g - 1] : 0;
-            p_hi = g + 1 < x.n_ranges ? x.spl[g] : last;
+            p_hi = g + 1 < x.n_ranges ? min(x.spl[g], last) : last;
         }
         load_run(x, threadIdx.x);
     }
