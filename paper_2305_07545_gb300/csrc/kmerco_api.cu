@@ -59,7 +59,8 @@ struct kmerco {
     DevCounters *ctr;        // device
     DevCounters *ctr_host;   // pinned, mapped mirror
     DevCounters *ctr_mirror; // the mirror's device address
-    uint64_t *table;         // distinct-key set: cap slots of kw words
+    uint64_t *table;         // distinct-key set: cap slots of kw words, and one for
+                             // the key that reads as a free slot
     uint64_t cap;
     uint32_t gen;            // generation tag of the set's current keys
     bool table_ok;           // the set holds exactly the list's keys (built when it is needed)
@@ -343,6 +344,8 @@ int device_error_status(unsigned err) {
     return KMERCO_OK;
 }
 
+uint64_t table_bytes(const kmerco_t *h, uint64_t cap) { return (cap + 1) * h->kw * 8; }
+
 // Makes every key of the distinct set read as a free slot: the next
 // generation tag, or a clear once the tags run out.
 int clean_table(kmerco_t *h) {
@@ -350,7 +353,7 @@ int clean_table(kmerco_t *h) {
     if (h->gen + 1 < tag_count(h)) {
         ++h->gen;
     } else {
-        KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, h->stream));
+        KM_CUDA(cudaMemsetAsync(h->table, 0xFF, table_bytes(h, h->cap), h->stream));
         h->gen = 0;
     }
     h->table_dirty = false;
@@ -395,14 +398,14 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
         if (want < h->cap + h->cap / 2) want = h->cap + h->cap / 2;
         if (want < 1024) want = 1024;
         void *q;
-        KM_TRY(dev_alloc(h, &q, want * h->kw * 8));
-        KM_CUDA(cudaMemsetAsync(q, 0xFF, want * h->kw * 8, h->stream));
+        KM_TRY(dev_alloc(h, &q, table_bytes(h, want)));
+        KM_CUDA(cudaMemsetAsync(q, 0xFF, table_bytes(h, want), h->stream));
         KM_CUDA(launch_reinsert(h->dlist, D < h->dlist_cap ? D : h->dlist_cap, nullptr, nullptr,
                                 h->kw, (uint64_t *)q, want, set_tag(h), nullptr, 0, h->ctr,
                                 h->G.probe_limit, h->stream));
         h->launches += D ? 1 : 0;
         KM_CUDA(cudaStreamSynchronize(h->stream));
-        dev_free(h, h->table, h->cap * h->kw * 8);
+        dev_free(h, h->table, table_bytes(h, h->cap));
         h->table = (uint64_t *)q;
         h->cap = want;
         h->table_ok = true;
@@ -970,7 +973,7 @@ int kmerco_estimate_bytes(const kmerco_config_t *cfg, uint64_t nreads, uint64_t 
         if (cfg->max_distinct && list > cfg->max_distinct) list = cfg->max_distinct;
         b += list * kw * 8 + grown(windows, 1);
         const InsertPlan ip = plan_insert(&t, windows, nbytes, true);
-        if (ip.table()) b += std::max<uint64_t>(2 * windows, 1024) * kw * 8;
+        if (ip.table()) b += table_bytes(&t, std::max<uint64_t>(2 * windows, 1024));
         if (ip.ranges) {
             b += grown(ip.dd.keys_a(), 8) + grown(ip.dd.keys_b(), 8) +
                  grown(ip.dd.mult_words(), 4) + grown(ip.dd.meta_bytes(), 1);
@@ -1107,7 +1110,7 @@ void kmerco_destroy(kmerco_t *h) {
         if (h->out_stream) cudaStreamSynchronize(h->out_stream);
         dev_free(h, h->G.cells, h->G.words * 8);
         dev_free(h, h->ctr, kCtrBytes);
-        dev_free(h, h->table, h->cap * h->kw * 8);
+        dev_free(h, h->table, table_bytes(h, h->cap));
         dev_free(h, h->dlist, h->dlist_cap * h->kw * 8);
         dev_free(h, h->dlist2, h->dlist2_cap * h->kw * 8);
         dev_free(h, h->union_scratch, h->union_scratch_cap * 4);
@@ -1910,7 +1913,7 @@ int batch_build_args(kmerco_batch *b, int chunk) {
 int batch_reset_device(kmerco_batch *b) {
     for (kmerco_t *h : b->h) {
         KM_CUDA(cudaMemsetAsync(h->G.cells, 0, h->G.words * 8, b->stream));
-        if (h->table) KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, b->stream));
+        if (h->table) KM_CUDA(cudaMemsetAsync(h->table, 0xFF, table_bytes(h, h->cap), b->stream));
         KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), b->stream));
     }
     return KMERCO_OK;
@@ -1997,7 +2000,7 @@ int batch_launch_sliced(kmerco_batch *b, int S, bool reset) {
         if (reset) {
             KM_CUDA(cudaMemsetAsync(h->G.cells, 0, h->G.words * 8, st));
             if (h->table && b->plans[i].table())
-                KM_CUDA(cudaMemsetAsync(h->table, 0xFF, h->cap * h->kw * 8, st));
+                KM_CUDA(cudaMemsetAsync(h->table, 0xFF, table_bytes(h, h->cap), st));
             KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), st));
         }
         const unsigned long long *bo = &b->bound_host[(size_t)i * kBoundOutWords];

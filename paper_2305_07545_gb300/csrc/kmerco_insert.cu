@@ -112,7 +112,8 @@ __device__ __forceinline__ void sat_increment(uint64_t *cells, uint64_t c, unsig
 // A slot stores the key with the set's generation tag in the unused top bits
 // of its top word (SetTag): a slot whose tag differs from the current one is
 // free, so a reset only moves to the next tag instead of clearing the table.
-// Without spare bits (mask 0) a free slot is all ones, cleared at reset.
+// Without spare bits (mask 0) a free slot is all ones, cleared at reset; the key
+// that is all ones itself has the place after the last slot.
 // For one-word keys `first` is an already loaded value of the home slot
 // (kEmptyKey - 1 when none was loaded, a value no slot holds); for two-word
 // keys *first2 is, when not null.
@@ -126,6 +127,8 @@ __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64
                                            uint32_t limit, unsigned *err, uint64_t pol,
                                            uint64_t first = kEmptyKey - 1,
                                            const ulonglong2 *first2 = nullptr) {
+    if (!t.mask && klo == kEmptyKey && (KW == 1 || khi == kEmptyKey))
+        return atomicExch((unsigned long long *)(table + cap * KW), 0ull) != 0ull;
     uint64_t slot = __umul64hi(th, cap);
     for (uint32_t it = 0;; ++it) {
         if (KW == 1) {

@@ -9,8 +9,7 @@
 namespace countbf {
 
 // ---------------------------------------------------------------- constants
-constexpr uint64_t kEmptyKey = ~0ull;      // empty slot of the distinct-key set;
-                                           // no canonical key is all ones
+constexpr uint64_t kEmptyKey = ~0ull;      // empty slot of the distinct-key set
 constexpr int kChunk = 2048;               // window starts per insert work unit
 constexpr int kSmallChunk = 512;           // the same for inputs too small to fill the GPU
 constexpr int kPartMaxHash = 4;            // hashes the partitioned update groups at a time
