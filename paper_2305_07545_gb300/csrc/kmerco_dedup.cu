@@ -32,8 +32,9 @@
 // through the same shared memory.  A range with more distinct keys than fit
 // is handled in several rounds over sub-ranges of it.
 //
-// Two-word keys are cut by their top 64 bits (the prefix); equal prefixes stay
-// in one range and are told apart in dedup_kernel.
+// Keys are cut by their prefix (their top 64 bits), two-word keys whose prefixes
+// are equal by their low word: reads with a common beginning of 32 bases and
+// more would else all meet in one range, which is one block's.
 #include "kmerco_dedup.cuh"
 #include "kmerco_stage.cuh"
 
@@ -113,30 +114,83 @@ __device__ __forceinline__ Key<2> canonical_key(const Key<2> &f, const Key<2> &r
     return hf < hr ? f : r;
 }
 
-// Index of a prefix among the n ranges of n - 1 sorted splitters: how many of
-// those are at or below it.
-// lut[i] = splitters whose (value - lo) >> sh is below i, with kMany set when
-// more than one falls into cell i: one comparison decides nearly every prefix
-// without a branch.  spl is followed by an all-ones value.
-constexpr unsigned kMany = 0x8000u;
+// A place to cut two-word keys at: the prefix, and the low word for keys with
+// that prefix.
+struct __align__(16) Cut2 {
+    uint64_t p, lo;
+    __device__ __forceinline__ bool operator<(const Cut2 &o) const {
+        return p < o.p || (p == o.p && lo < o.lo);
+    }
+};
 
-__device__ __forceinline__ unsigned find_range(const uint64_t *spl, const uint16_t *lut, unsigned n,
-                                               uint64_t lo, int sh, uint64_t x) {
-    const unsigned e = lut[(unsigned)((x - lo) >> sh)];
-    unsigned a = e & (kMany - 1);
+__device__ __forceinline__ uint64_t shfl_xor(uint64_t v, int m) {
+    return __shfl_xor_sync(0xffffffffu, v, m);
+}
+__device__ __forceinline__ Cut2 shfl_xor(const Cut2 &v, int m) {
+    return Cut2{shfl_xor(v.p, m), shfl_xor(v.lo, m)};
+}
+
+// What samples of keys are sorted by.
+template <int KW> struct SampleOf { using T = uint64_t; };
+template <> struct SampleOf<2> { using T = Cut2; };
+__device__ __forceinline__ uint64_t sample_of(const Key<1> &k, int) { return k.lo; }
+__device__ __forceinline__ Cut2 sample_of(const Key<2> &k, int K) {
+    return Cut2{prefix_of<2>(k, K), k.lo};
+}
+__device__ __forceinline__ void largest_sample(uint64_t &v) { v = ~0ull; }
+__device__ __forceinline__ void largest_sample(Cut2 &v) { v.p = v.lo = ~0ull; }
+
+// Index of a key among the n ranges of n - 1 sorted splitters: how many of those
+// are at or below it.  x is the key's prefix and low its low word; spl has the
+// splitters' prefixes, low_of(i) gives the low word of a two-word splitter: 0 where
+// no other splitter has the prefix.
+// lut[i] = splitters whose (prefix - lo) >> sh is below i, with kMany set when
+// more than one falls into cell i, so that one comparison of prefixes decides
+// nearly every key without a branch; in the other cells it bisects the cell's
+// splitters.  kTies is set where prefixes are equal among them, and only there low
+// words are compared (they stay in global memory; comparing them in every such cell made
+// refine_kernel 5% slower).  spl is followed by an all-ones value.
+constexpr unsigned kMany = 0x8000u, kTies = 0x4000u, kLutIndex = 0x3fffu;
+static_assert(kMaxRanges <= kLutIndex, "an index beside the flags");
+
+template <int KW, typename F>
+__device__ __forceinline__ unsigned find_range(const uint64_t *spl, F low_of, const uint16_t *lut,
+                                               unsigned n, uint64_t lo, int sh, uint64_t x,
+                                               uint64_t low) {
+    const unsigned c = (unsigned)((x - lo) >> sh), e = lut[c];
+    unsigned a = e & kLutIndex;
     a += spl[a] <= x ? 1u : 0u;
-    if (e & kMany)
-        while (spl[a] <= x && spl[a] != ~0ull) ++a;
+    if (e & kMany) {
+        a = e & kLutIndex;
+        unsigned b = c + 1 < kLutStride ? lut[c + 1] & kLutIndex : n - 1;
+        if (KW == 2 && (e & kTies)) {
+            while (a < b) {
+                const unsigned m = (a + b) / 2;
+                const uint64_t s = spl[m];
+                if (s < x || (s == x && low_of(m) <= low))
+                    a = m + 1;
+                else
+                    b = m;
+            }
+        } else {
+            while (a < b) {
+                const unsigned m = (a + b) / 2;
+                const bool at_or_below = spl[m] <= x;
+                a = at_or_below ? m + 1 : a;
+                b = at_or_below ? b : m;
+            }
+        }
+    }
     return min(a, n - 1);   // an all-ones prefix passes the end
 }
 
 // Ascending bitonic sort of 1024 * E values, E consecutive ones to a thread in
-// v (1,024 threads); xch: 1024 * E words of shared memory.  Strides inside a
-// thread are register swaps, inside a warp shuffles; only the 15 steps of
-// larger strides go through shared memory (105 of a plain network of 16,384
+// v (1,024 threads); xch: room for 1024 * E values in shared memory.  Strides
+// inside a thread are register swaps, inside a warp shuffles; only the 15 steps
+// of larger strides go through shared memory (105 of a plain network of 16,384
 // values).
-template <int E>
-__device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
+template <int E, typename V>
+__device__ __forceinline__ void block_sort(V (&v)[E], V *xch) {
     constexpr unsigned P = 1024 * E;
     const unsigned tid = threadIdx.x, i0 = tid * E;
     for (unsigned k = 2; k <= P; k <<= 1) {
@@ -150,14 +204,14 @@ __device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
                 const bool lower = (i0 & j) == 0, up = (i0 & k) == 0;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const uint64_t o = xch[e * 1024 + other];
+                    const V o = xch[e * 1024 + other];
                     v[e] = (lower == up) == (o < v[e]) ? o : v[e];
                 }
             } else if (j >= E) {   // in another lane
                 const bool lower = (i0 & j) == 0, up = (i0 & k) == 0;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const uint64_t o = __shfl_xor_sync(0xffffffffu, v[e], j / E);
+                    const V o = shfl_xor(v[e], (int)(j / E));
                     v[e] = (lower == up) == (o < v[e]) ? o : v[e];
                 }
             } else {   // in this thread
@@ -168,8 +222,8 @@ __device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
                     for (int e = 0; e < E; ++e) {
                         if (e & b) continue;
                         const bool up = ((i0 + e) & k) == 0;
-                        const uint64_t x = v[e], y = v[e | b];
-                        const bool swap = (x > y) == up;
+                        const V x = v[e], y = v[e | b];
+                        const bool swap = (y < x) == up;
                         v[e] = swap ? y : x;
                         v[e | b] = swap ? x : y;
                     }
@@ -180,9 +234,12 @@ __device__ __forceinline__ void block_sort(uint64_t (&v)[E], uint64_t *xch) {
 }
 
 // The lookup table of n - 1 splitters of the range [lo, last], v the thread's
-// (1,024 threads, n <= kMaxRanges); cells: 32 KiB of shared memory.
-__device__ __forceinline__ void write_lut(unsigned *cells, uint64_t v, bool any, unsigned n,
-                                          uint64_t lo, uint64_t last, uint16_t *lut) {
+// prefix (1,024 threads, n <= kMaxRanges), tie: whether another one has it and their
+// low words decide; cells: 32 KiB of shared memory.  In two-word keys' last cell a
+// key may have the prefix of the unused splitters, all ones: whole keys there too.
+template <int KW>
+__device__ __forceinline__ void write_lut(unsigned *cells, uint64_t v, bool tie, bool any,
+                                          unsigned n, uint64_t lo, uint64_t last, uint16_t *lut) {
     static_assert(kMaxRanges <= 1024, "a splitter a thread");
     constexpr unsigned E = (1u << kLutBits) / 1024;
     const unsigned j = threadIdx.x;
@@ -192,19 +249,33 @@ __device__ __forceinline__ void write_lut(unsigned *cells, uint64_t v, bool any,
     __syncthreads();
     if (j + 1 < n && any) {   // splitters in every cell of the table
         const uint64_t c = (v - lo) >> sh;
-        if (c < (1u << kLutBits)) atomicAdd(cells + c, 1u);
+        if (c < (1u << kLutBits)) atomicAdd(cells + c, tie ? 0x10001u : 1u);
     }
     __syncthreads();
     unsigned c[E], sum = 0;
 #pragma unroll
-    for (unsigned q = 0; q < E; ++q) sum += c[q] = cells[j * E + q];
+    for (unsigned q = 0; q < E; ++q) sum += (c[q] = cells[j * E + q]) & 0xffffu;
     unsigned tot;
     unsigned pre = block_exclusive_scan<unsigned, 1024>(sum, tot);
 #pragma unroll
     for (unsigned q = 0; q < E; ++q) {
-        lut[j * E + q] = (uint16_t)(pre | (c[q] > 1 ? kMany : 0u));
-        pre += c[q];
+        unsigned flags = (c[q] & 0xffffu) > 1 ? kMany : 0u;
+        if (KW == 2 && (c[q] > 0xffffu || j * E + q == (unsigned)((last - lo) >> sh)))
+            flags = kMany | kTies;
+        lut[j * E + q] = (uint16_t)(pre | flags);
+        pre += c[q] & 0xffffu;
     }
+}
+
+// Whether a neighbour among the n splitters has the prefix p of thread j's one too
+// (seen: shared memory for the prefixes).
+__device__ __forceinline__ bool shares_prefix(uint64_t *seen, unsigned j, unsigned n, uint64_t p) {
+    __syncthreads();
+    if (j < n) seen[j] = p;
+    __syncthreads();
+    const bool shared = j < n && ((j && seen[j - 1] == p) || (j + 1 < n && seen[j + 1] == p));
+    __syncthreads();
+    return shared;
 }
 
 __device__ __forceinline__ uint64_t mix64(uint64_t x) { return fmix64(x + 0x9E3779B97F4A7C15ull); }
@@ -303,18 +374,20 @@ __device__ __forceinline__ Key<2> revcomp(const Key<2> &f, int K) {
 // ----------------------------------------------------------- 2. splitters
 constexpr unsigned kSampleTile = 1024;   // samples a block sorts
 
-// Prefixes of the keys at n random valid window starts of the pass's `span` bases (a
-// few tries each), as sorted tiles of kSampleTile; the last one is filled up with
+// The keys at n random valid window starts of the pass's `span` bases (a few tries
+// each), as sorted tiles of kSampleTile: samples has their prefixes, samples_lo the
+// low words of two-word keys (0 in tiles of different prefixes); the last one is filled up with
 // all ones.  Whole prefixes: copies of a repeat have long beginnings in common,
 // and cutting by their top 31 bits left more than twice as many windows in some
 // ranges (dedup_big_kernel 2.8 instead of 1.8 ms for 3.8e8 two-word windows).
 template <int KW>
 __global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int canonical,
                                                       uint64_t span, unsigned n,
-                                                      uint64_t *samples, DedupMeta *meta) {
-    __shared__ uint64_t xch[kSampleTile];
+                                                      uint64_t *samples, uint64_t *samples_lo,
+                                                      DedupMeta *meta) {
+    __shared__ typename SampleOf<KW>::T xch[kSampleTile];
     const unsigned i = blockIdx.x * kSampleTile + threadIdx.x;
-    uint64_t v[1] = {~0ull};
+    Key<KW> key;
     bool found = false;
     for (unsigned t = 0; t < 4 && i < n && !found; ++t) {
         // window starts spread evenly over the pass, jittered; then anywhere
@@ -324,25 +397,44 @@ __global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int can
         if (!((x.valid[at >> 4] >> (at & 15)) & 1u)) continue;
         Key<KW> f;
         window_at((const uint64_t *)x.codes, at, K, f);
-        v[0] = prefix_of<KW>(canonical_key(f, revcomp(f, K), canonical), K);
+        key = canonical_key(f, revcomp(f, K), canonical);
         found = true;
     }
     const int c = __syncthreads_count(found);
     if (threadIdx.x == 0 && c) atomicAdd(&meta->sampled, (unsigned)c);
-    block_sort<1>(v, xch);
+    const uint64_t p = found ? prefix_of<KW>(key, K) : ~0ull;
+    uint64_t v[1] = {p}, low = 0;
+    block_sort<1>(v, (uint64_t *)xch);
+    if constexpr (KW == 2) {
+        // equal prefixes in the tile, which are rare: in the order of the whole keys
+        uint64_t *const seen = (uint64_t *)xch;
+        __syncthreads();
+        seen[threadIdx.x] = v[0];
+        __syncthreads();
+        const bool same = threadIdx.x && v[0] != ~0ull && seen[threadIdx.x - 1] == v[0];
+        if (__syncthreads_or(same)) {
+            Cut2 w[1] = {Cut2{p, found ? key.lo : ~0ull}};
+            block_sort<1>(w, xch);
+            v[0] = w[0].p;
+            low = w[0].lo;
+        }
+        samples_lo[i] = low;
+    }
     samples[i] = v[0];
 }
 
 // The samples of even ranks among the n of all tiles become the n_ranges - 1
 // splitters.  Block b ranks tile b: a sample's place in it, and by bisection its
-// places in the other tiles (all of them in shared memory; of equal samples the
+// places in the other tiles (their prefixes in shared memory; of equal samples the
 // ones of earlier tiles come first).  The last block to finish builds the lookup
 // table.  One block that sorted all samples took 20 us for 4,096 of them and 80 for
 // 16,384, a fifth to a third of a piece of 5e5 windows.
-__global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples, unsigned n,
+template <int KW>
+__global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
+                                                    const uint64_t *samples_lo, unsigned n,
                                                     unsigned n_ranges, uint64_t last,
                                                     DedupMeta *meta, uint64_t *spl,
-                                                    uint16_t *lut) {
+                                                    uint64_t *spl_lo, uint16_t *lut) {
     extern __shared__ ulonglong2 s2[];
     __shared__ bool is_last;
     uint64_t *const s = (uint64_t *)s2;
@@ -350,22 +442,38 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples, uns
     for (unsigned i = tid; i < n / 2; i += 1024) s2[i] = ((const ulonglong2 *)samples)[i];
     __syncthreads();
     const uint64_t v = s[own * kSampleTile + tid];
+    const uint64_t low = KW == 2 ? samples_lo[own * kSampleTile + tid] : 0;
     unsigned rank = tid;
     for (unsigned c = 0; c < n / kSampleTile; ++c) {
         if (c == own) continue;
-        const uint64_t *const t = s + c * kSampleTile;
-        unsigned at = 0;   // samples of the tile in front of v
+        const unsigned t0 = c * kSampleTile;
+        unsigned at = 0;   // samples of the tile below v's prefix
 #pragma unroll
         for (unsigned step = kSampleTile / 2; step; step >>= 1)
-            if (t[at + step - 1] < v || (c < own && t[at + step - 1] == v)) at += step;
-        rank += at + (t[at] < v || (c < own && t[at] == v) ? 1 : 0);
+            if (s[t0 + at + step - 1] < v) at += step;
+        if (s[t0 + at] < v) ++at;
+        if (at < kSampleTile && s[t0 + at] == v) {   // and those of the same prefix in front
+            unsigned hi = kSampleTile;
+            while (at < hi) {
+                const unsigned m = (at + hi) / 2;
+                const uint64_t w = KW == 2 && s[t0 + m] == v ? samples_lo[t0 + m] : low;
+                if (s[t0 + m] == v && (w < low || (w == low && c < own)))
+                    at = m + 1;
+                else
+                    hi = m;
+            }
+        }
+        rank += at;
     }
     const unsigned valid = meta->sampled;
     if (rank < valid) {   // splitter k - 1 is the sample of rank k * valid / n_ranges
         const uint64_t r = rank;
         for (uint64_t k = (r * n_ranges + valid - 1) / valid;
              k < n_ranges && k * valid / n_ranges == r; ++k)
-            if (k) spl[k - 1] = v;
+            if (k) {
+                spl[k - 1] = v;
+                if (KW == 2) spl_lo[k - 1] = low;
+            }
     }
     __threadfence();
     __syncthreads();
@@ -376,9 +484,16 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples, uns
     uint64_t f = ~0ull;   // the last of the n: what find_range stops at
     if (valid && tid + 1 < n_ranges)
         f = __ldcg(spl + tid);
-    else if (tid < n_ranges)
+    else if (tid < n_ranges) {
         spl[tid] = f;
-    write_lut((unsigned *)s, f, valid != 0, n_ranges, 0, last, lut);
+        if (KW == 2) spl_lo[tid] = f;
+    }
+    bool tie = false;
+    if (KW == 2 && valid) {
+        tie = shares_prefix(s, tid, n_ranges - 1, f);
+        if (!tie && tid < n_ranges) spl_lo[tid] = tid + 1 < n_ranges ? 0 : ~0ull;
+    }
+    write_lut<KW>((unsigned *)s, f, tie, valid != 0, n_ranges, 0, last, lut);
 }
 
 // ------------------------------------------------- grouping keys by range
@@ -486,7 +601,9 @@ __global__ void __launch_bounds__(CHUNK / 8, CHUNK >= 4096 ? 2 : 6)
             key[i] = canonical_key(f, r, CANON);
             br[i] = kNoKey;
             if ((valid >> i) & 1u) {
-                const unsigned bin = find_range(S.spl, S.lut, nr, 0, sh, prefix_of<KW>(key[i], K));
+                const unsigned bin = find_range<KW>(
+                    S.spl, [&](unsigned m) { return __ldg(x.spl_lo + m); }, S.lut, nr, 0, sh,
+                    prefix_of<KW>(key[i], K), key[i].lo);
                 br[i] = (bin << 16) | atomicAdd(&S.hist[bin], 1u);
             }
             const uint64_t c = next >> 62;
@@ -631,50 +748,100 @@ __global__ void __launch_bounds__(1024) tile_map_kernel(const uint32_t *totals, 
 }
 
 // Splitters of the fine ranges inside range b: keys of random places of
-// random pieces' runs.  One block per range.
+// random pieces' runs.  One block per range.  Prefixes alone, unless kCrowd
+// neighbouring splitters are equal: then half as many samples of whole keys, in the
+// same shared memory.  (A prefix of fewer ranges' windows is left together, to
+// dedup_big_kernel's few rounds: 2.8e8 windows of copied repeats have many of them,
+// and sorting whole keys at two equal ones took 910 instead of 500 us there.)
+constexpr unsigned kCrowd = 5;
 template <int KW, int E>
 __global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int K, unsigned n,
                                                               uint64_t last) {
-    extern __shared__ uint64_t s[];
+    extern __shared__ ulonglong2 s2[];
     __shared__ unsigned valid;
-    const unsigned b = blockIdx.x;
-    if (threadIdx.x == 0) valid = 0;
+    uint64_t *const s = (uint64_t *)s2;
+    const unsigned b = blockIdx.x, j = threadIdx.x;
+    if (j == 0) valid = 0;
     __syncthreads();
     const uint64_t lo = b ? x.spl[b - 1] : 0;
     const uint64_t hi = b + 1 < x.n_ranges ? x.spl[b] : last;
-    uint64_t v[E];
-    unsigned found = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const unsigned i = e * 1024 + threadIdx.x;
-        v[e] = ~0ull;
-        for (unsigned t = 0; i < n && t < 4; ++t) {
+    const auto draw = [&](unsigned i, Key<KW> &k) {
+        for (unsigned t = 0; t < 4; ++t) {
             const uint64_t z = mix64(((uint64_t)b << 32) | (i * 4 + t));
             const unsigned c = (unsigned)__umul64hi(z, (uint64_t)x.n_chunks);
             const unsigned s0 = x.starts[(uint64_t)b * x.n_chunks + c];
             const unsigned m = x.starts[(uint64_t)(b + 1) * x.n_chunks + c] - s0;
             if (!m) continue;
             const unsigned o = (unsigned)(((z & 0xffffffffu) * m) >> 32);
-            v[e] = prefix_of<KW>(load_key<KW>(x.in, (uint64_t)x.piece[c] + s0 + o), K);
-            ++found;
-            break;
+            k = load_key<KW>(x.in, (uint64_t)x.piece[c] + s0 + o);
+            return 1u;
         }
-    }
-    if (found) atomicAdd(&valid, found);
-    block_sort<E>(v, s);
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e) s[threadIdx.x * E + e] = v[e];
-    __syncthreads();
+        return 0u;
+    };
     // as many ranges as this one's windows fill, so that only the fine samples
     // spread the sizes; the others stay empty (all-ones splitters)
     const unsigned nf = max(1u, min(x.n_fine, (x.totals[b] + x.target - 1) / x.target));
-    const unsigned j = threadIdx.x;
-    uint64_t f = ~0ull;
-    if (valid && j + 1 < nf) f = s[(uint64_t)(j + 1) * valid / nf];
+    uint64_t f = ~0ull, f_lo = ~0ull;
+    {
+        uint64_t v[E];
+        unsigned found = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            Key<KW> k;
+            v[e] = ~0ull;
+            if (e * 1024 + j < n && draw(e * 1024 + j, k)) {
+                v[e] = prefix_of<KW>(k, K);
+                ++found;
+            }
+        }
+        if (found) atomicAdd(&valid, found);
+        block_sort<E>(v, s);
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) s[j * E + e] = v[e];
+    }
+    __syncthreads();
+    bool same = false, tie = false;
+    if (valid && j + 1 < nf) {
+        f = s[(uint64_t)(j + 1) * valid / nf];
+        f_lo = 0;
+        same = KW == 2 && j + kCrowd < nf && f == s[(uint64_t)(j + kCrowd) * valid / nf];
+    }
+    if constexpr (KW == 2) {
+        constexpr int E2 = (E < 4 ? 4 : E) / 2;
+        if (__syncthreads_or(same)) {
+            if (j == 0) valid = 0;
+            __syncthreads();
+            Cut2 v[E2], *const c = (Cut2 *)s2;
+            unsigned found = 0;
+#pragma unroll
+            for (int e = 0; e < E2; ++e) {
+                Key<KW> k;
+                largest_sample(v[e]);
+                if (e * 1024 + j < n && draw(e * 1024 + j, k)) {
+                    v[e] = sample_of(k, K);
+                    ++found;
+                }
+            }
+            if (found) atomicAdd(&valid, found);
+            block_sort<E2>(v, c);
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < E2; ++e) c[j * E2 + e] = v[e];
+            __syncthreads();
+            if (valid && j + 1 < nf) {
+                const Cut2 at = c[(uint64_t)(j + 1) * valid / nf];
+                f = at.p;
+                f_lo = at.lo;
+            }
+            tie = shares_prefix(s, j, valid ? nf - 1 : 0, f);
+            if (!tie && valid && j + 1 < nf) f_lo = 0;
+        }
+        if (j < x.n_fine) x.fine_lo[(uint64_t)b * kMaxRanges + j] = f_lo;
+    }
     if (j < x.n_fine) x.fine_spl[(uint64_t)b * kMaxRanges + j] = f;
     __syncthreads();
-    write_lut((unsigned *)s, f, valid != 0, nf, lo, hi, x.fine_lut + (uint64_t)b * kLutStride);
+    write_lut<KW>((unsigned *)s, f, tie, valid != 0, nf, lo, hi, x.fine_lut + (uint64_t)b * kLutStride);
 }
 
 // One tile of a range: gather its keys from the pieces, group them by fine
@@ -756,7 +923,9 @@ __global__ void __launch_bounds__(kRefineThreads, 2) refine_kernel(RefineArgs x,
             br[q] = kNoKey;
             if (i < n) {
                 key[q] = load_key<KW>(S.g.keys, i);
-                const unsigned bin = find_range(S.g.spl, S.g.lut, nf, lo, sh, prefix_of<KW>(key[q], K));
+                const unsigned bin = find_range<KW>(
+                    S.g.spl, [&](unsigned m) { return __ldg(x.fine_lo + (uint64_t)b * kMaxRanges + m); },
+                    S.g.lut, nf, lo, sh, prefix_of<KW>(key[q], K), key[q].lo);
                 br[q] = (bin << 16) | atomicAdd(&S.g.hist[bin], 1u);
             }
         }
@@ -778,12 +947,11 @@ __global__ void __launch_bounds__(kRefineThreads, 2) refine_kernel(RefineArgs x,
 
 // -------------------------------------------------------------- 4. dedup
 // A final range as its block reads it: its runs, one in every piece (one level)
-// or in every tile of its coarse range (two levels), the prefixes it spans, and
-// this thread's run of the first NT.
+// or in every tile of its coarse range (two levels), and this thread's run of the
+// first NT.
 struct RangeRuns {
     const uint16_t *row0;
     unsigned n_runs, first;
-    uint64_t p_lo, p_hi;
     unsigned src, n;
 
     __device__ __forceinline__ void load_run(const DedupArgs &x, unsigned r) {
@@ -794,29 +962,74 @@ struct RangeRuns {
             src = (x.n_fine ? (first + r) * (unsigned)kRefineTile : x.piece[r]) + s0;
         }
     }
-    __device__ __forceinline__ void load(const DedupArgs &x, unsigned g, uint64_t last) {
+    __device__ __forceinline__ void load(const DedupArgs &x, unsigned g) {
         first = 0;
         if (x.n_fine) {
             const unsigned b = g / x.n_fine, f = g % x.n_fine;
             first = x.tile_base[b];
             n_runs = x.tile_base[b + 1] - first;
             row0 = x.starts + (uint64_t)first * (x.n_fine + 1) + (uint64_t)f * n_runs;
-            const uint64_t *fs = x.fine_spl + (uint64_t)b * kMaxRanges;
-            p_lo = f ? fs[f - 1] : b ? x.spl[b - 1] : 0;
-            // unused splitters are all ones: the last range in use ends where its
-            // coarse one does (taken for all the key space, its keys fall into one
-            // cut and the block sorts them by the whole bitonic network)
-            const uint64_t end = b + 1 < x.n_ranges ? x.spl[b] : last;
-            p_hi = f + 1 < x.n_fine ? min(fs[f], end) : end;
         } else {
             n_runs = x.n_chunks;
             row0 = x.starts + (uint64_t)g * n_runs;
-            p_lo = g ? x.spl[g - 1] : 0;
-            p_hi = g + 1 < x.n_ranges ? min(x.spl[g], last) : last;
         }
         load_run(x, threadIdx.x);
     }
 };
+
+// How a range's keys are cut evenly into kSubBins2: by their prefixes, or by their
+// low words where all of them have one prefix.  One thread finds it out and leaves it
+// in shared memory while the block gathers the range (every thread waiting for the
+// bounds took 4% of dedup_kernel).
+struct RangeCut {
+    uint64_t base;     // the smallest prefix (or low word) there can be
+    int sh;            // kSubBits2 bits of the difference to it make a cut
+    unsigned by_low;
+};
+
+template <int KW>
+__device__ __forceinline__ RangeCut range_cut(const DedupArgs &x, unsigned g, uint64_t last) {
+    // the range's bounds: prefixes, and of two-word keys the low words
+    uint64_t lo = 0, hi = last, lo2 = 0, hi2 = ~0ull;
+    const auto below = [&](const uint64_t *p, const uint64_t *rest, uint64_t i) {
+        lo = p[i];
+        if (KW == 2) lo2 = rest[i];
+    };
+    const auto above = [&](const uint64_t *p, const uint64_t *rest, uint64_t i) {
+        const uint64_t v = p[i], w = KW == 2 ? rest[i] : 0;
+        // unused splitters are all ones: the last range in use ends where its coarse one
+        // does (taken for all the key space, its keys fall into one cut and the block
+        // sorts them by the whole bitonic network)
+        if (v < hi || (KW == 2 && v == hi && w < hi2)) {
+            hi = v;
+            hi2 = w;
+        }
+    };
+    if (x.n_fine) {
+        const unsigned b = g / x.n_fine, f = g % x.n_fine;
+        const uint64_t fs = (uint64_t)b * kMaxRanges + f;
+        if (f)
+            below(x.fine_spl, x.fine_lo, fs - 1);
+        else if (b)
+            below(x.spl, x.spl_lo, b - 1);
+        if (b + 1 < x.n_ranges) above(x.spl, x.spl_lo, b);
+        if (f + 1 < x.n_fine) above(x.fine_spl, x.fine_lo, fs);
+    } else {
+        if (g) below(x.spl, x.spl_lo, g - 1);
+        if (g + 1 < x.n_ranges) above(x.spl, x.spl_lo, g);
+    }
+    RangeCut c;
+    c.by_low = KW == 2 && lo == hi ? 1 : 0;
+    c.base = c.by_low ? lo2 : lo;
+    c.sh = max(bit_len(c.by_low ? hi2 - lo2 : hi - lo) - kSubBits2, 0);
+    return c;
+}
+
+template <int KW>
+__device__ __forceinline__ unsigned cut_of(const RangeCut &c, const Key<KW> &k, int K) {
+    const uint64_t v = KW == 2 && c.by_low ? k.lo : prefix_of<KW>(k, K);
+    return (unsigned)((v - c.base) >> c.sh);
+}
 
 template <int KW>
 __device__ __forceinline__ unsigned key_hash(const Key<KW> &k) {
@@ -907,6 +1120,7 @@ struct __align__(16) SmallSmem {
     unsigned src[kSmallThreads];
     unsigned pos[kSmallThreads + 1];
     unsigned lists, crowded, out0;   // lists: entries of left above, of list below
+    RangeCut cut;
 };
 
 constexpr unsigned kNoPlace = 0xffffu;
@@ -920,12 +1134,9 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
     const unsigned tid = threadIdx.x;
     const uint64_t last = K >= 32 ? ~0ull : (1ull << (2 * K)) - 1;
     RangeRuns next;
-    if (blockIdx.x < x.n_total) next.load(x, blockIdx.x, last);
+    if (blockIdx.x < x.n_total) next.load(x, blockIdx.x);
     for (unsigned g = blockIdx.x; g < x.n_total; g += gridDim.x) {
         const RangeRuns cur = next;
-        const uint64_t p_lo = cur.p_lo;
-        int sh = bit_len(cur.p_hi - p_lo) - kSubBits2;
-        if (sh < 0) sh = 0;
         // all windows of the range
         unsigned n = cur.n;
         for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
@@ -938,7 +1149,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
                 else
                     x.counts[g] = 0;
             }
-            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x);
             continue;
         }
         for (unsigned r0 = 0, m0 = 0; r0 < cur.n_runs; r0 += NT) {
@@ -962,7 +1173,10 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
             const uint4 none = make_uint4(~0u, ~0u, ~0u, ~0u);
             for (unsigned i = tid; i < kTableSlots / 8; i += NT) ((uint4 *)S.table)[i] = none;
             for (unsigned i = tid; i < (unsigned)kSubBins2; i += NT) S.sub[i] = 0;
-            if (tid == 0) S.lists = S.crowded = 0;
+            if (tid == 0) {
+                S.lists = S.crowded = 0;
+                if (x.ordered) S.cut = range_cut<KW>(x, g, last);
+            }
         }
         copies_done();
         __syncthreads();
@@ -1016,7 +1230,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
         const unsigned n_left = S.lists >> 16;
         if (n_left > kMaxLeft) {   // a crowded table: the other kernel's
             if (tid == 0) x.big[atomicAdd(&x.meta->n_big, 1u)] = g;
-            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+            if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x);
             __syncthreads();
             continue;
         }
@@ -1052,7 +1266,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
             }
             any = __syncthreads_or(mine);
         }
-        if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x, last);
+        if (g + gridDim.x < x.n_total) next.load(x, g + gridDim.x);
         const unsigned nd = S.lists & 0xffffu;
         if (!x.ordered) {
             if (tid == 0) S.out0 = atomicAdd(&x.meta->out_cursor, nd);
@@ -1066,8 +1280,9 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
             continue;
         }
         // their order
+        const RangeCut cut = S.cut;
         for (unsigned p = tid; p < nd; p += NT)
-            atomicAdd(&S.sub[(prefix_of<KW>(load_key<KW>(S.stage, S.list[p]), K) - p_lo) >> sh], 1u);
+            atomicAdd(&S.sub[cut_of(cut, load_key<KW>(S.stage, S.list[p]), K)], 1u);
         if (tid == 0) {
             S.out0 = atomicAdd(&x.meta->out_cursor, nd);
             x.places[g] = S.out0;
@@ -1081,7 +1296,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
         uint16_t *ord = S.table;   // the table is done with
         for (unsigned p = tid; p < nd; p += NT) {
             const unsigned i = S.list[p];
-            const unsigned c = (unsigned)((prefix_of<KW>(load_key<KW>(S.stage, i), K) - p_lo) >> sh);
+            const unsigned c = cut_of(cut, load_key<KW>(S.stage, i), K);
             ord[atomicAdd(&S.sub[c], 1u)] = (uint16_t)i;
         }
         __syncthreads();
@@ -1094,7 +1309,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
             const Key<KW> k = load_key<KW>(S.stage, i);
             unsigned rk = p;
             if (!crowded) {   // a cut's keys end at its cursor and begin at the one before
-                const unsigned c = (unsigned)((prefix_of<KW>(k, K) - p_lo) >> sh);
+                const unsigned c = cut_of(cut, k, K);
                 const unsigned a0 = c ? S.sub[c - 1] : 0u, a1 = S.sub[c];
                 if (a1 - a0 > 1) {
                     rk = a0;
@@ -1113,9 +1328,11 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
 // an open-addressing table, which counts them; whoever puts a key there first
 // appends its slot to a list, and everything after works on the list.  A range
 // with more distinct keys than the table takes is handled in rounds over
-// sub-ranges [lo, hi) of it: a round that overflows ends below the median of up
-// to 32 of the keys in the table instead (so it leaves some of them out, and the
-// rounds end).
+// sub-ranges [lo, hi) of it: a round that overflows stops, and begins again up to
+// the median of up to 32 of the keys in the table (so it leaves some of them out,
+// and the rounds end); a round that succeeds goes on to the bound before.  D keys
+// take about 4 D / slots rounds, half of them broken off.
+constexpr unsigned kBoundsMax = 16;
 template <int KW>
 struct __align__(16) DedupSmem {
     static constexpr int SLOTS = kDedupSlots<KW>;
@@ -1129,6 +1346,7 @@ struct __align__(16) DedupSmem {
     unsigned pos[kDedupThreads + 1]; // and place among the range's windows
     unsigned nd, over, crowded, ones, out0, cut;
     Key<KW> pivot;
+    Key<KW> bounds[kBoundsMax];      // the rounds' ends to come, the nearest last
 };
 static_assert(kDedupSlots<1> * 2 <= kDedupStage<1> * 8 && kDedupSlots<2> * 2 <= kDedupStage<2> * 16,
               "the slots in key order take the batch's place");
@@ -1195,21 +1413,27 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
     for (unsigned q = blockIdx.x; q < n_big; q += gridDim.x) {
         const unsigned g = x.big[q];
         RangeRuns cur;
-        cur.load(x, g, last);
-        const uint64_t p_lo = cur.p_lo;
-        int sh = bit_len(cur.p_hi - p_lo) - kSubBits2;
-        if (sh < 0) sh = 0;
-        unsigned done = 0;   // distinct keys written
+        cur.load(x, g);
+        const RangeCut cut = range_cut<KW>(x, g, last);
+        if (x.ordered) {   // the range's place in the output: room for all its windows
+            unsigned n = cur.n;
+            for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
+                n += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
+            block_exclusive_scan<unsigned, NT>(n, n);
+            if (tid == 0) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n);
+        }
+        unsigned done = 0;    // distinct keys written
+        unsigned depth = 0;   // bounds held
         Key<KW> lo, hi;
         lo.lo = lo.hi = 0;
         hi = lo;
         bool from = false, until = false;   // whether lo and hi bound this round
-        for (bool again = true, begun = false; again;) {
+        for (bool again = true; again;) {
             __syncthreads();   // the last round's table is cleared
             if (tid == 0) S.nd = S.over = S.crowded = S.ones = 0;
             for (unsigned i = tid; i < (unsigned)kSubBins2; i += NT) S.sub[i] = 0;
-            unsigned n_all = 0;
-            for (unsigned r0 = 0; r0 < cur.n_runs; r0 += NT) {
+            bool over = false;   // the same in every thread
+            for (unsigned r0 = 0; r0 < cur.n_runs && !over; r0 += NT) {
                 RangeRuns seg = cur;
                 if (r0) seg.load_run(x, r0 + tid);
                 unsigned m;
@@ -1217,10 +1441,9 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                 S.src[tid] = seg.src;
                 S.pos[tid] = pre;
                 if (tid == 0) S.pos[NT] = m;
-                n_all += m;
                 __syncthreads();
                 const unsigned nr = min((unsigned)NT, cur.n_runs - r0);
-                for (unsigned p0 = 0; p0 < m; p0 += kDedupStage<KW>) {
+                for (unsigned p0 = 0; p0 < m && !over; p0 += kDedupStage<KW>) {
                     const unsigned p1 = min(m, p0 + (unsigned)kDedupStage<KW>);
                     gather_runs<KW, NT>(x.in, S.src, S.pos, nr, p0, p1, S.stage,
                                         KW == 2 ? S.ref : nullptr);
@@ -1232,14 +1455,11 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                         table_add(S, k, x.in, KW == 2 ? S.ref[i] : 0u);
                     }
                     __syncthreads();
+                    over = S.over != 0;   // written between the barriers around the additions
                 }
             }
-            if (!begun) {   // the range's place in the output
-                begun = true;
-                if (tid == 0 && x.ordered) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n_all);
-            }
             const unsigned nd = S.nd;
-            if (!S.over && !x.ordered) {
+            if (!over && !x.ordered) {
                 const bool ones = KW == 1 && S.ones && !until;
                 if (tid == 0) S.out0 = atomicAdd(&x.meta->out_cursor, nd + (ones ? 1u : 0u));
                 __syncthreads();
@@ -1253,13 +1473,10 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                     x.mult[S.out0 + nd] = S.ones;
                 }
                 again = until;
-                lo = hi;
-                from = from || until;
-                until = false;
-            } else if (!S.over) {
+            } else if (!over) {
                 for (unsigned i = tid; i < nd; i += NT) {
                     const Key<KW> k = table_key(S, x.in, S.list[i]);
-                    atomicAdd(&S.sub[(prefix_of<KW>(k, K) - p_lo) >> sh], 1u);
+                    atomicAdd(&S.sub[cut_of(cut, k, K)], 1u);
                 }
                 __syncthreads();
                 unsigned most;
@@ -1269,7 +1486,7 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                 for (unsigned i = tid; i < nd; i += NT) {
                     const unsigned slot = S.list[i];
                     const Key<KW> k = table_key(S, x.in, slot);
-                    ord[atomicAdd(&S.sub[(prefix_of<KW>(k, K) - p_lo) >> sh], 1u)] = (uint16_t)slot;
+                    ord[atomicAdd(&S.sub[cut_of(cut, k, K)], 1u)] = (uint16_t)slot;
                 }
                 __syncthreads();
                 const uint64_t at = (uint64_t)S.out0 + done;
@@ -1278,7 +1495,7 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                     for (unsigned i = tid; i < nd; i += NT) {
                         const unsigned slot = ord[i];
                         const Key<KW> k = table_key(S, x.in, slot);
-                        const unsigned c = (unsigned)((prefix_of<KW>(k, K) - p_lo) >> sh);
+                        const unsigned c = cut_of(cut, k, K);
                         const unsigned a0 = c ? S.sub[c - 1] : 0u, a1 = S.sub[c];
                         unsigned rk = a0;
                         if (a1 - a0 > 1)
@@ -1304,9 +1521,6 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                     ++done;
                 }
                 again = until;
-                lo = hi;
-                from = from || until;
-                until = false;
             } else {
                 // too many distinct keys: the round ends below the median of the
                 // first keys found in 32 stretches of the table
@@ -1334,12 +1548,22 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                     }
                 }
                 __syncthreads();
+                if (until && depth < kBoundsMax) {   // (else the rounds go on to the one before it)
+                    if (tid == 0) S.bounds[depth] = hi;
+                    ++depth;
+                }
                 hi = S.pivot;
                 until = true;
                 again = S.cut != 0;   // a full stretch of the table holds two keys at least
                 if (!again && tid == 0) atomicOr(&x.ctr->error, kErrProbeLimit);
             }
             __syncthreads();
+            if (!over && again) {   // on to the next bound
+                lo = hi;
+                from = true;
+                until = depth != 0;
+                if (until) hi = S.bounds[--depth];
+            }
             for (unsigned i = tid; i < nd; i += NT) {
                 const unsigned slot = S.list[i];
                 S.slot[slot] = kFree;
@@ -1686,14 +1910,17 @@ struct MetaLayout {
         size += (bytes + 255) & ~255ull;
         return at;
     }
-    uint64_t meta, codes, valid, samples, spl, lut, piece, starts, places, counts, offsets, big;
-    uint64_t prefix, totals, tile_base, map, fine_spl, fine_lut, fine_starts;
+    uint64_t meta, codes, valid, samples, samples_lo, spl, spl_lo, lut, piece, starts, places;
+    uint64_t counts, offsets, big;
+    uint64_t prefix, totals, tile_base, map, fine_spl, fine_lo, fine_lut, fine_starts;
     explicit MetaLayout(const DedupPlan &p) {
         meta = take(sizeof(DedupMeta));
         codes = take(p.chunks * p.chunk / 4 + 64);   // and 128 bases after the last chunk
         valid = take(p.chunks * p.chunk / 8);
         samples = take(round_up(p.samples, kSampleTile) * 8ull);
+        samples_lo = take(p.kw == 2 ? round_up(p.samples, kSampleTile) * 8ull : 0);
         spl = take(kMaxRanges * 8ull);
+        spl_lo = take(p.kw == 2 ? kMaxRanges * 8ull : 0);
         lut = take(kLutStride * 2ull);
         piece = take(p.chunks * 4);
         starts = take((p.n_ranges + 1ull) * p.chunks * 2);
@@ -1701,13 +1928,14 @@ struct MetaLayout {
         counts = take(p.total() * 4);
         offsets = take((p.total() + 1) * 4);
         big = take(p.total() * 4);
-        prefix = totals = tile_base = map = fine_spl = fine_lut = fine_starts = size;
+        prefix = totals = tile_base = map = fine_spl = fine_lo = fine_lut = fine_starts = size;
         if (p.n_fine) {
             prefix = take((uint64_t)p.n_ranges * p.chunks * 4);
             totals = take(p.n_ranges * 4ull);
             tile_base = take((p.n_ranges + 1) * 4ull);
             map = take(p.tiles() * sizeof(TileMap));
             fine_spl = take((uint64_t)p.n_ranges * kMaxRanges * 8);
+            fine_lo = take(p.kw == 2 ? (uint64_t)p.n_ranges * kMaxRanges * 8 : 0);
             fine_lut = take((uint64_t)p.n_ranges * kLutStride * 2);
             fine_starts = take(p.tiles() * (p.n_fine + 1) * 2);
         }
@@ -1756,6 +1984,7 @@ RefineArgs refine_args(const DedupPlan &p, const DedupBufs &d, const MetaLayout 
     r.n_fine = p.n_fine;
     r.target = p.target;
     r.spl = (const uint64_t *)(d.meta + m.spl);
+    r.spl_lo = (const uint64_t *)(d.meta + m.spl_lo);
     r.piece = (const uint32_t *)(d.meta + m.piece);
     r.prefix = (const uint32_t *)(d.meta + m.prefix);
     r.totals = (const uint32_t *)(d.meta + m.totals);
@@ -1763,6 +1992,7 @@ RefineArgs refine_args(const DedupPlan &p, const DedupBufs &d, const MetaLayout 
     r.starts = (const uint16_t *)(d.meta + m.starts);
     r.map = (const TileMap *)(d.meta + m.map);
     r.fine_spl = (uint64_t *)(d.meta + m.fine_spl);
+    r.fine_lo = (uint64_t *)(d.meta + m.fine_lo);
     r.fine_lut = (uint16_t *)(d.meta + m.fine_lut);
     r.fine_starts = (uint16_t *)(d.meta + m.fine_starts);
     r.meta = (DedupMeta *)(d.meta + m.meta);
@@ -1806,7 +2036,9 @@ cudaError_t finish_variant(const DedupPlan &p, const DedupBufs &d, DevCounters *
     x.n_ranges = p.n_ranges;
     x.n_total = (unsigned)p.total();
     x.spl = (const uint64_t *)(d.meta + m.spl);
+    x.spl_lo = (const uint64_t *)(d.meta + m.spl_lo);
     x.fine_spl = (const uint64_t *)(d.meta + m.fine_spl);
+    x.fine_lo = (const uint64_t *)(d.meta + m.fine_lo);
     x.places = (uint32_t *)(d.meta + m.places);
     x.counts = (uint32_t *)(d.meta + m.counts);
     x.meta = meta;
@@ -1907,20 +2139,23 @@ cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical,
     pa.valid = (uint16_t *)(d.meta + m.valid);
     DD_TRY(cudaMemsetAsync(meta, 0, sizeof(DedupMeta), s));
     uint64_t *samples = (uint64_t *)(d.meta + m.samples);
+    uint64_t *samples_lo = (uint64_t *)(d.meta + m.samples_lo);
     const unsigned n = round_up(p.samples, kSampleTile), tiles = n / kSampleTile;
     const size_t smem = std::max(n * sizeof(uint64_t), sizeof(unsigned) << kLutBits);
     auto *sk = p.kw == 1 ? sample_kernel<1> : sample_kernel<2>;
-    sk<<<tiles, 1024, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, meta);
-    DD_TRY(set_smem(rank_kernel, smem));
-    rank_kernel<<<tiles, 1024, smem, s>>>(samples, n, p.n_ranges, last_prefix(p.K), meta,
-                                          (uint64_t *)(d.meta + m.spl),
-                                          (uint16_t *)(d.meta + m.lut));
+    sk<<<tiles, 1024, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, samples_lo, meta);
+    auto *rk = p.kw == 1 ? rank_kernel<1> : rank_kernel<2>;
+    DD_TRY(set_smem(rk, smem));
+    rk<<<tiles, 1024, smem, s>>>(samples, samples_lo, n, p.n_ranges, last_prefix(p.K), meta,
+                                 (uint64_t *)(d.meta + m.spl), (uint64_t *)(d.meta + m.spl_lo),
+                                 (uint16_t *)(d.meta + m.lut));
     ExtractArgs x;
     x.codes = pa.codes;
     x.valid = pa.valid;
     x.n_chunks = (unsigned)n_chunks;
     x.n_ranges = p.n_ranges;
     x.spl = (const uint64_t *)(d.meta + m.spl);
+    x.spl_lo = (const uint64_t *)(d.meta + m.spl_lo);
     x.lut = (const uint16_t *)(d.meta + m.lut);
     x.out = d.a;
     x.piece = (uint32_t *)(d.meta + m.piece);

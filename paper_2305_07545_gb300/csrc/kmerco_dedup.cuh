@@ -56,7 +56,7 @@ struct ExtractArgs {
     const uint16_t *valid;
     unsigned n_chunks;     // chunks of the pass
     unsigned n_ranges;
-    const uint64_t *spl;
+    const uint64_t *spl, *spl_lo;   // prefixes of the splitters, low words of two-word keys
     const uint16_t *lut;
     uint64_t *out;
     uint32_t *piece;       // first key of every chunk's piece
@@ -69,11 +69,11 @@ struct RefineArgs {
     uint64_t *out;
     unsigned n_chunks, n_ranges, n_fine;
     unsigned target;         // windows of a fine range
-    const uint64_t *spl;
+    const uint64_t *spl, *spl_lo;
     const uint32_t *piece, *prefix, *totals, *tile_base;
     const uint16_t *starts;
     const TileMap *map;
-    uint64_t *fine_spl;      // kMaxRanges per range
+    uint64_t *fine_spl, *fine_lo;   // kMaxRanges per range
     uint16_t *fine_lut;      // kLutStride per range
     uint16_t *fine_starts;   // per range: n_fine + 1 rows of its tiles
     DedupMeta *meta;
@@ -87,7 +87,7 @@ struct DedupArgs {
     unsigned n_fine;         // two levels: fine ranges per coarse range; 0: one level
     unsigned n_ranges, n_total;
     int ordered;             // write every range's keys in order, and where they are
-    const uint64_t *spl, *fine_spl;
+    const uint64_t *spl, *spl_lo, *fine_spl, *fine_lo;
     const uint32_t *piece, *tile_base;
     const uint16_t *starts;  // of the last level
     uint32_t *places, *counts;   // per range: first key in out, distinct keys

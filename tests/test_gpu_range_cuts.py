@@ -1,0 +1,93 @@
+"""Where the key space is cut into ranges, bit-exact and in its cost.
+
+Long keys with a common beginning (a constant flank, a primer, an adapter) have
+equal 64-bit prefixes and are cut by their low words; ranges that the samples
+say nothing about hold far more keys than a block's table and are counted in
+rounds, in key order and (a further call that goes to the distinct set) in none.
+"""
+import numpy as np
+import pytest
+
+import readsim
+
+torch = pytest.importorskip("torch")
+import paper_2305_07545_gb300 as kc  # noqa: E402
+from test_gpu_parity import _dev, check  # noqa: E402
+from test_gpu_set_keys import _count, _join  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _bases(st, *shape):
+    return readsim.ASCII[st.integers(int(np.prod(shape)), 4).astype(np.uint8)].reshape(shape)
+
+
+def _even(x):
+    return x.reshape(-1), np.arange(len(x) + 1, dtype=np.uint64) * np.uint64(x.shape[1])
+
+
+def _flanked(n, length, flank, seed):
+    st = readsim.Stream(seed)
+    head = np.broadcast_to(_bases(st, 1, flank), (n, flank))
+    return _even(np.concatenate([head, _bases(st, n, length - flank)], axis=1))
+
+
+@pytest.mark.parametrize("K,length,flank", [(33, 70, 40), (55, 70, 40), (64, 90, 50)])
+@pytest.mark.parametrize("n", [9000, 60000])   # one level of ranges, and two
+@pytest.mark.parametrize("forward_only", [False, True])
+def test_keys_with_a_common_beginning(K, length, flank, n, forward_only):
+    parts = [_flanked(n, length, flank, seed=K + n)]
+    g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
+    check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
+
+
+@pytest.mark.parametrize("K", [40, 55])
+@pytest.mark.parametrize("first", [3000, 14000])   # merged into the list, put in the set
+def test_a_further_call_with_a_common_beginning(K, first):
+    parts = [readsim.random_reads(first, 150, 150, seed=K), _flanked(9000, 72, 40, seed=K + 1),
+             _flanked(9000, 72, 40, seed=K + 1)]
+    g = _count(parts, K, 1 << 22, 8, 3, 2)
+    check(g, *_join(parts), K, 8, 3, 2, cross_check=False)
+
+
+@pytest.mark.parametrize("K,forward_only", [(21, False), (32, True), (33, False), (55, False),
+                                            (64, True)])
+@pytest.mark.parametrize("first", [0, 14000])   # in key order, then in none
+def test_ranges_that_the_samples_miss(K, forward_only, first):
+    # 25,000 windows among 6e7 bases of reads too short to hold one: the samples,
+    # spread over the bases, meet next to none of them, so a range has thousands of
+    # keys; of a further call every window comes seven times
+    st = readsim.Stream(K)
+    some = _bases(st, 250, K + 99)
+    some[0] = ord("T")   # forward strand: the largest key there is
+    if first:
+        some = np.tile(some, (7, 1))
+    short = _bases(st, 3_000_000, 20)
+    cut = len(short) // 3
+    parts = [_even(short[:cut]), _even(some), _even(short[cut:])]
+    call = _join(parts)
+    calls = [readsim.random_reads(first, 150, 150, seed=K), call] if first else [call]
+    g = _count(calls, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
+    check(g, *_join(calls), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
+
+
+def _insert_ms(b, o, K, m=1 << 24):
+    d = _dev(b), _dev(o)
+    with kc.CountBF(K, m, 4, 4, 3) as bf:
+        ms = []
+        for _ in range(4):
+            bf.reset()
+            bf.insert(*d)
+            bf.classify()
+            ms.append(bf.stats()["insert_ms"])
+    return min(ms)
+
+
+def test_a_common_beginning_costs_no_rounds():
+    # as many windows and distinct keys as random reads have; cut by prefixes alone a
+    # block took a hundred times as long for its share of the keys.  Eight times
+    # leaves room for more bisecting and crowded cuts.
+    n, K = 60000, 55
+    flanked = _insert_ms(*_flanked(n, 70, 40, seed=1), K)
+    uniform = _insert_ms(*readsim.random_reads(n, 70, 70, seed=2), K)
+    assert flanked < 8 * uniform, (flanked, uniform)
