@@ -153,8 +153,10 @@ __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64
             ulonglong2 v = it == 0 && first2 ? *first2 : __ldcg((const ulonglong2 *)(table + 2 * slot));
             for (;;) {
                 if (v.x == klo && v.y == whi) return false;
-                const bool free = t.mask ? slot_free(v.y, t) : (v.x == kEmptyKey || v.y == kEmptyKey);
-                if (!free && v.y != whi) break;
+                const bool free = t.mask ? slot_free(v.y, t) : (v.x == kEmptyKey && v.y == kEmptyKey);
+                // without a tag: one word of all ones is a key's, or not written yet
+                const bool unsure = !t.mask && !free && (v.x == kEmptyKey || v.y == kEmptyKey);
+                if (!free && !unsure && v.y != whi) break;
                 const uint64_t elo = free ? v.x : kEmptyKey, ehi = free ? v.y : kEmptyKey;
                 uint64_t olo, ohi;
                 cas128(table + 2 * slot, elo, ehi, klo, whi, olo, ohi);

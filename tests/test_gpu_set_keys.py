@@ -78,3 +78,20 @@ def test_the_key_of_all_ones_added_merged_and_after_a_reset(K):
             other.classify()
             assert other.stats()["distinct"] == n
             bf.reset()
+
+
+@pytest.mark.parametrize("sizes", [(1, 1), (40, 40, 40)])
+def test_64_mers_with_a_half_of_t(sizes):
+    # one word of such a key is all ones, as both are of a free slot; every key comes
+    # several times, and other keys probe past it
+    st = readsim.Stream(64)
+    half = readsim.ASCII[st.integers(60 * 32, 4).astype(np.uint8)].reshape(60, 32)
+    t = np.full((60, 32), ord("T"), np.uint8)
+    some = np.concatenate([np.concatenate([half, t], axis=1), np.concatenate([t, half], axis=1)])
+    own = some.reshape(-1), np.arange(121, dtype=np.uint64) * np.uint64(64)
+    parts = [_join([own, readsim.random_reads(n, 64, 100, seed=n + i), own])
+             for i, n in enumerate(sizes)]
+    g = _count(parts, 64, 1 << 14, 8, 3, 2, forward_only=True)
+    check(g, *_join(parts), 64, 8, 3, 2, forward_only=True)
+    more = _count(parts, 64, 1 << 14, 8, 3, 2)
+    check(more, *_join(parts), 64, 8, 3, 2)
