@@ -27,10 +27,11 @@
 //      distinct list.
 //
 // A range is cut by splitters taken from the data itself, so skewed
-// compositions only move the splitters; one key held by very many windows
-// makes one large range with few distinct keys, which dedup_kernel streams
-// through the same shared memory.  A range with more distinct keys than fit
-// is handled in several rounds over sub-ranges of it.
+// compositions only move the splitters.  A key held by very many windows is
+// more than one splitter: the last of them becomes the next key, so that the
+// range before it holds this key alone and is counted by the lengths of its
+// runs.  A range with more distinct keys than fit is handled in several rounds
+// over sub-ranges of it.
 //
 // Keys are cut by their prefix (their top 64 bits), two-word keys whose prefixes
 // are equal by their low word: reads with a common beginning of 32 bases and
@@ -267,6 +268,52 @@ __device__ __forceinline__ void write_lut(unsigned *cells, uint64_t v, bool tie,
     }
 }
 
+// The cut right behind the cut (p, low), when that is a key: whether it is one, and
+// not the largest.  A two-word cut whose low word does not go with its prefix (a
+// sample that stands for all keys of its prefix has 0 there) is none.
+template <int KW>
+__device__ __forceinline__ bool next_cut(uint64_t &p, uint64_t &low, int K) {
+    if (KW == 1) {
+        if (p == ~0ull) return false;
+        ++p;
+        return true;
+    }
+    Key<2> k;
+    k.hi = p >> (128 - 2 * K);
+    k.lo = low;
+    if (prefix_of<2>(k, K) != p || (p == ~0ull && low == ~0ull)) return false;
+    k.hi += ++k.lo == 0 ? 1 : 0;
+    const uint64_t q = prefix_of<2>(k, K);
+    low = q == p ? k.lo : 0;   // (q, 0): in front of all keys of the next prefix
+    p = q;
+    return true;
+}
+
+// Splitter j of n, (p, low), where at(i, p, low) reads splitter i: the last one of
+// equal splitters moves behind their key, which is held by more windows than a range
+// then has.  Whether there are equal ones.
+template <int KW, typename F>
+__device__ __forceinline__ bool part_equal(F at, unsigned j, unsigned n, uint64_t &p, uint64_t &low,
+                                           int K) {
+    p = low = ~0ull;
+    if (j >= n) return false;
+    at(j, p, low);
+    const auto as = [&](unsigned i) {
+        uint64_t q, r = low;
+        at(i, q, r);
+        return q == p && (KW == 1 || r == low);
+    };
+    const bool prev = j && as(j - 1), next = j + 1 < n && as(j + 1);
+    if (prev && !next) {
+        uint64_t q = p, r = low;
+        if (next_cut<KW>(q, r, K)) {
+            p = q;
+            low = r;
+        }
+    }
+    return prev || next;
+}
+
 // Whether a neighbour among the n splitters has the prefix p of thread j's one too
 // (seen: shared memory for the prefixes).
 __device__ __forceinline__ bool shares_prefix(uint64_t *seen, unsigned j, unsigned n, uint64_t p) {
@@ -432,7 +479,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int can
 template <int KW>
 __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
                                                     const uint64_t *samples_lo, unsigned n,
-                                                    unsigned n_ranges, uint64_t last,
+                                                    unsigned n_ranges, int K, uint64_t last,
                                                     DedupMeta *meta, uint64_t *spl,
                                                     uint64_t *spl_lo, uint16_t *lut) {
     extern __shared__ ulonglong2 s2[];
@@ -481,17 +528,22 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    uint64_t f = ~0ull;   // the last of the n: what find_range stops at
-    if (valid && tid + 1 < n_ranges)
-        f = __ldcg(spl + tid);
-    else if (tid < n_ranges) {
-        spl[tid] = f;
-        if (KW == 2) spl_lo[tid] = f;
-    }
+    uint64_t f, f_lo;   // all ones at the last of the n: what find_range stops at
+    const bool equal = part_equal<KW>(
+        [&](unsigned i, uint64_t &p, uint64_t &low) {
+            p = __ldcg(spl + i);
+            if (KW == 2) low = __ldcg(spl_lo + i);
+        },
+        tid, valid ? n_ranges - 1 : 0, f, f_lo, K);
+    __syncthreads();
     bool tie = false;
     if (KW == 2 && valid) {
-        tie = shares_prefix(s, tid, n_ranges - 1, f);
-        if (!tie && tid < n_ranges) spl_lo[tid] = tid + 1 < n_ranges ? 0 : ~0ull;
+        tie = shares_prefix(s, tid, n_ranges - 1, f) || equal;
+        if (!tie && tid + 1 < n_ranges) f_lo = 0;
+    }
+    if (tid < n_ranges) {
+        spl[tid] = f;
+        if (KW == 2) spl_lo[tid] = f_lo;
     }
     write_lut<KW>((unsigned *)s, f, tie, valid != 0, n_ranges, 0, last, lut);
 }
@@ -801,14 +853,20 @@ __global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int 
         for (int e = 0; e < E; ++e) s[j * E + e] = v[e];
     }
     __syncthreads();
-    bool same = false, tie = false;
-    if (valid && j + 1 < nf) {
-        f = s[(uint64_t)(j + 1) * valid / nf];
-        f_lo = 0;
-        same = KW == 2 && j + kCrowd < nf && f == s[(uint64_t)(j + kCrowd) * valid / nf];
-    }
-    if constexpr (KW == 2) {
+    const unsigned used = valid ? nf - 1 : 0;   // splitters
+    bool tie = false;
+    if constexpr (KW == 1) {
+        part_equal<1>(
+            [&](unsigned i, uint64_t &p, uint64_t &) { p = s[(uint64_t)(i + 1) * valid / nf]; }, j, used,
+            f, f_lo, K);
+    } else {
         constexpr int E2 = (E < 4 ? 4 : E) / 2;
+        bool same = false;
+        if (j < used) {
+            f = s[(uint64_t)(j + 1) * valid / nf];
+            f_lo = 0;
+            same = j + kCrowd < nf && f == s[(uint64_t)(j + kCrowd) * valid / nf];
+        }
         if (__syncthreads_or(same)) {
             if (j == 0) valid = 0;
             __syncthreads();
@@ -829,12 +887,14 @@ __global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int 
 #pragma unroll
             for (int e = 0; e < E2; ++e) c[j * E2 + e] = v[e];
             __syncthreads();
-            if (valid && j + 1 < nf) {
-                const Cut2 at = c[(uint64_t)(j + 1) * valid / nf];
-                f = at.p;
-                f_lo = at.lo;
-            }
-            tie = shares_prefix(s, j, valid ? nf - 1 : 0, f);
+            tie = part_equal<2>(
+                [&](unsigned i, uint64_t &p, uint64_t &low) {
+                    const Cut2 at = c[(uint64_t)(i + 1) * valid / nf];
+                    p = at.p;
+                    low = at.lo;
+                },
+                j, valid ? nf - 1 : 0, f, f_lo, K);
+            tie = shares_prefix(s, j, valid ? nf - 1 : 0, f) || tie;
             if (!tie && valid && j + 1 < nf) f_lo = 0;
         }
         if (j < x.n_fine) x.fine_lo[(uint64_t)b * kMaxRanges + j] = f_lo;
@@ -984,13 +1044,15 @@ struct RangeRuns {
 struct RangeCut {
     uint64_t base;     // the smallest prefix (or low word) there can be
     int sh;            // kSubBits2 bits of the difference to it make a cut
-    unsigned by_low;
+    uint16_t by_low, pure;   // pure: the range is one key, whose cut is lo, lo2
+    uint64_t lo, lo2;
 };
 
 template <int KW>
-__device__ __forceinline__ RangeCut range_cut(const DedupArgs &x, unsigned g, uint64_t last) {
+__device__ __forceinline__ RangeCut range_cut(const DedupArgs &x, unsigned g, int K, uint64_t last) {
     // the range's bounds: prefixes, and of two-word keys the low words
     uint64_t lo = 0, hi = last, lo2 = 0, hi2 = ~0ull;
+    bool open = false;   // hi is a splitter: the range ends in front of it
     const auto below = [&](const uint64_t *p, const uint64_t *rest, uint64_t i) {
         lo = p[i];
         if (KW == 2) lo2 = rest[i];
@@ -1003,6 +1065,7 @@ __device__ __forceinline__ RangeCut range_cut(const DedupArgs &x, unsigned g, ui
         if (v < hi || (KW == 2 && v == hi && w < hi2)) {
             hi = v;
             hi2 = w;
+            open = true;
         }
     };
     if (x.n_fine) {
@@ -1022,13 +1085,19 @@ __device__ __forceinline__ RangeCut range_cut(const DedupArgs &x, unsigned g, ui
     c.by_low = KW == 2 && lo == hi ? 1 : 0;
     c.base = c.by_low ? lo2 : lo;
     c.sh = max(bit_len(c.by_low ? hi2 - lo2 : hi - lo) - kSubBits2, 0);
+    c.lo = lo;
+    c.lo2 = lo2;
+    if (open)
+        c.pure = next_cut<KW>(lo, lo2, K) && lo == hi && (KW == 1 || lo2 == hi2);
+    else
+        c.pure = lo == last && (KW == 1 || lo2 == ~0ull);
     return c;
 }
 
 template <int KW>
 __device__ __forceinline__ unsigned cut_of(const RangeCut &c, const Key<KW> &k, int K) {
     const uint64_t v = KW == 2 && c.by_low ? k.lo : prefix_of<KW>(k, K);
-    return (unsigned)((v - c.base) >> c.sh);
+    return min((unsigned)((v - c.base) >> c.sh), (unsigned)kSubBins2 - 1);
 }
 
 template <int KW>
@@ -1175,7 +1244,7 @@ __global__ void __launch_bounds__(kSmallThreads, 4) dedup_kernel(DedupArgs x, in
             for (unsigned i = tid; i < (unsigned)kSubBins2; i += NT) S.sub[i] = 0;
             if (tid == 0) {
                 S.lists = S.crowded = 0;
-                if (x.ordered) S.cut = range_cut<KW>(x, g, last);
+                if (x.ordered) S.cut = range_cut<KW>(x, g, K, last);
             }
         }
         copies_done();
@@ -1414,14 +1483,28 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
         const unsigned g = x.big[q];
         RangeRuns cur;
         cur.load(x, g);
-        const RangeCut cut = range_cut<KW>(x, g, last);
-        if (x.ordered) {   // the range's place in the output: room for all its windows
-            unsigned n = cur.n;
-            for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
-                n += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
-            block_exclusive_scan<unsigned, NT>(n, n);
-            if (tid == 0) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n);
+        const RangeCut cut = range_cut<KW>(x, g, K, last);
+        unsigned n_all = cur.n;   // windows of the range
+        for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
+            n_all += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
+        block_exclusive_scan<unsigned, NT>(n_all, n_all);
+        if (cut.pure) {   // one key, however many windows
+            if (tid == 0) {
+                const unsigned at = atomicAdd(&x.meta->out_cursor, 1u);
+                Key<KW> k;
+                k.lo = KW == 1 ? cut.lo : cut.lo2;
+                k.hi = KW == 1 ? 0 : cut.lo >> (128 - 2 * K);
+                store_key<KW>(x.out, at, k);
+                x.mult[at] = n_all;
+                if (x.ordered) {
+                    x.places[g] = at;
+                    x.counts[g] = 1;
+                }
+            }
+            continue;
         }
+        // the range's place in the output: room for all its windows
+        if (tid == 0 && x.ordered) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n_all);
         unsigned done = 0;    // distinct keys written
         unsigned depth = 0;   // bounds held
         Key<KW> lo, hi;
@@ -2146,7 +2229,7 @@ cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical,
     sk<<<tiles, 1024, 0, s>>>(pa, p.K, canonical, span, p.samples, samples, samples_lo, meta);
     auto *rk = p.kw == 1 ? rank_kernel<1> : rank_kernel<2>;
     DD_TRY(set_smem(rk, smem));
-    rk<<<tiles, 1024, smem, s>>>(samples, samples_lo, n, p.n_ranges, last_prefix(p.K), meta,
+    rk<<<tiles, 1024, smem, s>>>(samples, samples_lo, n, p.n_ranges, p.K, last_prefix(p.K), meta,
                                  (uint64_t *)(d.meta + m.spl), (uint64_t *)(d.meta + m.spl_lo),
                                  (uint16_t *)(d.meta + m.lut));
     ExtractArgs x;

@@ -91,3 +91,44 @@ def test_a_common_beginning_costs_no_rounds():
     flanked = _insert_ms(*_flanked(n, 70, 40, seed=1), K)
     uniform = _insert_ms(*readsim.random_reads(n, 70, 70, seed=2), K)
     assert flanked < 8 * uniform, (flanked, uniform)
+
+
+@pytest.mark.parametrize("K,forward_only", [(13, False), (21, False), (32, True), (33, True),
+                                            (55, False), (64, True)])
+@pytest.mark.parametrize("n", [1500, 12000])   # one level of ranges, and two
+def test_keys_held_by_very_many_windows(K, forward_only, n):
+    # reads of one base each (the smallest and the largest keys there are), of T's and a
+    # last A (the largest key but three), one read and one with another last base many times
+    st = readsim.Stream(n + K)
+    x = _bases(st, n, 150)
+    x[: n // 8] = ord("T")
+    x[n // 8: n // 6] = ord("A")
+    x[n // 6: n // 4, :K] = ord("T")
+    x[n // 6: n // 4, K - 1] = ord("A")
+    x[n // 4: n // 3] = x[n // 4]
+    x[n // 3: n // 2] = x[n // 4]
+    x[n // 3: n // 2, K - 1] = ord("C")
+    parts = [_even(x[_shuffled(n, st)])]
+    g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
+    check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
+    # the same as a further call that goes to the set
+    parts = [readsim.random_reads(10 * n, 150, 150, seed=K)] + parts
+    g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
+    check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
+
+
+def _shuffled(n, st):
+    return np.argsort(st.uniform(n))
+
+
+@pytest.mark.parametrize("K", [31, 55])
+def test_a_key_of_very_many_windows_costs_no_more_than_others(K):
+    # a tenth of the reads of one base: their windows were one block's, which took 15
+    # times as long as all the others for the rest
+    n = 200000
+    b, o = readsim.random_reads(n, 150, 150, seed=1)
+    uniform = _insert_ms(b, o, K, m=1 << 26)
+    x = b.reshape(n, 150).copy()
+    x[::10] = ord("G")
+    hot = _insert_ms(x.reshape(-1), o, K, m=1 << 26)
+    assert hot < 2 * uniform, (hot, uniform)
