@@ -617,15 +617,15 @@ PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
     return pp;
 }
 
-// By key ranges: calls of enough windows, unless the handle limits retries or
-// its list (those limits are the window-by-window kernel's).
+// By key ranges: calls of enough windows, unless the handle limits retries (those
+// limits are the window-by-window kernel's).
 InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool fresh,
                        bool may_merge = false) {
     InsertPlan ip;
     ip.bound = bound;
     ip.fresh = fresh;
-    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->max_distinct ||
-        h->G.cas_limit != kCasLimit || nbytes < bound)
+    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->G.cas_limit != kCasLimit ||
+        nbytes < bound)
         return ip;
     // windows one pass takes (1.9e9 two-word windows: 239 ms with their classification
     // in one pass, 244 in two that keep to the ranges' target)
@@ -644,7 +644,8 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     if (ip.ranges) ip.pp = plan_partition(h, ip.dd.bound);
     // (a call of several passes into an empty handle would else put its keys into a
     // set and sort them: 2.4e9 windows 170 ms and 50 to classify, merged 143 and 28)
-    ip.merge = ip.ranges && may_merge && h->d_ub + bound < 0xFFFFFFFFull &&
+    // (a list with a cap keeps to its buffer)
+    ip.merge = ip.ranges && may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull &&
                (fresh ? ip.passes > 1 : h->list_sorted && bound * kMergeShare >= h->d_ub);
     return ip;
 }
@@ -848,9 +849,11 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
                               std::min(ce * chunk, nbytes) - cb * chunk, h->sms, s, launches));
         const bool fresh = ip.fresh && pass == 0;
         const bool ordered = fresh || ip.merge;
-        KM_CUDA(dedup_finish(ip.dd, b.dd, h->ctr, ce - cb, ordered, fresh, h->sms, s, launches));
+        KM_CUDA(dedup_finish(ip.dd, b.dd, h->ctr, ce - cb, ordered, fresh, h->dlist_cap, h->sms, s,
+                             launches));
         EmitArgs e = dedup_result(ip.dd, b.dd, h->G, h->ctr, ordered);
         e.dlist = fresh ? h->dlist : ip.merge ? merge_input(ip, b) : nullptr;
+        e.dlist_cap = fresh ? h->dlist_cap : ~0ull;
         e.sure = fresh && ip.sure ? h->sure : nullptr;
         e.tau = h->tau;
         KM_TRY(launch_updates(h, ip, b, e, s, launches));
@@ -864,7 +867,8 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
         if (!ip.table()) continue;
         // the pass's keys into the distinct set (the first pass of an empty
         // handle: its list as it stands)
-        KM_CUDA(launch_reinsert(fresh ? h->dlist : e.keys, ip.dd.bound,
+        KM_CUDA(launch_reinsert(fresh ? h->dlist : e.keys,
+                                fresh ? std::min(ip.dd.bound, h->dlist_cap) : ip.dd.bound,
                                 fresh ? &e.meta->distinct : &e.meta->out_cursor, nullptr, h->kw,
                                 h->table, h->cap, set_tag(h), fresh ? nullptr : h->dlist,
                                 h->dlist_cap, h->ctr, h->G.probe_limit, s));

@@ -1660,7 +1660,7 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
 // offsets[g] = distinct keys in ranges before g, offsets[n] = all; one block.
 __global__ void __launch_bounds__(1024) scan_counts_kernel(const uint32_t *counts, unsigned n,
                                                            uint32_t *offsets, DedupMeta *meta,
-                                                           DevCounters *ctr) {
+                                                           DevCounters *ctr, uint64_t list_cap) {
     constexpr unsigned E = 16;
     unsigned carry = 0;
     for (unsigned i0 = 0; i0 < n; i0 += 1024 * E) {
@@ -1684,7 +1684,10 @@ __global__ void __launch_bounds__(1024) scan_counts_kernel(const uint32_t *count
     if (threadIdx.x == 0) {
         offsets[n] = carry;
         meta->distinct = carry;
-        if (ctr) ctr->distinct = carry;   // the list holds exactly these
+        if (ctr) {
+            ctr->distinct = carry;   // the list holds exactly these
+            if (carry > list_cap) atomicOr(&ctr->error, kErrListFull);
+        }
     }
 }
 
@@ -1814,7 +1817,7 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_kernel(EmitArgs e) {
                 const uint64_t at = e.ordered ? place_in(off, plc, i) : i;
                 key[q] = load_key<KW>(e.keys, at);
                 w[q] = (uint32_t)min((uint64_t)e.mult[at], G.maxc);
-                if (e.dlist) store_key<KW>(e.dlist, i, key[q]);
+                if (e.dlist && i < e.dlist_cap) store_key<KW>(e.dlist, i, key[q]);
                 if (e.sure) e.sure[i] = w[q] > e.tau;
             }
         }
@@ -1938,7 +1941,7 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_atomic_kernel(EmitArgs e
         const uint64_t at = e.ordered ? place_in(off, plc, i) : i;
         const Key<KW> key = load_key<KW>(e.keys, at);
         const uint64_t w = min((uint64_t)e.mult[at], G.maxc);
-        if (e.dlist) store_key<KW>(e.dlist, i, key);
+        if (e.dlist && i < e.dlist_cap) store_key<KW>(e.dlist, i, key);
         if (e.sure) e.sure[i] = w > e.tau;
         const uint64_t k1m = KW == 1 ? premix8(key.lo) : 0;
         for (int a0 = 0; a0 < G.nhash; a0 += 4) {
@@ -2084,8 +2087,8 @@ RefineArgs refine_args(const DedupPlan &p, const DedupBufs &d, const MetaLayout 
 
 template <int KW>
 cudaError_t finish_variant(const DedupPlan &p, const DedupBufs &d, DevCounters *ctr,
-                           uint64_t n_chunks, bool ordered, bool fresh, int sms, cudaStream_t s,
-                           uint64_t &launches) {
+                           uint64_t n_chunks, bool ordered, bool fresh, uint64_t list_cap, int sms,
+                           cudaStream_t s, uint64_t &launches) {
     const MetaLayout m(p);
     DedupMeta *meta = (DedupMeta *)(d.meta + m.meta);
     const unsigned nc = (unsigned)n_chunks;
@@ -2137,7 +2140,8 @@ cudaError_t finish_variant(const DedupPlan &p, const DedupBufs &d, DevCounters *
     launches += 2;
     if (!ordered) return cudaGetLastError();
     scan_counts_kernel<<<1, 1024, 0, s>>>(x.counts, (unsigned)p.total(),
-                                          (uint32_t *)(d.meta + m.offsets), meta, fresh ? ctr : nullptr);
+                                          (uint32_t *)(d.meta + m.offsets), meta, fresh ? ctr : nullptr,
+                                          list_cap);
     launches += 1;
     return cudaGetLastError();
 }
@@ -2255,10 +2259,11 @@ cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical,
 }
 
 cudaError_t dedup_finish(const DedupPlan &p, const DedupBufs &d, DevCounters *ctr,
-                         uint64_t n_chunks, bool ordered, bool fresh, int sms, cudaStream_t s,
-                         uint64_t &launches) {
-    return p.kw == 1 ? finish_variant<1>(p, d, ctr, n_chunks, ordered, fresh, sms, s, launches)
-                     : finish_variant<2>(p, d, ctr, n_chunks, ordered, fresh, sms, s, launches);
+                         uint64_t n_chunks, bool ordered, bool fresh, uint64_t list_cap, int sms,
+                         cudaStream_t s, uint64_t &launches) {
+    return p.kw == 1
+               ? finish_variant<1>(p, d, ctr, n_chunks, ordered, fresh, list_cap, sms, s, launches)
+               : finish_variant<2>(p, d, ctr, n_chunks, ordered, fresh, list_cap, sms, s, launches);
 }
 
 EmitArgs dedup_result(const DedupPlan &p, const DedupBufs &d, const Geometry &G, DevCounters *ctr,

@@ -104,6 +104,7 @@ struct EmitArgs {
     int ordered;             // keys in the order of the ranges (places, offsets), else as they stand
     unsigned begin, end;     // distinct keys of this pass
     uint64_t *dlist;         // distinct list to write, or null
+    uint64_t dlist_cap;      // keys it holds: those after them are left out
     uint8_t *sure;           // key i has more than tau windows (or null)
     uint32_t tau;
     int coarse_shift, slot_bits, w_bits;
@@ -152,15 +153,15 @@ DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk);
 // after these); then the windows' keys are cut into ranges (span: bases of the
 // pass); then everything up to the distinct keys with their multiplicities.
 // ordered: in ascending order; fresh: the handle's list is empty (ctr->distinct
-// becomes the call's count).
+// becomes the call's count, and more than list_cap of them the list-full error).
 cudaError_t dedup_pack(const DedupPlan &p, const DedupBufs &d, const InsertArgs &a, uint64_t chunk0,
                        uint64_t n_chunks, uint64_t begin, uint64_t end, int sms, cudaStream_t s,
                        uint64_t &launches);
 cudaError_t dedup_extract(const DedupPlan &p, const DedupBufs &d, int canonical, uint64_t n_chunks,
                           uint64_t span, int sms, cudaStream_t s, uint64_t &launches);
 cudaError_t dedup_finish(const DedupPlan &p, const DedupBufs &d, DevCounters *ctr,
-                         uint64_t n_chunks, bool ordered, bool fresh, int sms, cudaStream_t s,
-                         uint64_t &launches);
+                         uint64_t n_chunks, bool ordered, bool fresh, uint64_t list_cap, int sms,
+                         cudaStream_t s, uint64_t &launches);
 // The arguments every consumer of the distinct keys takes.  Of a pass that is not
 // ordered, e.keys holds them one after the other in no order, e.meta->out_cursor of them.
 EmitArgs dedup_result(const DedupPlan &p, const DedupBufs &d, const Geometry &G, DevCounters *ctr,
