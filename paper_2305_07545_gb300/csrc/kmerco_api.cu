@@ -617,14 +617,14 @@ PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
     return pp;
 }
 
-// By key ranges: calls of enough windows, unless the handle limits retries (those
-// limits are the window-by-window kernel's).
+// By key ranges: calls of enough windows, unless the handle limits retries to few
+// (window by window then, whose loops contend for slots and counters).
 InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool fresh,
                        bool may_merge = false) {
     InsertPlan ip;
     ip.bound = bound;
     ip.fresh = fresh;
-    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->G.cas_limit != kCasLimit ||
+    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->G.cas_limit < kRangesRetries ||
         nbytes < bound)
         return ip;
     // windows one pass takes (1.9e9 two-word windows: 239 ms with their classification
@@ -1773,7 +1773,7 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
     // ascending lists: copied into an empty handle, merged into an ordered one
     dst->sure_ok = false;
     const bool ordered = src->list_sorted && sc.distinct && !dst->max_distinct &&
-                         dst->G.probe_limit == kProbeLimit;
+                         dst->G.probe_limit >= kRangesRetries;
     bool listed = false;
     if (ordered && dst->d_ub == 0) {
         KM_TRY(ensure_set_capacity(dst, sc.distinct, false));

@@ -41,6 +41,9 @@ constexpr int kRadixBins = 1 << kRadixBits;
 constexpr int kSplitTile = 4096;
 constexpr uint32_t kCasLimit = 1u << 22;   // retries of one counter update
 constexpr uint32_t kProbeLimit = 1u << 20; // probes of one distinct-set insert
+// A caller's retry limit from which inserts go by key ranges: no insert into a set at a load
+// factor of 1/2 probes as often.  Smaller ones are there to be met, window by window.
+constexpr uint32_t kRangesRetries = 1024;
 
 // Device error bits (DevCounters::error).
 constexpr unsigned kErrCasLimit = 1u;
