@@ -491,13 +491,17 @@ bool use_partitioned(const kmerco_t *h, uint64_t bound) {
     if (h->update_mode == 1) return false;
     const bool able = h->G.words <= (1ull << (kMaxCoarseShift + 6));
     if (h->update_mode == 2) return able;
-    // smaller countBFs stay L2-resident.  The partitioned update takes about 10 ps
-    // an increment and 3 to 4.3 ps a cell (it reads and writes them all); a random
-    // update 20 ps while the countBF is about the size of L2 (2^25 cells are
-    // 256 MiB), 33 to 60 ps beyond.  A third to nearly all of the windows are
-    // distinct keys.
+    // smaller countBFs stay L2-resident.  The partitioned update takes about 20 ps an
+    // increment and 2.4 ps a cell (it reads and writes them all); a random one 30 ps
+    // while the countBF fits L2 (2^24 cells are 128 MiB), 40 at twice that, 53
+    // beyond.  So the lines would lie at 0.25, 0.13 and 0.08 increments a cell were all
+    // windows distinct keys, and at three times that where a third of them are:
+    // between the two (4e6 distinct windows of four hashes into 2^25 cells: 0.84 ms by
+    // random updates, 0.54 partitioned; 1e6: 0.26 and 0.27).
     const uint64_t U = bound * (uint64_t)h->nhash, W = h->G.words;
-    return able && W >= (1ull << 17) && U >= (W <= (1ull << 25) ? W : W / 5);
+    // Its further launches cost as much as it saves on 3e6 increments.
+    const uint64_t least = W <= (1ull << 24) ? W / 2 : W <= (1ull << 25) ? W / 4 : W / 9;
+    return able && W >= (1ull << 17) && U >= std::max<uint64_t>(least, 3u << 20);
 }
 
 // Trial division; n is at most about 2^24 here.
