@@ -117,8 +117,7 @@ typedef struct {
                               stops, so the counts are incomplete, and the next classify or
                               stats returns KMERCO_ETIMEOUT; reset clears the state.  Small
                               values exist to exercise that path on contended input: below
-                              1,024 every window is inserted by itself, with compare-and-swap
-                              updates whatever update_mode says. */
+                              1,024 every window is put in the set by itself. */
     uint64_t max_distinct; /* most distinct keys the handle's distinct list may hold; 0: no
                               limit (it grows with the input).  Keys beyond it are left out of
                               the list and the next classify or stats returns KMERCO_ENOMEM;

@@ -25,10 +25,18 @@ constexpr int kCopyPieces = 8;   // pieces of a host input copied while earlier 
 constexpr uint64_t kHostBoundReads = 1ull << 16;
 
 // Windows from which an insert call goes by key ranges: below, its dozen
-// launches cost more than the window-by-window kernel takes.  A handle that
-// holds keys already also collects the call's keys into its distinct set.
+// launches cost more than the window-by-window kernel takes.  A call into a
+// handle that holds keys has to merge its keys with those too: eight pieces of
+// 2.5e6 windows take 3.9 ms by ranges and 3.3 window by window, of 5e6 6.3 and 5.9
+// when nearly all windows differ, 3.5 and 4.1 when they are five times as many.
 constexpr uint64_t kRangesMin = 1ull << 14;
-constexpr uint64_t kRangesMinMore = 1ull << 17;
+constexpr uint64_t kRangesMinMore = 1ull << 22;
+// Windows from which a call that goes window by window is packed first.
+constexpr uint64_t kPackMin = 1ull << 16;
+// Windows up to which a further call whose keys are not merged into an ordered list
+// goes window by window: 28 pieces of 1e7 windows 39 ms, by ranges and then into
+// the set 52 (five times as many windows as keys: 27.5 and 26.0).
+constexpr uint64_t kWindowsMost = 1ull << 26;
 
 // Distinct one-word keys above which classification takes the bucket sort
 // (its histogram readback and host-side merge cost more than a full radix
@@ -422,10 +430,12 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
     return KMERCO_OK;
 }
 
-// Calls that bring at least this share of the keys already held (bounds of
-// both) are merged into the ordered list: a union takes about 10 ps for every
-// key held or new, the distinct set 36 ps for every new one and the list then
-// has to be sorted.
+// Calls of at least this share of the keys already held (bounds of both, where the
+// counts are not known) are merged into the ordered list: a union takes about 13 ps
+// for every key held or new.  By ranges a call is 50 ps a window quicker than window by
+// window, but a handle that goes over to its set later has to build it from the
+// list, 36 ps a key: with four the sum is about even however many pieces come
+// (six pieces of 1e7 windows 8.1 ms, 8.7 all window by window; three 3.5 and 4.2).
 constexpr uint64_t kMergeShare = 4;
 
 // Room for the union of the list and at most `add` more keys.
@@ -486,8 +496,8 @@ int validate(const kmerco_config_t *c) {
 }
 
 // Whether a call of at most `bound` windows applies its increments with the
-// partitioned update.
-bool use_partitioned(const kmerco_t *h, uint64_t bound) {
+// partitioned update; staged: all the windows', not its distinct keys' alone.
+bool use_partitioned(const kmerco_t *h, uint64_t bound, bool staged) {
     if (h->update_mode == 1) return false;
     const bool able = h->G.words <= (1ull << (kMaxCoarseShift + 6));
     if (h->update_mode == 2) return able;
@@ -500,7 +510,8 @@ bool use_partitioned(const kmerco_t *h, uint64_t bound) {
     // random updates, 0.54 partitioned; 1e6: 0.26 and 0.27).
     const uint64_t U = bound * (uint64_t)h->nhash, W = h->G.words;
     // Its further launches cost as much as it saves on 3e6 increments.
-    const uint64_t least = W <= (1ull << 24) ? W / 2 : W <= (1ull << 25) ? W / 4 : W / 9;
+    const uint64_t least = W <= (1ull << 24) ? W / (staged ? 4 : 2)
+                           : W <= (1ull << 25) ? W / (staged ? 8 : 4) : W / (staged ? 12 : 9);
     return able && W >= (1ull << 17) && U >= std::max<uint64_t>(least, 3u << 20);
 }
 
@@ -556,9 +567,12 @@ struct PartPlan {
 };
 
 // How one insert call runs: window by window, or by key ranges in `passes`
-// passes over consecutive chunks of its reads.
+// passes over consecutive chunks of its reads.  Window by window and packed: the input
+// is packed first; with pp.part the insert kernel then writes the windows' keys down
+// and their increments are partitioned.
 struct InsertPlan {
     bool ranges = false;
+    bool packed = false;
     bool fresh = false;      // the handle holds no keys: the first pass writes the list
     bool sure = false;       // the list is the call's keys: which are sure is written too
     bool merge = false;      // the list stays in order: every pass's keys but the ones that
@@ -570,6 +584,31 @@ struct InsertPlan {
     // whether the call needs the distinct set
     bool table() const { return !(ranges && (merge || (fresh && passes == 1))); }
     uint64_t merges() const { return merge ? passes - (fresh ? 1 : 0) : 0; }
+    bool staged() const { return packed && pp.part; }
+    // keys whose increments a pass applies, at most
+    uint64_t keys_most() const { return ranges ? dd.bound : bound; }
+};
+
+// Bytes of the scratch of a plan: range keys twice, multiplicities, tables; increment
+// codes by region and by slice, their cursors.
+struct PlanScratch {
+    uint64_t n[7];
+    PlanScratch(const InsertPlan &ip, int kw) : n{} {
+        if (ip.ranges) {
+            n[0] = ip.dd.keys_a() * 8;
+            n[1] = ip.dd.keys_b() * 8;
+            n[2] = ip.dd.mult_words() * 4;
+            n[3] = ip.dd.meta_bytes();
+        } else if (ip.packed) {
+            n[0] = ip.pp.part ? ip.bound * kw * 8 : 0;
+            n[3] = ip.dd.meta_bytes();
+        }
+        if (ip.pp.part) {
+            n[4] = ip.pp.coarse_words() * 4;
+            n[5] = ip.pp.fine_words() * 4;
+            n[6] = ip.pp.ctr_words() * 8;
+        }
+    }
 };
 
 struct InsertBufs {
@@ -589,13 +628,13 @@ struct InsertBufs {
 // kCountLanes / eta cells, rounded down to a power of two) for alpha <= 15 and
 // enough increments a cell, compare-and-swap apply otherwise or when the slices
 // would be too many for one coarse region.
-PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
+PartPlan plan_partition(const kmerco_t *h, uint64_t bound, bool staged) {
     PartPlan pp;
-    if (!use_partitioned(h, bound) || bound == 0) return pp;
+    if (bound == 0 || bound > kMaxRangeWindows || !use_partitioned(h, bound, staged)) return pp;
     pp.part = true;
     const uint64_t W = h->G.words, nh = (uint64_t)h->nhash;
     pp.keys = std::min(bound, std::max<uint64_t>(h->pass_codes / nh, 1024));
-    if (bound > (1ull << 24)) pp.keys = std::min(pp.keys, (bound + 1) / 2);
+    if (bound > (1ull << 24) && !staged) pp.keys = std::min(pp.keys, (bound + 1) / 2);
     const uint64_t U = pp.keys * nh;   // increments per pass
     pp.coarse_shift = ceil_log2(W) - 6;
     if (pp.coarse_shift < 0) pp.coarse_shift = 0;
@@ -605,11 +644,10 @@ PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
     while ((2ull << count_shift) * (uint64_t)h->eta <= (uint64_t)kCountLanes) ++count_shift;
     // Counting apply: about 1 ps a counter of the countBF; compare-and-swap
     // apply: 4.3 ps a cell and 2.3 ps an increment more than counting (measured
-    // on 2^24 to 2^29 cells).  A third of the increments staged stand for
-    // distinct keys.
+    // on 2^24 to 2^29 cells).  A third of a call's windows stand for distinct keys.
     const double per_cell = (double)h->eta - 4.3;
     pp.count = h->alpha <= 15 && pp.coarse_shift - count_shift <= kMaxCoarseShift - kSliceShift &&
-               (double)(bound * nh) / 3 * 2.3 >= per_cell * (double)W;
+               (double)(bound * nh) / (staged ? 1 : 3) * 2.3 >= per_cell * (double)W;
     pp.slice_shift = pp.count ? count_shift : kSliceShift;
     pp.repart = pp.coarse_shift > pp.slice_shift;
     if (!pp.repart) pp.slice_shift = pp.coarse_shift;
@@ -621,16 +659,32 @@ PartPlan plan_partition(const kmerco_t *h, uint64_t bound) {
     return pp;
 }
 
+// Window by window; the increments partitioned where that is the faster update, the
+// input packed first for that and in calls that read it for more than some microseconds.
+InsertPlan plan_windows(const kmerco_t *h, uint64_t bound, uint64_t nbytes) {
+    InsertPlan ip;
+    ip.bound = bound;
+    ip.pp = plan_partition(h, bound, true);
+    ip.packed = ip.pp.part || bound >= kPackMin;
+    if (ip.packed) ip.dd = plan_pack(h->K, nbytes);
+    return ip;
+}
+
 // By key ranges: calls of enough windows, unless the handle limits retries to few
 // (window by window then, whose loops contend for slots and counters).
 InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool fresh,
                        bool may_merge = false) {
-    InsertPlan ip;
-    ip.bound = bound;
-    ip.fresh = fresh;
-    if (bound < (fresh ? kRangesMin : kRangesMinMore) || h->G.cas_limit < kRangesRetries ||
+    InsertPlan ip = plan_windows(h, bound, nbytes);
+    // (a list with a cap keeps to its buffer)
+    const bool merge = may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull;
+    const bool into_list = merge && h->list_sorted && bound * kMergeShare >= h->d_ub;
+    if (bound < (fresh ? kRangesMin : kRangesMinMore) ||
+        (!fresh && !into_list && bound <= kWindowsMost) || h->G.cas_limit < kRangesRetries ||
         nbytes < bound)
         return ip;
+    ip = InsertPlan();
+    ip.bound = bound;
+    ip.fresh = fresh;
     // windows one pass takes (1.9e9 two-word windows: 239 ms with their classification
     // in one pass, 244 in two that keep to the ranges' target)
     uint64_t most = kMaxRangeWindows;
@@ -645,12 +699,11 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
         if (ip.dd.on || pc == 1) break;   // else its chunks may hold more windows than a pass takes
     }
     ip.ranges = ip.dd.on;
-    if (ip.ranges) ip.pp = plan_partition(h, ip.dd.bound);
+    if (!ip.ranges) return plan_windows(h, bound, nbytes);
+    ip.pp = plan_partition(h, ip.dd.bound, false);
     // (a call of several passes into an empty handle would else put its keys into a
     // set and sort them: 2.4e9 windows 170 ms and 50 to classify, merged 143 and 28)
-    // (a list with a cap keeps to its buffer)
-    ip.merge = ip.ranges && may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull &&
-               (fresh ? ip.passes > 1 : h->list_sorted && bound * kMergeShare >= h->d_ub);
+    ip.merge = fresh ? merge && ip.passes > 1 : into_list;
     return ip;
 }
 
@@ -737,7 +790,8 @@ uint64_t insert_chunk(const kmerco_t *h, uint64_t nbytes) {
 
 // Chunks of the insert's first_read table at most.
 uint64_t first_read_entries(const kmerco_t *h, const InsertPlan &ip, uint64_t nbytes) {
-    const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
+    const uint64_t chunk =
+        ip.ranges || ip.packed ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
     return (nbytes + chunk - 1) / chunk;
 }
 
@@ -767,10 +821,11 @@ int launch_updates(const kmerco_t *h, const InsertPlan &ip, const InsertBufs &b,
     e.coarse_written = b.ctr + kCoarseBins;
     unsigned long long *fine_cursor = b.ctr + 2 * kCoarseBins;
     unsigned long long *fine_written = fine_cursor + pp.nslices;
-    for (uint64_t k0 = 0; k0 < ip.dd.bound; k0 += pp.keys) {
+    const uint64_t most = ip.keys_most();
+    for (uint64_t k0 = 0; k0 < most; k0 += pp.keys) {
         KM_CUDA(cudaMemsetAsync(b.ctr, 0, pp.ctr_words() * 8, s));
         e.begin = (unsigned)k0;
-        e.end = (unsigned)std::min(k0 + pp.keys, ip.dd.bound);
+        e.end = (unsigned)std::min(k0 + pp.keys, most);
         KM_CUDA(launch_emit(e, h->kw, h->sms, s));
         if (pp.repart) {
             PartArgs p;
@@ -799,7 +854,7 @@ int launch_updates(const kmerco_t *h, const InsertPlan &ip, const InsertBufs &b,
         ap.codes = pp.repart ? b.fine : b.coarse;
         ap.cap = pp.repart ? pp.fine_cap : pp.coarse_cap;
         ap.lane_codes = pp.repart && pp.count ? 1 : 0;
-        ap.guard = ip.dd.bound * (uint64_t)h->nhash >= (1ull << 32) ? 1 : 0;
+        ap.guard = most * (uint64_t)h->nhash >= (1ull << 32) ? 1 : 0;
         ap.written = pp.repart ? fine_written : e.coarse_written;
         ap.ctr = h->ctr;
         KM_CUDA(pp.count ? launch_apply_count(ap, pp.nslices, s) : launch_apply(ap, pp.nslices, s));
@@ -824,7 +879,8 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
                          const InsertBufs &b, cudaStream_t s, uint64_t &launches,
                          const HostCopy *hc = nullptr, cudaEvent_t input_read = nullptr) {
     const uint64_t nbytes = a.last - a.first;
-    const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
+    const uint64_t chunk =
+        ip.ranges || ip.packed ? (uint64_t)ip.dd.chunk : insert_chunk(h, nbytes);
     const uint64_t nchunks = (nbytes + chunk - 1) / chunk;
     KM_CUDA(launch_first_read(a.offsets, a.nreads, a.first, nchunks, chunk, h->first_read, s));
     launches += nchunks ? 1 : 0;
@@ -838,7 +894,7 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
             const uint64_t c0 = cb + (ce - cb) * j / qq, c1 = cb + (ce - cb) * (j + 1) / qq;
             // the pieces holding this range's bytes and the K - 1 after it
             KM_TRY(wait_pieces(hc, c0 * chunk, std::min(c1 * chunk + (uint64_t)a.K - 1, nbytes), s));
-            if (!ip.ranges) {
+            if (!ip.ranges && !ip.packed) {
                 a.chunk_begin = c0;
                 a.nchunks = c1;
                 KM_CUDA(launch_insert(a, h->grid_atomic, (int)chunk, s));
@@ -848,6 +904,24 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
             KM_CUDA(dedup_pack(ip.dd, b.dd, a, cb, ce - cb, c0, c1, h->sms, s, launches));
         }
         if (input_read && pass + 1 == ip.passes) KM_CUDA(cudaEventRecord(input_read, s));
+        if (ip.packed) {
+            const Packed in = packed_input(ip.dd, b.dd);
+            a.codes = in.codes;
+            a.valid = in.valid;
+            if (ip.staged()) {
+                a.staged = b.dd.a;
+                a.n_staged = &in.meta->out_cursor;
+                KM_CUDA(cudaMemsetAsync(in.meta, 0, sizeof(DedupMeta), s));
+            }
+            const int own = chunk == kExtractSmall ? kSmallChunk : kChunk;   // half a packed one
+            static_assert(kExtractSmall == 2 * kSmallChunk && kExtractChunk == 2 * kChunk, "halves");
+            a.chunk_begin = 0;
+            a.nchunks = nchunks * 2;
+            KM_CUDA(launch_insert(a, h->grid_atomic, own, s));
+            launches += 1;
+            if (ip.staged())
+                KM_TRY(launch_updates(h, ip, b, windows_result(b.dd.a, in.meta, h->G, h->ctr), s, launches));
+        }
         if (!ip.ranges) continue;
         KM_CUDA(dedup_extract(ip.dd, b.dd, a.canonical, ce - cb,
                               std::min(ce * chunk, nbytes) - cb * chunk, h->sms, s, launches));
@@ -881,22 +955,23 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
     return KMERCO_OK;
 }
 
+int ensure_scratch(kmerco_t *h, const InsertPlan &ip) {
+    const PlanScratch need(ip, h->kw);
+    if (need.n[0]) KM_TRY(ensure(h, &h->range_a, &h->range_a_cap, need.n[0] / 8));
+    if (need.n[1]) KM_TRY(ensure(h, &h->range_b, &h->range_b_cap, need.n[1] / 8));
+    if (need.n[2]) KM_TRY(ensure(h, &h->mult, &h->mult_cap, need.n[2] / 4));
+    KM_TRY(ensure(h, &h->range_meta, &h->range_meta_cap, need.n[3]));
+    if (!ip.pp.part) return KMERCO_OK;
+    KM_TRY(ensure(h, &h->coarse, &h->coarse_alloc, need.n[4] / 4));
+    if (need.n[5]) KM_TRY(ensure(h, &h->fine, &h->fine_alloc, need.n[5] / 4));
+    return ensure(h, &h->part_ctr, &h->part_ctr_alloc, need.n[6] / 8);
+}
+
 // The buffers of a plan from the handle's: the ranges' scratch, the list, the set
-// or the union's buffers, first reads.  `held` becomes the keys held before, at most.
+// or the union's buffers, first reads; then the scratch of packed windows, without
+// which they are counted from the bases.  `held` becomes the keys held before, at most.
 int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) {
-    const DedupPlan &d = ip.dd;
-    const PartPlan &pp = ip.pp;
-    if (ip.ranges) {
-        KM_TRY(ensure(h, &h->range_a, &h->range_a_cap, d.keys_a()));
-        KM_TRY(ensure(h, &h->range_b, &h->range_b_cap, d.keys_b()));
-        KM_TRY(ensure(h, &h->mult, &h->mult_cap, d.mult_words()));
-        KM_TRY(ensure(h, &h->range_meta, &h->range_meta_cap, d.meta_bytes()));
-        if (pp.part) {
-            KM_TRY(ensure(h, &h->coarse, &h->coarse_alloc, pp.coarse_words()));
-            if (pp.repart) KM_TRY(ensure(h, &h->fine, &h->fine_alloc, pp.fine_words()));
-            KM_TRY(ensure(h, &h->part_ctr, &h->part_ctr_alloc, pp.ctr_words()));
-        }
-    }
+    if (ip.ranges) KM_TRY(ensure_scratch(h, ip));
     if (ip.merge) {
         const int st = ensure_union(h, ip.bound);
         if (st == KMERCO_ENOMEM)
@@ -913,6 +988,14 @@ int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) 
         h->d_ub += ip.bound;
     ip.sure = !ip.table() && ip.fresh && ip.passes == 1 &&
               ensure(h, &h->sure, &h->sure_cap, ip.bound) == KMERCO_OK;
+    if (ip.packed) {
+        h->scratch_busy = true;   // its buffers do not make room for each other
+        if (ensure_scratch(h, ip) != KMERCO_OK) {
+            ip.packed = h->scratch_busy = false;
+            ip.pp = PartPlan();
+            KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
+        }
+    }
     return KMERCO_OK;
 }
 
@@ -982,14 +1065,10 @@ int kmerco_estimate_bytes(const kmerco_config_t *cfg, uint64_t nreads, uint64_t 
         b += list * kw * 8 + grown(windows, 1);
         const InsertPlan ip = plan_insert(&t, windows, nbytes, true);
         if (ip.table()) b += table_bytes(&t, std::max<uint64_t>(2 * windows, 1024));
-        if (ip.ranges) {
-            b += grown(ip.dd.keys_a(), 8) + grown(ip.dd.keys_b(), 8) +
-                 grown(ip.dd.mult_words(), 4) + grown(ip.dd.meta_bytes(), 1);
-            if (ip.pp.part) {
-                b += grown(ip.pp.coarse_words(), 4) + grown(ip.pp.ctr_words(), 8);
-                if (ip.pp.repart) b += grown(ip.pp.fine_words(), 4);
-            }
-        }
+        const PlanScratch scratch(ip, t.kw);
+        const uint64_t elem[7] = {8, 8, 4, 1, 4, 4, 8};
+        for (int q = 0; q < 7; ++q)
+            if (scratch.n[q]) b += grown(scratch.n[q] / elem[q], elem[q]);
         const uint64_t chunk = ip.ranges ? (uint64_t)ip.dd.chunk : kSmallChunk;   // the most chunks
         b += grown((nbytes + chunk - 1) / chunk, 4);
         // classification of at most `windows` distinct keys
@@ -1230,6 +1309,7 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
         first = h->ctr_host->first;
         last = h->ctr_host->last;
         bound = h->ctr_host->bound;
+        h->d_ub = std::min<uint64_t>(h->d_ub, h->ctr_host->distinct);   // known by the way
     }
     if (h->whole_file)   // the reads are one sequence of last - first bases
         bound = last - first >= (uint64_t)K ? last - first - K + 1 : 0;
@@ -1260,9 +1340,9 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
         // window by window, which needs the list and the set alone (24 bytes a
         // window and key word instead of 34 and more)
         release_scratch(h);
-        ip = InsertPlan();
-        ip.bound = bound;
+        ip = plan_windows(h, bound, nbytes);
         st = secure_insert(h, ip, nbytes, held);
+        h->scratch_busy = false;
     }
     KM_TRY(st);
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
@@ -1966,13 +2046,8 @@ void batch_scratch(InsertBufs &f, void **ptrs[7]) {
 bool batch_alloc_scratch(kmerco_batch *b) {
     uint64_t need[7] = {0, 0, 0, 0, 0, 0, 0};
     for (const InsertPlan &ip : b->plans) {
-        if (!ip.ranges) continue;
-        const uint64_t n[7] = {ip.dd.keys_a() * 8, ip.dd.keys_b() * 8, ip.dd.mult_words() * 4,
-                               ip.dd.meta_bytes(),
-                               ip.pp.part ? ip.pp.coarse_words() * 4 : 0,
-                               ip.pp.part ? ip.pp.fine_words() * 4 : 0,
-                               ip.pp.part ? ip.pp.ctr_words() * 8 : 0};
-        for (int q = 0; q < 7; ++q) need[q] = std::max(need[q], n[q]);
+        const PlanScratch scratch(ip, b->kw);
+        for (int q = 0; q < 7; ++q) need[q] = std::max(need[q], scratch.n[q]);
     }
     for (int k = 0; k < kBatchStreams; ++k) {
         if (!b->aux[k] && cudaStreamCreateWithFlags(&b->aux[k], cudaStreamNonBlocking) != cudaSuccess)

@@ -1816,7 +1816,7 @@ __global__ void __launch_bounds__(kEmitThreads, 4) emit_kernel(EmitArgs e) {
             if (i < i1) {
                 const uint64_t at = e.ordered ? place_in(off, plc, i) : i;
                 key[q] = load_key<KW>(e.keys, at);
-                w[q] = (uint32_t)min((uint64_t)e.mult[at], G.maxc);
+                w[q] = e.mult ? (uint32_t)min((uint64_t)e.mult[at], G.maxc) : 1u;
                 if (e.dlist && i < e.dlist_cap) store_key<KW>(e.dlist, i, key[q]);
                 if (e.sure) e.sure[i] = w[q] > e.tau;
             }
@@ -2194,6 +2194,21 @@ DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk) {
     return p;
 }
 
+DedupPlan plan_pack(int K, uint64_t nbytes) {
+    DedupPlan p;
+    p.K = K;
+    p.kw = K <= 32 ? 1 : 2;
+    p.chunk = dedup_chunk(nbytes);
+    p.chunks = (nbytes + p.chunk - 1) / p.chunk;
+    return p;
+}
+
+Packed packed_input(const DedupPlan &p, const DedupBufs &d) {
+    const MetaLayout m(p);
+    return Packed{(const uint32_t *)(d.meta + m.codes), (const uint16_t *)(d.meta + m.valid),
+                  (DedupMeta *)(d.meta + m.meta)};
+}
+
 cudaError_t dedup_pack(const DedupPlan &p, const DedupBufs &d, const InsertArgs &a, uint64_t chunk0,
                        uint64_t n_chunks, uint64_t begin, uint64_t end, int sms, cudaStream_t s,
                        uint64_t &launches) {
@@ -2282,6 +2297,18 @@ EmitArgs dedup_result(const DedupPlan &p, const DedupBufs &d, const Geometry &G,
     e.end = ~0u;
     e.ctr = ctr;
     e.meta = (const DedupMeta *)(d.meta + m.meta);
+    return e;
+}
+
+EmitArgs windows_result(const uint64_t *keys, const DedupMeta *meta, const Geometry &G,
+                        DevCounters *ctr) {
+    EmitArgs e;
+    memset(&e, 0, sizeof(e));
+    e.G = G;
+    e.keys = keys;
+    e.end = ~0u;
+    e.ctr = ctr;
+    e.meta = meta;
     return e;
 }
 

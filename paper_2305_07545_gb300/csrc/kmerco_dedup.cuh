@@ -99,7 +99,7 @@ struct DedupArgs {
 struct EmitArgs {
     Geometry G;
     const uint64_t *keys;
-    const uint32_t *mult, *places, *offsets;
+    const uint32_t *mult, *places, *offsets;   // mult null: each key once
     unsigned n_total;        // ranges
     int ordered;             // keys in the order of the ranges (places, offsets), else as they stand
     unsigned begin, end;     // distinct keys of this pass
@@ -148,6 +148,16 @@ int dedup_chunk(uint64_t nbytes);
 // that is more than one pass takes.
 DedupPlan plan_dedup(int K, uint64_t bound, uint64_t chunks, int chunk);
 
+// A call that is only packed (kmerco_insert.cu then takes its windows one by one).
+DedupPlan plan_pack(int K, uint64_t nbytes);
+// Where the packed input and the pass's counts are.
+struct Packed {
+    const uint32_t *codes;
+    const uint16_t *valid;
+    DedupMeta *meta;
+};
+Packed packed_input(const DedupPlan &p, const DedupBufs &d);
+
 // The pass over n_chunks chunks from chunk0 on: first its bases are packed,
 // chunk range [begin, end) by chunk range (nothing reads the caller's buffers
 // after these); then the windows' keys are cut into ranges (span: bases of the
@@ -166,6 +176,9 @@ cudaError_t dedup_finish(const DedupPlan &p, const DedupBufs &d, DevCounters *ct
 // ordered, e.keys holds them one after the other in no order, e.meta->out_cursor of them.
 EmitArgs dedup_result(const DedupPlan &p, const DedupBufs &d, const Geometry &G, DevCounters *ctr,
                       bool ordered);
+// n keys of one window each, in no order, their number in meta->out_cursor.
+EmitArgs windows_result(const uint64_t *keys, const DedupMeta *meta, const Geometry &G,
+                        DevCounters *ctr);
 cudaError_t launch_emit(const EmitArgs &e, int kw, int sms, cudaStream_t s);
 cudaError_t launch_emit_atomic(const EmitArgs &e, int kw, int sms, cudaStream_t s);
 

@@ -7,8 +7,8 @@
 //    kernels that apply those in the partitioned update are here
 //    (repartition_kernel, apply_count_kernel, apply_kernel);
 //  - window by window (insert_kernel, insert_batch_kernel here): for small
-//    calls, handles with a retry limit or a cap on their distinct list, and
-//    when the buffers of the first way cannot be had.
+//    calls, handles with a small retry limit, and when the buffers of the
+//    first way cannot be had.
 //
 // insert_kernel: a work unit is a chunk of consecutive window starts of the
 // flat bases array, regardless of read boundaries, so long and short reads
@@ -24,9 +24,13 @@
 //      into the distinct-key set (open addressing, linear probing); keys new
 //      to the set are staged in shared memory and appended to the distinct
 //      list with one global atomic per chunk.
+// Larger calls have their input packed first (pack_kernel): steps 1 and 2 read codes
+// and window bits, and the caller's buffers are read within microseconds.  For the
+// partitioned update the counters are left out and the windows' keys written to
+// memory instead: pieces of 2.5e6 windows into 2^18 cells then take 238 us each
+// with their increments, 282 with a compare-and-swap per window and hash.
 //
-// Partitioned update of the first way (at most 2^30 cells): emit_kernel has
-// appended the increments as 32-bit codes to 64 coarse countBF regions;
+// Partitioned update (at most 2^30 cells): emit_kernel has appended the increments as 32-bit codes to 64 coarse countBF regions;
 // repartition_kernel splits every region into slices, and one block per
 // slice applies its increments in shared memory: apply_count_kernel
 // (alpha <= 15) sums them in 32-bit lanes and adds the sums with saturation
@@ -47,6 +51,7 @@ struct __align__(16) InsertSmem {
     uint64_t fresh[CHUNK * KW];                 // keys new to the distinct set
     unsigned nvalid;
     unsigned nfresh;
+    unsigned staged_base;
     unsigned long long fresh_base;
 };
 
@@ -176,7 +181,7 @@ __device__ __forceinline__ bool set_insert(uint64_t *table, uint64_t cap, uint64
 
 // One chunk of CHUNK window starts (the steps above) for the sample
 // described by `a`; counts its windows into my_windows / my_skipped.
-template <int KW, int CHUNK>
+template <int KW, int CHUNK, bool PACKED = false, bool STAGED = false>
 __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chunk,
                                               InsertSmem<KW, CHUNK> &S, uint64_t pol_keep,
                                               uint64_t pol_stream,
@@ -186,7 +191,13 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = a.K;
     const Geometry &G = a.G;
-    const unsigned nb = stage_chunk<CHUNK, kInsertThreads>(a, chunk, S.st);
+    unsigned nb = 0;
+    if (PACKED) {
+        const uint32_t *codes = a.codes + chunk * (CHUNK / 16);
+        for (int i = tid; i < kPack32; i += kInsertThreads) S.st.pk[i] = codes[i];
+    } else {
+        nb = stage_chunk<CHUNK, kInsertThreads>(a, chunk, S.st);
+    }
     if (tid == 0) {
         S.nvalid = 0;
         S.nfresh = 0;
@@ -200,10 +211,15 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
     const uint64_t maskK1 = (1ull << (K - 1)) - 1;
     for (int p0 = 0; p0 < CHUNK; p0 += kInsertThreads) {
         unsigned p = (unsigned)(p0 + tid);
-        bool window = p + (unsigned)K <= nb && (bits_at(brk64, p + 1) & maskK1) == 0;
-        bool valid = window && (bits_at(inv64, p) & maskK) == 0;
-        my_windows += window;
-        my_skipped += window && !valid;
+        bool valid;
+        if (PACKED) {   // the windows were counted when they were packed
+            valid = (a.valid[chunk * (CHUNK / 16) + (p >> 4)] >> (p & 15)) & 1u;
+        } else {
+            const bool window = p + (unsigned)K <= nb && (bits_at(brk64, p + 1) & maskK1) == 0;
+            valid = window && (bits_at(inv64, p) & maskK) == 0;
+            my_windows += window;
+            my_skipped += window && !valid;
+        }
         unsigned bal = __ballot_sync(0xffffffffu, valid);
         unsigned base = 0;
         if (lane == 0 && bal) base = atomicAdd(&S.nvalid, (unsigned)__popc(bal));
@@ -213,8 +229,13 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
     __syncthreads();
 
     // per valid window: canonical key, hashes, counter updates, set insert
-    for (int i = tid; i < kPack32 / 2; i += kInsertThreads) S.st.brk[i] = 0;   // for the next chunk
+    for (int i = tid; !PACKED && i < kPack32 / 2; i += kInsertThreads)
+        S.st.brk[i] = 0;   // for the next chunk
     const unsigned nvalid = S.nvalid;
+    if (STAGED) {
+        if (tid == 0 && nvalid) S.staged_base = atomicAdd(a.n_staged, nvalid);
+        __syncthreads();
+    }
     const uint64_t *pk64 = (const uint64_t *)S.st.pk;
     for (unsigned i0 = (unsigned)warp * 32; i0 < nvalid; i0 += kInsertThreads) {
         const unsigned i = i0 + lane;
@@ -274,10 +295,22 @@ __device__ __forceinline__ void process_chunk(const InsertArgs &a, uint64_t chun
 
         uint64_t table_hash = 0, table_first = kEmptyKey - 1;
         const uint64_t k1m = KW == 1 ? premix8(klo) : 0;
+        if (STAGED && active) {
+            const uint64_t at = (uint64_t)S.staged_base + i;
+            uint64_t h1;
+            if (KW == 1) {
+                __stcs((unsigned long long *)a.staged + at, (unsigned long long)klo);
+                murmur8(k1m, 0u, h1, table_hash);
+                table_first = load_hint(a.table + __umul64hi(table_hash, a.cap), pol_stream);
+            } else {
+                __stcs((ulonglong2 *)a.staged + at, make_ulonglong2(klo, khi));
+                murmur16(klo, khi, 0u, h1, table_hash);
+            }
+        }
         // All loads of a group of four hashes (and, in the first group, the
         // distinct-set home slot) are issued together, then all first
         // compare-and-swap attempts; only failed attempts retry.
-        for (int a0 = 0; a0 < G.nhash; a0 += 4) {
+        for (int a0 = 0; !STAGED && a0 < G.nhash; a0 += 4) {
             uint64_t cell[4], cur[4], prev[4];
             unsigned sh[4], slot[4];
             bool use[4], need[4];
@@ -372,7 +405,7 @@ __device__ __forceinline__ void flush_totals(DevCounters *ctr, unsigned long lon
     k = 0;
 }
 
-template <int KW, int CHUNK>
+template <int KW, int CHUNK, bool PACKED, bool STAGED>
 __global__ void __launch_bounds__(kInsertThreads, 4) insert_kernel(InsertArgs a) {
     __shared__ InsertSmem<KW, CHUNK> S;
     for (int i = threadIdx.x; i < ChunkDims<CHUNK>::kPack32 / 2; i += kInsertThreads) S.st.brk[i] = 0;
@@ -380,8 +413,9 @@ __global__ void __launch_bounds__(kInsertThreads, 4) insert_kernel(InsertArgs a)
     const uint64_t pol_keep = policy_keep(), pol_stream = policy_stream();
     unsigned long long my_windows = 0, my_skipped = 0;
     for (uint64_t chunk = a.chunk_begin + blockIdx.x; chunk < a.nchunks; chunk += gridDim.x)
-        process_chunk<KW, CHUNK>(a, chunk, S, pol_keep, pol_stream, my_windows, my_skipped);
-    flush_totals(a.ctr, my_windows, my_skipped);
+        process_chunk<KW, CHUNK, PACKED, STAGED>(a, chunk, S, pol_keep, pol_stream, my_windows,
+                                                 my_skipped);
+    if (!PACKED) flush_totals(a.ctr, my_windows, my_skipped);
 }
 
 // Many samples in one persistent launch (atomic update design): the chunks
@@ -950,9 +984,9 @@ __global__ void __launch_bounds__(kApplyThreads, 2) apply_count_kernel(ApplyArgs
 int insert_blocks_per_sm(int kw) {
     int n = 0;
     const cudaError_t e =
-        kw == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<1, kChunk>,
+        kw == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<1, kChunk, false, false>,
                                                                 kInsertThreads, 0)
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<2, kChunk>,
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, insert_kernel<2, kChunk, false, false>,
                                                                 kInsertThreads, 0);
     return e == cudaSuccess && n > 0 ? n : 1;
 }
@@ -1069,15 +1103,22 @@ cudaError_t launch_apply_count(const ApplyArgs &p, uint64_t nslices, cudaStream_
     return cudaGetLastError();
 }
 
+template <bool PACKED, bool STAGED>
+auto insert_variant(int K, int chunk) -> void (*)(InsertArgs) {
+    if (K <= 32)
+        return chunk == kChunk ? insert_kernel<1, kChunk, PACKED, STAGED>
+                               : insert_kernel<1, kSmallChunk, PACKED, STAGED>;
+    return chunk == kChunk ? insert_kernel<2, kChunk, PACKED, STAGED>
+                           : insert_kernel<2, kSmallChunk, PACKED, STAGED>;
+}
+
 cudaError_t launch_insert(const InsertArgs &a, int grid, int chunk, cudaStream_t s) {
     if (a.nchunks <= a.chunk_begin) return cudaSuccess;
     const uint64_t n = a.nchunks - a.chunk_begin;
     const unsigned g = (unsigned)(n < (uint64_t)grid ? n : (uint64_t)grid);
     if (chunk != kChunk && chunk != kSmallChunk) return cudaErrorInvalidValue;
-    void (*k)(InsertArgs) = a.K <= 32 ? (chunk == kChunk ? insert_kernel<1, kChunk>
-                                                         : insert_kernel<1, kSmallChunk>)
-                                      : (chunk == kChunk ? insert_kernel<2, kChunk>
-                                                         : insert_kernel<2, kSmallChunk>);
+    auto *k = !a.codes   ? insert_variant<false, false>(a.K, chunk)
+              : a.staged ? insert_variant<true, true>(a.K, chunk) : insert_variant<true, false>(a.K, chunk);
     k<<<g, kInsertThreads, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -323,6 +323,10 @@ struct InsertArgs {
     SetTag set_tag;              // current generation of the set
     uint64_t *dlist;             // distinct keys in arrival order
     uint64_t dlist_cap;
+    const uint32_t *codes;       // launch_insert: the packed input (PackArgs); null: its bases
+    const uint16_t *valid;
+    uint64_t *staged;            // with codes: receives every window's key in no order, and
+    unsigned *n_staged;          // their number; no counter is updated then (null: updated here)
     DevCounters *ctr;
 };
 
