@@ -26,11 +26,9 @@ constexpr uint64_t kHostBoundReads = 1ull << 16;
 
 // Windows from which an insert call goes by key ranges: below, its dozen
 // launches cost more than the window-by-window kernel takes.  A call into a
-// handle that holds keys has to merge its keys with those too: eight pieces of
-// 2.5e6 windows take 3.9 ms by ranges and 3.3 window by window, of 5e6 6.3 and 5.9
-// when nearly all windows differ, 3.5 and 4.1 when they are five times as many.
+// handle that holds keys has to merge its keys with those too.
 constexpr uint64_t kRangesMin = 1ull << 14;
-constexpr uint64_t kRangesMinMore = 1ull << 22;
+constexpr uint64_t kRangesMinMore = 1ull << 17;
 // Windows from which a call that goes window by window is packed first.
 constexpr uint64_t kPackMin = 1ull << 16;
 // Windows up to which a further call whose keys are not merged into an ordered list
@@ -82,6 +80,9 @@ struct kmerco {
     uint64_t *dlist2;        // the list's other place: a union is written there
     uint64_t dlist2_cap;
     uint64_t d_ub;           // upper bound of the distinct keys held
+    uint64_t *pend, *pend2;  // ascending keys of the last calls, not merged into the list yet
+    uint64_t pend_cap, pend2_cap;   // (two buffers take turns), and at most how many
+    uint64_t pend_ub;
     uint8_t *in_bases;       // staging of host inputs
     uint64_t in_bases_cap;
     uint64_t *in_offsets;
@@ -233,8 +234,12 @@ void release_scratch(kmerco_t *h) {
     give_back(&h->coarse, &h->coarse_alloc, 4);
     give_back(&h->fine, &h->fine_alloc, 4);
     give_back(&h->part_ctr, &h->part_ctr_alloc, 8);
-    give_back(&h->dlist2, &h->dlist2_cap, (uint64_t)h->kw * 8);
-    give_back(&h->union_scratch, &h->union_scratch_cap, 4);
+    give_back(&h->pend2, &h->pend2_cap, (uint64_t)h->kw * 8);
+    if (!h->pend_ub) {   // else what merges them stays too
+        give_back(&h->pend, &h->pend_cap, (uint64_t)h->kw * 8);
+        give_back(&h->dlist2, &h->dlist2_cap, (uint64_t)h->kw * 8);
+        give_back(&h->union_scratch, &h->union_scratch_cap, 4);
+    }
     give_back(&h->sure, &h->sure_cap, 1);
     h->sure_ok = false;
 }
@@ -372,7 +377,7 @@ int clean_table(kmerco_t *h) {
 // distinct set over all keys held, at a load factor of 1/2 at most for every
 // key the next launch could add: cap >= 2 * (distinct so far + new windows).
 // The set is built when a call first needs it: an insert by key ranges into an
-// empty handle writes the list alone.
+// empty handle writes the list alone.  Nothing is pending.
 int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
     uint64_t need = h->d_ub + add;
     const bool grow_table = want_table && 2 * need > h->cap;
@@ -430,39 +435,72 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
     return KMERCO_OK;
 }
 
-// Calls of at least this share of the keys already held (bounds of both, where the
-// counts are not known) are merged into the ordered list: a union takes about 13 ps
-// for every key held or new.  By ranges a call is 50 ps a window quicker than window by
-// window, but a handle that goes over to its set later has to build it from the
-// list, 36 ps a key: with four the sum is about even however many pieces come
-// (six pieces of 1e7 windows 8.1 ms, 8.7 all window by window; three 3.5 and 4.2).
-constexpr uint64_t kMergeShare = 4;
+// Whether a call of at most `bound` windows is merged into the ordered list of `held`
+// keys at most.  By ranges a call is the quicker the larger it is and the more
+// often its keys come; window by window it costs no union, but the set has to be
+// built from the list first, 75 ps a key, and the keys sorted again at the end.  So large
+// calls are merged however many come, smaller ones only into a list of about their
+// own length (two calls of 1.3e6 windows 0.65 ms, 0.77 window by window; twelve of
+// 1.2e6 3.2 and 4.8 when more are merged).
+bool merges(uint64_t bound, uint64_t held) {
+    return bound >= (1ull << 21) ? bound * 32 >= held : bound * 3 >= held * 2;
+}
+// The share of the keys held from which another handle's list is merged with them.
+constexpr uint64_t kUnionShare = 4;
 
-// Room for the union of the list and at most `add` more keys.
+// A union takes about 13 ps for every key held or new, so a long list is not merged with
+// every small call: the call's keys join those pending, which are merged into the
+// list when they are as many calls' as the list is times theirs.  P equal calls are
+// then P^1.5 calls' keys of unions, not P^2 / 2 (sixteen of 1e7 windows, nearly all
+// different, 24.9 ms, 26.2 merged each; 28 with five times as many windows as keys 23.7
+// and 30.6).
+bool pending_full(uint64_t list, uint64_t pending, uint64_t call) {
+    return (double)pending * (double)pending >= (double)list * (double)call;
+}
+
+// The bounds of what is held, when the counters have just been read.
+void know_counts(kmerco_t *h) {
+    const uint64_t list = std::min<uint64_t>(h->d_ub - h->pend_ub, h->ctr_host->distinct);
+    h->pend_ub = std::min<uint64_t>(h->pend_ub, h->ctr_host->pending);
+    h->d_ub = list + h->pend_ub;
+}
+
+// Room for the union of what is held and at most `add` more keys.
 int ensure_union(kmerco_t *h, uint64_t add) {
     // a bound of what is held will do while the list is small; for a large one the
     // call waits to learn its length
     if (h->d_ub && h->d_ub + add > h->dlist2_cap && (h->d_ub + add) * h->kw > (1ull << 28)) {
         KM_TRY(read_counters(h));
-        h->d_ub = h->ctr_host->distinct;
+        know_counts(h);
     }
     KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub + add, (uint64_t)h->kw * 8));
     // several passes: each one's list into what is held by then
     return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub + add, add));
 }
 
-// Merges an ascending list of *nb32 or *nb64 keys, at most nb_most, into the
-// handle's ascending list (after ensure_union).
-int merge_keys(kmerco_t *h, const uint64_t *keys, uint64_t nb_most, const unsigned *nb32,
-               const unsigned long long *nb64) {
-    KM_CUDA(launch_union(h->dlist, h->d_ub, keys, nb_most, nb32, nb64, h->kw, h->dlist2,
+// Merges an ascending list of *count keys, at most nb_most, into the handle's ascending
+// list, which has na_most at most (after ensure_union).
+int merge_keys(kmerco_t *h, uint64_t na_most, const uint64_t *keys, uint64_t nb_most,
+               const unsigned long long *count) {
+    KM_CUDA(launch_union(h->dlist, na_most, keys, nb_most, nullptr, count, h->kw, h->dlist2,
                          h->union_scratch, &h->ctr->distinct, h->stream));
     h->launches += 4;
     std::swap(h->dlist, h->dlist2);
     std::swap(h->dlist_cap, h->dlist2_cap);
-    h->d_ub += nb_most;
     h->table_ok = h->sure_ok = false;
     h->list_sorted = true;
+    return KMERCO_OK;
+}
+
+// Merges the keys pending into the list: for whatever reads or extends the list itself.
+int merge_pending(kmerco_t *h) {
+    if (!h->pend_ub) return KMERCO_OK;
+    const uint64_t list = h->d_ub - h->pend_ub;
+    KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub, (uint64_t)h->kw * 8));
+    KM_TRY(ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(list, h->pend_ub)));
+    KM_TRY(merge_keys(h, list, h->pend, h->pend_ub, &h->ctr->pending));
+    KM_CUDA(cudaMemsetAsync(&h->ctr->pending, 0, sizeof(h->ctr->pending), h->stream));
+    h->pend_ub = 0;
     return KMERCO_OK;
 }
 
@@ -577,6 +615,8 @@ struct InsertPlan {
     bool sure = false;       // the list is the call's keys: which are sure is written too
     bool merge = false;      // the list stays in order: every pass's keys but the ones that
                              // begin a list are merged into it
+    bool pend = false;       // into the pending list instead; full: which then goes into
+    bool full = false;       // the list
     uint64_t passes = 1;
     uint64_t bound = 0;      // windows of the call at most
     DedupPlan dd;
@@ -620,6 +660,7 @@ struct InsertBufs {
     uint64_t *list, *list2;
     unsigned *union_scratch;
     uint64_t held;
+    unsigned long long *count;   // of the list's keys
 };
 
 // Increment-code buffers sized for one pass of at most pass_codes increments,
@@ -677,7 +718,7 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     InsertPlan ip = plan_windows(h, bound, nbytes);
     // (a list with a cap keeps to its buffer)
     const bool merge = may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull;
-    const bool into_list = merge && h->list_sorted && bound * kMergeShare >= h->d_ub;
+    const bool into_list = merge && h->list_sorted && merges(bound, h->d_ub);
     if (bound < (fresh ? kRangesMin : kRangesMinMore) ||
         (!fresh && !into_list && bound <= kWindowsMost) || h->G.cas_limit < kRangesRetries ||
         nbytes < bound)
@@ -930,15 +971,19 @@ int launch_sample_insert(const kmerco_t *h, InsertArgs a, const InsertPlan &ip,
         KM_CUDA(dedup_finish(ip.dd, b.dd, h->ctr, ce - cb, ordered, fresh, h->dlist_cap, h->sms, s,
                              launches));
         EmitArgs e = dedup_result(ip.dd, b.dd, h->G, h->ctr, ordered);
-        e.dlist = fresh ? h->dlist : ip.merge ? merge_input(ip, b) : nullptr;
+        const bool first_pending = ip.pend && !b.held;
+        e.dlist = fresh ? h->dlist : first_pending ? list : ip.merge ? merge_input(ip, b) : nullptr;
         e.dlist_cap = fresh ? h->dlist_cap : ~0ull;
         e.sure = fresh && ip.sure ? h->sure : nullptr;
         e.tau = h->tau;
         KM_TRY(launch_updates(h, ip, b, e, s, launches));
-        if (ip.merge && !fresh) {
+        if (first_pending) {
+            KM_CUDA(cudaMemcpyAsync(b.count, &e.meta->distinct, sizeof(e.meta->distinct),
+                                    cudaMemcpyDeviceToDevice, s));   // its upper half is zero
+        } else if (ip.merge && !fresh) {
             const uint64_t before = std::min(b.held + pass * ip.dd.bound, b.held + ip.bound);
             KM_CUDA(launch_union(list, before, e.dlist, ip.dd.bound, &e.meta->distinct, nullptr,
-                                 h->kw, list2, b.union_scratch, &h->ctr->distinct, s));
+                                 h->kw, list2, b.union_scratch, b.count, s));
             launches += 4;
             std::swap(list, list2);
         }
@@ -969,7 +1014,8 @@ int ensure_scratch(kmerco_t *h, const InsertPlan &ip) {
 
 // The buffers of a plan from the handle's: the ranges' scratch, the list, the set
 // or the union's buffers, first reads; then the scratch of packed windows, without
-// which they are counted from the bases.  `held` becomes the keys held before, at most.
+// which they are counted from the bases.  `held` becomes the keys that a merged call
+// meets, at most.
 int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) {
     if (ip.ranges) KM_TRY(ensure_scratch(h, ip));
     if (ip.merge) {
@@ -979,7 +1025,16 @@ int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) 
         else
             KM_TRY(st);
     }
-    held = h->d_ub;
+    if (ip.merge && ip.passes == 1) {
+        const uint64_t pending = h->pend_ub + ip.bound;
+        ip.full = pending_full(h->d_ub - h->pend_ub, pending, ip.bound);
+        uint64_t **to = h->pend_ub ? &h->pend2 : &h->pend;   // the first keys pending as they come
+        ip.pend = (h->pend_ub || !ip.full) &&
+                  ensure(h, to, h->pend_ub ? &h->pend2_cap : &h->pend_cap, pending,
+                         (uint64_t)h->kw * 8) == KMERCO_OK;
+    }
+    if (!ip.pend) KM_TRY(merge_pending(h));
+    held = ip.pend ? h->pend_ub : h->d_ub;
     KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
     // a call merged once writes its list into the other buffer alone
     if (!ip.merge || ip.passes > 1)
@@ -1200,6 +1255,8 @@ void kmerco_destroy(kmerco_t *h) {
         dev_free(h, h->table, table_bytes(h, h->cap));
         dev_free(h, h->dlist, h->dlist_cap * h->kw * 8);
         dev_free(h, h->dlist2, h->dlist2_cap * h->kw * 8);
+        dev_free(h, h->pend, h->pend_cap * h->kw * 8);
+        dev_free(h, h->pend2, h->pend2_cap * h->kw * 8);
         dev_free(h, h->union_scratch, h->union_scratch_cap * 4);
         dev_free(h, h->sure, h->sure_cap);
         dev_free(h, h->in_bases, h->in_bases_cap);
@@ -1247,7 +1304,7 @@ int kmerco_reset(kmerco_t *h) {
     KM_CUDA(cudaMemsetAsync(h->G.cells, 0, h->G.words * 8, h->stream));
     KM_TRY(clean_table(h));
     KM_CUDA(cudaMemsetAsync(h->ctr, 0, sizeof(DevCounters), h->stream));
-    h->d_ub = 0;
+    h->d_ub = h->pend_ub = 0;
     h->table_ok = true;
     h->list_sorted = h->sure_ok = false;
     h->classified = false;
@@ -1309,7 +1366,7 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
         first = h->ctr_host->first;
         last = h->ctr_host->last;
         bound = h->ctr_host->bound;
-        h->d_ub = std::min<uint64_t>(h->d_ub, h->ctr_host->distinct);   // known by the way
+        know_counts(h);
     }
     if (h->whole_file)   // the reads are one sequence of last - first bases
         bound = last - first >= (uint64_t)K ? last - first - K + 1 : 0;
@@ -1347,11 +1404,20 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
     KM_TRY(st);
     const InsertArgs a = sample_args(h, d_bases, d_off, nreads, first, last);
     const InsertBufs bufs = {{h->range_a, h->range_b, h->mult, h->range_meta}, h->coarse, h->fine,
-                             h->part_ctr, h->dlist, h->dlist2, h->union_scratch, held};
+                             h->part_ctr, ip.pend ? h->pend : h->dlist,
+                             ip.pend ? h->pend2 : h->dlist2, h->union_scratch, held,
+                             ip.pend ? &h->ctr->pending : &h->ctr->distinct};
     KM_CUDA(cudaEventRecord(h->ev[0], h->stream));
     KM_TRY(launch_sample_insert(h, a, ip, bufs, h->stream, h->launches, copying ? &hc : nullptr,
                                 copying || host_offsets ? h->input_read : nullptr));
-    if (ip.merges() & 1) {
+    if (ip.pend) {
+        if (held) {
+            std::swap(h->pend, h->pend2);
+            std::swap(h->pend_cap, h->pend2_cap);
+        }
+        h->pend_ub += ip.bound;
+        if (ip.full) KM_TRY(merge_pending(h));
+    } else if (ip.merges() & 1) {
         std::swap(h->dlist, h->dlist2);
         std::swap(h->dlist_cap, h->dlist2_cap);
     }
@@ -1414,6 +1480,7 @@ int kmerco_classify(kmerco_t *h) {
     if (!h) return KMERCO_EINVAL;
     if (h->classified) return KMERCO_OK;
     DeviceGuard guard(h->device);
+    KM_TRY(merge_pending(h));
     KM_TRY(read_counters(h));
     KM_TRY(device_error_status(h->ctr_host->error));
     const uint64_t D = h->ctr_host->distinct;
@@ -1564,6 +1631,7 @@ sorted_done:
 int kmerco_stats(kmerco_t *h, kmerco_stats_t *s) {
     if (!h || !s) return KMERCO_EINVAL;
     DeviceGuard guard(h->device);
+    KM_TRY(merge_pending(h));   // the totals count every key once
     KM_CUDA(launch_count_saturated(h->G, h->ctr, h->stream));
     h->launches += 1;
     KM_TRY(read_counters(h));
@@ -1654,6 +1722,7 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
         KM_CUDA(cudaMemcpyAsync(*stage, keys, words * 8, cudaMemcpyHostToDevice, h->stream));
         d_keys = *stage;
     }
+    KM_TRY(merge_pending(h));
     KM_TRY(ensure_set_capacity(h, n, true));
     KM_CUDA(launch_reinsert(d_keys, n, nullptr, nullptr, h->kw, h->table, h->cap, set_tag(h),
                             h->dlist, h->dlist_cap, h->ctr, h->G.probe_limit, h->stream));
@@ -1851,6 +1920,8 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
         dst->nhash != src->nhash || dst->canonical != src->canonical || dst->device != src->device)
         return KMERCO_EINVAL;
     DeviceGuard guard(dst->device);
+    KM_TRY(merge_pending(src));
+    KM_TRY(merge_pending(dst));
     KM_TRY(read_counters(src));
     KM_TRY(device_error_status(src->ctr_host->error));
     const DevCounters sc = *src->ctr_host;
@@ -1867,12 +1938,13 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
                                 cudaMemcpyDeviceToDevice, dst->stream));
         dst->table_ok = false;
         listed = dst->list_sorted = true;
-    } else if (ordered && dst->list_sorted && sc.distinct * kMergeShare >= dst->d_ub &&
+    } else if (ordered && dst->list_sorted && sc.distinct * kUnionShare >= dst->d_ub &&
                dst->d_ub + sc.distinct < 0xFFFFFFFFull) {
         const int st = ensure_union(dst, sc.distinct);
         if (st != KMERCO_ENOMEM) {
             KM_TRY(st);
-            KM_TRY(merge_keys(dst, src->dlist, sc.distinct, nullptr, &src->ctr->distinct));
+            KM_TRY(merge_keys(dst, dst->d_ub, src->dlist, sc.distinct, &src->ctr->distinct));
+            dst->d_ub += sc.distinct;
             listed = true;
         }
     }
@@ -2123,6 +2195,7 @@ void batch_mark_inserted(kmerco_batch *b) {
         h->n_distinct = h->n_trusted = 0;
         h->insert_timed = h->classify_timed = false;
         h->d_ub = std::max(h->d_ub, b->load[i]);
+        h->pend_ub = 0;   // merged before, or reset with the rest
         h->sure_ok = false;
         if (b->sched == 1 && !b->plans[i].table()) {   // the list alone was written, in order
             h->table_ok = false;
@@ -2277,6 +2350,7 @@ int kmerco_batch_insert(kmerco_batch_t *b, const char *const *bases,
     for (int i = 0; i < b->n; ++i) {
         kmerco_t *h = b->h[i];
         if (reset) KM_TRY(kmerco_reset(h));
+        KM_TRY(merge_pending(h));
         const unsigned long long *bo = &b->bound_host[(size_t)i * kBoundOutWords];
         uint64_t bound = bo[0];
         if (h->whole_file)   // the sample's reads are one sequence
@@ -2394,6 +2468,7 @@ int kmerco_batch_classify(kmerco_batch_t *b) {
     Range range("kmerco_batch_classify");
     if (!b) return KMERCO_EINVAL;
     DeviceGuard guard(b->device);
+    for (kmerco_t *h : b->h) KM_TRY(merge_pending(h));
     // one readback of every sample's totals
     for (kmerco_t *h : b->h)
         KM_CUDA(cudaMemcpyAsync(h->ctr_host, h->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost,

@@ -57,6 +57,7 @@ struct DevCounters {
     unsigned long long skipped;
     unsigned long long inserted;
     unsigned long long distinct;    // keys appended to the distinct list
+    unsigned long long pending;     // keys of the handle's pending list
     unsigned long long trusted;     // written by classify
     unsigned long long bound;       // window upper bound of the last batch
     unsigned long long first;       // offsets[0] of the last batch
