@@ -29,6 +29,9 @@ constexpr uint64_t kHostBoundReads = 1ull << 16;
 // handle that holds keys has to merge its keys with those too.
 constexpr uint64_t kRangesMin = 1ull << 14;
 constexpr uint64_t kRangesMinMore = 1ull << 17;
+// Windows from which a call that goes window by window sets an ordered list aside,
+// instead of building the set from it.
+constexpr uint64_t kAsideMin = 1ull << 17;
 // Windows from which a call that goes window by window is packed first.
 constexpr uint64_t kPackMin = 1ull << 16;
 // Windows up to which a further call whose keys are not merged into an ordered list
@@ -80,9 +83,11 @@ struct kmerco {
     uint64_t *dlist2;        // the list's other place: a union is written there
     uint64_t dlist2_cap;
     uint64_t d_ub;           // upper bound of the distinct keys held
-    uint64_t *pend, *pend2;  // ascending keys of the last calls, not merged into the list yet
-    uint64_t pend_cap, pend2_cap;   // (two buffers take turns), and at most how many
-    uint64_t pend_ub;
+    uint64_t *pend, *pend2;  // ascending keys not merged into the list yet (two buffers
+    uint64_t pend_cap, pend2_cap;   // take turns), and at most how many: those of the
+    uint64_t pend_ub;        // last calls beside an ordered list, or of the first ones
+                             // beside an unordered list with a set of its own
+    bool polled;             // totals were asked for between calls with keys pending
     uint8_t *in_bases;       // staging of host inputs
     uint64_t in_bases_cap;
     uint64_t *in_offsets;
@@ -377,11 +382,11 @@ int clean_table(kmerco_t *h) {
 // distinct set over all keys held, at a load factor of 1/2 at most for every
 // key the next launch could add: cap >= 2 * (distinct so far + new windows).
 // The set is built when a call first needs it: an insert by key ranges into an
-// empty handle writes the list alone.  Nothing is pending.
+// empty handle writes the list alone.
 int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
-    uint64_t need = h->d_ub + add;
+    uint64_t D = h->d_ub - h->pend_ub;   // 0: nothing inserted since create or reset
+    uint64_t need = D + add;
     const bool grow_table = want_table && 2 * need > h->cap;
-    uint64_t D = h->d_ub;   // 0: nothing inserted since create or reset
     if (D && (need > h->dlist_cap || grow_table)) {
         KM_TRY(read_counters(h));
         D = h->ctr_host->distinct;
@@ -431,19 +436,20 @@ int ensure_set_capacity(kmerco_t *h, uint64_t add, bool want_table) {
         h->table_ok = true;
     }
     if (want_table) h->table_dirty = true;
-    h->d_ub = need;
+    h->d_ub = need + h->pend_ub;
     return KMERCO_OK;
 }
 
 // Whether a call of at most `bound` windows is merged into the ordered list of `held`
-// keys at most.  By ranges a call is the quicker the larger it is and the more
-// often its keys come; window by window it costs no union, but the set has to be
-// built from the list first, 75 ps a key, and the keys sorted again at the end.  So large
-// calls are merged however many come, smaller ones only into a list of about their
-// own length (two calls of 1.3e6 windows 0.65 ms, 0.77 window by window; twelve of
-// 1.2e6 3.2 and 4.8 when more are merged).
-bool merges(uint64_t bound, uint64_t held) {
-    return bound >= (1ull << 21) ? bound * 32 >= held : bound * 3 >= held * 2;
+// keys at most.  By ranges a call is the quicker the larger it is and the more often
+// its keys come (1e7 windows: 50 ps a window); window by window it needs no union.
+// So large calls are merged however many come, smaller ones only into a list of about
+// their own length, of two-word keys of some calls': two calls of 1.3e6 windows 0.65
+// ms, 0.77 window by window; 15 of 3.5e6 6.0 ms and 7.5 all merged; three of 1.3e6
+// 55-mers 1.23 and 1.54.
+bool merges(int kw, uint64_t bound, uint64_t held) {
+    if (bound >= (1ull << 23)) return bound * 32 >= held;
+    return kw == 2 && bound >= (1ull << 20) ? bound * 7 >= held * 2 : bound * 3 >= held * 2;
 }
 // The share of the keys held from which another handle's list is merged with them.
 constexpr uint64_t kUnionShare = 4;
@@ -478,11 +484,11 @@ int ensure_union(kmerco_t *h, uint64_t add) {
     return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub + add, add));
 }
 
-// Merges an ascending list of *count keys, at most nb_most, into the handle's ascending
-// list, which has na_most at most (after ensure_union).
-int merge_keys(kmerco_t *h, uint64_t na_most, const uint64_t *keys, uint64_t nb_most,
-               const unsigned long long *count) {
-    KM_CUDA(launch_union(h->dlist, na_most, keys, nb_most, nullptr, count, h->kw, h->dlist2,
+// Merges an ascending list of *count keys, at most nb_most, into the handle's list,
+// which is ascending in `list` and has na_most at most (after ensure_union).
+int merge_keys(kmerco_t *h, const uint64_t *list, uint64_t na_most, const uint64_t *keys,
+               uint64_t nb_most, const unsigned long long *count) {
+    KM_CUDA(launch_union(list, na_most, keys, nb_most, nullptr, count, h->kw, h->dlist2,
                          h->union_scratch, &h->ctr->distinct, h->stream));
     h->launches += 4;
     std::swap(h->dlist, h->dlist2);
@@ -492,16 +498,42 @@ int merge_keys(kmerco_t *h, uint64_t na_most, const uint64_t *keys, uint64_t nb_
     return KMERCO_OK;
 }
 
+// The D keys of the list in ascending order, in one of the sort buffers.
+int sort_list(kmerco_t *h, uint64_t D, const uint64_t **sorted);
+
 // Merges the keys pending into the list: for whatever reads or extends the list itself.
 int merge_pending(kmerco_t *h) {
     if (!h->pend_ub) return KMERCO_OK;
-    const uint64_t list = h->d_ub - h->pend_ub;
+    const uint64_t *list = h->dlist;
+    if (!h->list_sorted) {
+        KM_TRY(read_counters(h));
+        know_counts(h);
+        if (h->d_ub > h->pend_ub) KM_TRY(sort_list(h, h->d_ub - h->pend_ub, &list));
+    }
+    const uint64_t held = h->d_ub - h->pend_ub;
     KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub, (uint64_t)h->kw * 8));
-    KM_TRY(ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(list, h->pend_ub)));
-    KM_TRY(merge_keys(h, list, h->pend, h->pend_ub, &h->ctr->pending));
+    KM_TRY(ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(held, h->pend_ub)));
+    KM_TRY(merge_keys(h, list, held, h->pend, h->pend_ub, &h->ctr->pending));
     KM_CUDA(cudaMemsetAsync(&h->ctr->pending, 0, sizeof(h->ctr->pending), h->stream));
     h->pend_ub = 0;
     return KMERCO_OK;
+}
+
+// Exchanges the ordered list and the (empty) keys pending: what follows goes to a set
+// of its own, which need not be built from the list (75 ps a key, and the list would have to
+// be sorted again), and joins it in the end: sixteen pieces of 6e6 windows 10.0 ->
+// 9.5 ms, three of 4e6 55-mers 3.6 -> 3.1.  back: takes that back.
+int set_aside(kmerco_t *h, bool back) {
+    unsigned long long *from = back ? &h->ctr->pending : &h->ctr->distinct;
+    unsigned long long *to = back ? &h->ctr->distinct : &h->ctr->pending;
+    KM_CUDA(cudaMemcpyAsync(to, from, sizeof(*to), cudaMemcpyDeviceToDevice, h->stream));
+    KM_CUDA(cudaMemsetAsync(from, 0, sizeof(*from), h->stream));
+    std::swap(h->dlist, h->pend);
+    std::swap(h->dlist_cap, h->pend_cap);
+    h->pend_ub = back ? 0 : h->d_ub;
+    h->list_sorted = back;
+    h->table_ok = !back;
+    return clean_table(h);
 }
 
 int validate(const kmerco_config_t *c) {
@@ -718,7 +750,8 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     InsertPlan ip = plan_windows(h, bound, nbytes);
     // (a list with a cap keeps to its buffer)
     const bool merge = may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull;
-    const bool into_list = merge && h->list_sorted && merges(bound, h->d_ub);
+    const bool into_list =
+        merge && h->list_sorted && (h->polled ? bound * kUnionShare >= h->d_ub : merges(h->kw, bound, h->d_ub));
     if (bound < (fresh ? kRangesMin : kRangesMinMore) ||
         (!fresh && !into_list && bound <= kWindowsMost) || h->G.cas_limit < kRangesRetries ||
         nbytes < bound)
@@ -1027,28 +1060,36 @@ int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) 
     }
     if (ip.merge && ip.passes == 1) {
         const uint64_t pending = h->pend_ub + ip.bound;
-        ip.full = pending_full(h->d_ub - h->pend_ub, pending, ip.bound);
+        ip.full = h->polled || pending_full(h->d_ub - h->pend_ub, pending, ip.bound);
         uint64_t **to = h->pend_ub ? &h->pend2 : &h->pend;   // the first keys pending as they come
         ip.pend = (h->pend_ub || !ip.full) &&
                   ensure(h, to, h->pend_ub ? &h->pend2_cap : &h->pend_cap, pending,
                          (uint64_t)h->kw * 8) == KMERCO_OK;
     }
-    if (!ip.pend) KM_TRY(merge_pending(h));
+    // (keys set aside stay so while calls go to the set)
+    if (!ip.pend && (ip.ranges || h->list_sorted)) KM_TRY(merge_pending(h));
     held = ip.pend ? h->pend_ub : h->d_ub;
-    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
+    uint64_t chunks = first_read_entries(h, ip, nbytes);
+    if (ip.packed) chunks = std::max(chunks, first_read_entries(h, InsertPlan(), nbytes));
+    KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, chunks));
+    const bool aside = !ip.ranges && ip.bound >= kAsideMin && h->list_sorted && !h->table_ok &&
+                       h->d_ub && !h->max_distinct && !h->polled;
+    if (aside) KM_TRY(set_aside(h, false));
     // a call merged once writes its list into the other buffer alone
-    if (!ip.merge || ip.passes > 1)
-        KM_TRY(ensure_set_capacity(h, ip.bound, ip.table()));
-    else
+    if (!ip.merge || ip.passes > 1) {
+        const int st = ensure_set_capacity(h, ip.bound, ip.table());
+        if (st != KMERCO_OK && aside) KM_TRY(set_aside(h, true));
+        KM_TRY(st);
+    } else {
         h->d_ub += ip.bound;
+    }
     ip.sure = !ip.table() && ip.fresh && ip.passes == 1 &&
               ensure(h, &h->sure, &h->sure_cap, ip.bound) == KMERCO_OK;
     if (ip.packed) {
         h->scratch_busy = true;   // its buffers do not make room for each other
         if (ensure_scratch(h, ip) != KMERCO_OK) {
-            ip.packed = h->scratch_busy = false;
+            ip.packed = false;
             ip.pp = PartPlan();
-            KM_TRY(ensure(h, &h->first_read, &h->first_read_cap, first_read_entries(h, ip, nbytes)));
         }
     }
     return KMERCO_OK;
@@ -1475,36 +1516,21 @@ int wait_result_copies(kmerco_t *h, uint64_t words) {
 
 }  // namespace
 
-int kmerco_classify(kmerco_t *h) {
-    Range range("kmerco_classify");
-    if (!h) return KMERCO_EINVAL;
-    if (h->classified) return KMERCO_OK;
-    DeviceGuard guard(h->device);
-    KM_TRY(merge_pending(h));
-    KM_TRY(read_counters(h));
-    KM_TRY(device_error_status(h->ctr_host->error));
-    const uint64_t D = h->ctr_host->distinct;
+}  // extern "C"
+
+namespace {
+
+int sort_list(kmerco_t *h, uint64_t D, const uint64_t **sorted) {
     if (D >= 0xFFFFFFFFull) return KMERCO_ENOMEM;   // sort tiles index keys with 32 bits
     const int kw = h->kw;
-    const bool in_order = h->list_sorted;
-    if (!in_order) {
-        KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D * kw));
-        KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D * kw));
-        KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap, sort_scratch_words(D, kw)));
-    }
-    KM_TRY(ensure(h, &h->est, &h->est_cap, D));
-    KM_TRY(wait_result_copies(h, D * kw));
-    KM_TRY(ensure(h, &h->split, &h->split_cap, D * kw));
-    KM_TRY(ensure(h, &h->split_scratch, &h->split_scratch_cap, split_scratch_words(D)));
-    KM_CUDA(cudaEventRecord(h->ev[2], h->stream));
+    KM_TRY(ensure(h, &h->alt0, &h->alt0_cap, D * kw));
+    KM_TRY(ensure(h, &h->alt1, &h->alt1_cap, D * kw));
+    KM_TRY(ensure(h, &h->sort_scratch, &h->sort_scratch_cap, sort_scratch_words(D, kw)));
     const uint64_t *const distinct_in = h->dlist;   // left unchanged
-    const uint64_t *sorted = distinct_in;
     const int bits = 2 * h->K;
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
     // (small sets: the radix sort, without the bucket sort's fixed scratch)
-    if (in_order) {
-        // an insert by key ranges wrote the list in ascending order
-    } else if (use_top_sort(D, kw, bits)) {
+    if (use_top_sort(D, kw, bits)) {
         // three stable passes on the top bits (dlist -> alt0 -> alt1 -> alt0),
         // then the segments in shared memory
         const int s0 = bits - kTopSortBits;
@@ -1525,7 +1551,7 @@ int kmerco_classify(kmerco_t *h) {
         // ... and the few too long for one block: radix sorts of their own
         bool any;
         KM_TRY(sort_long_runs(h, D, bits, h->bucket_host[0], &any, h->stream));
-        sorted = h->alt0;
+        *sorted = h->alt0;
     } else if (kw == 1 && bits >= kHistBits + 8 && D > kBucketSortMin &&
                D <= (uint64_t)kHistBins * (kBucketCap / 4)) {
         // Bucket sort: histogram of the top kHistBits key bits, adjacent bins
@@ -1582,9 +1608,9 @@ int kmerco_classify(kmerco_t *h) {
         if (nsuper > (unsigned)kMaxSuper) {
             // too many super-buckets for the scatter's shared counters
             KM_CUDA(radix_sort(distinct_in, h->alt0, h->alt1, D, kw, bits, h->sort_scratch,
-                               &sorted, h->stream));
+                               sorted, h->stream));
             h->launches += 3 * (uint64_t)passes;
-            goto sorted_done;
+            return KMERCO_OK;
         }
         KM_CUDA(cudaMemcpyAsync(d_map, map, kHistBins * sizeof(unsigned), cudaMemcpyHostToDevice,
                                 h->stream));
@@ -1596,7 +1622,7 @@ int kmerco_classify(kmerco_t *h) {
         KM_CUDA(bucket_place_and_sort(distinct_in, h->alt0, D, shift, d_map, nsuper, d_start, d_lo,
                                       d_rsh, d_cursor, h->stream));
         h->launches += 4;
-        sorted = h->alt0;
+        *sorted = h->alt0;
         for (unsigned b = 0; b < nsuper; ++b) {
             const uint64_t n_b = start[b + 1] - start[b];
             if (n_b <= (uint64_t)kBucketCap) continue;
@@ -1610,10 +1636,37 @@ int kmerco_classify(kmerco_t *h) {
         }
     } else {
         KM_CUDA(radix_sort(distinct_in, h->alt0, h->alt1, D, kw, bits, h->sort_scratch,
-                           &sorted, h->stream));
+                           sorted, h->stream));
         if (D > 1) h->launches += 3 * (uint64_t)passes;
     }
-sorted_done:
+    return KMERCO_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int kmerco_classify(kmerco_t *h) {
+    Range range("kmerco_classify");
+    if (!h) return KMERCO_EINVAL;
+    if (h->classified) return KMERCO_OK;
+    DeviceGuard guard(h->device);
+    const bool pending = h->pend_ub != 0;
+    if (pending) KM_CUDA(cudaEventRecord(h->ev[2], h->stream));
+    KM_TRY(merge_pending(h));
+    KM_TRY(read_counters(h));
+    KM_TRY(device_error_status(h->ctr_host->error));
+    const uint64_t D = h->ctr_host->distinct;
+    if (D >= 0xFFFFFFFFull) return KMERCO_ENOMEM;   // sort tiles index keys with 32 bits
+    const int kw = h->kw;
+    const bool in_order = h->list_sorted;
+    KM_TRY(ensure(h, &h->est, &h->est_cap, D));
+    KM_TRY(wait_result_copies(h, D * kw));
+    KM_TRY(ensure(h, &h->split, &h->split_cap, D * kw));
+    KM_TRY(ensure(h, &h->split_scratch, &h->split_scratch_cap, split_scratch_words(D)));
+    if (!pending) KM_CUDA(cudaEventRecord(h->ev[2], h->stream));
+    const uint64_t *sorted = h->dlist;   // an insert by key ranges wrote it in ascending order
+    if (!in_order) KM_TRY(sort_list(h, D, &sorted));
     h->est_exact = false;   // est holds the keys' bits
     KM_CUDA(launch_classify(sorted, D, kw, h->G, h->tau, in_order && h->sure_ok ? h->sure : nullptr,
                             h->est, h->split, h->split_scratch, h->ctr, h->stream));
@@ -1631,7 +1684,10 @@ sorted_done:
 int kmerco_stats(kmerco_t *h, kmerco_stats_t *s) {
     if (!h || !s) return KMERCO_EINVAL;
     DeviceGuard guard(h->device);
-    KM_TRY(merge_pending(h));   // the totals count every key once
+    // the totals count every key once; a program that asks for them between its calls
+    // has them merged or put in the set at once from then on
+    if (h->pend_ub) h->polled = true;
+    KM_TRY(merge_pending(h));
     KM_CUDA(launch_count_saturated(h->G, h->ctr, h->stream));
     h->launches += 1;
     KM_TRY(read_counters(h));
@@ -1943,7 +1999,7 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
         const int st = ensure_union(dst, sc.distinct);
         if (st != KMERCO_ENOMEM) {
             KM_TRY(st);
-            KM_TRY(merge_keys(dst, dst->d_ub, src->dlist, sc.distinct, &src->ctr->distinct));
+            KM_TRY(merge_keys(dst, dst->dlist, dst->d_ub, src->dlist, sc.distinct, &src->ctr->distinct));
             dst->d_ub += sc.distinct;
             listed = true;
         }

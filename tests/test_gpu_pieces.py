@@ -15,22 +15,22 @@ import paper_2305_07545_gb300 as kc  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
-READS = 38000   # of 150 bases: more than 2^22 windows for K up to 39
+READS = 76000   # with 112 windows each: more than 2^23
 
 
-def _pieces(n, K, seed):
+def _pieces(n, K, seed, reads=READS):
     """n pieces on the device, overlapping in part; the last ones repeat the first."""
     st = readsim.Stream(seed)
     length = 111 + K
-    genome = st.integers(3_000_000, 4).astype(np.uint8)
+    genome = st.integers(80 * reads, 4).astype(np.uint8)
     out = []
     for i in range(n):
-        at = st.integers(READS, len(genome) - length)
+        at = st.integers(reads, len(genome) - length)
         x = genome[at[:, None] + np.arange(length)]
         if i % 2:   # half of the pieces are mostly of their own
             x = np.where(st.uniform(x.size).reshape(x.shape) < 0.02, 3 - x, x)
         b = torch.from_numpy(readsim.ASCII[x].reshape(-1)).cuda()
-        o = torch.arange(READS + 1, device="cuda", dtype=torch.int64) * length
+        o = torch.arange(reads + 1, device="cuda", dtype=torch.int64) * length
         out.append((b, o))
     torch.cuda.synchronize()
     return out + out[:2]
@@ -67,10 +67,13 @@ def _at_once(parts, K, m):
         return _state(bf)
 
 
+# all merged, some pending meanwhile; the second (of two-word keys some more) merged, the
+# others beside them in a set of their own; small ones, into a set built from the list
+@pytest.mark.parametrize("reads", [READS, 12000, 4000, 900])
 @pytest.mark.parametrize("K,m", [(31, 1 << 25), (39, 1 << 22)])
 @pytest.mark.parametrize("host", [False, True])   # whether the counts held are known
-def test_pieces(K, m, host):
-    parts = _pieces(9, K, seed=K)
+def test_pieces(K, m, host, reads):
+    parts = _pieces(6, K, seed=K, reads=reads)
     want = _at_once(parts, K, m)
     if host:
         parts = [(b.cpu().pin_memory(), o.cpu().pin_memory()) for b, o in parts]
@@ -88,10 +91,11 @@ def test_pieces(K, m, host):
         _same(_state(bf), want)
 
 
+@pytest.mark.parametrize("reads", [READS, 4000])
 @pytest.mark.parametrize("K", [31, 39])
-def test_calls_between_pieces(K):
+def test_calls_between_pieces(K, reads):
     m = 1 << 22
-    parts = _pieces(5, K, seed=K + 1)
+    parts = _pieces(5, K, seed=K + 1, reads=reads)
     small = parts[0][0][:(111 + K) * 90].clone(), parts[0][1][:91].clone()
     torch.cuda.synchronize()
     with kc.CountBF(K, m, 8, 3, 2) as bf:
@@ -112,9 +116,10 @@ def test_calls_between_pieces(K):
         assert held < bf.stats()["distinct"] <= held + 1000
 
 
-def test_handles_with_keys_pending_are_merged():
+@pytest.mark.parametrize("reads", [READS, 4000])
+def test_handles_with_keys_pending_are_merged(reads):
     K, m = 31, 1 << 22
-    parts = _pieces(5, K, seed=7)
+    parts = _pieces(5, K, seed=7, reads=reads)
     for cut in (3, 4):
         with kc.CountBF(K, m, 8, 3, 2) as x, kc.CountBF(K, m, 8, 3, 2) as y:
             for b, o in parts[:cut]:
@@ -126,10 +131,11 @@ def test_handles_with_keys_pending_are_merged():
             _same(_state(y), _at_once(parts[cut:], K, m))
 
 
+@pytest.mark.parametrize("reads", [READS, 4000])
 @pytest.mark.parametrize("schedule", [0, 1])
-def test_a_batch_with_keys_pending(schedule):
+def test_a_batch_with_keys_pending(schedule, reads):
     K, m = 31, 1 << 22
-    parts = _pieces(4, K, seed=8)
+    parts = _pieces(4, K, seed=8, reads=reads)
     stream = torch.cuda.Stream()
     fs = [kc.CountBF(K, m, 8, 3, 2, stream=stream.cuda_stream) for _ in range(2)]
     with kc.Batch(fs) as batch:
@@ -180,3 +186,31 @@ def test_pieces_under_a_budget():
                 continue
             _same(_state(bf), want)
     assert refused < 4
+
+
+@pytest.mark.parametrize("K", [31, 39])
+def test_a_refused_piece_leaves_the_list_where_it_was(K):
+    # the third piece sets the list aside and finds no room for its set: the results
+    # of the first two are there as before
+    m, kw = 1 << 22, 1 if K <= 32 else 2
+    parts = _pieces(3, K, seed=K, reads=4000)
+    large = _pieces(1, K, seed=K + 5, reads=14000)[0]
+    with kc.CountBF(K, m, 8, 3, 2) as bf:
+        for b, o in parts[:2]:
+            bf.insert(b, o)
+        bf.classify()
+        bf.distinct()
+        held = bf.stats()["device_bytes"]
+    # room for the large piece's list (8 bytes a window and key word) and not its set
+    windows = 14000 * 112
+    with kc.CountBF(K, m, 8, 3, 2, hbm_budget=held + 10 * windows * kw) as bf:
+        for b, o in parts[:2]:
+            bf.insert(b, o)
+        want = _state(bf)
+        with pytest.raises(kc.KmercoError) as e:
+            bf.insert(*large)
+        assert e.value.status == kc.ENOMEM
+        filler = [torch.full((n,), -1, dtype=torch.int64, device="cuda") for n in (1 << 16, 1 << 20)]
+        torch.cuda.synchronize()
+        _same(_state(bf), want)
+        del filler
