@@ -3,7 +3,8 @@
 Long keys with a common beginning (a constant flank, a primer, an adapter) have
 equal 64-bit prefixes and are cut by their low words; ranges that the samples
 say nothing about hold far more keys than a block's table and are counted in
-rounds, in key order and (a further call that goes to the distinct set) in none.
+rounds.  Keys leave the ranges in key order, or in none: so do the later passes of
+a call into a list with a cap, whose keys go to the distinct set.
 """
 import numpy as np
 import pytest
@@ -41,34 +42,40 @@ def test_keys_with_a_common_beginning(K, length, flank, n, forward_only):
     check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
 
 
+def _unordered(windows, passes):
+    """Options that make the passes after a call's first one unordered (three hashes)."""
+    return dict(max_distinct=1 << 28, pass_codes=3 * (windows // passes + 1))
+
+
 @pytest.mark.parametrize("K", [40, 55])
-@pytest.mark.parametrize("first", [3000, 14000])   # merged into the list, put in the set
-def test_a_further_call_with_a_common_beginning(K, first):
-    parts = [readsim.random_reads(first, 150, 150, seed=K), _flanked(9000, 72, 40, seed=K + 1),
+@pytest.mark.parametrize("second", ["call", "passes"])   # merged into the list, put in the set
+def test_a_further_part_with_a_common_beginning(K, second):
+    parts = [readsim.random_reads(3000, 150, 150, seed=K), _flanked(9000, 72, 40, seed=K + 1),
              _flanked(9000, 72, 40, seed=K + 1)]
-    g = _count(parts, K, 1 << 22, 8, 3, 2)
-    check(g, *_join(parts), K, 8, 3, 2, cross_check=False)
+    b, o = _join(parts)
+    if second == "call":
+        g = _count(parts, K, 1 << 22, 8, 3, 2)
+    else:
+        windows = 3000 * (151 - K) + 18000 * (73 - K)
+        g = _count([(b, o)], K, 1 << 22, 8, 3, 2, **_unordered(windows, 4))
+    check(g, b, o, K, 8, 3, 2, cross_check=False)
 
 
 @pytest.mark.parametrize("K,forward_only", [(21, False), (32, True), (33, False), (55, False),
                                             (64, True)])
-@pytest.mark.parametrize("first", [0, 14000])   # in key order, then in none
-def test_ranges_that_the_samples_miss(K, forward_only, first):
+@pytest.mark.parametrize("unordered", [False, True])
+def test_ranges_that_the_samples_miss(K, forward_only, unordered):
     # 25,000 windows among 6e7 bases of reads too short to hold one: the samples,
-    # spread over the bases, meet next to none of them, so a range has thousands of
-    # keys; of a further call every window comes seven times
+    # spread over the bases, meet next to none of them, so a range has thousands of keys
     st = readsim.Stream(K)
     some = _bases(st, 250, K + 99)
     some[0] = ord("T")   # forward strand: the largest key there is
-    if first:
-        some = np.tile(some, (7, 1))
     short = _bases(st, 3_000_000, 20)
-    cut = len(short) // 3
-    parts = [_even(short[:cut]), _even(some), _even(short[cut:])]
-    call = _join(parts)
-    calls = [readsim.random_reads(first, 150, 150, seed=K), call] if first else [call]
-    g = _count(calls, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
-    check(g, *_join(calls), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
+    cut = 3 * len(short) // 4   # in the second of two passes
+    b, o = _join([_even(short[:cut]), _even(some), _even(short[cut:])])
+    kw = _unordered(25000, 2) if unordered else {}
+    g = _count([(b, o)], K, 1 << 22, 8, 3, 2, forward_only=forward_only, **kw)
+    check(g, b, o, K, 8, 3, 2, forward_only=forward_only, cross_check=False)
 
 
 def _insert_ms(b, o, K, m=1 << 24):
@@ -111,9 +118,8 @@ def test_keys_held_by_very_many_windows(K, forward_only, n):
     parts = [_even(x[_shuffled(n, st)])]
     g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
     check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
-    # the same as a further call that goes to the set
-    parts = [readsim.random_reads(10 * n, 150, 150, seed=K)] + parts
-    g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only)
+    g = _count(parts, K, 1 << 22, 8, 3, 2, forward_only=forward_only,
+               **_unordered(n * (151 - K), 3))
     check(g, *_join(parts), K, 8, 3, 2, forward_only=forward_only, cross_check=False)
 
 
