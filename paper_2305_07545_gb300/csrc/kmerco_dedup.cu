@@ -419,11 +419,15 @@ __device__ __forceinline__ Key<2> revcomp(const Key<2> &f, int K) {
 }
 
 // ----------------------------------------------------------- 2. splitters
+// Equal prefixes among a level's splitters, or a tile's samples, from which on the low
+// words of two-word keys decide too.
+constexpr unsigned kCrowd = 5;
+
 constexpr unsigned kSampleTile = 1024;   // samples a block sorts
 
 // The keys at n random valid window starts of the pass's `span` bases (a few tries
 // each), as sorted tiles of kSampleTile: samples has their prefixes, samples_lo the
-// low words of two-word keys (0 in tiles of different prefixes); the last one is filled up with
+// low words of two-word keys (0 in tiles without more than kCrowd samples of a prefix); the last one is filled up with
 // all ones.  Whole prefixes: copies of a repeat have long beginnings in common,
 // and cutting by their top 31 bits left more than twice as many windows in some
 // ranges (dedup_big_kernel 2.8 instead of 1.8 ms for 3.8e8 two-word windows).
@@ -453,13 +457,15 @@ __global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int can
     uint64_t v[1] = {p}, low = 0;
     block_sort<1>(v, (uint64_t *)xch);
     if constexpr (KW == 2) {
-        // equal prefixes in the tile, which are rare: in the order of the whole keys
+        // many equal prefixes in the tile, which is rare: in the order of the whole keys
         uint64_t *const seen = (uint64_t *)xch;
+        const unsigned tid = threadIdx.x;
         __syncthreads();
-        seen[threadIdx.x] = v[0];
+        seen[tid] = v[0];
         __syncthreads();
-        const bool same = threadIdx.x && v[0] != ~0ull && seen[threadIdx.x - 1] == v[0];
+        const bool same = tid >= kCrowd && v[0] != ~0ull && seen[tid - kCrowd] == v[0];
         if (__syncthreads_or(same)) {
+            if (tid == 0) atomicOr(&meta->crowd, 1u << blockIdx.x);
             Cut2 w[1] = {Cut2{p, found ? key.lo : ~0ull}};
             block_sort<1>(w, xch);
             v[0] = w[0].p;
@@ -489,7 +495,8 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
     for (unsigned i = tid; i < n / 2; i += 1024) s2[i] = ((const ulonglong2 *)samples)[i];
     __syncthreads();
     const uint64_t v = s[own * kSampleTile + tid];
-    const uint64_t low = KW == 2 ? samples_lo[own * kSampleTile + tid] : 0;
+    const unsigned crowd = KW == 2 ? meta->crowd : 0;   // without, all low words are 0
+    const uint64_t low = (crowd >> own) & 1u ? samples_lo[own * kSampleTile + tid] : 0;
     unsigned rank = tid;
     for (unsigned c = 0; c < n / kSampleTile; ++c) {
         if (c == own) continue;
@@ -500,10 +507,11 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
             if (s[t0 + at + step - 1] < v) at += step;
         if (s[t0 + at] < v) ++at;
         if (at < kSampleTile && s[t0 + at] == v) {   // and those of the same prefix in front
+            const bool lows = KW == 2 && ((crowd >> c | crowd >> own) & 1u);
             unsigned hi = kSampleTile;
             while (at < hi) {
                 const unsigned m = (at + hi) / 2;
-                const uint64_t w = KW == 2 && s[t0 + m] == v ? samples_lo[t0 + m] : low;
+                const uint64_t w = lows && s[t0 + m] == v ? samples_lo[t0 + m] : low;
                 if (s[t0 + m] == v && (w < low || (w == low && c < own)))
                     at = m + 1;
                 else
@@ -519,7 +527,7 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
              k < n_ranges && k * valid / n_ranges == r; ++k)
             if (k) {
                 spl[k - 1] = v;
-                if (KW == 2) spl_lo[k - 1] = low;
+                if (KW == 2 && crowd) spl_lo[k - 1] = low;
             }
     }
     __threadfence();
@@ -528,16 +536,21 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    uint64_t f, f_lo;   // all ones at the last of the n: what find_range stops at
-    const bool equal = part_equal<KW>(
-        [&](unsigned i, uint64_t &p, uint64_t &low) {
-            p = __ldcg(spl + i);
-            if (KW == 2) low = __ldcg(spl_lo + i);
-        },
-        tid, valid ? n_ranges - 1 : 0, f, f_lo, K);
+    uint64_t f = ~0ull, f_lo = ~0ull;   // of the last of the n: what find_range stops at
+    bool equal = false, tie = false;
+    if (KW == 1 || crowd) {
+        equal = part_equal<KW>(
+            [&](unsigned i, uint64_t &p, uint64_t &low) {
+                p = __ldcg(spl + i);
+                if (KW == 2) low = __ldcg(spl_lo + i);
+            },
+            tid, valid ? n_ranges - 1 : 0, f, f_lo, K);
+    } else if (valid && tid + 1 < n_ranges) {
+        f = __ldcg(spl + tid);
+        f_lo = 0;
+    }
     __syncthreads();
-    bool tie = false;
-    if (KW == 2 && valid) {
+    if (KW == 2 && valid && crowd) {
         tie = shares_prefix(s, tid, n_ranges - 1, f) || equal;
         if (!tie && tid + 1 < n_ranges) f_lo = 0;
     }
@@ -805,7 +818,6 @@ __global__ void __launch_bounds__(1024) tile_map_kernel(const uint32_t *totals, 
 // same shared memory.  (A prefix of fewer ranges' windows is left together, to
 // dedup_big_kernel's few rounds: 2.8e8 windows of copied repeats have many of them,
 // and sorting whole keys at two equal ones took 910 instead of 500 us there.)
-constexpr unsigned kCrowd = 5;
 template <int KW, int E>
 __global__ void __launch_bounds__(1024) fine_splitters_kernel(RefineArgs x, int K, unsigned n,
                                                               uint64_t last) {

@@ -37,7 +37,7 @@ struct DedupMeta {
     unsigned sampled;      // samples that are keys
     unsigned ranked;       // blocks of rank_kernel that are done
     unsigned n_big;        // ranges left to dedup_big_kernel
-    unsigned pad;
+    unsigned crowd;        // sample tiles that have the low words of two-word keys
 };
 
 struct TileMap {
