@@ -579,10 +579,12 @@ bool use_partitioned(const kmerco_t *h, uint64_t bound, bool staged) {
     // between the two (4e6 distinct windows of four hashes into 2^25 cells: 0.84 ms by
     // random updates, 0.54 partitioned; 1e6: 0.26 and 0.27).
     const uint64_t U = bound * (uint64_t)h->nhash, W = h->G.words;
-    // Its further launches cost as much as it saves on 3e6 increments.
-    const uint64_t least = W <= (1ull << 24) ? W / (staged ? 4 : 2)
+    // Below 2^22 cells its further launches weigh against the few updates that
+    // miss; 1e6 staged increments pay for theirs.
+    const uint64_t least = W <= (1ull << 22)   ? W
+                           : W <= (1ull << 24) ? W / (staged ? 4 : 2)
                            : W <= (1ull << 25) ? W / (staged ? 8 : 4) : W / (staged ? 12 : 9);
-    return able && W >= (1ull << 17) && U >= std::max<uint64_t>(least, 3u << 20);
+    return able && W >= (1ull << 17) && U >= least && (!staged || U >= (1ull << 20));
 }
 
 // Trial division; n is at most about 2^24 here.
