@@ -1426,6 +1426,7 @@ struct __align__(16) DedupSmem {
     unsigned src[kDedupThreads];     // runs: first key
     unsigned pos[kDedupThreads + 1]; // and place among the range's windows
     unsigned nd, over, crowded, ones, out0, cut;
+    RangeCut cut_by;
     Key<KW> pivot;
     Key<KW> bounds[kBoundsMax];      // the rounds' ends to come, the nearest last
 };
@@ -1494,14 +1495,22 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
     for (unsigned q = blockIdx.x; q < n_big; q += gridDim.x) {
         const unsigned g = x.big[q];
         RangeRuns cur;
+        if (tid == 0) S.cut_by = range_cut<KW>(x, g, K, last);
         cur.load(x, g);
-        const RangeCut cut = range_cut<KW>(x, g, K, last);
-        unsigned n_all = cur.n;   // windows of the range
-        for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
-            n_all += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
-        block_exclusive_scan<unsigned, NT>(n_all, n_all);
-        if (cut.pure) {   // one key, however many windows
+        unsigned n_all;   // windows of the range
+        const unsigned pre0 = block_exclusive_scan<unsigned, NT>(cur.n, n_all);
+        const unsigned m0 = n_all;
+        if (cur.n_runs > NT) {
+            unsigned n = 0;
+            for (unsigned r = NT + tid; r < cur.n_runs; r += NT)
+                n += (unsigned)cur.row0[(uint64_t)cur.n_runs + r] - cur.row0[r];
+            block_exclusive_scan<unsigned, NT>(n, n);
+            n_all += n;
+        }
+        if (S.cut_by.pure) {   // one key, however many windows
+            __syncthreads();   // every thread has seen it
             if (tid == 0) {
+                const RangeCut &cut = S.cut_by;
                 const unsigned at = atomicAdd(&x.meta->out_cursor, 1u);
                 Key<KW> k;
                 k.lo = KW == 1 ? cut.lo : cut.lo2;
@@ -1515,14 +1524,13 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
             }
             continue;
         }
-        // the range's place in the output: room for all its windows
-        if (tid == 0 && x.ordered) x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n_all);
         unsigned done = 0;    // distinct keys written
         unsigned depth = 0;   // bounds held
         Key<KW> lo, hi;
         lo.lo = lo.hi = 0;
         hi = lo;
         bool from = false, until = false;   // whether lo and hi bound this round
+        bool first = true;
         for (bool again = true; again;) {
             __syncthreads();   // the last round's table is cleared
             if (tid == 0) S.nd = S.over = S.crowded = S.ones = 0;
@@ -1530,9 +1538,11 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
             bool over = false;   // the same in every thread
             for (unsigned r0 = 0; r0 < cur.n_runs && !over; r0 += NT) {
                 RangeRuns seg = cur;
-                if (r0) seg.load_run(x, r0 + tid);
-                unsigned m;
-                const unsigned pre = block_exclusive_scan<unsigned, NT>(seg.n, m);
+                unsigned m = m0, pre = pre0;
+                if (r0) {
+                    seg.load_run(x, r0 + tid);
+                    pre = block_exclusive_scan<unsigned, NT>(seg.n, m);
+                }
                 S.src[tid] = seg.src;
                 S.pos[tid] = pre;
                 if (tid == 0) S.pos[NT] = m;
@@ -1542,6 +1552,12 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                     const unsigned p1 = min(m, p0 + (unsigned)kDedupStage<KW>);
                     gather_runs<KW, NT>(x.in, S.src, S.pos, nr, p0, p1, S.stage,
                                         KW == 2 ? S.ref : nullptr);
+                    if (first) {   // beside the first copies
+                        first = false;
+                        // the range's place in the output: room for all its windows
+                        if (tid == 0 && x.ordered)
+                            x.places[g] = S.out0 = atomicAdd(&x.meta->out_cursor, n_all);
+                    }
                     copies_done();
                     __syncthreads();
                     for (unsigned i = tid; i < p1 - p0; i += NT) {
@@ -1569,6 +1585,7 @@ __global__ void __launch_bounds__(kDedupThreads, 3) dedup_big_kernel(DedupArgs x
                 }
                 again = until;
             } else if (!over) {
+                const RangeCut cut = S.cut_by;
                 for (unsigned i = tid; i < nd; i += NT) {
                     const Key<KW> k = table_key(S, x.in, S.list[i]);
                     atomicAdd(&S.sub[cut_of(cut, k, K)], 1u);
