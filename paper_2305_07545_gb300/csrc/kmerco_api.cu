@@ -1769,6 +1769,7 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
     if (!h || (!keys && n)) return KMERCO_EINVAL;
     if (n == 0) return KMERCO_OK;
     DeviceGuard guard(h->device);
+    KM_TRY(merge_pending(h));   // (it may use the sort buffers)
     const uint64_t words = n * h->kw;
     const uint64_t *d_keys = keys;
     if (!is_device_ptr(keys)) {
@@ -1780,7 +1781,6 @@ int kmerco_add_distinct(kmerco_t *h, const uint64_t *keys, uint64_t n) {
         KM_CUDA(cudaMemcpyAsync(*stage, keys, words * 8, cudaMemcpyHostToDevice, h->stream));
         d_keys = *stage;
     }
-    KM_TRY(merge_pending(h));
     KM_TRY(ensure_set_capacity(h, n, true));
     KM_CUDA(launch_reinsert(d_keys, n, nullptr, nullptr, h->kw, h->table, h->cap, set_tag(h),
                             h->dlist, h->dlist_cap, h->ctr, h->G.probe_limit, h->stream));

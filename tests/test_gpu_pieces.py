@@ -107,13 +107,19 @@ def test_calls_between_pieces(K, reads):
                 _same(_state(bf), _at_once(parts[:n], K, m))
         bf.insert(*small)     # to the set
         _same(_state(bf), _at_once(parts + [small], K, m))
-        bf.reset()
+    with kc.CountBF(K, m, 8, 3, 2) as bf:
         for b, o in parts[:3]:
             bf.insert(b, o)
-        extra = np.arange(1000 * (2 if K > 32 else 1), dtype=np.uint64)
-        held = _at_once(parts[:3], K, m)[0][2]
+        kw = 2 if K > 32 else 1
+        extra = np.arange(1000 * kw, dtype=np.uint64) * np.uint64(3)   # host keys, staged
         kc.kmerco_add_distinct(bf.h, extra, 1000)
-        assert held < bf.stats()["distinct"] <= held + 1000
+        bf.classify()
+        got = bf.distinct()[0].reshape(-1, kw)
+    keys = np.concatenate([_at_once(parts[:3], K, m)[1][0].reshape(-1, kw), extra.reshape(-1, kw)])
+    order = np.lexsort(keys.T)
+    keys = keys[order]
+    new = np.concatenate([[True], (keys[1:] != keys[:-1]).any(axis=1)])
+    assert np.array_equal(got, keys[new])
 
 
 @pytest.mark.parametrize("reads", [READS, 4000])
@@ -190,21 +196,21 @@ def test_pieces_under_a_budget():
 
 @pytest.mark.parametrize("K", [31, 39])
 def test_a_refused_piece_leaves_the_list_where_it_was(K):
-    # the third piece sets the list aside and finds no room for its set: the results
-    # of the first two are there as before
+    # a large third piece finds no room, first by ranges, then for the set of its own
+    # beside the list set aside: the results of the first two are there as before
     m, kw = 1 << 22, 1 if K <= 32 else 2
-    parts = _pieces(3, K, seed=K, reads=4000)
-    large = _pieces(1, K, seed=K + 5, reads=14000)[0]
+    parts = _pieces(2, K, seed=K, reads=4000)[:2]
+    large = _pieces(1, K, seed=K + 5, reads=60000)[0]
     with kc.CountBF(K, m, 8, 3, 2) as bf:
-        for b, o in parts[:2]:
+        for b, o in parts:
             bf.insert(b, o)
         bf.classify()
         bf.distinct()
         held = bf.stats()["device_bytes"]
-    # room for the large piece's list (8 bytes a window and key word) and not its set
-    windows = 14000 * 112
-    with kc.CountBF(K, m, 8, 3, 2, hbm_budget=held + 10 * windows * kw) as bf:
-        for b, o in parts[:2]:
+    # the large piece's list and set alone take 160 MB a key word, twice what is held
+    assert 24 * 60000 * 112 * kw > 2 * held
+    with kc.CountBF(K, m, 8, 3, 2, hbm_budget=held + (4 << 20)) as bf:
+        for b, o in parts:
             bf.insert(b, o)
         want = _state(bf)
         with pytest.raises(kc.KmercoError) as e:
