@@ -252,7 +252,7 @@ __global__ void query_kernel(const uint64_t *keys, uint64_t n, int K, Geometry G
 // decides "erroneous" and the key's other counters are not read.  A key whose
 // `sure` byte is set has more than tau windows in this countBF, which never
 // underestimates: it is trustworthy without a look at its counters, which would
-// all k_h have to be read; the erroneous ones, 86% of the keys, cost one read each.
+// all k_h have to be read; an erroneous one mostly costs one read.
 // With the split on bits after it, classifying 2.1e8 keys against a 4 GiB countBF
 // takes 5.23 ms; a query of all counters, the split on its estimates, took 9.35.
 //

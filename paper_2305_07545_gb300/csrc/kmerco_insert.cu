@@ -30,7 +30,8 @@
 // memory instead: pieces of 2.5e6 windows into 2^18 cells then take 238 us each
 // with their increments, 282 with a compare-and-swap per window and hash.
 //
-// Partitioned update (at most 2^30 cells): emit_kernel has appended the increments as 32-bit codes to 64 coarse countBF regions;
+// Partitioned update (at most 2^30 cells): emit_kernel (kmerco_dedup.cu) has
+// appended the increments as 32-bit codes to 64 coarse countBF regions;
 // repartition_kernel splits every region into slices, and one block per
 // slice applies its increments in shared memory: apply_count_kernel
 // (alpha <= 15) sums them in 32-bit lanes and adds the sums with saturation

@@ -12,7 +12,7 @@ namespace countbf {
 constexpr uint64_t kEmptyKey = ~0ull;      // empty slot of the distinct-key set
 constexpr int kChunk = 2048;               // window starts per insert work unit
 constexpr int kSmallChunk = 512;           // the same for inputs too small to fill the GPU
-constexpr int kPartMaxHash = 4;            // hashes the partitioned update groups at a time
+constexpr int kPartMaxHash = 4;            // hashes up to which update_mode 2 is accepted
 constexpr int kCoarseBins = 64;            // coarse countBF regions of the partitioned design
 constexpr int kSliceShift = 13;            // 2^13 cells (64 KiB) per shared-memory slice
 constexpr int kMaxCoarseShift = 24;        // cell-in-region bits of an increment code
