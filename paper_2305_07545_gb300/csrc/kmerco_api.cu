@@ -471,14 +471,19 @@ void know_counts(kmerco_t *h) {
     h->d_ub = list + h->pend_ub;
 }
 
-// Room for the union of what is held and at most `add` more keys.
-int ensure_union(kmerco_t *h, uint64_t add) {
-    // a bound of what is held will do while the list is small; for a large one the
-    // call waits to learn its length
+// A bound of what is held will do for a union while the list is small; for a large one
+// the call waits to learn its length.
+int learn_held(kmerco_t *h, uint64_t add) {
     if (h->d_ub && h->d_ub + add > h->dlist2_cap && (h->d_ub + add) * h->kw > (1ull << 28)) {
         KM_TRY(read_counters(h));
         know_counts(h);
     }
+    return KMERCO_OK;
+}
+
+// Room for the union of what is held and at most `add` more keys.  (Merging what is
+// pending exchanges the list's two places: that comes before.)
+int ensure_union(kmerco_t *h, uint64_t add) {
     KM_TRY(ensure(h, &h->dlist2, &h->dlist2_cap, h->d_ub + add, (uint64_t)h->kw * 8));
     // several passes: each one's list into what is held by then
     return ensure(h, &h->union_scratch, &h->union_scratch_cap, union_scratch_words(h->d_ub + add, add));
@@ -1053,13 +1058,7 @@ int ensure_scratch(kmerco_t *h, const InsertPlan &ip) {
 // meets, at most.
 int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) {
     if (ip.ranges) KM_TRY(ensure_scratch(h, ip));
-    if (ip.merge) {
-        const int st = ensure_union(h, ip.bound);
-        if (st == KMERCO_ENOMEM)
-            ip.merge = false;   // the distinct set then
-        else
-            KM_TRY(st);
-    }
+    if (ip.merge) KM_TRY(learn_held(h, ip.bound));
     if (ip.merge && ip.passes == 1) {
         const uint64_t pending = h->pend_ub + ip.bound;
         ip.full = h->polled || pending_full(h->d_ub - h->pend_ub, pending, ip.bound);
@@ -1070,6 +1069,15 @@ int secure_insert(kmerco_t *h, InsertPlan &ip, uint64_t nbytes, uint64_t &held) 
     }
     // (keys set aside stay so while calls go to the set)
     if (!ip.pend && (ip.ranges || h->list_sorted)) KM_TRY(merge_pending(h));
+    if (ip.merge) {
+        const int st = ensure_union(h, ip.bound);
+        if (st == KMERCO_ENOMEM) {   // the distinct set then
+            ip.merge = ip.pend = false;
+            KM_TRY(merge_pending(h));
+        } else {
+            KM_TRY(st);
+        }
+    }
     held = ip.pend ? h->pend_ub : h->d_ub;
     uint64_t chunks = first_read_entries(h, ip, nbytes);
     if (ip.packed) chunks = std::max(chunks, first_read_entries(h, InsertPlan(), nbytes));
@@ -1998,6 +2006,7 @@ int kmerco_merge(kmerco_t *dst, kmerco_t *src) {
         listed = dst->list_sorted = true;
     } else if (ordered && dst->list_sorted && sc.distinct * kUnionShare >= dst->d_ub &&
                dst->d_ub + sc.distinct < 0xFFFFFFFFull) {
+        KM_TRY(learn_held(dst, sc.distinct));
         const int st = ensure_union(dst, sc.distinct);
         if (st != KMERCO_ENOMEM) {
             KM_TRY(st);

@@ -220,3 +220,33 @@ def test_a_refused_piece_leaves_the_list_where_it_was(K):
         torch.cuda.synchronize()
         _same(_state(bf), want)
         del filler
+
+
+@pytest.mark.parametrize("K", [31, 39])
+def test_a_call_of_several_passes_beside_pending_keys(K):
+    # the third piece's keys are pending; the fourth call is all pieces once more, in three
+    # passes, each merged into the list, which takes turns between its two places
+    m = 1 << 22
+    parts = _pieces(2, K, seed=K + 9)
+    whole = _join(parts)
+    with kc.CountBF(K, m, 8, 3, 2, pass_codes=3 * READS * 112 * 4 // 3) as bf:
+        for b, o in parts[:3]:
+            bf.insert(b, o)
+        bf.insert(*whole)
+        _same(_state(bf), _at_once(parts[:3] + [whole], K, m))
+
+
+def test_pieces_without_a_window_that_counts():
+    # pending keys whose count is none: pieces of N between others, all sizes known late
+    K, m = 31, 1 << 22
+    parts = _pieces(3, K, seed=12)
+    empty = [(torch.full_like(b, ord("N")), o) for b, o in parts[:2]]
+    torch.cuda.synchronize()
+    order = [parts[0], parts[1], empty[0], parts[2], empty[1], empty[0], parts[1], parts[2]]
+    want = _at_once(order, K, m)
+    for host in (False, True):
+        use = [(b.cpu().pin_memory(), o.cpu().pin_memory()) for b, o in order] if host else order
+        with kc.CountBF(K, m, 8, 3, 2) as bf:
+            for b, o in use:
+                bf.insert(b, o)
+            _same(_state(bf), want)
