@@ -234,7 +234,10 @@ int kmerco_insert(kmerco_t *h, const char *bases, const uint64_t *offsets, uint6
 int kmerco_classify(kmerco_t *h);
 
 /* Fill *s (host pointer) with the handle's totals.  Synchronises; counts
- * saturated counters on the device.  Errors: EINVAL (NULL), ECUDA. */
+ * saturated counters on the device, and merges the keys that large inserts
+ * keep beside the distinct list until it is read (a handle whose totals are
+ * asked for between such inserts merges them at once from then on).
+ * Errors: EINVAL (NULL), ENOMEM, ECUDA. */
 int kmerco_stats(kmerco_t *h, kmerco_stats_t *s);
 
 /*
