@@ -501,17 +501,21 @@ __global__ void __launch_bounds__(1024) rank_kernel(const uint64_t *samples,
     for (unsigned c = 0; c < n / kSampleTile; ++c) {
         if (c == own) continue;
         const unsigned t0 = c * kSampleTile;
-        unsigned at = 0;   // samples of the tile below v's prefix
+        const bool lows = KW == 2 && ((crowd >> c | crowd >> own) & 1u);
+        // samples of the tile in front of v; with low words, those below its prefix
+        const bool below = c < own && !lows;   // and its equals of earlier tiles
+        unsigned at = 0;
 #pragma unroll
-        for (unsigned step = kSampleTile / 2; step; step >>= 1)
-            if (s[t0 + at + step - 1] < v) at += step;
-        if (s[t0 + at] < v) ++at;
-        if (at < kSampleTile && s[t0 + at] == v) {   // and those of the same prefix in front
-            const bool lows = KW == 2 && ((crowd >> c | crowd >> own) & 1u);
+        for (unsigned step = kSampleTile / 2; step; step >>= 1) {
+            const uint64_t t = s[t0 + at + step - 1];
+            if (t < v || (below && t == v)) at += step;
+        }
+        if (s[t0 + at] < v || (below && s[t0 + at] == v)) ++at;
+        if (lows) {   // and those of the same prefix in front
             unsigned hi = kSampleTile;
             while (at < hi) {
                 const unsigned m = (at + hi) / 2;
-                const uint64_t w = lows && s[t0 + m] == v ? samples_lo[t0 + m] : low;
+                const uint64_t w = s[t0 + m] == v ? samples_lo[t0 + m] : low;
                 if (s[t0 + m] == v && (w < low || (w == low && c < own)))
                     at = m + 1;
                 else
