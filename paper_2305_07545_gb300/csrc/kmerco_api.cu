@@ -758,7 +758,8 @@ InsertPlan plan_insert(const kmerco_t *h, uint64_t bound, uint64_t nbytes, bool 
     // (a list with a cap keeps to its buffer)
     const bool merge = may_merge && !h->max_distinct && h->d_ub + bound < 0xFFFFFFFFull;
     const bool into_list =
-        merge && h->list_sorted && (h->polled ? bound * kUnionShare >= h->d_ub : merges(h->kw, bound, h->d_ub));
+        merge && h->list_sorted &&
+        (h->polled ? bound * kUnionShare >= h->d_ub : merges(h->kw, bound, h->d_ub));
     if (bound < (fresh ? kRangesMin : kRangesMinMore) ||
         (!fresh && !into_list && bound <= kWindowsMost) || h->G.cas_limit < kRangesRetries ||
         nbytes < bound)

@@ -427,10 +427,11 @@ constexpr unsigned kSampleTile = 1024;   // samples a block sorts
 
 // The keys at n random valid window starts of the pass's `span` bases (a few tries
 // each), as sorted tiles of kSampleTile: samples has their prefixes, samples_lo the
-// low words of two-word keys (0 in tiles without more than kCrowd samples of a prefix); the last one is filled up with
-// all ones.  Whole prefixes: copies of a repeat have long beginnings in common,
-// and cutting by their top 31 bits left more than twice as many windows in some
-// ranges (dedup_big_kernel 2.8 instead of 1.8 ms for 3.8e8 two-word windows).
+// low words of two-word keys (0 in tiles without more than kCrowd samples of a
+// prefix); the last tile is filled up with all ones.  Whole prefixes: copies of a
+// repeat have long beginnings in common, and cutting by their top 31 bits left more than
+// twice as many windows in some ranges (dedup_big_kernel 2.8 instead of 1.8 ms for
+// 3.8e8 two-word windows).
 template <int KW>
 __global__ void __launch_bounds__(1024) sample_kernel(PackArgs x, int K, int canonical,
                                                       uint64_t span, unsigned n,
